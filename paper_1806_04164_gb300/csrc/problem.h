@@ -47,6 +47,8 @@ struct Problem {
   int64_t T = 0, E = 0, N = 0;
   int64_t nnz = 0;      // near pair entries
   int64_t nleaf = 0;
+  double h_max = 0;     // longest edge of the mesh
+  double r_max = 0;     // largest distance of a centroid from the origin
   size_t bytes = 0;
   std::vector<void*> allocs;
 
@@ -93,6 +95,7 @@ struct Problem {
   void* coef = nullptr;          // [max_nrhs][T][6] complex (io precision)
   void* coef32 = nullptr;        // [T][6] complex float copy for the MIXED near part
   void* gsgd = nullptr;          // 2 x [max_nrhs][nleaf][5][P/2] antipodal sum / difference leaf patterns
+  size_t gsgd_bytes = 0;         // (the field maps use the same buffer as scratch)
   void* vec = nullptr;           // [N] complex (io precision), adjoint scratch
   void* vec2 = nullptr;          // [N] complex (io precision), single-layer scratch
   void* pot = nullptr;           // [max_nrhs][T][6] far-part potentials (near part too when pot2 is unused)

@@ -541,6 +541,9 @@ static pie_status setup_t(Problem& pr, cudaStream_t st) {
     }
     for (int d = 0; d < 3; ++d) cent[3 * i + d] = m.centroid[3 * tm + d];
     h2[i] = m.h2[tm];
+    pr.h_max = std::max(pr.h_max, std::sqrt(m.h2[tm]));
+    const double* ctr = &m.centroid[3 * tm];
+    pr.r_max = std::max(pr.r_max, std::sqrt(ctr[0] * ctr[0] + ctr[1] * ctr[1] + ctr[2] * ctr[2]));
     area[i] = m.area[tm];
     for (int k = 0; k < 3; ++k) {
       int32_t n = m.tri_edge[3 * tm + k];
@@ -758,7 +761,8 @@ static pie_status setup_t(Problem& pr, cudaStream_t st) {
   }
   const size_t cio = pr.io_f32() ? sizeof(cf) : sizeof(cd);
   const size_t nr = size_t(pr.par.max_nrhs);
-  pr.gsgd = zalloc(pr, sizeof(C2<Rf>) * 2 * nr * size_t(pr.lev[L].nb) * kComp * (P / 2), s);
+  pr.gsgd_bytes = sizeof(C2<Rf>) * 2 * nr * size_t(pr.lev[L].nb) * kComp * (P / 2);
+  pr.gsgd = zalloc(pr, pr.gsgd_bytes, s);
   pr.coef = zalloc(pr, cio * 6 * size_t(T) * nr, s);
   pr.pot = zalloc(pr, cio * 6 * size_t(T) * nr, s);
   pr.pot2 = zalloc(pr, cio * 6 * size_t(T) * nr, s);
