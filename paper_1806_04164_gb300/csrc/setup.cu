@@ -7,6 +7,7 @@
 //  - interpolation filter (degree rescale) and phases.
 #include <cstring>
 #include <cmath>
+#include <type_traits>
 
 #include "device.cuh"
 
@@ -15,166 +16,316 @@ namespace pie {
 constexpr double kFourPi = 4.0 * kPi;
 constexpr int kMaxTau = 30;
 
-// ------------------------------------------------------------ closed forms
-// int_T 1/|r-r'| dS' and int_T (r'-r)/|r-r'| dS' over the flat triangle
-// (v0, v1, v2) (Wilton et al. 1984; Graglia 1993).  With unit normal n, height
-// d = n.(r - v0), per edge a->b: tangent s, outward normal m = s x n,
-// l+ = (b-r).s, l- = (a-r).s, P0 = (a-r).m, R0^2 = P0^2 + d^2,
-// f = ln((R+ + l+)/(R- + l-)):
-//   I1 = sum [P0 f - |d|(atan(P0 l+/(R0^2+|d|R+)) - atan(P0 l-/(R0^2+|d|R-)))]
-//   Ir = 1/2 sum m [R0^2 f + l+R+ - l-R-] - d n I1.
-__device__ void static_potentials(const double* r, const double* v, double& I1, double* Ir) {
-  double e1[3], e2[3], n[3];
-  for (int i = 0; i < 3; ++i) {
-    e1[i] = v[3 + i] - v[i];
-    e2[i] = v[6 + i] - v[i];
-  }
-  n[0] = e1[1] * e2[2] - e1[2] * e2[1];
-  n[1] = e1[2] * e2[0] - e1[0] * e2[2];
-  n[2] = e1[0] * e2[1] - e1[1] * e2[0];
-  double nn = sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
-  for (int i = 0; i < 3; ++i) n[i] /= nn;
-  double d = n[0] * (r[0] - v[0]) + n[1] * (r[1] - v[1]) + n[2] * (r[2] - v[2]);
-  double ad = fabs(d);
-  I1 = 0;
-  double Ip[3] = {0, 0, 0};
-  for (int k = 0; k < 3; ++k) {
-    const double* a = v + 3 * k;
-    const double* b = v + 3 * ((k + 1) % 3);
-    double s[3] = {b[0] - a[0], b[1] - a[1], b[2] - a[2]};
-    double el = sqrt(s[0] * s[0] + s[1] * s[1] + s[2] * s[2]);
-    for (int i = 0; i < 3; ++i) s[i] /= el;
-    double m[3] = {s[1] * n[2] - s[2] * n[1], s[2] * n[0] - s[0] * n[2], s[0] * n[1] - s[1] * n[0]};
-    double lp = 0, lm = 0, P0 = 0, Rp2 = 0, Rm2 = 0;
-    for (int i = 0; i < 3; ++i) {
-      lp += (b[i] - r[i]) * s[i];
-      lm += (a[i] - r[i]) * s[i];
-      P0 += (a[i] - r[i]) * m[i];
-      Rp2 += (r[i] - b[i]) * (r[i] - b[i]);
-      Rm2 += (r[i] - a[i]) * (r[i] - a[i]);
-    }
-    double Rp = sqrt(Rp2), Rm = sqrt(Rm2);
-    double R02 = P0 * P0 + d * d;
-    double f = 0;
-    if (R02 > 1e-24 * el * el) {
-      if (lm >= 0)
-        f = log((Rp + lp) / (Rm + lm));
-      else if (lp <= 0)
-        f = log((Rm - lm) / (Rp - lp));
-      else
-        f = log((Rp + lp) * (Rm - lm) / R02);
-    }
-    double dp = R02 + ad * Rp, dm = R02 + ad * Rm;
-    double at = (dp > 0 ? atan(P0 * lp / dp) : 0.0) - (dm > 0 ? atan(P0 * lm / dm) : 0.0);
-    I1 += P0 * f - ad * at;
-    double c = 0.5 * (R02 * f + lp * Rp - lm * Rm);
-    for (int i = 0; i < 3; ++i) Ip[i] += c * m[i];
-  }
-  for (int i = 0; i < 3; ++i) Ir[i] = Ip[i] - d * I1 * n[i];
+// ------------------------------------------------------------ pair moments
+//
+// Both kernels below bind on the FP64 pipe (two fused multiply-adds per clock
+// and SM), so they are written for few double operations per point pair.  The
+// 7-point rule on a triangle is its centroid c and two orbits c + s_o v_k
+// (v_k = vertex k - c, s_o = 1 - 3 a_o, weights w_o), so sums over its points
+// need sum_o w_o g and sum_o w_o s_o g per corner only.  The stored centroid's
+// rounding e = sum_k v_k / 3 is added to the first moments at the end.
+// e^{ikR}/R needs no sincos: cos(kR) and sin(kR)/R are power series in (kR)^2,
+// NT terms of each.
+
+struct Rule7 {
+  double w0, w[2], s[2], ws[2];  // ws = w s
+};
+
+__device__ __forceinline__ Rule7 load_rule7(const double* __restrict__ r) {
+  const double s0 = 1.0 - 3.0 * r[5], s1 = 1.0 - 3.0 * r[17];
+  return Rule7{r[3], {r[7], r[19]}, {s0, s1}, {r[7] * s0, r[19] * s1}};
 }
 
-// (exp(ikR) - 1)/(4 pi R) without cancellation; ik/(4 pi) at R = 0.
-__device__ __forceinline__ void green_rem(double k, double R, double& gr, double& gi) {
-  if (R > 0) {
-    double sh = sin(0.5 * k * R);
-    gr = -2.0 * sh * sh / (kFourPi * R);
-    gi = sin(k * R) / (kFourPi * R);
-  } else {
-    gr = 0;
-    gi = k / kFourPi;
+// Coefficients in R^2 of cos(kR), sin(kR)/(kR) and 2 (1 - cos kR)/(kR)^2.
+constexpr int kNearTerms = 11;
+struct NearSeries {
+  double c[kNearTerms], s[kNearTerms], r[kNearTerms];
+};
+
+static NearSeries near_series(double k) {
+  NearSeries t;
+  double* v[3] = {t.c, t.s, t.r};
+  for (int N = 0; N < 3; ++N) {
+    double a = 1.0;
+    for (int n = 0; n < kNearTerms; ++n) {
+      if (n > 0) a *= -k * k / double((2 * n + N) * (2 * n + N - 1));
+      v[N][n] = a;
+    }
   }
+  return t;
+}
+
+// The first NT terms by Horner.
+template <int NT>
+__device__ __forceinline__ double even_series(const double* c, double z) {
+  double v = c[NT - 1];
+#pragma unroll
+  for (int n = NT - 2; n >= 0; --n) v = fma(v, z, c[n]);
+  return v;
+}
+
+// ln(a/b), a, b > 0 (normal): a is scaled by the power of two that brings a/b
+// into [2/3, 3/2], then ln = 2 atanh(t), t = (a - b)/(a + b), |t| <= 0.2, by its
+// Taylor series (11 terms: t^24/23 < 1e-17): one division for the ratio and the
+// logarithm together (25 double operations; log(a / b) took 41).
+__device__ __forceinline__ double log_ratio(double a, double b) {
+  const int ha = __double2hiint(a);
+  const int q = (ha - __double2hiint(b) + (1 << 19)) >> 20;
+  const double as = __hiloint2double(ha - (q << 20), __double2loint(a));
+  const double t = (as - b) / (as + b), z = t * t;
+  double p = 1.0 / 23;
+#pragma unroll
+  for (int n = 10; n >= 1; --n) p = fma(p, z, 1.0 / (2 * n + 1));
+  const double t2 = t + t, qd = double(q);
+  // ln 2 to 1e-33 as a sum of two doubles
+  return fma(qd, 0.69314718055994530942, fma(qd, 2.3190468138462996e-17, fma(t2 * z, p, t2)));
 }
 
 struct Moments {
   double m0r, m0i, mtr[3], mti[3], msr[3], msi[3], mtsr, mtsi;
 };
 
-__device__ void moments_regular(const double* vt, const double* ct, double At, const double* vs, const double* cs,
-                                double As, double k, const double* rule7, Moments& o) {
-  double rs[7][3], ws[7];
-  for (int j = 0; j < 7; ++j) {
-    for (int d = 0; d < 3; ++d)
-      rs[j][d] = rule7[4 * j] * vs[d] + rule7[4 * j + 1] * vs[3 + d] + rule7[4 * j + 2] * vs[6 + d];
-    ws[j] = rule7[4 * j + 3] * As;
-  }
-  o = Moments{};
-  for (int i = 0; i < 7; ++i) {
-    double ri[3];
-    for (int d = 0; d < 3; ++d)
-      ri[d] = rule7[4 * i] * vt[d] + rule7[4 * i + 1] * vt[3 + d] + rule7[4 * i + 2] * vt[6 + d];
-    double wi = rule7[4 * i + 3] * At;
-    double Kr = 0, Ki = 0, K1r[3] = {0, 0, 0}, K1i[3] = {0, 0, 0};
-    for (int j = 0; j < 7; ++j) {
-      double dx = ri[0] - rs[j][0], dy = ri[1] - rs[j][1], dz = ri[2] - rs[j][2];
-      double R = sqrt(dx * dx + dy * dy + dz * dz);
-      double sn, cs_;
-      sincos(k * R, &sn, &cs_);
-      double g = ws[j] / (kFourPi * R);
-      double gr = g * cs_, gi = g * sn;
-      Kr += gr;
-      Ki += gi;
-      for (int d = 0; d < 3; ++d) {
-        double u = rs[j][d] - cs[d];
-        K1r[d] += gr * u;
-        K1i[d] += gi * u;
-      }
-    }
-    o.m0r += wi * Kr;
-    o.m0i += wi * Ki;
-    for (int d = 0; d < 3; ++d) {
-      double u = ri[d] - ct[d];
-      o.mtr[d] += wi * u * Kr;
-      o.mti[d] += wi * u * Ki;
-      o.msr[d] += wi * K1r[d];
-      o.msi[d] += wi * K1i[d];
-      o.mtsr += wi * u * K1r[d];
-      o.mtsi += wi * u * K1i[d];
-    }
+// One outer point's share at weight w and weighted test offset wu = w (r - c_t):
+// K = sum_j w_j g, K1 = sum_j w_j u_j g.
+__device__ __forceinline__ void add_point(Moments& o, double w, const double (&wu)[3], double Kr, double Ki,
+                                          const double (&K1r)[3], const double (&K1i)[3]) {
+  o.m0r = fma(w, Kr, o.m0r);
+  o.m0i = fma(w, Ki, o.m0i);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    o.mtr[d] = fma(wu[d], Kr, o.mtr[d]);
+    o.mti[d] = fma(wu[d], Ki, o.mti[d]);
+    o.msr[d] = fma(w, K1r[d], o.msr[d]);
+    o.msi[d] = fma(w, K1i[d], o.msi[d]);
+    o.mtsr = fma(wu[d], K1r[d], o.mtsr);
+    o.mtsi = fma(wu[d], K1i[d], o.mtsi);
   }
 }
 
-__device__ void moments_singular(const double* vt, const double* ct, double At, const double* vs, const double* cs,
-                                 double As, double k, const double* rule7, const double* rule64, Moments& o) {
+// The centroid rounding e of the source triangle in the first moments.
+__device__ __forceinline__ void add_centroid(Moments& o, const double (&e)[3]) {
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    o.msr[d] = fma(e[d], o.m0r, o.msr[d]);
+    o.msi[d] = fma(e[d], o.m0i, o.msi[d]);
+    o.mtsr = fma(e[d], o.mtr[d], o.mtsr);
+    o.mtsi = fma(e[d], o.mti[d], o.mtsi);
+  }
+}
+
+// The row's test points for the regular pairs: r, w, w (r - c_t) of the 7-point rule.
+struct TestPoint {
+  double r[3], w, wu[3];
+};
+
+// Regular pair by the 7 x 7 rule.  NT = 0: sincos (boxes large in wavelengths).
+// The imaginary parts are summed without their factor k.
+template <int NT>
+__device__ __forceinline__ void moments_regular(const TestPoint* __restrict__ tp, const double* __restrict__ vs,
+                                                const double* __restrict__ cs, double As, double k,
+                                                const NearSeries& G, const Rule7& R, Moments& o) {
+  double v[3][3], e[3];
+  const double c[3] = {cs[0], cs[1], cs[2]};
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) v[q][d] = vs[3 * q + d] - c[d];
+    e[d] = (v[0][d] + v[1][d] + v[2][d]) / 3.0;
+  }
   o = Moments{};
-  for (int i = 0; i < 64; ++i) {
-    double ri[3];
-    for (int d = 0; d < 3; ++d)
-      ri[d] = rule64[4 * i] * vt[d] + rule64[4 * i + 1] * vt[3 + d] + rule64[4 * i + 2] * vt[6 + d];
-    double wi = rule64[4 * i + 3] * At;
-    double I1, Ir[3];
-    static_potentials(ri, vs, I1, Ir);
-    double Kr = I1 / kFourPi, Ki = 0;
-    double K1r[3], K1i[3] = {0, 0, 0};
-    for (int d = 0; d < 3; ++d) K1r[d] = (Ir[d] + (ri[d] - cs[d]) * I1) / kFourPi;
-    for (int j = 0; j < 7; ++j) {
-      double rj[3];
-      for (int d = 0; d < 3; ++d)
-        rj[d] = rule7[4 * j] * vs[d] + rule7[4 * j + 1] * vs[3 + d] + rule7[4 * j + 2] * vs[6 + d];
-      double wj = rule7[4 * j + 3] * As;
-      double dx = ri[0] - rj[0], dy = ri[1] - rj[1], dz = ri[2] - rj[2];
-      double gr, gi;
-      green_rem(k, sqrt(dx * dx + dy * dy + dz * dz), gr, gi);
-      gr *= wj;
-      gi *= wj;
-      Kr += gr;
-      Ki += gi;
+  // e^{ikR}/R = cos(kR)/R + i k sin(kR)/(kR)
+  auto green = [&](double q2, double& gr, double& gi) {
+    const double ri = rsqrt(q2);
+    if constexpr (NT == 0) {
+      double sn, cn;
+      sincos(k * (q2 * ri), &sn, &cn);
+      gr = ri * cn;
+      gi = ri * sn;
+    } else {
+      gr = ri * even_series<NT>(G.c, q2);
+      gi = even_series<NT>(G.s, q2);
+    }
+  };
+#pragma unroll 1
+  for (int i = 0; i < 7; ++i) {
+    const double x[3] = {tp[i].r[0] - c[0], tp[i].r[1] - c[1], tp[i].r[2] - c[2]};
+    double Kr, Ki, K1r[3] = {0, 0, 0}, K1i[3] = {0, 0, 0};
+    green(x[0] * x[0] + x[1] * x[1] + x[2] * x[2], Kr, Ki);
+    Kr *= R.w0;
+    Ki *= R.w0;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      double hr = 0, hi = 0;
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        const double dx = fma(-R.s[p], v[q][0], x[0]), dy = fma(-R.s[p], v[q][1], x[1]),
+                     dz = fma(-R.s[p], v[q][2], x[2]);
+        double gr, gi;
+        green(dx * dx + dy * dy + dz * dz, gr, gi);
+        Kr = fma(R.w[p], gr, Kr);
+        Ki = fma(R.w[p], gi, Ki);
+        hr = fma(R.ws[p], gr, hr);
+        hi = fma(R.ws[p], gi, hi);
+      }
+#pragma unroll
       for (int d = 0; d < 3; ++d) {
-        double u = rj[d] - cs[d];
-        K1r[d] += gr * u;
-        K1i[d] += gi * u;
+        K1r[d] = fma(v[q][d], hr, K1r[d]);
+        K1i[d] = fma(v[q][d], hi, K1i[d]);
       }
     }
-    o.m0r += wi * Kr;
-    o.m0i += wi * Ki;
+    const double wu[3] = {tp[i].wu[0], tp[i].wu[1], tp[i].wu[2]};
+    add_point(o, tp[i].w, wu, Kr, Ki, K1r, K1i);
+  }
+  add_centroid(o, e);
+  const double fr = As * (1.0 / kFourPi), fi = NT == 0 ? fr : fr * k;
+  o.m0r *= fr;
+  o.m0i *= fi;
+  o.mtsr *= fr;
+  o.mtsi *= fi;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    o.mtr[d] *= fr;
+    o.mti[d] *= fi;
+    o.msr[d] *= fr;
+    o.msi[d] *= fi;
+  }
+}
+
+// Near-singular pair, test triangle t, source s: outer 8 x 8 collapsed Gauss
+// rule (points lane, lane + NL, ...: NL lanes share the pair), the static
+// inner integrals int 1/R and int (r'-r)/R over the flat source triangle in
+// closed form (Wilton et al. 1984; Graglia 1993), the rest
+// (e^{ikR} - 1)/R by the 7-point rule.  With unit normal n, height
+// d = n.(r - v0), per edge a->b: tangent s, outward normal m = s x n,
+// l+ = (b-r).s, l- = (a-r).s, P0 = (a-r).m, R0^2 = P0^2 + d^2,
+// f = ln((R+ + l+)/(R- + l-)):
+//   I1 = sum P0 f - |d| W,  Ir = 1/2 sum m [R0^2 f + l+R+ - l-R-] - d n I1,
+// W the solid angle of the triangle, one arctangent by van Oosterom and
+// Strackee (1983) instead of two per edge.  Adds to o.
+template <int NT, int NL>
+__device__ __forceinline__ void moments_singular(const double* __restrict__ vt, const double* __restrict__ ct,
+                                                 double At, const double* __restrict__ vs,
+                                                 const double* __restrict__ cs, double As, double k,
+                                                 const NearSeries& G, const Rule7& R7,
+                                                 const double* __restrict__ rule64, int lane, Moments& o) {
+  double v[3][3], s[3][3], m[3][3], n[3], el[3], e[3];
+  const double c[3] = {cs[0], cs[1], cs[2]};
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) v[q][d] = vs[3 * q + d] - c[d];
+    e[d] = (v[0][d] + v[1][d] + v[2][d]) / 3.0;
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) s[q][d] = vs[3 * ((q + 1) % 3) + d] - vs[3 * q + d];
+    el[q] = sqrt(s[q][0] * s[q][0] + s[q][1] * s[q][1] + s[q][2] * s[q][2]);
+  }
+  // the normal from s_0 x s_1 = e1 x (e2 - e1) = e1 x e2
+  n[0] = s[0][1] * s[1][2] - s[0][2] * s[1][1];
+  n[1] = s[0][2] * s[1][0] - s[0][0] * s[1][2];
+  n[2] = s[0][0] * s[1][1] - s[0][1] * s[1][0];
+  const double nn = sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) n[d] /= nn;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) s[q][d] /= el[q];
+    m[q][0] = s[q][1] * n[2] - s[q][2] * n[1];
+    m[q][1] = s[q][2] * n[0] - s[q][0] * n[2];
+    m[q][2] = s[q][0] * n[1] - s[q][1] * n[0];
+  }
+  const double fr = -0.5 * k * k * As, fi = k * As;
+  Moments a{};
+#pragma unroll 1
+  for (int i = lane; i < 64; i += NL) {
+    double wu[3], x[3];
+    const double wi = rule64[4 * i + 3] * (At * (1.0 / kFourPi));
+#pragma unroll
     for (int d = 0; d < 3; ++d) {
-      double u = ri[d] - ct[d];
-      o.mtr[d] += wi * u * Kr;
-      o.mti[d] += wi * u * Ki;
-      o.msr[d] += wi * K1r[d];
-      o.msi[d] += wi * K1i[d];
-      o.mtsr += wi * u * K1r[d];
-      o.mtsi += wi * u * K1i[d];
+      const double r = rule64[4 * i] * vt[d] + rule64[4 * i + 1] * vt[3 + d] + rule64[4 * i + 2] * vt[6 + d];
+      wu[d] = wi * (r - ct[d]);
+      x[d] = r - c[d];
     }
+    // static part
+    double p[3][3], Rv[3];  // r - vertex, its length
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) p[q][d] = x[d] - v[q][d];
+      Rv[q] = sqrt(p[q][0] * p[q][0] + p[q][1] * p[q][1] + p[q][2] * p[q][2]);
+    }
+    const double h = n[0] * p[0][0] + n[1] * p[0][1] + n[2] * p[0][2], ah = fabs(h);
+    double I1 = 0, Ip[3] = {0, 0, 0}, den = Rv[0] * Rv[1] * Rv[2];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const int q1 = (q + 1) % 3;
+      const double Rm = Rv[q], Rp = Rv[q1];
+      const double lm = -(p[q][0] * s[q][0] + p[q][1] * s[q][1] + p[q][2] * s[q][2]), lp = lm + el[q];
+      const double P0 = -(p[q][0] * m[q][0] + p[q][1] * m[q][1] + p[q][2] * m[q][2]);
+      const double R02 = P0 * P0 + h * h;
+      const bool right = lm >= 0, left = lp <= 0;
+      const double up = left ? Rm - lm : right ? Rp + lp : (Rp + lp) * (Rm - lm);
+      const double dn = left ? Rp - lp : right ? Rm + lm : R02;
+      const double f = R02 > 1e-24 * el[q] * el[q] ? log_ratio(up, dn) : 0.0;
+      I1 = fma(P0, f, I1);
+      const double w = 0.5 * (R02 * f + lp * Rp - lm * Rm);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) Ip[d] = fma(w, m[q][d], Ip[d]);
+      den = fma(p[q][0] * p[q1][0] + p[q][1] * p[q1][1] + p[q][2] * p[q1][2], Rv[(q + 2) % 3], den);
+    }
+    I1 -= 2.0 * ah * atan2(ah * nn, den);
+    // the rest, (e^{ikR} - 1)/R = -k^2/2 R [2 (1 - cos kR)/(kR)^2] + i k sin(kR)/(kR)
+    double gr, gi, Kr, Ki, K1r[3] = {0, 0, 0}, K1i[3] = {0, 0, 0};
+    auto rem = [&](double q2) {
+      gr = q2 * rsqrt(q2 + 1e-300) * even_series<NT>(G.r, q2);  // R = 0 at a shared point
+      gi = even_series<NT>(G.s, q2);
+    };
+    rem(x[0] * x[0] + x[1] * x[1] + x[2] * x[2]);
+    Kr = R7.w0 * gr;
+    Ki = R7.w0 * gi;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      double hr = 0, hi = 0;
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        const double dx = fma(-R7.s[b], v[q][0], x[0]), dy = fma(-R7.s[b], v[q][1], x[1]),
+                     dz = fma(-R7.s[b], v[q][2], x[2]);
+        rem(dx * dx + dy * dy + dz * dz);
+        Kr = fma(R7.w[b], gr, Kr);
+        Ki = fma(R7.w[b], gi, Ki);
+        hr = fma(R7.ws[b], gr, hr);
+        hi = fma(R7.ws[b], gi, hi);
+      }
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        K1r[d] = fma(v[q][d], hr, K1r[d]);
+        K1i[d] = fma(v[q][d], hi, K1i[d]);
+      }
+    }
+    Kr = fma(fr, Kr, I1);
+    Ki *= fi;
+    // (only the rule's imaginary part takes the centroid's rounding: the
+    // static part is exact about c and dwarfs the real remainder)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      K1r[d] = fma(fr, K1r[d], fma(fma(-h, n[d], x[d]), I1, Ip[d]));
+      K1i[d] = fma(e[d], Ki, fi * K1i[d]);
+    }
+    add_point(a, wi, wu, Kr, Ki, K1r, K1i);
+  }
+  o.m0r += a.m0r;
+  o.m0i += a.m0i;
+  o.mtsr += a.mtsr;
+  o.mtsi += a.mtsi;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    o.mtr[d] += a.mtr[d];
+    o.mti[d] += a.mti[d];
+    o.msr[d] += a.msr[d];
+    o.msi[d] += a.msi[d];
   }
 }
 
@@ -188,13 +339,15 @@ __device__ __forceinline__ bool near_singular(const double* ct, const double* cs
 
 // Near-part set-up in three passes, so that the few expensive near-singular
 // pairs do not stall the warps computing the regular ones:
-//  1. k_count_singular: count the near-singular pairs with t <= s;
+//  1. k_count_singular: count the near-singular pairs with t < s;
 //  2. k_near_regular: regular pairs by the 7 x 7 rule; near-singular pairs
-//     with t <= s are appended to a list;
-//  3. k_near_singular: one thread per listed pair computes the rule in both
-//     orders, averages, and writes the (t,s) and (s,t) entries (mt and ms
-//     swapped), which keeps Z^T = Z.
-// Lanes walk a test row flat, as the product kernel does.
+//     are appended to a list;
+//  3. k_near_singular: kSingLanes lanes per listed pair compute the rule in
+//     both orders and average; then the pairs (t, t).
+// Every unordered pair is computed once and written as (t,s) and (s,t) (mt and
+// ms swapped), which keeps Z^T = Z: a row lists its sources in ascending order,
+// so the pairs t < s of a row are its tail past t's own position, and lanes
+// walk that tail flat, as the product kernel does.
 struct NearGeom {
   const int32_t* leaf_of;
   const int32_t* leaf_start;
@@ -208,6 +361,14 @@ struct NearGeom {
   const double* h2;
 };
 
+// Position of source s within the row of a triangle of box b (-1: not near).
+__device__ __forceinline__ int row_position(const NearGeom& g, int b, int64_t s) {
+  const int bs = g.leaf_of[s];
+  for (int q = g.near_ptr[b]; q < g.near_ptr[b + 1]; ++q)
+    if (g.near_idx[q] == bs) return g.near_off[q] + int(s - g.leaf_start[bs]);
+  return -1;
+}
+
 __global__ void __launch_bounds__(256) k_count_singular(int64_t T, NearGeom g, unsigned long long* count) {
   int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   int lane = threadIdx.x & 31;
@@ -217,10 +378,10 @@ __global__ void __launch_bounds__(256) k_count_singular(int64_t T, NearGeom g, u
   const int len = int(g.row_ptr[t + 1] - g.row_ptr[t]);
   int qi = q0;
   unsigned n = 0;
-  for (int j = lane; j < len; j += 32) {
+  for (int j = row_position(g, b, t) + 1 + lane; j < len; j += 32) {
     while (qi + 1 < q1 && g.near_off[qi + 1] <= j) ++qi;
     const int64_t s = g.leaf_start[g.near_idx[qi]] + (j - g.near_off[qi]);
-    if (t <= s && near_singular(g.cent + 3 * t, g.cent + 3 * s, g.h2[t], g.h2[s])) ++n;
+    if (near_singular(g.cent + 3 * t, g.cent + 3 * s, g.h2[t], g.h2[s])) ++n;
   }
   n = __reduce_add_sync(0xffffffffu, n);
   if (lane == 0 && n) atomicAdd(count, (unsigned long long)n);
@@ -243,11 +404,14 @@ __device__ __forceinline__ void store_moments(C2<Rm>* mom, int64_t nnz, int64_t 
   mom[7 * nnz + e] = mk<Rm>(Rm(m.mtsr), Rm(m.mtsi));
 }
 
-template <typename Rm>
-__global__ void __launch_bounds__(128) k_near_regular(int64_t T, int64_t nnz, NearGeom g, double k,
+// 20,480 triangles (2.75e6 unordered pairs): 8.6 ms; 34.4 ms with both orders,
+// sincos and a division per point pair.
+template <typename Rm, int NT>
+__global__ void __launch_bounds__(128) k_near_regular(int64_t T, int64_t nnz, NearGeom g, double k, NearSeries G,
                                                       const double* __restrict__ rule7, C2<Rm>* __restrict__ mom,
                                                       SingPair* __restrict__ list, unsigned long long* __restrict__ nlist,
                                                       unsigned long long cap) {
+  __shared__ TestPoint tps[4][7];
   int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   int lane = threadIdx.x & 31;
   if (t >= T) return;
@@ -255,61 +419,83 @@ __global__ void __launch_bounds__(128) k_near_regular(int64_t T, int64_t nnz, Ne
   const int q0 = g.near_ptr[b], q1 = g.near_ptr[b + 1];
   const int64_t e0 = g.row_ptr[t];
   const int len = int(g.row_ptr[t + 1] - e0);
-  const double* vt = g.vert + 9 * t;
   const double* ct = g.cent + 3 * t;
+  const Rule7 R = load_rule7(rule7);
+  TestPoint* tp = tps[threadIdx.x >> 5];
+  if (lane < 7) {
+    const double* vt = g.vert + 9 * t;
+    const double* q = rule7 + 4 * lane;
+    tp[lane].w = q[3] * g.area[t];
+    for (int d = 0; d < 3; ++d) {
+      tp[lane].r[d] = q[0] * vt[d] + q[1] * vt[3 + d] + q[2] * vt[6 + d];
+      tp[lane].wu[d] = tp[lane].w * (tp[lane].r[d] - ct[d]);
+    }
+  }
+  __syncwarp();
   int qi = q0;
-  for (int j = lane; j < len; j += 32) {
+  for (int j = row_position(g, b, t) + 1 + lane; j < len; j += 32) {
     while (qi + 1 < q1 && g.near_off[qi + 1] <= j) ++qi;
     const int64_t s = g.leaf_start[g.near_idx[qi]] + (j - g.near_off[qi]);
     const int64_t e = e0 + j;
     if (near_singular(ct, g.cent + 3 * s, g.h2[t], g.h2[s])) {
-      if (t <= s) {
-        unsigned long long slot = atomicAdd(nlist, 1ull);
-        if (slot < cap) list[slot] = SingPair{int32_t(t), int32_t(s), e};
-      }
+      unsigned long long slot = atomicAdd(nlist, 1ull);
+      if (slot < cap) list[slot] = SingPair{int32_t(t), int32_t(s), e};
       continue;
     }
     Moments m;
-    moments_regular(vt, ct, g.area[t], g.vert + 9 * s, g.cent + 3 * s, g.area[s], k, rule7, m);
+    moments_regular<NT>(tp, g.vert + 9 * s, g.cent + 3 * s, g.area[s], k, G, R, m);
     store_moments(mom, nnz, e, m, false);
+    const int p = row_position(g, g.near_idx[qi], t);
+    if (p >= 0) store_moments(mom, nnz, g.row_ptr[s] + p, m, true);
   }
 }
 
-template <typename Rm>
-__global__ void __launch_bounds__(128) k_near_singular(int64_t npairs, int64_t nnz, NearGeom g, double k,
+// Eight lanes per pair: a small mesh's few thousand pairs still give every SM
+// warps, and the 64 outer points of each order split evenly.  SELF: the pairs
+// (t, t), one order each (no list).  20,480 triangles: 24.1 ms (22.5 + 1.6);
+// 84.1 ms with a thread per pair, two arctangents and a logarithm of a quotient
+// per edge and three sines per point pair.
+constexpr int kSingLanes = 8;
+template <typename Rm, int NT, bool SELF>
+__global__ void __launch_bounds__(128) k_near_singular(int64_t npairs, int64_t nnz, NearGeom g, double k, NearSeries G,
                                                        const double* __restrict__ rule7,
                                                        const double* __restrict__ rule64,
                                                        const SingPair* __restrict__ list, C2<Rm>* __restrict__ mom) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= npairs) return;
-  const SingPair pq = list[i];
-  const int64_t t = pq.t, s = pq.s;
-  Moments m, m2;
-  moments_singular(g.vert + 9 * t, g.cent + 3 * t, g.area[t], g.vert + 9 * s, g.cent + 3 * s, g.area[s], k, rule7,
-                   rule64, m);
-  moments_singular(g.vert + 9 * s, g.cent + 3 * s, g.area[s], g.vert + 9 * t, g.cent + 3 * t, g.area[t], k, rule7,
-                   rule64, m2);
-  // two-sided average, as seen from t (test) and s (source)
-  m.m0r = 0.5 * (m.m0r + m2.m0r);
-  m.m0i = 0.5 * (m.m0i + m2.m0i);
-  m.mtsr = 0.5 * (m.mtsr + m2.mtsr);
-  m.mtsi = 0.5 * (m.mtsi + m2.mtsi);
-  for (int d = 0; d < 3; ++d) {
-    const double tr = 0.5 * (m.mtr[d] + m2.msr[d]), ti = 0.5 * (m.mti[d] + m2.msi[d]);
-    const double sr = 0.5 * (m.msr[d] + m2.mtr[d]), si = 0.5 * (m.msi[d] + m2.mti[d]);
-    m.mtr[d] = tr;
-    m.mti[d] = ti;
-    m.msr[d] = sr;
-    m.msi[d] = si;
+  const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kSingLanes;
+  const int lane = threadIdx.x % kSingLanes;
+  // lanes past the end repeat the last pair (every lane joins the shuffles)
+  const int64_t ii = min(i, npairs - 1);
+  const int64_t pt = SELF ? ii : list[ii].t, ps = SELF ? ii : list[ii].s;
+  const Rule7 R = load_rule7(rule7);
+  // both orders into one set of moments as seen from t (test) and s (source):
+  // mt and ms change places between them
+  Moments m{};
+#pragma unroll 1
+  for (int order = 0; order < (SELF ? 1 : 2); ++order) {
+    const int64_t t = order ? ps : pt, s = order ? pt : ps;
+    moments_singular<NT, kSingLanes>(g.vert + 9 * t, g.cent + 3 * t, g.area[t], g.vert + 9 * s, g.cent + 3 * s,
+                                     g.area[s], k, G, R, rule64, lane, m);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const double x = m.mtr[d], y = m.mti[d];
+      m.mtr[d] = SELF ? 0.5 * (x + m.msr[d]) : m.msr[d];
+      m.mti[d] = SELF ? 0.5 * (y + m.msi[d]) : m.msi[d];
+      m.msr[d] = SELF ? m.mtr[d] : x;
+      m.msi[d] = SELF ? m.mti[d] : y;
+    }
   }
-  store_moments(mom, nnz, pq.e, m, false);
-  if (s != t) {
-    // entry (s, t): row s, at the position of t inside the near box of t
-    const int bs = g.leaf_of[s], bt = g.leaf_of[t];
-    int64_t e2 = -1;
-    for (int qi = g.near_ptr[bs]; qi < g.near_ptr[bs + 1]; ++qi)
-      if (g.near_idx[qi] == bt) e2 = g.row_ptr[s] + g.near_off[qi] + (t - g.leaf_start[bt]);
-    if (e2 >= 0) store_moments(mom, nnz, e2, m, true);
+  double* f = reinterpret_cast<double*>(&m);
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+#pragma unroll
+    for (int w = 1; w < kSingLanes; w *= 2) f[q] += __shfl_xor_sync(0xffffffffu, f[q], w);
+    if (!SELF) f[q] *= 0.5;
+  }
+  if (i >= npairs || lane != 0) return;
+  store_moments(mom, nnz, SELF ? g.row_ptr[pt] + row_position(g, g.leaf_of[pt], pt) : list[ii].e, m, false);
+  if constexpr (!SELF) {
+    const int p = row_position(g, g.leaf_of[ps], pt);
+    if (p >= 0) store_moments(mom, nnz, g.row_ptr[ps] + p, m, true);
   }
 }
 
@@ -686,10 +872,40 @@ static pie_status setup_t(Problem& pr, cudaStream_t st) {
   if ((s = cuda_check(cudaStreamSynchronize(st), "count sync")) != PIE_OK) return s;
   SingPair* list = static_cast<SingPair*>(zalloc(pr, sizeof(SingPair) * std::max<unsigned long long>(nsing, 1), s));
   if (s != PIE_OK) return s;
-  k_near_regular<Rm><<<unsigned((T * 32 + 127) / 128), 128, 0, st>>>(
-      T, pr.nnz, ng, pr.k0, pr.rule7, static_cast<C2<Rm>*>(pr.mom), list, dcount + 1, nsing);
-  k_near_singular<Rm><<<unsigned((nsing + 127) / 128), 128, 0, st>>>(int64_t(nsing), pr.nnz, ng, pr.k0, pr.rule7,
-                                                                     pr.rule64, list, static_cast<C2<Rm>*>(pr.mom));
+  // Series terms by the largest kR: points of near triangles are at most
+  // 2 sqrt(3) leaf sides and two thirds of an edge each way apart (h <= leaf /
+  // 1.5), 4.4 leaf sides; near-singular pairs at most 2.9 h.  First omitted
+  // term below 1e-17: x^(2 NT)/(2 NT)!, or 2 x^(2 NT)/(2 NT + 2)!; k h is at most 0.52.
+  {
+    C2<Rm>* mom = static_cast<C2<Rm>*>(pr.mom);
+    const unsigned rb = unsigned((T * 32 + 127) / 128);
+    const double xr = 4.4 * pr.k0 * aL, xs = 2.9 * pr.k0 * pr.h_max;
+    const NearSeries G = near_series(pr.k0);
+    auto regular = [&](auto nt) {
+      k_near_regular<Rm, decltype(nt)::value><<<rb, 128, 0, st>>>(T, pr.nnz, ng, pr.k0, G, pr.rule7, mom, list,
+                                                                  dcount + 1, nsing);
+    };
+    auto singular = [&](auto nt, auto self, int64_t n) {
+      if (n == 0) return;
+      k_near_singular<Rm, decltype(nt)::value, decltype(self)::value>
+          <<<unsigned((n * kSingLanes + 127) / 128), 128, 0, st>>>(n, pr.nnz, ng, pr.k0, G, pr.rule7, pr.rule64, list,
+                                                                   mom);
+    };
+    if (xr < 0.028)
+      regular(std::integral_constant<int, 4>());
+    else if (xr < 0.59)
+      regular(std::integral_constant<int, 8>());
+    else
+      regular(std::integral_constant<int, 0>());
+    auto both = [&](auto nt) {
+      singular(nt, std::false_type(), int64_t(nsing));
+      singular(nt, std::true_type(), T);
+    };
+    if (xs < 0.04)
+      both(std::integral_constant<int, 4>());
+    else
+      both(std::integral_constant<int, kNearTerms>());
+  }
   if ((s = cuda_check(cudaGetLastError(), "near build")) != PIE_OK) return s;
 
   // leaf radiation tables
