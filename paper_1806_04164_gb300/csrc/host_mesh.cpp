@@ -233,62 +233,54 @@ pie_status build_tree(const Mesh& m, int L, double root_side, Tree& tr) {
     tr.leaf_start[b] = std::lower_bound(leafkey.begin(), leafkey.end(), lk[b]) - leafkey.begin();
   tr.leaf_start[lk.size()] = T;
 
-  auto find_box = [&](int l, int64_t ix, int64_t iy, int64_t iz) -> int64_t {
-    int64_t n = int64_t(1) << (l - 1);
-    if (ix < 0 || iy < 0 || iz < 0 || ix >= n || iy >= n || iz >= n) return -1;
-    int64_t k = morton(ix, iy, iz, l - 1);
-    const auto& ks = tr.keys[l];
-    auto it = std::lower_bound(ks.begin(), ks.end(), k);
-    if (it == ks.end() || *it != k) return -1;
-    return it - ks.begin();
-  };
-  // near lists at the leaves
-  tr.near_ptr.assign(1, 0);
-  tr.near_idx.clear();
-  for (size_t b = 0; b < lk.size(); ++b) {
-    int64_t ix, iy, iz;
-    demorton(lk[b], L - 1, ix, iy, iz);
-    std::vector<int64_t> nb;
-    for (int dx = -1; dx <= 1; ++dx)
-      for (int dy = -1; dy <= 1; ++dy)
-        for (int dz = -1; dz <= 1; ++dz) {
-          int64_t q = find_box(L, ix + dx, iy + dy, iz + dz);
-          if (q >= 0) nb.push_back(q);
-        }
-    std::sort(nb.begin(), nb.end());
-    tr.near_idx.insert(tr.near_idx.end(), nb.begin(), nb.end());
-    tr.near_ptr.push_back(int64_t(tr.near_idx.size()));
-  }
-  // interaction lists at levels 3..L
+  // Box indices per level, then near and interaction lists from the top down:
+  // the boxes around b are the children of the boxes around its parent, near
+  // when their indices differ by at most one, in b's interaction list
+  // otherwise.  Parents' lists are ascending and children of one parent
+  // contiguous, so both lists come out ascending.
+  int off_code[7][7][7];
+  for (int dx = -3; dx <= 3; ++dx)
+    for (int dy = -3; dy <= 3; ++dy)
+      for (int dz = -3; dz <= 3; ++dz) off_code[dx + 3][dy + 3][dz + 3] = offset_code(dx, dy, dz);
   tr.il_ptr.assign(L + 1, {});
   tr.il_idx.assign(L + 1, {});
   tr.il_off.assign(L + 1, {});
-  for (int l = 3; l <= L; ++l) {
+  std::vector<int64_t> up_ptr = {0, 1}, up_idx = {0};  // near lists one level up (the root's: itself)
+  std::vector<int64_t> ij;                             // box indices of the level
+  for (int l = 2; l <= L; ++l) {
+    const auto& ks = tr.keys[l];
+    const int64_t nb = int64_t(ks.size());
+    ij.resize(3 * nb);
+    for (int64_t b = 0; b < nb; ++b) demorton(ks[b], l - 1, ij[3 * b], ij[3 * b + 1], ij[3 * b + 2]);
     auto& ptr = tr.il_ptr[l];
     auto& idx = tr.il_idx[l];
     auto& off = tr.il_off[l];
-    ptr.assign(1, 0);
-    for (size_t b = 0; b < tr.keys[l].size(); ++b) {
-      int64_t ix, iy, iz;
-      demorton(tr.keys[l][b], l - 1, ix, iy, iz);
-      std::vector<std::pair<int64_t, int32_t>> cand;
-      int64_t px = ix >> 1, py = iy >> 1, pz = iz >> 1;
-      for (int64_t qx = 2 * (px - 1); qx <= 2 * (px + 1) + 1; ++qx)
-        for (int64_t qy = 2 * (py - 1); qy <= 2 * (py + 1) + 1; ++qy)
-          for (int64_t qz = 2 * (pz - 1); qz <= 2 * (pz + 1) + 1; ++qz) {
-            int64_t dx = ix - qx, dy = iy - qy, dz = iz - qz;
-            if (std::max(std::llabs(dx), std::max(std::llabs(dy), std::llabs(dz))) <= 1) continue;
-            int64_t q = find_box(l, qx, qy, qz);
-            if (q >= 0) cand.push_back({q, int32_t(offset_code(int(dx), int(dy), int(dz)))});
+    std::vector<int64_t> nptr(1, 0), nidx;
+    if (l >= 3) ptr.assign(1, 0);
+    for (int64_t b = 0; b < nb; ++b) {
+      const int64_t p = tr.parent[l][b];
+      for (int64_t u = up_ptr[p]; u < up_ptr[p + 1]; ++u) {
+        const int64_t c1 = tr.child_start[l - 1][up_idx[u] + 1];
+        for (int64_t q = tr.child_start[l - 1][up_idx[u]]; q < c1; ++q) {
+          const int dx = int(ij[3 * b] - ij[3 * q]), dy = int(ij[3 * b + 1] - ij[3 * q + 1]),
+                    dz = int(ij[3 * b + 2] - ij[3 * q + 2]);
+          const int code = off_code[dx + 3][dy + 3][dz + 3];
+          if (code < 0) {
+            nidx.push_back(q);
+          } else if (l >= 3) {
+            idx.push_back(q);
+            off.push_back(code);
           }
-      std::sort(cand.begin(), cand.end());
-      for (auto& c : cand) {
-        idx.push_back(c.first);
-        off.push_back(c.second);
+        }
       }
-      ptr.push_back(int64_t(idx.size()));
+      nptr.push_back(int64_t(nidx.size()));
+      if (l >= 3) ptr.push_back(int64_t(idx.size()));
     }
+    up_ptr.swap(nptr);
+    up_idx.swap(nidx);
   }
+  tr.near_ptr.swap(up_ptr);
+  tr.near_idx.swap(up_idx);
   return PIE_OK;
 }
 
