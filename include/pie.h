@@ -416,7 +416,9 @@ pie_status pie_nearfield(pie_problem* pr, const void* x, const void* rho, const 
  *    0 = the caller's stream alone, stages in order.
  *  near_ctas_per_sm: grid of the near kernel when overlapped, in CTAs of 256
  *    threads per SM (each warp walks test triangles with a grid stride), so
- *    that it takes a bounded share of every SM beside the far kernels;
+ *    that it takes a bounded share of every SM beside the far kernels (a
+ *    complex double near part: one block of 128 threads per SM for every two,
+ *    as its integer multiply-adds leave the FP64 pipe to the far part);
  *    0 = one warp per test triangle.  0..32.
  *  rhs_chunk: right-hand sides per pass over the operator, 1..max_nrhs.
  *  near_rhs_block: right-hand sides that one pass of the near kernel
@@ -435,8 +437,9 @@ pie_status pie_nearfield(pie_problem* pr, const void* x, const void* rho, const 
  *    and group of up to 4 right-hand sides, the box's source coefficients
  *    in shared memory), 0 = automatic (box-staged for passes of one column,
  *    warp per triangle otherwise).  Both take the same operations in the
- *    same order.  A complex double near part, and near_rhs_block 8, always
- *    use the warp-per-triangle kernel.
+ *    same order.  near_rhs_block 8 always uses the warp-per-triangle kernel.
+ *    A complex double near part runs in fixed point, one column per block,
+ *    whatever near_rhs_block and near_kernel say.
  * Defaults at pie_problem_create: overlap 1, near_ctas_per_sm 2, rhs_chunk
  * max_nrhs, near_rhs_block 0, far_rows 0, near_kernel 0.  Per-stage
  * profiling (pie_profile_begin) runs the stages in order whatever overlap

@@ -8,6 +8,7 @@
 #include <cuda_fp16.h>
 
 #include "handles.h"
+#include "near_fixed.cuh"
 
 namespace pie {
 static thread_local std::string g_err;
@@ -384,6 +385,31 @@ pie_status pie_problem_stage(pie_problem* h, int which, int level, double* out, 
     src = pr.mom;
     n = size_t(pr.nnz) * kMom;
     f32 = pr.near_f32();
+    if (!f32) {  // fixed point times the row's exponents (near_fixed.cuh)
+      const size_t nnz = size_t(pr.nnz);
+      std::vector<int32_t> m(4 * n), row(2 * size_t(pr.T)), delta(size_t(pr.nleaf)), leaf(size_t(pr.T));
+      std::vector<int64_t> ptr(size_t(pr.T) + 1);
+      auto get = [&](auto& h, const void* d) {
+        if (s == PIE_OK) s = cuda_check(cudaMemcpy(h.data(), d, h.size() * sizeof(h[0]), cudaMemcpyDeviceToHost), "stage copy");
+      };
+      get(m, pr.mom);
+      get(row, pr.fixed_row);
+      get(delta, pr.fixed_delta);
+      get(leaf, pr.leaf_of);
+      get(ptr, pr.row_ptr);
+      if (s != PIE_OK) return s;
+      for (size_t t = 0; t < size_t(pr.T); ++t)
+        for (size_t q = 0; q < kMom; ++q) {
+          const bool test = (q >= 1 && q <= 3) || q == 7;
+          const int x = row[2 * t + test] + (q >= 4 ? delta[leaf[t]] : 0);
+          for (size_t i = q * nnz + ptr[t]; i < q * nnz + ptr[t + 1]; ++i)
+            for (int c = 0; c < 2; ++c)
+              out[2 * i + c] = row[2 * t] == kFixedNan
+                                   ? std::nan("")
+                                   : std::ldexp(double(m[4 * i + 2 * c]) * (1 << kLimb) + m[4 * i + 2 * c + 1], x);
+        }
+      return PIE_OK;
+    }
     if (pr.near_h16()) {  // half pairs times the plane scales
       std::vector<__half2> tmp(n);
       s = cuda_check(cudaMemcpy(tmp.data(), src, n * sizeof(__half2), cudaMemcpyDeviceToHost), "stage copy");

@@ -7,7 +7,7 @@
 #include <cstdio>
 #include <type_traits>
 
-#include "device.cuh"
+#include "near_fixed.cuh"
 
 namespace pie {
 
@@ -346,6 +346,243 @@ static pie_status near_box_prepare() {
                             "near smem attribute");
   if (s == PIE_OK && bit >= 0) done.fetch_or(uint64_t(1) << bit);
   return s;
+}
+
+// a1, PIE_FP64: near part in fixed point (near_fixed.cuh).  A block per (leaf
+// box, share of its test triangles) and right-hand side (blockIdx.y), grid
+// stride over the pairs: the box's source coefficients are staged as
+// integers kFixedStage at a time, then its warps take the test triangles in
+// turn, lanes over the row.  nsplit shares a box among several blocks when the
+// leaf boxes alone do not fill the SMs.  81,920 triangles: 0.63 ms alone (2.2 ms
+// with FP64 multiply-adds), 24,576 of a cube: 0.66 ms (1.78); beside the far part
+// one block an SM does, since the two use different pipes: the product of 81,920
+// triangles 3.27 ms (5.11).
+
+// A warp-wide 64-bit multiply-add issues every two clocks and takes four, so the
+// limb products are taken kind by kind over all sums (KIND 0: h h', 1: h l',
+// 2: l h'; HALF 0: real, 1: imaginary part of c) and not sum by sum.
+struct FixedSum {
+  int64_t hh, x;
+};
+template <int KIND, int HALF>
+__device__ __forceinline__ void fixed_cfma(FixedSum (&s)[12], int i, const int4& c, const int4& m) {
+  const int cc = HALF ? (KIND == 2 ? c.w : c.z) : (KIND == 2 ? c.y : c.x);
+  const int mx = KIND == 1 ? m.y : m.x, my = KIND == 1 ? m.w : m.z;
+  int64_t& re = KIND == 0 ? s[2 * i].hh : s[2 * i].x;
+  int64_t& im = KIND == 0 ? s[2 * i + 1].hh : s[2 * i + 1].x;
+  re += HALF ? int64_t(-cc) * my : int64_t(cc) * mx;
+  im += int64_t(cc) * (HALF ? mx : my);
+}
+
+// The twelve products of one pair; m: m0, mt(3), ms(3), mts; c: a, beta(3), sigma, d.
+template <typename F, typename C, typename M>
+__device__ __forceinline__ void near_products(F f, const C& c, const M& m) {
+  f(1, c[0], m[4]);
+  f(2, c[0], m[5]);
+  f(3, c[0], m[6]);
+  f(0, c[0], m[7]);
+  f(4, c[4], m[0]);
+  f(1, c[1], m[0]);
+  f(0, c[1], m[1]);
+  f(2, c[2], m[0]);
+  f(5, c[5], m[0]);
+  f(0, c[2], m[2]);
+  f(3, c[3], m[0]);
+  f(0, c[3], m[3]);
+}
+
+// Entries j0 .. j1 of row t in double, for a stage with a coefficient that is
+// not finite: lane i < 12 returns component i of the six sums.
+__device__ __noinline__ double near_row_double(const FixedNear& nf, int64_t nnz, int64_t t, int b, int64_t e0, int j0,
+                                               int j1, int q0, int q1, const int32_t* leaf_start,
+                                               const int32_t* near_idx, const int32_t* near_off, const cd* coef) {
+  const int lane = threadIdx.x & 31;
+  cd acc[6];
+  for (int i = 0; i < 6; ++i) acc[i] = mk<double>(0, 0);
+  int qi = q0;
+  for (int j = j0 + lane; j < j1; j += 32) {
+    while (qi + 1 < q1 && near_off[qi + 1] <= j) ++qi;
+    const cd* c = coef + 6 * (int64_t(leaf_start[near_idx[qi]]) + (j - near_off[qi]));
+    cd m[kMom];
+    for (int q = 0; q < kMom; ++q) m[q] = fixed_moment(nf, nnz, q, e0 + j, t, b);
+    near_products([&](int i, cd x, cd y) { cfma(acc[i], x, y); }, c, m);
+  }
+  double out = 0;
+  for (int i = 0; i < 12; ++i) {
+    const double v = warp_sum(i % 2 ? acc[i / 2].y : acc[i / 2].x);
+    if (lane == i) out = v;
+  }
+  return out;
+}
+
+// Shared memory: the stage's coefficients [6][kFixedStage], then two buffers of
+// 32 entries' moments [2][8][32] per warp.
+constexpr size_t kFixedSmem = sizeof(int4) * (6 * kFixedStage + 4 * 2 * kMom * 32);
+
+__global__ void __launch_bounds__(128, 3)
+    k_near_fixed(int64_t nleaf, int nsplit, int64_t nnz, const int32_t* __restrict__ leaf_start,
+                 const int32_t* __restrict__ near_ptr, const int32_t* __restrict__ near_idx,
+                 const int32_t* __restrict__ near_off, const int64_t* __restrict__ row_ptr, const FixedNear nf,
+                 const cd* __restrict__ coef, double mu0, cd* __restrict__ pot, int64_t sc = 0, int64_t sp = 0) {
+  extern __shared__ __align__(16) unsigned char fixed_smem[];
+  int4(*cs)[kFixedStage] = reinterpret_cast<int4(*)[kFixedStage]>(fixed_smem);
+  __shared__ int fields[4][4];  // [warp][group]
+  coef += blockIdx.y * sc;
+  double* out = reinterpret_cast<double*>(pot + blockIdx.y * sp);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int4(*ms)[kMom][32] = reinterpret_cast<int4(*)[kMom][32]>(cs + 6) + 2 * warp;
+  for (int64_t bi = blockIdx.x; bi < nleaf * nsplit; bi += gridDim.x) {
+    const int64_t b = bi / nsplit;
+    const int q0 = near_ptr[b], q1 = near_ptr[b + 1];
+    const int t0 = leaf_start[b] + int(bi % nsplit) * 4 + warp, t1 = leaf_start[b + 1];
+    const int len = int(row_ptr[leaf_start[b] + 1] - row_ptr[leaf_start[b]]);
+    const int dl = nf.delta[b];
+    for (int j0 = 0; j0 < len; j0 += kFixedStage) {
+      const int j1 = min(len, j0 + kFixedStage);
+      // largest exponent fields of the stage's a, beta, sigma, d
+      int x[4] = {1, 1, 1, 1};
+      int qi = q0;
+      for (int j = j0 + int(threadIdx.x); j < j1; j += blockDim.x) {
+        while (qi + 1 < q1 && near_off[qi + 1] <= j) ++qi;
+        const cd* c = coef + 6 * (int64_t(leaf_start[near_idx[qi]]) + (j - near_off[qi]));
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+          const cd v = c[k];
+          int& r = x[k == 0 ? 0 : k < 4 ? 1 : k - 2];
+          r = max(r, max(exponent_field(v.x), exponent_field(v.y)));
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[i] = __reduce_max_sync(0xffffffffu, x[i]);
+      __syncthreads();  // the previous stage's readers are done
+      if (lane < 4) fields[warp][lane] = lane == 0 ? x[0] : lane == 1 ? x[1] : lane == 2 ? x[2] : x[3];
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[i] = max(max(fields[0][i], fields[1][i]), max(fields[2][i], fields[3][i]));
+      const bool finite = max(max(x[0], x[1]), max(x[2], x[3])) < 0x7ff;
+      // beta's field covers a and delta; a takes beta's less delta
+      x[1] = max(x[1], x[0] + dl);
+      x[0] = x[1] - dl;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[i] += 53 - kCoefBits;
+      qi = q0;
+      for (int j = j0 + int(threadIdx.x); j < j1 && finite; j += blockDim.x) {
+        while (qi + 1 < q1 && near_off[qi + 1] <= j) ++qi;
+        const cd* c = coef + 6 * (int64_t(leaf_start[near_idx[qi]]) + (j - near_off[qi]));
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+          const cd v = c[k];
+          const int f = x[k == 0 ? 0 : k < 4 ? 1 : k - 2];
+          const int2 r = fixed_encode(v.x, f), i = fixed_encode(v.y, f);
+          cs[k][j - j0] = make_int4(r.x, r.y, i.x, i.y);
+        }
+      }
+      __syncthreads();
+      // the warp's (test triangle, 32 entries) steps in one sequence: each step's
+      // moments are on their way while the step before is multiplied, across rows
+      // too (rows of a box have one length, one after the other)
+      const int64_t base = row_ptr[leaf_start[b]];
+      const int per_row = (j1 - j0 + 31) / 32;
+      auto fetch = [&](int t, int i, int slot) {
+        const int j = j0 + 32 * i + lane;
+        if (t < t1 && j < j1 && finite) {
+          const int4* src = nf.mom + base + int64_t(t - leaf_start[b]) * len + j;
+#pragma unroll
+          for (int q = 0; q < kMom; ++q) cp_async(&ms[slot][q][lane], src + q * nnz);
+        }
+        cp_async_commit();
+      };
+      int slot = 0;
+      fetch(t0, 0, 0);
+      for (int t = t0; t < t1; t += 4 * nsplit) {
+        const int64_t e0 = base + int64_t(t - leaf_start[b]) * len;
+        double v;
+        if (finite) {
+          FixedSum sum[12];
+#pragma unroll
+          for (int i = 0; i < 12; ++i) sum[i] = FixedSum{0, 0};
+          for (int i = 0; i < per_row; ++i) {
+            const bool last = i + 1 == per_row;
+            fetch(last ? t + 4 * nsplit : t, last ? 0 : i + 1, slot ^ 1);
+            cp_async_wait<1>();
+            const int j = 32 * i + lane;
+            if (j0 + j < j1) {
+              int4 m[kMom], c[6];
+#pragma unroll
+              for (int q = 0; q < kMom; ++q) m[q] = ms[slot][q][lane];
+#pragma unroll
+              for (int k = 0; k < 6; ++k) c[k] = cs[k][j];
+              near_products([&](int k, const int4& a, const int4& b) { fixed_cfma<0, 0>(sum, k, a, b); }, c, m);
+              near_products([&](int k, const int4& a, const int4& b) { fixed_cfma<1, 0>(sum, k, a, b); }, c, m);
+              near_products([&](int k, const int4& a, const int4& b) { fixed_cfma<2, 0>(sum, k, a, b); }, c, m);
+              near_products([&](int k, const int4& a, const int4& b) { fixed_cfma<0, 1>(sum, k, a, b); }, c, m);
+              near_products([&](int k, const int4& a, const int4& b) { fixed_cfma<1, 1>(sum, k, a, b); }, c, m);
+              near_products([&](int k, const int4& a, const int4& b) { fixed_cfma<2, 1>(sum, k, a, b); }, c, m);
+            }
+            slot ^= 1;
+          }
+          // value = hh 2^56 + x 2^28: x carried into hh but for 28 bits below it, and
+          // the warp's totals in pieces of 27 bits
+          int p0 = 0, p1 = 0, p2 = 0, p3 = 0;
+#pragma unroll
+          for (int i = 0; i < 12; ++i) {
+            const int64_t h = sum[i].hh + (sum[i].x >> kLimb);
+            const int r0 = int(__reduce_add_sync(0xffffffffu, (uint32_t(sum[i].x) & ((1u << kLimb) - 1)) >> 1));
+            const int r1 = int(__reduce_add_sync(0xffffffffu, uint32_t(h) & ((1u << 27) - 1)));
+            const int r2 = int(__reduce_add_sync(0xffffffffu, uint32_t(h >> 27) & ((1u << 27) - 1)));
+            const int r3 = __reduce_add_sync(0xffffffffu, int(h >> 54));
+            if (lane == i) p0 = r0, p1 = r1, p2 = r2, p3 = r3;
+          }
+          // 96 bits: the totals above the point less five bits, then 5 + 27 bits
+          const uint64_t mid = (uint64_t(uint32_t(p2)) << 27) + uint32_t(p1);
+          const uint64_t low = uint64_t(uint32_t(p0)) + ((mid & 31) << 27);
+          const int64_t hi = int64_t(p3) * (int64_t(1) << 49) + int64_t(mid >> 5) + int64_t(low >> 32);
+          const FixedRow row = nf.row[t];
+          const int e = (lane < 2 ? row.mt : row.m0) + (lane < 8 ? x[1] : lane < 10 ? x[2] : x[3]) - 1075;
+          v = fixed_scale(hi, uint32_t(low), e + 2 * kLimb - 27);
+          if (row.m0 == kFixedNan) v = nan("");
+        } else {
+          v = near_row_double(nf, nnz, t, int(b), e0, j0, j1, q0, q1, leaf_start, near_idx, near_off, coef);
+        }
+        if (lane < 12) {
+          if (lane < 8) v *= mu0;
+          out[12 * int64_t(t) + lane] = j0 ? out[12 * int64_t(t) + lane] + v : v;
+        }
+      }
+      cp_async_wait_all();  // (the step past the last row: nothing in it)
+    }
+  }
+}
+
+pie_status near_fixed_prepare() {
+  static std::atomic<uint64_t> done{0};
+  int bit = -1;
+  if (device_done(done, &bit)) return PIE_OK;
+  pie_status s = cuda_check(
+      cudaFuncSetAttribute(k_near_fixed, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kFixedSmem)),
+      "near smem attribute");
+  if (s == PIE_OK && bit >= 0) done.fetch_or(uint64_t(1) << bit);
+  return s;
+}
+
+// Launch of the fixed-point near part for nrhs columns on a grid of at most
+// max_blocks (0: no bound).
+static void near_fixed(const Problem& pr, const cd* coef, cd* pot, int nrhs, int64_t max_blocks, cudaStream_t st) {
+  const FixedNear nf{static_cast<const int4*>(pr.mom), static_cast<const FixedRow*>(pr.fixed_row), pr.fixed_delta};
+  // shares per box: the least rounds of three blocks an SM, staging (about
+  // 1/50 of a box's rows) once a share; at least four test triangles each
+  const int64_t slots = 3 * int64_t(pr.nsm), most = std::min<int64_t>(16, (pr.T / pr.nleaf + 3) / 4);
+  int nsplit = 1;
+  double best = 0;
+  for (int64_t s = 1; s <= most; ++s) {
+    const double cost = double((pr.nleaf * s + slots - 1) / slots) * (1.0 / double(s) + 0.02);
+    if (s == 1 || cost < best) best = cost, nsplit = int(s);
+  }
+  int64_t grid = pr.nleaf * nsplit;
+  if (max_blocks > 0) grid = std::min(grid, max_blocks);
+  k_near_fixed<<<dim3(unsigned(grid), unsigned(nrhs)), 128, kFixedSmem, st>>>(
+      pr.nleaf, nsplit, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr, nf, coef, kMu0, pot,
+      6 * pr.T, 6 * pr.T);
 }
 
 // Antipode of half-grid sample q (theta rows 0..ntheta/2-1): -khat_q is
@@ -1151,21 +1388,21 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
       near_grid = std::min<unsigned>(near_grid, unsigned(pr.nsm * pr.tune.near_ctas_per_sm));
   }
   prof_mark(pr, 1, false, st);
-  // the near part reads each pair's moments once for RB right-hand sides
+  // the float near part reads each pair's moments once for RB right-hand sides
   // (RB chosen per call: a wide accumulator set costs occupancy when unused)
   auto near_launch = [&](auto rb) {
-    constexpr int RB = decltype(rb)::value;
-    k_near<Rm, Rio, RB, H16><<<dim3(near_grid, unsigned((nrhs + RB - 1) / RB)), 256, 0, sn>>>(
-        pr.T, pr.nnz, pr.leaf_of, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr,
-        static_cast<const C2<Rm>*>(pr.mom), static_cast<const __half2*>(pr.mom), mom_scale(pr), ncoef, Rm(kMu0),
-        pot2, nrhs, sT, sT);
+    if constexpr (sizeof(Rm) == 4)
+      k_near<Rm, Rio, decltype(rb)::value, H16><<<dim3(near_grid, nblk(nrhs, decltype(rb)::value)), 256, 0, sn>>>(
+          pr.T, pr.nnz, pr.leaf_of, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr,
+          static_cast<const C2<Rm>*>(pr.mom), static_cast<const __half2*>(pr.mom), mom_scale(pr), ncoef, Rm(kMu0),
+          pot2, nrhs, sT, sT);
   };
   // float near part: the box-staged kernel (RB 1, 2 or 4) for one column,
   // or for any pass when tune.near_kernel is 2; otherwise one warp per test
   // triangle (RB 1, 2, 4 or 8).  The box kernel measured slower on passes of
   // many columns of small meshes whose rows outgrow its staging buffer.
   int rb = pr.tune.near_rhs_block;
-  if (rb == 0) rb = nrhs == 1 ? 1 : (nrhs == 2 || sizeof(Rm) == 8) ? 2 : nrhs <= 4 ? 4 : 8;
+  if (rb == 0) rb = nrhs == 1 ? 1 : nrhs == 2 ? 2 : nrhs <= 4 ? 4 : 8;
   const bool boxed = sizeof(Rm) == 4 && (pr.tune.near_kernel == 2 || (pr.tune.near_kernel == 0 && rb == 1));
   auto box_launch = [&](auto rbc) -> pie_status {
     if constexpr (sizeof(Rm) == 4) {
@@ -1185,6 +1422,9 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
   };
   if (!with_near) {
     pot2 = nullptr;
+  } else if constexpr (sizeof(Rm) == 8) {  // PIE_FP64: fixed point, each column by itself
+    near_fixed(pr, coef, pot2, nrhs,
+               overlap && pr.tune.near_ctas_per_sm > 0 ? int64_t(pr.nsm) * ((pr.tune.near_ctas_per_sm + 1) / 2) : 0, sn);
   } else if (boxed && (rb == 1 || rb == 2 || rb == 4)) {
     pie_status s = rb == 1   ? box_launch(std::integral_constant<int, 1>())
                    : rb == 2 ? box_launch(std::integral_constant<int, 2>())
@@ -1335,21 +1575,18 @@ static pie_status apply_near_t(Problem& pr, const void* xv, void* yv, cudaStream
   const C2<Rm>* ncoef = split ? reinterpret_cast<const C2<Rm>*>(coef32) : reinterpret_cast<const C2<Rm>*>(coef);
   k_coef<Rio><<<nblk(pr.T, 256), 256, 0, st>>>(pr.T, pr.E, static_cast<const C2<Rio>*>(xv), pr.perm, pr.tri_edge,
                                                pr.tri_c, pr.tri_dcp, pr.w * pr.w * eps0(), coef, coef32);
-  bool boxed = false;  // the box-staged kernel (float near part, unless tuned off)
-  if constexpr (sizeof(Rm) == 4) {
-    if (pr.tune.near_kernel != 1) {
-      k_near_box<Rio, H16, 1><<<unsigned(pr.nleaf), kNearBoxThreads, near_box_smem<1>(), st>>>(
-          pr.nleaf, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr,
-          static_cast<const cf*>(pr.mom), static_cast<const __half2*>(pr.mom), mom_scale(pr), ncoef, float(kMu0),
-          pot);
-      boxed = true;
-    }
-  }
-  if (!boxed)
+  if constexpr (sizeof(Rm) == 8) {
+    near_fixed(pr, coef, pot, 1, 0, st);
+  } else if (pr.tune.near_kernel != 1) {  // the box-staged kernel, unless tuned off
+    k_near_box<Rio, H16, 1><<<unsigned(pr.nleaf), kNearBoxThreads, near_box_smem<1>(), st>>>(
+        pr.nleaf, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr,
+        static_cast<const cf*>(pr.mom), static_cast<const __half2*>(pr.mom), mom_scale(pr), ncoef, float(kMu0), pot);
+  } else {
     k_near<Rm, Rio, 1, H16><<<nblk(pr.T * 32, 256), 256, 0, st>>>(
         pr.T, pr.nnz, pr.leaf_of, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr,
         static_cast<const C2<Rm>*>(pr.mom), static_cast<const __half2*>(pr.mom), mom_scale(pr), ncoef, Rm(kMu0),
         pot);
+  }
   k_assemble<Rio><<<nblk(pr.N, 256), 256, 0, st>>>(pr.N, pr.E, pr.edge_tt, pr.edge_k, pr.tri_c, pr.tri_dcp,
                                                    pr.inv_perm, pot, static_cast<C2<Rio>*>(yv));
   return cuda_check(cudaGetLastError(), "apply_near launch");
@@ -1827,10 +2064,7 @@ pie_status apply_near_scratch(Problem& pr, const void* x, void* y, void* coef, v
           static_cast<const cf*>(pr.mom), nullptr, mom_scale(pr), static_cast<const cf*>(coef), float(kMu0),
           static_cast<cd*>(pot));
     else
-      k_near<double, double><<<nblk(pr.T * 32, 256), 256, 0, st>>>(
-          pr.T, pr.nnz, pr.leaf_of, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr,
-          static_cast<const cd*>(pr.mom), nullptr, mom_scale(pr), static_cast<const cd*>(coef), kMu0,
-          static_cast<cd*>(pot));
+      near_fixed(pr, static_cast<const cd*>(coef), static_cast<cd*>(pot), 1, 0, st);
     k_assemble<double><<<nblk(pr.N, 256), 256, 0, st>>>(pr.N, pr.E, pr.edge_tt, pr.edge_k, pr.tri_c, pr.tri_dcp,
                                                         pr.inv_perm, static_cast<const cd*>(pot), static_cast<cd*>(y));
   }

@@ -80,7 +80,9 @@ struct Problem {
   double* rule64 = nullptr;      // [64][4] collapsed Gauss 8 x 8
 
   // operator tables
-  void* mom = nullptr;           // [8][nnz] complex (near precision)
+  void* mom = nullptr;           // [8][nnz] complex (near precision; PIE_FP64: fixed point, near_fixed.cuh)
+  void* fixed_row = nullptr;     // PIE_FP64: [T] FixedRow, exponents of the fixed-point moments
+  int32_t* fixed_delta = nullptr;  // PIE_FP64: [nleaf]
   void* Pi = nullptr;            // [T][P/2]
   void* M = nullptr;             // [T][3][P/2] radiation tables (half grid), triangle-major
   void* PiR = nullptr;           // [P/2][T]    the same tables, sample-major (receiving side)
@@ -134,6 +136,8 @@ pie_status apply_batch(Problem& pr, const void* x, void* y, int nrhs, cudaStream
 pie_status apply_cols(Problem& pr, const void* x, void* y, int nrhs, cudaStream_t st);
 // one-time kernel attributes of the product (not allowed inside a stream capture)
 pie_status prepare_apply(Problem& pr);
+// the shared-memory limit of the fixed-point near kernel on the current device (set-up of PIE_FP64 problems)
+pie_status near_fixed_prepare();
 // records the start (end = false) or end of stage `stage` of the current apply when profiling
 void prof_mark(Problem& pr, int stage, bool end, cudaStream_t st);
 pie_status apply_near_one(Problem& pr, const void* x, void* y, cudaStream_t st);

@@ -9,7 +9,7 @@
 #include <cmath>
 #include <type_traits>
 
-#include "device.cuh"
+#include "near_fixed.cuh"
 
 namespace pie {
 
@@ -499,6 +499,70 @@ __global__ void __launch_bounds__(128) k_near_singular(int64_t npairs, int64_t n
   }
 }
 
+// delta of a leaf box (FixedRow): the exponent of its longest edge, near boxes included.
+__global__ void k_fixed_delta(int64_t nleaf, NearGeom g, int32_t* __restrict__ delta) {
+  const int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  if (b >= nleaf) return;
+  int e = -100000;
+  for (int q = g.near_ptr[b]; q < g.near_ptr[b + 1]; ++q)
+    for (int s = g.leaf_start[g.near_idx[q]] + int(threadIdx.x & 31); s < g.leaf_start[g.near_idx[q] + 1]; s += 32)
+      e = max(e, ilogb(g.h2[s]));
+  e = __reduce_max_sync(0xffffffffu, e);
+  if ((threadIdx.x & 31) == 0) delta[b] = (e >> 1) + 1;
+}
+
+// The FP64 pair moments into fixed point, in place (near_fixed.cuh): a warp per
+// row, one pass for the row's exponents and one to convert.
+__global__ void __launch_bounds__(128) k_moments_fixed(int64_t T, int64_t nnz, NearGeom g,
+                                                       const int32_t* __restrict__ delta, FixedRow* __restrict__ row,
+                                                       cd* mom) {
+  const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  if (t >= T) return;
+  const int lane = threadIdx.x & 31, dl = delta[g.leaf_of[t]];
+  const int64_t e0 = g.row_ptr[t], e1 = g.row_ptr[t + 1];
+  int x[4] = {1, 1, 1, 1};  // largest exponent fields of m0, mt, ms, mts
+  // largest sums over one lane's entries of a product stage, as they meet in a
+  // sum of the product: m0 with one ms, mt's three with mts
+  double a0 = 0, at = 0, s0 = 0, st = 0;
+  const double dw = scalbn(1.0, -dl);
+  for (int64_t e = e0 + lane; e < e1; e += 32) {
+    if (((e - e0) % kFixedStage) < 32) s0 = st = 0;
+    double v[kMom];
+#pragma unroll
+    for (int q = 0; q < kMom; ++q) {
+      const cd m = mom[q * nnz + e];
+      int& r = x[(q + 2) / 3];
+      r = max(r, max(exponent_field(m.x), exponent_field(m.y)));
+      v[q] = fabs(m.x) + fabs(m.y);
+    }
+    s0 += v[0] + dw * fmax(v[4], fmax(v[5], v[6]));
+    st += v[1] + v[2] + v[3] + dw * v[7];
+    a0 = fmax(a0, s0);
+    at = fmax(at, st);
+  }
+  int top = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    x[i] = __reduce_max_sync(0xffffffffu, x[i]);
+    top = max(top, x[i]);
+  }
+  // exponent fields: the largest integer below 2^kMomentBits, the sums below 2^kLaneBits
+  auto field = [&](int xa, int xb, double sum) {
+    const int lane_e = __reduce_max_sync(0xffffffffu, sum > 0 ? exponent_field(sum) + 53 - kLaneBits : -100000);
+    return max(max(xa, xb - dl) + 53 - kMomentBits, lane_e);
+  };
+  const int f0 = field(x[0], x[2], a0), ft = field(x[1], x[3], at);
+  if (lane == 0) row[t] = top == 0x7ff ? FixedRow{kFixedNan, kFixedNan} : FixedRow{f0 - 1075, ft - 1075};
+  for (int64_t e = e0 + lane; e < e1; e += 32)
+#pragma unroll
+    for (int q = 0; q < kMom; ++q) {
+      const cd m = mom[q * nnz + e];
+      const int f = ((q >= 1 && q <= 3) || q == 7 ? ft : f0) + (q >= 4 ? dl : 0);
+      const int2 r = fixed_encode(m.x, f), i = fixed_encode(m.y, f);
+      reinterpret_cast<int4*>(mom)[q * nnz + e] = make_int4(r.x, r.y, i.x, i.y);
+    }
+}
+
 // Leaf radiation tables at kappa_L: Pi_t(p) = int_t exp(-i kappa khat_p.(r - C_b)),
 // M_t(p) = int_t (r - c_t) exp(-i kappa khat_p.(r - C_b)); 7-point rule.
 // Called with P = the half grid (theta rows 0..ntheta/2-1): the other half
@@ -905,6 +969,15 @@ static pie_status setup_t(Problem& pr, cudaStream_t st) {
       both(std::integral_constant<int, 4>());
     else
       both(std::integral_constant<int, kNearTerms>());
+  }
+  if constexpr (sizeof(Rm) == 8) {
+    FixedRow* row = static_cast<FixedRow*>(pr.fixed_row = zalloc(pr, sizeof(FixedRow) * size_t(T), s));
+    pr.fixed_delta = static_cast<int32_t*>(zalloc(pr, sizeof(int32_t) * size_t(nleaf), s));
+    if (s == PIE_OK) s = near_fixed_prepare();
+    if (s != PIE_OK) return s;
+    k_fixed_delta<<<unsigned((nleaf * 32 + 127) / 128), 128, 0, st>>>(nleaf, ng, pr.fixed_delta);
+    k_moments_fixed<<<unsigned((T * 32 + 127) / 128), 128, 0, st>>>(T, pr.nnz, ng, pr.fixed_delta, row,
+                                                                    static_cast<cd*>(pr.mom));
   }
   if ((s = cuda_check(cudaGetLastError(), "near build")) != PIE_OK) return s;
 

@@ -14,7 +14,7 @@
 #include <complex>
 #include <vector>
 
-#include "device.cuh"
+#include "near_fixed.cuh"
 
 namespace pie {
 
@@ -36,14 +36,25 @@ __device__ int64_t near_entry(int64_t t, int64_t s, const int32_t* leaf_of, cons
   return -1;
 }
 
+// Moment q of entry e (row t of leaf box b) in double, from float or fixed-point moments.
+struct FloatNear {
+  const cf* mom;
+};
+__device__ __forceinline__ cd moment(const FloatNear& f, int64_t nnz, int q, int64_t e, int64_t, int) {
+  return cvt<double>(f.mom[q * nnz + e]);
+}
+__device__ __forceinline__ cd moment(const FixedNear& f, int64_t nnz, int q, int64_t e, int64_t t, int b) {
+  return fixed_moment(f, nnz, q, e, t, b);
+}
+
 // |Z_ii|^{-1/2} for every unknown (mesh order), from the near pair moments.
-template <typename Rm>
+template <typename Near>
 __global__ void k_diag_scale(int64_t N, int64_t E, int64_t nnz, const int32_t* __restrict__ edge_tt,
                              const int8_t* __restrict__ edge_k, const double* __restrict__ tri_c,
                              const double* __restrict__ tri_dcp, const int64_t* __restrict__ inv_perm,
                              const int32_t* __restrict__ leaf_of, const int32_t* __restrict__ leaf_start,
                              const int32_t* __restrict__ near_ptr, const int32_t* __restrict__ near_idx,
-                             const int64_t* __restrict__ row_ptr, const C2<Rm>* __restrict__ mom, double w2e,
+                             const int64_t* __restrict__ row_ptr, const Near mom, double w2e,
                              double* __restrict__ dscale) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= N) return;
@@ -58,25 +69,26 @@ __global__ void k_diag_scale(int64_t N, int64_t E, int64_t nnz, const int32_t* _
         const double* d1 = tri_dcp + 9 * t1 + 3 * k1;
         const double* d2 = tri_dcp + 9 * t2 + 3 * k2;
         double cc = kMu0 * tri_c[3 * t1 + k1] * tri_c[3 * t2 + k2];
-        C2<Rm> m0 = mom[e], mts = mom[7 * nnz + e];
-        double vr = double(mts.x), vi = double(mts.y), dd = 0;
+        const int bt = leaf_of[t1];
+        const cd m0 = moment(mom, nnz, 0, e, t1, bt), mts = moment(mom, nnz, 7, e, t1, bt);
+        double vr = mts.x, vi = mts.y, dd = 0;
         for (int d = 0; d < 3; ++d) {
-          C2<Rm> mt = mom[(1 + d) * nnz + e], ms = mom[(4 + d) * nnz + e];
-          vr += d1[d] * double(ms.x) + double(mt.x) * d2[d];
-          vi += d1[d] * double(ms.y) + double(mt.y) * d2[d];
+          const cd mt = moment(mom, nnz, 1 + d, e, t1, bt), ms = moment(mom, nnz, 4 + d, e, t1, bt);
+          vr += d1[d] * ms.x + mt.x * d2[d];
+          vi += d1[d] * ms.y + mt.y * d2[d];
           dd += d1[d] * d2[d];
         }
-        vr += dd * double(m0.x);
-        vi += dd * double(m0.y);
+        vr += dd * m0.x;
+        vi += dd * m0.y;
         zr += cc * vr;
         zi += cc * vi;
       }
   } else {
     int64_t t = inv_perm[i - E];
     int64_t e = near_entry(t, t, leaf_of, leaf_start, near_ptr, near_idx, row_ptr);
-    C2<Rm> m0 = mom[e];
-    zr = w2e * double(m0.x);
-    zi = w2e * double(m0.y);
+    const cd m0 = moment(mom, nnz, 0, e, t, leaf_of[t]);
+    zr = w2e * m0.x;
+    zi = w2e * m0.y;
   }
   double a = sqrt(zr * zr + zi * zi);
   dscale[i] = a > 0 ? 1.0 / sqrt(a) : 1.0;
@@ -84,17 +96,17 @@ __global__ void k_diag_scale(int64_t N, int64_t E, int64_t nnz, const int32_t* _
 
 // |S_tt|^{-1/2} for the single layer of Eq. (3) (pulse t in mesh order):
 // S_tt = int_t int_t g, the self-pair moment m0.
-template <typename Rm>
-__global__ void k_diag_single(int64_t T, const int64_t* __restrict__ inv_perm, const int32_t* __restrict__ leaf_of,
+template <typename Near>
+__global__ void k_diag_single(int64_t T, int64_t nnz, const int64_t* __restrict__ inv_perm, const int32_t* __restrict__ leaf_of,
                               const int32_t* __restrict__ leaf_start, const int32_t* __restrict__ near_ptr,
                               const int32_t* __restrict__ near_idx, const int64_t* __restrict__ row_ptr,
-                              const C2<Rm>* __restrict__ mom, double* __restrict__ dscale) {
+                              const Near mom, double* __restrict__ dscale) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= T) return;
   int64_t t = inv_perm[i];
   int64_t e = near_entry(t, t, leaf_of, leaf_start, near_ptr, near_idx, row_ptr);
-  C2<Rm> m0 = mom[e];
-  double a = sqrt(double(m0.x) * double(m0.x) + double(m0.y) * double(m0.y));
+  const cd m0 = moment(mom, nnz, 0, e, t, leaf_of[t]);
+  double a = sqrt(m0.x * m0.x + m0.y * m0.y);
   dscale[i] = a > 0 ? 1.0 / sqrt(a) : 1.0;
 }
 
@@ -582,21 +594,20 @@ static pie_status arnoldi_cycle(Ctx& c, C2<B>* V, Cycle& cy, double beta, double
 // |Z_ii|^{-1/2} (op 0) or |S_tt|^{-1/2} (op 1) from the near pair moments.
 static void diag_scaling(Problem& pr, int op, int64_t N, double* d, cudaStream_t st) {
   const double w2e = pr.w * pr.w * eps0();
-  if (op == 1) {
-    if (pr.near_f32())
-      k_diag_single<float><<<nb_(N, 256), 256, 0, st>>>(N, pr.inv_perm, pr.leaf_of, pr.leaf_start, pr.near_ptr,
-                                                        pr.near_idx, pr.row_ptr, static_cast<const cf*>(pr.mom), d);
+  auto scale = [&](auto near) {
+    using Near = decltype(near);
+    if (op == 1)
+      k_diag_single<Near><<<nb_(N, 256), 256, 0, st>>>(N, pr.nnz, pr.inv_perm, pr.leaf_of, pr.leaf_start, pr.near_ptr,
+                                                       pr.near_idx, pr.row_ptr, near, d);
     else
-      k_diag_single<double><<<nb_(N, 256), 256, 0, st>>>(N, pr.inv_perm, pr.leaf_of, pr.leaf_start, pr.near_ptr,
-                                                         pr.near_idx, pr.row_ptr, static_cast<const cd*>(pr.mom), d);
-  } else if (pr.near_f32())
-    k_diag_scale<float><<<nb_(N, 256), 256, 0, st>>>(N, pr.E, pr.nnz, pr.edge_tt, pr.edge_k, pr.tri_c, pr.tri_dcp,
-                                                     pr.inv_perm, pr.leaf_of, pr.leaf_start, pr.near_ptr, pr.near_idx,
-                                                     pr.row_ptr, static_cast<const cf*>(pr.mom), w2e, d);
-  else
-    k_diag_scale<double><<<nb_(N, 256), 256, 0, st>>>(N, pr.E, pr.nnz, pr.edge_tt, pr.edge_k, pr.tri_c, pr.tri_dcp,
+      k_diag_scale<Near><<<nb_(N, 256), 256, 0, st>>>(N, pr.E, pr.nnz, pr.edge_tt, pr.edge_k, pr.tri_c, pr.tri_dcp,
                                                       pr.inv_perm, pr.leaf_of, pr.leaf_start, pr.near_ptr,
-                                                      pr.near_idx, pr.row_ptr, static_cast<const cd*>(pr.mom), w2e, d);
+                                                      pr.near_idx, pr.row_ptr, near, w2e, d);
+  };
+  if (pr.near_f32())
+    scale(FloatNear{static_cast<const cf*>(pr.mom)});
+  else
+    scale(FixedNear{static_cast<const int4*>(pr.mom), static_cast<const FixedRow*>(pr.fixed_row), pr.fixed_delta});
 }
 
 // Restarted GMRES with the Krylov basis in type B (double for PIE_FP64,
