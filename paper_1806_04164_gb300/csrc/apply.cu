@@ -181,7 +181,8 @@ __global__ void __launch_bounds__(256) k_near(int64_t T, int64_t nnz, const int3
 // lanes over the row as in k_near (lane j, j + 32, ...): each moment is read
 // once for the RB right-hand sides, and every right-hand side sees the same
 // operations in the same order as in k_near, so the same result to the last
-// bit.  Rows longer than kNearStage read the coefficients from global
+// bit.  nsplit shares a box's test triangles among several blocks when the
+// leaf boxes alone do not fill the SMs.  Rows longer than kNearStage read the coefficients from global
 // memory instead.
 constexpr int kNearStage = 512;
 constexpr int kNearBoxThreads = 128;  // threads per block (per leaf box); 256 measured 8 % slower (FP32H)
@@ -191,7 +192,7 @@ constexpr size_t near_box_smem() {
 }
 template <typename Rio, bool H16, int RB>
 __global__ void __launch_bounds__(kNearBoxThreads, RB == 1 ? 6 : (RB == 2 ? 4 : 2))
-    k_near_box(int64_t nleaf, int64_t nnz, const int32_t* __restrict__ leaf_start,
+    k_near_box(int64_t nleaf, int nsplit, int64_t nnz, const int32_t* __restrict__ leaf_start,
                const int32_t* __restrict__ near_ptr, const int32_t* __restrict__ near_idx,
                const int32_t* __restrict__ near_off, const int64_t* __restrict__ row_ptr,
                const cf* __restrict__ mom, const __half2* __restrict__ momh, MomScale msc,
@@ -204,7 +205,8 @@ __global__ void __launch_bounds__(kNearBoxThreads, RB == 1 ? 6 : (RB == 2 ? 4 : 
   coef += r0 * sc;
   pot += r0 * sp;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-  for (int64_t b = blockIdx.x; b < nleaf; b += gridDim.x) {
+  for (int64_t bi = blockIdx.x; bi < nleaf * nsplit; bi += gridDim.x) {
+    const int64_t b = bi / nsplit;
     const int q0 = near_ptr[b], q1 = near_ptr[b + 1];
     const int t0 = leaf_start[b], t1 = leaf_start[b + 1];
     const int len = int(row_ptr[t0 + 1] - row_ptr[t0]);
@@ -222,7 +224,7 @@ __global__ void __launch_bounds__(kNearBoxThreads, RB == 1 ? 6 : (RB == 2 ? 4 : 
     }
     cp_async_wait_all();
     __syncthreads();
-    for (int t = t0 + warp; t < t1; t += nwarp) {
+    for (int t = t0 + int(bi % nsplit) * nwarp + warp; t < t1; t += nwarp * nsplit) {
       const int64_t e0 = row_ptr[t];
       cf acc[RB][6];
 #pragma unroll
@@ -666,6 +668,88 @@ __global__ void k_agg(int P, int ntheta, int64_t nb, const int32_t* __restrict__
   }
 }
 
+// a2 with the twenty real sums of a (box, half-grid sample) shared by several
+// threads: a thread per leaf box (threadIdx.y), sample (threadIdx.x) and sum --
+// A with one part of c (blockIdx.z even: real, odd: imaginary) or B with the
+// other (threadIdx.z) -- NC components each; the two meet in shared memory and
+// give that part of S(q) and S(-q).  Every sum runs in k_agg's order.  One
+// thread for all twenty leaves a small tree's few hundred warps on one SM
+// scheduler each, at 67 clocks a double operation: 56 leaf boxes 51 -> 15 us,
+// 272 81 -> 35 us, 4400 (double) 358 -> 336 us; from about 10,000 boxes in double
+// and 9,000 in float k_agg is as fast or faster (its loads are wider).
+template <typename Rf, int NC>
+__global__ void k_agg_split(int P, int ntheta, int64_t nb, const int32_t* __restrict__ leaf_start,
+                      const C2<Rf>* __restrict__ Pi, const C2<Rf>* __restrict__ M, const C2<Rf>* __restrict__ coef,
+                      Rf mu0, C2<Rf>* __restrict__ S, int64_t sc = 0, int64_t sS = 0) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int X = threadIdx.z, part = blockIdx.z & 1, ri = X ? 1 - part : part, c0 = NC * int(blockIdx.z >> 1);
+  const int nq = blockDim.x;
+  Rf* sums = reinterpret_cast<Rf*>(smem_raw) + threadIdx.y * 2 * NC * nq + threadIdx.x;  // [A, B][component][q]
+  const int64_t b = int64_t(blockIdx.x) * blockDim.y + threadIdx.y;
+  const bool live = b < nb;
+  const Rf* cr = reinterpret_cast<const Rf*>(coef + blockIdx.y * sc) + ri;
+  const Rf* pr = reinterpret_cast<const Rf*>(Pi) + X;
+  const Rf* mr = reinterpret_cast<const Rf*>(M) + X;
+  const int Ph = P / 2;
+  const int t0 = live ? leaf_start[b] : 0, t1 = live ? leaf_start[b + 1] : 0;
+  for (int q0 = 0; q0 < Ph; q0 += nq) {
+    const int q = q0 + threadIdx.x;
+    Rf acc[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) acc[c] = 0;
+    if (q < Ph) {
+      // UT triangles' loads together, their multiply-adds in triangle order
+      constexpr int UT = NC == 1 ? 4 : 2;
+      struct Tri {
+        Rf a, c[NC], pi, m[NC];
+      };
+      auto load = [&](int64_t t, Tri& r) {
+        r.a = cr[12 * t];
+        r.pi = pr[2 * (t * Ph + q)];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          r.c[c] = cr[12 * t + 2 * (1 + c0 + c)];
+          if (c0 + c < 3) r.m[c] = mr[2 * ((t * 3 + c0 + c) * Ph + q)];
+        }
+      };
+      auto accumulate = [&](const Tri& r) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          if (c0 + c < 3) acc[c] = fma(r.m[c], r.a, acc[c]);
+          acc[c] = fma(r.pi, r.c[c], acc[c]);
+        }
+      };
+      int t = t0;
+      for (; t + UT <= t1; t += UT) {
+        Tri r[UT];
+#pragma unroll
+        for (int u = 0; u < UT; ++u) load(t + u, r[u]);
+#pragma unroll
+        for (int u = 0; u < UT; ++u) accumulate(r[u]);
+      }
+      for (; t < t1; ++t) {
+        Tri r;
+        load(t, r);
+        accumulate(r);
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < NC; ++c) sums[(X * NC + c) * nq] = acc[c];
+    __syncthreads();
+    if (live && q < Ph) {
+      // real part: A - B at q, A + B at -q; imaginary part: A + B at q, A - B at -q
+      Rf* o = reinterpret_cast<Rf*>(S + blockIdx.y * sS + (b * kComp + c0) * P + (X ? antipode(q, ntheta) : q)) + part;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        const Rf f = c0 + c < 3 ? mu0 : Rf(1);
+        const Rf A = sums[c * nq], B = sums[(NC + c) * nq];
+        o[2 * c * P] = X == part ? f * (A - B) : f * (A + B);
+      }
+    }
+  }
+}
+
 // a3: interpolation from level l+1 to its parents at level l:
 // S_l[b] = sum_children phase_o (F S_child); one block per parent, one thread
 // per sample.  The children's patterns are staged in shared memory cg at a
@@ -804,7 +888,7 @@ __device__ __forceinline__ void fft16(C2<R>* x, C2<R>* out) {
     for (int k2 = 0; k2 < 4; ++k2) out[k1 + 4 * k2] = x[4 * k1 + k2];
 }
 
-constexpr int kFftBatch = 4;  // children per batch in the factorised filter kernels
+constexpr int kFftBatch = 4;  // (child, component) units per warp of the factorised filter kernels
 
 // Mirror-split blocks of K_m (or of K_m^T when TR) in shared memory:
 // KE[m][i][k], KO[m][i][k], i, k < NT/2.
@@ -846,11 +930,13 @@ __device__ __forceinline__ void apply_split_block(const C2<Rf>* a, const Rf* KE,
   }
 }
 
+// Shared memory of a factorised filter block of nw warps: the mirror-split K_m
+// blocks, then one region of kFftBatch spectra per warp (below 48 KB for 4).
+constexpr int kFftWarps = 4;
 template <int NT, typename Rf>
-__host__ __device__ constexpr size_t fft_smem_bytes(bool interp) {
-  constexpr int NPHI = 2 * NT, P = NT * NPHI;
-  return sizeof(C2<Rf>) * (size_t(kFftBatch) * kComp * NPHI * (NT + 1) + (interp ? size_t(kComp) * P : 0)) +
-         sizeof(Rf) * 2 * NPHI * (NT / 2) * (NT / 2);
+__host__ __device__ constexpr size_t fft_smem_bytes(int nw) {
+  constexpr int NPHI = 2 * NT;
+  return sizeof(C2<Rf>) * (size_t(kFftBatch) * nw * NPHI * (NT + 1)) + sizeof(Rf) * 2 * NPHI * (NT / 2) * (NT / 2);
 }
 
 // One K_m block in place on a spectrum column (NT theta rows, stride 1):
@@ -869,181 +955,229 @@ __device__ __forceinline__ void filter_column(C2<Rf>* col, int m, const Rf* KE, 
   apply_split_block<NT, 1>(a, KE + m * H * H, KO + m * H * H, col);
 }
 
-// a3 (factorised): one block per parent box, kFftBatch children at a time.
-// Per (child, component) one shared-memory region of NPHI x (NT+1) complex
-// holds, in turn, the row spectra [m][i], the filtered spectra (the K_m
-// blocks act in place on each column m), and the shifted child pattern, row
-// i written over the row's own spectra ([j][i]) before it is added to the
-// parent's.  Threads:
-// one per (child, component, theta row) for the DFTs, one per (child,
-// component, azimuthal frequency) for the K_m blocks.
+// a3, a5 (factorised).  A unit is one component of one child box (P
+// consecutive samples of the child level's patterns); a warp takes kFftBatch
+// consecutive units, whatever their parents, so every lane of every warp but
+// the last has work: one lane per (unit, theta row) for the DFTs, one per
+// (unit, azimuthal frequency) and turn for the K_m blocks.  (A block per parent
+// with its children four at a time ran surfaces' 3.8 children on 93 % of its
+// lanes, with block barriers between the steps.)  Per unit one shared-memory
+// region of NPHI x (NT+1) complex holds, in turn, the row spectra [m][i], the
+// filtered spectra (in place on each column m) and the result [j][i]; a warp
+// owns its regions, so the steps are separated by warp barriers only.  Blocks
+// of kFftWarps warps share the K_m tables; one warp on small levels, which
+// spreads them over the SMs.  327,680 triangles: interpolation 1.36 -> 1.15 ms,
+// anterpolation 1.40 -> 1.14 ms; 81,920: 0.44 -> 0.33 and 0.46 -> 0.33 ms.
 template <int NT, typename Rf>
-__global__ void __launch_bounds__(kFftBatch * kComp * NT, 3) k_interp_fft(
-    const int32_t* __restrict__ child_start, const int8_t* __restrict__ oct_child, const C2<Rf>* __restrict__ Sc,
-    const Rf* __restrict__ Kf, const C2<Rf>* __restrict__ phase, C2<Rf>* __restrict__ Sp, int64_t sSc = 0,
-    int64_t sSp = 0) {
-  static_assert(NT == 8, "the register DFT is the 16-point one");
-  Sc += blockIdx.y * sSc;
-  Sp += blockIdx.y * sSp;
-  constexpr int NPHI = 2 * NT, P = NT * NPHI, NB = kFftBatch, H = NT / 2;
+struct FftUnits {
+  static_assert(NT == 8 && kFftBatch * NT == 32, "16-point register DFT, one warp per kFftBatch units");
+  static constexpr int NPHI = 2 * NT, P = NT * NPHI, H = NT / 2;
   // AP: column stride of the spectra (padded by one so that lanes striding
   // over columns hit distinct banks)
-  constexpr int AP = NT + 1, REG = NPHI * AP;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C2<Rf>* A = reinterpret_cast<C2<Rf>*>(smem_raw);  // [slot][c] regions of REG complex
-  C2<Rf>* acc = A + NB * kComp * REG;                 // parent pattern [c][p]
-  Rf* KE = reinterpret_cast<Rf*>(acc + kComp * P);    // mirror-split K_m blocks
-  Rf* KO = KE + NPHI * H * H;
-  const int tid = threadIdx.x, nth = blockDim.x;
-  load_split_blocks<NT, false>(Kf, KE, KO, tid, nth);
-  for (int i = tid; i < kComp * P; i += nth) acc[i] = mk<Rf>(0, 0);
-  const int b = blockIdx.x, c0 = child_start[b], c1 = child_start[b + 1];
-  const int slot = tid / (kComp * NT), c = (tid / NT) % kComp, i = tid % NT;
-  for (int base = c0; base < c1; base += NB) {
-    const int nb = min(NB, c1 - base);
-    C2<Rf>* R = A + (slot * kComp + c) * REG;
-    __syncthreads();
-    if (slot < nb) {  // forward DFT of every row
-      C2<Rf> x[NPHI], X[NPHI];
-      const C2<Rf>* src = Sc + ((int64_t)(base + slot) * kComp + c) * P + i * NPHI;
-#pragma unroll
-      for (int j = 0; j < NPHI; ++j) x[j] = src[j];
+  static constexpr int AP = NT + 1, REG = NPHI * AP;
+  const Rf *KE, *KO;  // mirror-split K_m blocks
+  C2<Rf>* A;          // the warp's regions
+  int lane, n;        // units of the warp: first .. first + n - 1
+  int64_t first;
+  __device__ __forceinline__ FftUnits(unsigned char* smem, int64_t units) {
+    Rf* k = reinterpret_cast<Rf*>(smem);
+    KE = k;
+    KO = k + NPHI * H * H;
+    lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
+    A = reinterpret_cast<C2<Rf>*>(k + 2 * NPHI * H * H) + warp * kFftBatch * REG;
+    first = (int64_t(blockIdx.x) * (blockDim.x >> 5) + warp) * kFftBatch;
+    n = int(max(int64_t(0), min(int64_t(kFftBatch), units - first)));
+  }
+  // the lane's row x through the forward DFT, the K_m blocks and the inverse DFT
+  __device__ __forceinline__ void filter(C2<Rf>* x, C2<Rf>* X) {
+    const int slot = lane / NT, i = lane % NT;
+    C2<Rf>* R = A + slot * REG;
+    if (slot < n) {
       fft16<false>(x, X);
 #pragma unroll
       for (int m = 0; m < NPHI; ++m) R[m * AP + i] = X[m];
     }
-    __syncthreads();
-    for (int it = tid; it < nb * kComp * NPHI; it += nth)  // K_m blocks, in place
+    __syncwarp();
+    for (int it = lane; it < n * NPHI; it += 32)
       filter_column<NT>(A + (it / NPHI) * REG + (it % NPHI) * AP, it % NPHI, KE, KO);
-    __syncthreads();
-    if (slot < nb) {  // inverse DFT, phase shift to the parent centre, in the row's own column
-      C2<Rf> x[NPHI], X[NPHI];
+    __syncwarp();
+    if (slot < n) {
 #pragma unroll
       for (int m = 0; m < NPHI; ++m) x[m] = R[m * AP + i];
       fft16<true>(x, X);
-      const C2<Rf>* ph = phase + oct_child[base + slot] * P + i * NPHI;
-#pragma unroll
-      for (int j = 0; j < NPHI; ++j) R[j * AP + i] = cmul(ph[j], X[j]);
-    }
-    __syncthreads();
-    for (int k = tid; k < kComp * P; k += nth) {
-      const int cc = k / P, row = (k / NPHI) % NT, j = k % NPHI;
-      C2<Rf> v = acc[k];
-      for (int s = 0; s < nb; ++s) {
-        const C2<Rf> u = A[(s * kComp + cc) * REG + j * AP + row];
-        v.x += u.x;
-        v.y += u.y;
-      }
-      acc[k] = v;
     }
   }
-  __syncthreads();
-  for (int k = tid; k < kComp * P; k += nth) Sp[(int64_t)b * kComp * P + k] = acc[k];
-}
+  // f(sample index from the warp's first unit, value) over the regions, coalesced
+  template <typename F>
+  __device__ __forceinline__ void each(F f) {
+    __syncwarp();
+    for (int k = lane; k < n * P; k += 32) f(k, A[(k / P) * REG + (k % NPHI) * AP + (k % P) / NPHI]);
+  }
+};
 
-// a5 (factorised): one block per parent box; its children take
-// F^T (conj(phase_o) G_parent), added to their incoming patterns.  Same
-// shared-memory regions as k_interp_fft, without the parent accumulator.
+// a3: the children's patterns filtered and shifted to their parents' centres,
+// Uc[unit] = phase_o (F S_child); k_child_sum adds them up.
 template <int NT, typename Rf>
-__global__ void __launch_bounds__(kFftBatch * kComp * NT, 4) k_anterp_fft(
-    const int32_t* __restrict__ child_start, const int8_t* __restrict__ oct_child, const C2<Rf>* __restrict__ Gp,
-    const Rf* __restrict__ Kf, const C2<Rf>* __restrict__ phase, C2<Rf>* __restrict__ Gc, int64_t sGp = 0,
-    int64_t sGc = 0) {
-  static_assert(NT == 8, "the register DFT is the 16-point one");
-  Gp += blockIdx.y * sGp;
-  Gc += blockIdx.y * sGc;
-  constexpr int NPHI = 2 * NT, P = NT * NPHI, NB = kFftBatch, H = NT / 2;
-  constexpr int AP = NT + 1, REG = NPHI * AP;
+__global__ void __launch_bounds__(32 * kFftWarps, 4) k_interp_fft(int64_t units, const int8_t* __restrict__ oct_child,
+                                                                  const C2<Rf>* __restrict__ Sc,
+                                                                  const Rf* __restrict__ Kf,
+                                                                  const C2<Rf>* __restrict__ phase,
+                                                                  C2<Rf>* __restrict__ Uc, int64_t sc = 0) {
+  using Units = FftUnits<NT, Rf>;
+  constexpr int NPHI = Units::NPHI, P = Units::P;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C2<Rf>* A = reinterpret_cast<C2<Rf>*>(smem_raw);
-  Rf* KE = reinterpret_cast<Rf*>(A + NB * kComp * REG);
-  Rf* KO = KE + NPHI * H * H;
-  const int tid = threadIdx.x, nth = blockDim.x;
-  load_split_blocks<NT, true>(Kf, KE, KO, tid, nth);
-  const int b = blockIdx.x, c0 = child_start[b], c1 = child_start[b + 1];
-  const int slot = tid / (kComp * NT), c = (tid / NT) % kComp, i = tid % NT;
-  for (int base = c0; base < c1; base += NB) {
-    const int nb = min(NB, c1 - base);
-    C2<Rf>* R = A + (slot * kComp + c) * REG;
-    __syncthreads();
-    if (slot < nb) {
-      C2<Rf> x[NPHI], X[NPHI];
-      const C2<Rf>* src = Gp + ((int64_t)b * kComp + c) * P + i * NPHI;
-      const C2<Rf>* ph = phase + oct_child[base + slot] * P + i * NPHI;
+  Units w(smem_raw, units);
+  load_split_blocks<NT, false>(Kf, const_cast<Rf*>(w.KE), const_cast<Rf*>(w.KO), threadIdx.x, blockDim.x);
+  __syncthreads();
+  Sc += blockIdx.y * sc + w.first * P;
+  Uc += blockIdx.y * sc + w.first * P;
+  const int slot = w.lane / NT, i = w.lane % NT;
+  C2<Rf> x[NPHI], X[NPHI];
+  if (slot < w.n) {
 #pragma unroll
-      for (int j = 0; j < NPHI; ++j) {
-        C2<Rf> g = src[j], w = ph[j];
-        x[j] = mk<Rf>(w.x * g.x + w.y * g.y, w.x * g.y - w.y * g.x);  // conj(w) g
-      }
-      fft16<false>(x, X);
-#pragma unroll
-      for (int m = 0; m < NPHI; ++m) R[m * AP + i] = X[m];
-    }
-    __syncthreads();
-    for (int it = tid; it < nb * kComp * NPHI; it += nth)  // transposed K_m blocks, in place
-      filter_column<NT>(A + (it / NPHI) * REG + (it % NPHI) * AP, it % NPHI, KE, KO);
-    __syncthreads();
-    if (slot < nb) {
-      C2<Rf> x[NPHI], X[NPHI];
-#pragma unroll
-      for (int m = 0; m < NPHI; ++m) x[m] = R[m * AP + i];
-      fft16<true>(x, X);
-      C2<Rf>* dst = Gc + ((int64_t)(base + slot) * kComp + c) * P + i * NPHI;
-#pragma unroll
-      for (int j = 0; j < NPHI; ++j) {
-        C2<Rf> g = dst[j];
-        dst[j] = mk<Rf>(g.x + X[j].x, g.y + X[j].y);
-      }
-    }
+    for (int j = 0; j < NPHI; ++j) x[j] = Sc[slot * P + i * NPHI + j];
   }
+  w.filter(x, X);
+  if (slot < w.n) {  // phase shift to the parent centre, in the row's own spectra
+    const C2<Rf>* ph = phase + oct_child[(w.first + slot) / kComp] * P + i * NPHI;
+#pragma unroll
+    for (int j = 0; j < NPHI; ++j) w.A[slot * Units::REG + j * Units::AP + i] = cmul(ph[j], X[j]);
+  }
+  w.each([&](int k, C2<Rf> v) { Uc[k] = v; });
 }
 
-// a4: translation at one level: G[d] = sum_{s in IL(d)} T[off] * S[s];
-// one destination box per threadIdx.y row of a block (several rows for small
-// angular grids), one thread per sample, five components.  In float the
-// list is walked U = 4 entries at a time: their loads are issued together
-// and the multiply-adds follow in list order (the order of the one-entry
-// loop), so a thread waits for one load latency per four entries instead of
-// per entry (the small-grid float levels are latency-bound).  In double the
-// FP64 pipe bounds the kernel and U = 1 (measured: U = 2 was 0.5 % slower).
+// The sum over a parent's children, in order: one thread per (parent,
+// component, sample), blocks of (P samples, one component).
 template <typename Rf>
-__global__ void k_trans(int P, int64_t nb, const int32_t* __restrict__ il_ptr, const int32_t* __restrict__ il_idx,
-                        const int32_t* __restrict__ il_off, const C2<Rf>* __restrict__ Tt,
-                        const C2<Rf>* __restrict__ S, C2<Rf>* __restrict__ G, int64_t sS = 0) {
-  constexpr int U = sizeof(Rf) == 4 ? 4 : 1;
-  const int64_t d = int64_t(blockIdx.x) * blockDim.y + threadIdx.y;
-  if (d >= nb) return;
-  S += blockIdx.y * sS;
-  G += blockIdx.y * sS;
-  const int j0 = il_ptr[d], j1 = il_ptr[d + 1];
-  for (int p = threadIdx.x; p < P; p += blockDim.x) {
-    C2<Rf> acc[kComp];
+__global__ void k_child_sum(int P, const int32_t* __restrict__ child_start, const C2<Rf>* __restrict__ Uc,
+                            C2<Rf>* __restrict__ Sp, int64_t sc = 0, int64_t sp = 0) {
+  const int64_t b = blockIdx.x;
+  const int k = blockIdx.z * P + threadIdx.x;
+  Uc += blockIdx.y * sc;
+  C2<Rf> v = mk<Rf>(0, 0);
+  const int c1 = child_start[b + 1];
+#pragma unroll 4
+  for (int c = child_start[b]; c < c1; ++c) {
+    const C2<Rf> u = Uc[(int64_t)c * kComp * P + k];
+    v.x += u.x;
+    v.y += u.y;
+  }
+  Sp[blockIdx.y * sp + b * kComp * P + k] = v;
+}
+
+// a5: children take F^T (conj(phase_o) G_parent), added to their incoming patterns.
+template <int NT, typename Rf>
+__global__ void __launch_bounds__(32 * kFftWarps, 4)
+    k_anterp_fft(int64_t units, const int32_t* __restrict__ parent, const int8_t* __restrict__ oct_child,
+                 const C2<Rf>* __restrict__ Gp, const Rf* __restrict__ Kf, const C2<Rf>* __restrict__ phase,
+                 C2<Rf>* __restrict__ Gc, int64_t sGp = 0, int64_t sGc = 0) {
+  using Units = FftUnits<NT, Rf>;
+  constexpr int NPHI = Units::NPHI, P = Units::P;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  Units w(smem_raw, units);
+  load_split_blocks<NT, true>(Kf, const_cast<Rf*>(w.KE), const_cast<Rf*>(w.KO), threadIdx.x, blockDim.x);
+  __syncthreads();
+  const int slot = w.lane / NT, i = w.lane % NT;
+  C2<Rf> x[NPHI], X[NPHI];
+  if (slot < w.n) {
+    const int64_t ch = (w.first + slot) / kComp, c = (w.first + slot) % kComp;
+    const C2<Rf>* src = Gp + blockIdx.y * sGp + (int64_t(parent[ch]) * kComp + c) * P + i * NPHI;
+    const C2<Rf>* ph = phase + oct_child[ch] * P + i * NPHI;
 #pragma unroll
-    for (int c = 0; c < kComp; ++c) acc[c] = mk<Rf>(0, 0);
+    for (int j = 0; j < NPHI; ++j) {
+      C2<Rf> g = src[j], w = ph[j];
+      x[j] = mk<Rf>(w.x * g.x + w.y * g.y, w.x * g.y - w.y * g.x);  // conj(w) g
+    }
+  }
+  w.filter(x, X);
+  if (slot < w.n) {
+#pragma unroll
+    for (int j = 0; j < NPHI; ++j) w.A[slot * Units::REG + j * Units::AP + i] = X[j];
+  }
+  Gc += blockIdx.y * sGc + w.first * P;
+  w.each([&](int k, C2<Rf> v) {
+    const C2<Rf> g = Gc[k];
+    Gc[k] = mk<Rf>(g.x + v.x, g.y + v.y);
+  });
+}
+
+// The levels of one translation launch, most boxes first (the leaf level's
+// blocks start first, the coarse levels fill in behind them).
+constexpr int kMaxTrans = 19;  // levels 3 .. 21
+struct TransLevel {
+  int64_t first;  // number of the level's first box in the launch
+  const int32_t *ptr, *idx, *off;
+  const void* T;
+  const void* S;
+  void* G;
+  int64_t stride;  // between right-hand sides
+};
+struct TransArgs {
+  int n = 0;
+  int64_t total = 0;
+  TransLevel l[kMaxTrans];
+};
+__device__ __forceinline__ int trans_level(const TransArgs& a, int64_t box) {
+  int k = 0;
+  while (k + 1 < a.n && box >= a.l[k + 1].first) ++k;
+  return k;
+}
+
+// a4: translation, all levels at once: G[d] = sum_{s in IL(d)} T[off] * S[s];
+// one destination box per threadIdx.y row of a block (several rows for small
+// angular grids), one thread per sample and NC components (the others in
+// blockIdx.z: five components a thread where the boxes fill the SMs, one on
+// small trees).  In float the list is walked U = 4 entries at a time: their
+// loads are issued together and the multiply-adds follow in list order (the
+// order of the one-entry loop), so a thread waits for one load latency per
+// four entries instead of per entry (the small-grid float levels are
+// latency-bound).  In double the FP64 pipe bounds the kernel and U = 1
+// (measured: U = 2 was 0.5 % slower).  With a launch per level the coarse levels
+// left most SMs idle in turn: 327,680 triangles (double) 4.58 -> 4.40 ms, 81,920
+// 1.25 -> 1.12 ms, 56 boxes 46 -> 20 us, float patterns of 32 samples at 327,680
+// triangles 135 -> 97 us.
+template <typename Rf, int NC>
+__global__ void k_trans(int P, const TransArgs args) {
+  constexpr int U = sizeof(Rf) == 4 ? 4 : 1;
+  const int64_t box = int64_t(blockIdx.x) * blockDim.y + threadIdx.y;
+  if (box >= args.total) return;
+  const TransLevel& lv = args.l[trans_level(args, box)];
+  const int64_t d = box - lv.first;
+  const int32_t* __restrict__ il_idx = lv.idx;
+  const int32_t* __restrict__ il_off = lv.off;
+  const C2<Rf>* __restrict__ Tt = static_cast<const C2<Rf>*>(lv.T);
+  const C2<Rf>* __restrict__ S = static_cast<const C2<Rf>*>(lv.S) + blockIdx.y * lv.stride + blockIdx.z * NC * P;
+  C2<Rf>* __restrict__ G = static_cast<C2<Rf>*>(lv.G) + blockIdx.y * lv.stride + blockIdx.z * NC * P;
+  const int j0 = lv.ptr[d], j1 = lv.ptr[d + 1];
+  for (int p = threadIdx.x; p < P; p += blockDim.x) {
+    C2<Rf> acc[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) acc[c] = mk<Rf>(0, 0);
     int j = j0;
     for (; j + U <= j1; j += U) {
-      C2<Rf> tv[U], sv[U][kComp];
+      C2<Rf> tv[U], sv[U][NC];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         tv[u] = Tt[(int64_t)il_off[j + u] * P + p];
         const C2<Rf>* src = S + (int64_t)il_idx[j + u] * kComp * P + p;
 #pragma unroll
-        for (int c = 0; c < kComp; ++c) sv[u][c] = src[c * P];
+        for (int c = 0; c < NC; ++c) sv[u][c] = src[c * P];
       }
 #pragma unroll
       for (int u = 0; u < U; ++u)
 #pragma unroll
-        for (int c = 0; c < kComp; ++c) cfma(acc[c], tv[u], sv[u][c]);
+        for (int c = 0; c < NC; ++c) cfma(acc[c], tv[u], sv[u][c]);
     }
     for (; j < j1; ++j) {
       int s = il_idx[j];
       C2<Rf> tv = Tt[(int64_t)il_off[j] * P + p];
       const C2<Rf>* src = S + (int64_t)s * kComp * P + p;
 #pragma unroll
-      for (int c = 0; c < kComp; ++c) cfma(acc[c], tv, src[c * P]);
+      for (int c = 0; c < NC; ++c) cfma(acc[c], tv, src[c * P]);
     }
 #pragma unroll
-    for (int c = 0; c < kComp; ++c) G[((int64_t)d * kComp + c) * P + p] = acc[c];
+    for (int c = 0; c < NC; ++c) G[((int64_t)d * kComp + c) * P + p] = acc[c];
   }
 }
 
@@ -1055,65 +1189,67 @@ __global__ void k_trans(int P, int64_t nb, const int32_t* __restrict__ il_ptr, c
 // this shortens the chain of dependent loads a thread waits through.  The
 // order of operations depends on the list alone, never on the launch shape.
 constexpr int kTransSplit = 4;
-template <typename Rf>
-__global__ void k_trans_split(int P, int64_t nb, const int32_t* __restrict__ il_ptr,
-                              const int32_t* __restrict__ il_idx, const int32_t* __restrict__ il_off,
-                              const C2<Rf>* __restrict__ Tt, const C2<Rf>* __restrict__ S, C2<Rf>* __restrict__ G,
-                              int64_t sS = 0) {
+template <typename Rf, int NC>
+__global__ void k_trans_split(int P, const TransArgs args) {
   constexpr int U = 4;
   extern __shared__ unsigned char smem_raw[];
   C2<Rf>* part = reinterpret_cast<C2<Rf>*>(smem_raw);  // [row][chunk][component][P]
   const int r = threadIdx.y / kTransSplit, k = threadIdx.y % kTransSplit, p = threadIdx.x;
-  const int64_t d = int64_t(blockIdx.x) * (blockDim.y / kTransSplit) + r;
-  const bool live = d < nb && p < P;
-  S += blockIdx.y * sS;
-  G += blockIdx.y * sS;
-  C2<Rf> acc[kComp];
+  const int64_t box = int64_t(blockIdx.x) * (blockDim.y / kTransSplit) + r;
+  const bool live = box < args.total && p < P;
+  const TransLevel& lv = args.l[trans_level(args, min(box, args.total - 1))];
+  const int64_t d = box - lv.first;
+  const int32_t* __restrict__ il_idx = lv.idx;
+  const int32_t* __restrict__ il_off = lv.off;
+  const C2<Rf>* __restrict__ Tt = static_cast<const C2<Rf>*>(lv.T);
+  const C2<Rf>* __restrict__ S = static_cast<const C2<Rf>*>(lv.S) + blockIdx.y * lv.stride + blockIdx.z * NC * P;
+  C2<Rf>* __restrict__ G = static_cast<C2<Rf>*>(lv.G) + blockIdx.y * lv.stride + blockIdx.z * NC * P;
+  C2<Rf> acc[NC];
 #pragma unroll
-  for (int c = 0; c < kComp; ++c) acc[c] = mk<Rf>(0, 0);
+  for (int c = 0; c < NC; ++c) acc[c] = mk<Rf>(0, 0);
   if (live) {
-    const int j0 = il_ptr[d], len = il_ptr[d + 1] - j0;
+    const int j0 = lv.ptr[d], len = lv.ptr[d + 1] - j0;
     const int q = (len + kTransSplit - 1) / kTransSplit;
     const int a = j0 + min(len, k * q), b = j0 + min(len, (k + 1) * q);
     int j = a;
     for (; j + U <= b; j += U) {
-      C2<Rf> tv[U], sv[U][kComp];
+      C2<Rf> tv[U], sv[U][NC];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         tv[u] = Tt[(int64_t)il_off[j + u] * P + p];
         const C2<Rf>* src = S + (int64_t)il_idx[j + u] * kComp * P + p;
 #pragma unroll
-        for (int c = 0; c < kComp; ++c) sv[u][c] = src[c * P];
+        for (int c = 0; c < NC; ++c) sv[u][c] = src[c * P];
       }
 #pragma unroll
       for (int u = 0; u < U; ++u)
 #pragma unroll
-        for (int c = 0; c < kComp; ++c) cfma(acc[c], tv[u], sv[u][c]);
+        for (int c = 0; c < NC; ++c) cfma(acc[c], tv[u], sv[u][c]);
     }
     for (; j < b; ++j) {
       C2<Rf> tv = Tt[(int64_t)il_off[j] * P + p];
       const C2<Rf>* src = S + (int64_t)il_idx[j] * kComp * P + p;
 #pragma unroll
-      for (int c = 0; c < kComp; ++c) cfma(acc[c], tv, src[c * P]);
+      for (int c = 0; c < NC; ++c) cfma(acc[c], tv, src[c * P]);
     }
   }
-  C2<Rf>* mine = part + ((int64_t)(r * kTransSplit + k) * kComp) * P;
+  C2<Rf>* mine = part + ((int64_t)(r * kTransSplit + k) * NC) * P;
   if (p < P && k > 0)
 #pragma unroll
-    for (int c = 0; c < kComp; ++c) mine[c * P + p] = acc[c];
+    for (int c = 0; c < NC; ++c) mine[c * P + p] = acc[c];
   __syncthreads();
   if (!live || k > 0) return;
 #pragma unroll
   for (int kk = 1; kk < kTransSplit; ++kk) {
-    const C2<Rf>* o = part + ((int64_t)(r * kTransSplit + kk) * kComp) * P;
+    const C2<Rf>* o = part + ((int64_t)(r * kTransSplit + kk) * NC) * P;
 #pragma unroll
-    for (int c = 0; c < kComp; ++c) {
+    for (int c = 0; c < NC; ++c) {
       acc[c].x += o[c * P + p].x;
       acc[c].y += o[c * P + p].y;
     }
   }
 #pragma unroll
-  for (int c = 0; c < kComp; ++c) G[((int64_t)d * kComp + c) * P + p] = acc[c];
+  for (int c = 0; c < NC; ++c) G[((int64_t)d * kComp + c) * P + p] = acc[c];
 }
 
 // a5: anterpolation from level l to level l+1:
@@ -1259,6 +1395,104 @@ __global__ void __launch_bounds__(256) k_disagg(int64_t T, int P, const int32_t*
   for (int i = 0; i < 6; ++i) o[i] = mk<Rio>(Rio(acc[i].x), Rio(acc[i].y));
 }
 
+// a6 with the twelve real sums of a triangle shared by five threads
+// (threadIdx.y, one warp each for the block's 32 triangles): U real, U
+// imaginary, the three V real, the three V imaginary, T1 and T2; 6, 6, 6, 6 and
+// 8 multiply-adds a sample pair, each sum in k_disagg's order.  In double a
+// warp's multiply-add occupies an SM scheduler for 67 clocks, so k_disagg's
+// 2048 of them a triangle run one after the other on as many schedulers as
+// there are warps of triangles (with the sum / difference patterns: 1280
+// triangles 140 -> 36 us, 11,250 172 -> 63 us, 81,920 426 -> 322 us, 327,680
+// 1232 -> 1204 us).  Float patterns of many triangles keep k_disagg, which reads
+// each table entry once.
+template <typename Rf, typename Rio>
+__global__ void __launch_bounds__(160) k_disagg_split(int64_t T, int P, const int32_t* __restrict__ leaf_of,
+                                                      const C2<Rf>* __restrict__ PiR, const C2<Rf>* __restrict__ MR,
+                                                      const C2<Rf>* __restrict__ GS, const C2<Rf>* __restrict__ GD,
+                                                      C2<Rio>* __restrict__ pot, int64_t sH = 0, int64_t sp = 0) {
+  const int64_t t = blockIdx.x * (int64_t)32 + threadIdx.x;
+  if (t >= T) return;
+  const int Ph = P / 2;
+  const Rf* gs = reinterpret_cast<const Rf*>(GS + blockIdx.y * sH + (int64_t)leaf_of[t] * kComp * Ph);
+  const Rf* gd = reinterpret_cast<const Rf*>(GD + blockIdx.y * sH + (int64_t)leaf_of[t] * kComp * Ph);
+  Rio* o = reinterpret_cast<Rio*>(pot + blockIdx.y * sp + 6 * t);
+  // NS sums over the sample pairs: load(q, d) gives the operands of sum (or
+  // step) d, step(d) its two multiply-adds; four sample pairs' loads are issued
+  // ahead of the four being summed
+  struct Op {
+    C2<Rf> x;
+    Rf s, d;
+  };
+  auto run = [&](auto n, auto load, auto step) {
+    constexpr int N = decltype(n)::value, U = sizeof(Rf) == 8 ? 2 : 4;
+    Op a[U][N], b[U][N];
+    auto fetch = [&](int q, Op(&v)[U][N]) {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (q + u < Ph)
+#pragma unroll
+          for (int d = 0; d < N; ++d) v[u][d] = load(q + u, d);
+    };
+    auto sum = [&](int q, const Op(&v)[U][N]) {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (q + u < Ph)
+#pragma unroll
+          for (int d = 0; d < N; ++d) step(d, v[u][d]);
+    };
+    fetch(0, a);
+    for (int q = 0; q < Ph; q += 2 * U) {
+      fetch(q + U, b);
+      sum(q, a);
+      fetch(q + 2 * U, a);
+      sum(q + U, b);
+    }
+  };
+  auto at = [&](const Rf* g, int c, int q, int im) { return g[2 * (c * Ph + q) + im]; };
+  // im = 0: real part, += x.x s.x + x.y d.y; im = 1: imaginary part, += x.x s.y - x.y d.x
+  auto U = [&](auto imc) {
+    constexpr int im = decltype(imc)::value;
+    Rf u = 0;
+    run(
+        std::integral_constant<int, 3>(),
+        [&](int q, int d) { return Op{MR[((int64_t)d * Ph + q) * T + t], at(gs, d, q, im), at(gd, d, q, 1 - im)}; },
+        [&](int, const Op& v) {
+          u = fma(v.x.x, v.s, u);
+          u = fma(im ? -v.x.y : v.x.y, v.d, u);
+        });
+    o[im] = Rio(u);
+  };
+  auto V = [&](auto imc) {
+    constexpr int im = decltype(imc)::value;
+    Rf v[3] = {0, 0, 0};
+    run(
+        std::integral_constant<int, 3>(),
+        [&](int q, int d) { return Op{PiR[(int64_t)q * T + t], at(gs, d, q, im), at(gd, d, q, 1 - im)}; },
+        [&](int d, const Op& w) {
+          v[d] = fma(w.x.x, w.s, v[d]);
+          v[d] = fma(im ? -w.x.y : w.x.y, w.d, v[d]);
+        });
+#pragma unroll
+    for (int d = 0; d < 3; ++d) o[2 + 2 * d + im] = Rio(v[d]);
+  };
+  switch (threadIdx.y) {
+    case 0: return U(std::integral_constant<int, 0>());
+    case 1: return U(std::integral_constant<int, 1>());
+    case 2: return V(std::integral_constant<int, 0>());
+    case 3: return V(std::integral_constant<int, 1>());
+  }
+  Rf v[4] = {0, 0, 0, 0};  // T1 real, imaginary, T2 real, imaginary
+  run(
+      std::integral_constant<int, 4>(),
+      [&](int q, int d) { return Op{PiR[(int64_t)q * T + t], at(gs, 3 + d / 2, q, d % 2), at(gd, 3 + d / 2, q, 1 - d % 2)}; },
+      [&](int d, const Op& w) {
+        v[d] = fma(w.x.x, w.s, v[d]);
+        v[d] = fma(d % 2 ? -w.x.y : w.x.y, w.d, v[d]);
+      });
+#pragma unroll
+  for (int d = 0; d < 4; ++d) o[8 + d] = Rio(v[d]);
+}
+
 // Per-triangle potential j of the product: near + far (each rounded to the
 // io precision, summed in double, rounded again), or pot alone.
 template <typename Rio>
@@ -1309,6 +1543,13 @@ __global__ void k_assemble(int64_t N, int64_t E, const int32_t* __restrict__ edg
 
 static inline unsigned nblk(int64_t n, int b) { return unsigned((n + b - 1) / b); }
 
+// Blocks per leaf box of k_near_box: enough to give an SM its six, at least
+// four test triangles each.
+static int near_box_split(const Problem& pr) {
+  const int64_t want = (6 * int64_t(pr.nsm) + pr.nleaf - 1) / pr.nleaf, most = (pr.T / pr.nleaf + 3) / 4;
+  return int(std::max<int64_t>(1, std::min({want, most, int64_t(16)})));
+}
+
 static inline MomScale mom_scale(const Problem& pr) {
   MomScale m;
   for (int q = 0; q < kMom; ++q) m.s[q] = pr.mom_scale[q];
@@ -1318,28 +1559,6 @@ static inline MomScale mom_scale(const Problem& pr) {
 void prof_mark(Problem& pr, int stage, bool end, cudaStream_t st) {
   if (pr.prof_n >= pr.prof_cap) return;
   cudaEventRecord(pr.prof_ev[(size_t(pr.prof_n) * kStages + stage) * 2 + (end ? 1 : 0)], st);
-}
-
-template <int NT, typename Rf>
-static size_t fft_smem(bool interp) {
-  return fft_smem_bytes<NT, Rf>(interp);
-}
-
-// Opt the factorised filter kernels into their (above 48 KB) dynamic shared memory.
-template <int NT, typename Rf>
-static pie_status fft_prepare() {
-  static std::atomic<uint64_t> done{0};  // per device, as near_box_prepare
-  int bit = -1;
-  if (device_done(done, &bit)) return PIE_OK;
-  pie_status s = cuda_check(cudaFuncSetAttribute(k_interp_fft<NT, Rf>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 int(fft_smem<NT, Rf>(true))),
-                            "smem attribute");
-  if (s == PIE_OK)
-    s = cuda_check(cudaFuncSetAttribute(k_anterp_fft<NT, Rf>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        int(fft_smem<NT, Rf>(false))),
-                   "smem attribute");
-  if (s == PIE_OK && bit >= 0) done.fetch_or(uint64_t(1) << bit);
-  return s;
 }
 
 template <typename Rm, typename Rf, typename Rio, bool H16 = false>
@@ -1409,11 +1628,12 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
       constexpr int RB = decltype(rbc)::value;
       pie_status s = near_box_prepare<Rio, H16, RB>();
       if (s != PIE_OK) return s;
-      unsigned grid = unsigned(pr.nleaf);
+      const int nsplit = near_box_split(pr);
+      unsigned grid = unsigned(pr.nleaf * nsplit);
       if (overlap && pr.tune.near_ctas_per_sm > 0)  // in CTAs of 256 threads per SM
         grid = std::min<unsigned>(grid, unsigned(pr.nsm * pr.tune.near_ctas_per_sm * (256 / kNearBoxThreads)));
       k_near_box<Rio, H16, RB><<<dim3(grid, unsigned((nrhs + RB - 1) / RB)), kNearBoxThreads, near_box_smem<RB>(),
-                                 sn>>>(pr.nleaf, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off,
+                                 sn>>>(pr.nleaf, nsplit, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off,
                                        pr.row_ptr, static_cast<const cf*>(pr.mom),
                                        static_cast<const __half2*>(pr.mom), mom_scale(pr),
                                        reinterpret_cast<const cf*>(ncoef), float(kMu0), pot2, nrhs, sT, sT);
@@ -1456,13 +1676,32 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
     const int r = pr.tune.far_rows > 0 ? pr.tune.far_rows : (threads < 64 ? 128 / threads : 1);
     return std::max(1, std::min(r, 1024 / threads));
   };
+  // grids of fewer warps than kWideWarps an SM (eight a scheduler) give each
+  // warp less to do (components and sums over more threads); the arithmetic
+  // stays the same
+  constexpr int kWideWarps = 32;
+  auto narrow = [&](int64_t warps) { return warps < int64_t(kWideWarps) * pr.nsm; };
   {
     // half-grid threads per box
     const int ath = P / 2 < 32 ? P / 2 : ((P / 2 + 31) / 32) * 32;
-    const int abp = far_rows(ath);
-    k_agg<Rf><<<dim3(nblk(pr.lev[L].nb, abp), nr), dim3(ath, abp), 0, sf>>>(
-        P, pr.par.ntheta, pr.lev[L].nb, pr.leaf_start, Pi, M, fcoef, Rf(kMu0), static_cast<C2<Rf>*>(pr.lev[L].S),
-        sT, sl(L));
+    const int64_t warps = (pr.lev[L].nb * ath + 31) / 32 * nr;  // of the whole-sample kernel
+    C2<Rf>* SL = static_cast<C2<Rf>*>(pr.lev[L].S);
+    auto split = [&](auto ncc) {
+      constexpr int NC = decltype(ncc)::value;
+      const int sth = std::min(512, ath), abp = std::max(1, std::min(far_rows(2 * sth), 512 / sth));
+      k_agg_split<Rf, NC><<<dim3(nblk(pr.lev[L].nb, abp), nr, 2 * kComp / NC), dim3(sth, abp, 2),
+                            sizeof(Rf) * 2 * NC * sth * abp, sf>>>(P, pr.par.ntheta, pr.lev[L].nb, pr.leaf_start, Pi,
+                                                                   M, fcoef, Rf(kMu0), SL, sT, sl(L));
+    };
+    if (narrow(2 * warps)) {
+      split(std::integral_constant<int, 1>());
+    } else if (narrow(sizeof(Rf) == 8 ? warps / 4 : warps)) {
+      split(std::integral_constant<int, kComp>());
+    } else {
+      const int abp = far_rows(ath);
+      k_agg<Rf><<<dim3(nblk(pr.lev[L].nb, abp), nr), dim3(ath, abp), 0, sf>>>(
+          P, pr.par.ntheta, pr.lev[L].nb, pr.leaf_start, Pi, M, fcoef, Rf(kMu0), SL, sT, sl(L));
+    }
   }
   prof_mark(pr, 2, true, st);
   const size_t sm = sizeof(C2<Rf>) * kComp * P;
@@ -1475,16 +1714,19 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
   const int fbp = std::max(1, std::min(far_rows(tpb), int((49152 - fsm_bytes) / sm)));
   const int cg = int(std::max<size_t>(1, std::min<size_t>(8, (49152 - fsm_bytes) / (sm * fbp))));
   const bool fft8 = pr.par.ntheta == 8;
-  if (fft8) {
-    pie_status s = fft_prepare<8, Rf>();
-    if (s != PIE_OK) return s;
-  }
   prof_mark(pr, 3, false, st);
+  // units of the factorised filter between level l and its children, and warps per block
+  auto fft_units = [&](int l) { return pr.lev[l + 1].nb * kComp; };
+  auto fft_nw = [&](int l) { return narrow(fft_units(l) / kFftBatch * nr) ? 1 : kFftWarps; };
   for (int l = L - 1; l >= 3 && fft8; --l) {
-    k_interp_fft<8, Rf><<<dim3(unsigned(pr.lev[l].nb), nr), kFftBatch * kComp * 8, fft_smem<8, Rf>(true), sf>>>(
-        pr.lev[l].child_start, pr.lev[l + 1].octant, static_cast<const C2<Rf>*>(pr.lev[l + 1].S),
-        static_cast<const Rf*>(pr.lev[l].Kf), static_cast<const C2<Rf>*>(pr.lev[l].phase),
-        static_cast<C2<Rf>*>(pr.lev[l].S), sl(l + 1), sl(l));
+    const int nw = fft_nw(l);
+    // the shifted child patterns pass through the child level's G, free until the translation
+    C2<Rf>* U = static_cast<C2<Rf>*>(pr.lev[l + 1].G);
+    k_interp_fft<8, Rf><<<dim3(nblk(fft_units(l), kFftBatch * nw), nr), 32 * nw, fft_smem_bytes<8, Rf>(nw), sf>>>(
+        fft_units(l), pr.lev[l + 1].octant, static_cast<const C2<Rf>*>(pr.lev[l + 1].S),
+        static_cast<const Rf*>(pr.lev[l].Kf), static_cast<const C2<Rf>*>(pr.lev[l].phase), U, sl(l + 1));
+    k_child_sum<Rf><<<dim3(unsigned(pr.lev[l].nb), nr, kComp), P, 0, sf>>>(
+        P, pr.lev[l].child_start, U, static_cast<C2<Rf>*>(pr.lev[l].S), sl(l + 1), sl(l));
   }
   for (int l = L - 1; l >= 3 && !fft8; --l) {
     k_interp<Rf><<<dim3(nblk(pr.lev[l].nb, fbp), nr), dim3(tpb, fbp), fsm_bytes + sm * fbp * cg, sf>>>(
@@ -1494,37 +1736,43 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
   }
   prof_mark(pr, 3, true, st);
   prof_mark(pr, 4, false, st);
-  for (int l = 3; l <= L; ++l) {
+  TransArgs ta;
+  for (int l = L; l >= 3; --l) {
     if (!((pr.far_mask >> l) & 1u)) {  // level left out: no incoming pattern of its own
       pie_status s = cuda_check(cudaMemsetAsync(pr.lev[l].G, 0, sizeof(C2<Rf>) * sl(l) * nr, sf), "memset");
       if (s != PIE_OK) return s;
       continue;
     }
-    bool split_done = false;
-    if constexpr (sizeof(Rf) == 4) {
-      if (tpb <= 128) {  // float, small grid: each list cut into kTransSplit chunks
-        const int tbp = far_rows(tpb * kTransSplit);
-        k_trans_split<Rf><<<dim3(nblk(pr.lev[l].nb, tbp), nr), dim3(tpb, tbp * kTransSplit),
-                            sizeof(C2<Rf>) * kComp * P * kTransSplit * tbp, sf>>>(
-            P, pr.lev[l].nb, pr.lev[l].il_ptr, pr.lev[l].il_idx, pr.lev[l].il_off,
-            static_cast<const C2<Rf>*>(pr.lev[l].trans), static_cast<const C2<Rf>*>(pr.lev[l].S),
-            static_cast<C2<Rf>*>(pr.lev[l].G), sl(l));
-        split_done = true;
-      }
-    }
-    if (!split_done) {
+    ta.l[ta.n++] = TransLevel{ta.total,       pr.lev[l].il_ptr, pr.lev[l].il_idx, pr.lev[l].il_off,
+                              pr.lev[l].trans, pr.lev[l].S,      pr.lev[l].G,      sl(l)};
+    ta.total += pr.lev[l].nb;
+  }
+  if (ta.total > 0) {
+    // per right-hand side: components a thread takes
+    const bool one = narrow(ta.total * (tpb / 32) * int64_t(nr));
+    auto launch = [&](auto ncc) {
+      constexpr int NC = decltype(ncc)::value;
+      if constexpr (sizeof(Rf) == 4)
+        if (tpb <= 128) {  // float, small grid: each list cut into kTransSplit chunks
+          const int tbp = far_rows(tpb * kTransSplit);
+          k_trans_split<Rf, NC><<<dim3(nblk(ta.total, tbp), nr, kComp / NC), dim3(tpb, tbp * kTransSplit),
+                                  sizeof(C2<Rf>) * NC * P * kTransSplit * tbp, sf>>>(P, ta);
+          return;
+        }
       const int tbp = far_rows(tpb);  // destination boxes per block
-      k_trans<Rf><<<dim3(nblk(pr.lev[l].nb, tbp), nr), dim3(tpb, tbp), 0, sf>>>(
-          P, pr.lev[l].nb, pr.lev[l].il_ptr, pr.lev[l].il_idx, pr.lev[l].il_off,
-          static_cast<const C2<Rf>*>(pr.lev[l].trans), static_cast<const C2<Rf>*>(pr.lev[l].S),
-          static_cast<C2<Rf>*>(pr.lev[l].G), sl(l));
-    }
+      k_trans<Rf, NC><<<dim3(nblk(ta.total, tbp), nr, kComp / NC), dim3(tpb, tbp), 0, sf>>>(P, ta);
+    };
+    if (one)
+      launch(std::integral_constant<int, 1>());
+    else
+      launch(std::integral_constant<int, kComp>());
   }
   prof_mark(pr, 4, true, st);
   prof_mark(pr, 5, false, st);
   for (int l = 3; l < L && fft8; ++l) {
-    k_anterp_fft<8, Rf><<<dim3(unsigned(pr.lev[l].nb), nr), kFftBatch * kComp * 8, fft_smem<8, Rf>(false), sf>>>(
-        pr.lev[l].child_start, pr.lev[l + 1].octant, static_cast<const C2<Rf>*>(pr.lev[l].G),
+    const int nw = fft_nw(l);
+    k_anterp_fft<8, Rf><<<dim3(nblk(fft_units(l), kFftBatch * nw), nr), 32 * nw, fft_smem_bytes<8, Rf>(nw), sf>>>(
+        fft_units(l), pr.lev[l + 1].parent, pr.lev[l + 1].octant, static_cast<const C2<Rf>*>(pr.lev[l].G),
         static_cast<const Rf*>(pr.lev[l].Kf), static_cast<const C2<Rf>*>(pr.lev[l].phase),
         static_cast<C2<Rf>*>(pr.lev[l + 1].G), sl(l), sl(l + 1));
   }
@@ -1543,9 +1791,17 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
     k_gsgd<Rf><<<dim3(unsigned(pr.lev[L].nb), nr), 128, 0, sf>>>(P, pr.par.ntheta,
                                                                  static_cast<const C2<Rf>*>(pr.lev[L].G), GS, GD,
                                                                  sl(L), sH);
-    k_disagg<Rf, Rio><<<dim3(nblk(pr.T, 256), nr), 256, 0, sf>>>(
-        pr.T, P, pr.leaf_of, static_cast<const C2<Rf>*>(pr.PiR), static_cast<const C2<Rf>*>(pr.MR), GS, GD, pot, sH,
-        sT);
+    const C2<Rf>* PiR = static_cast<const C2<Rf>*>(pr.PiR);
+    const C2<Rf>* MR = static_cast<const C2<Rf>*>(pr.MR);
+    bool whole = false;  // a thread per triangle
+    if constexpr (sizeof(Rf) == 4) whole = !narrow((pr.T + 31) / 32 * nr);
+    if (whole) {
+      if constexpr (sizeof(Rf) == 4)
+        k_disagg<Rf, Rio><<<dim3(nblk(pr.T, 256), nr), 256, 0, sf>>>(pr.T, P, pr.leaf_of, PiR, MR, GS, GD, pot, sH, sT);
+    } else {
+      k_disagg_split<Rf, Rio><<<dim3(nblk(pr.T, 32), nr), dim3(32, 5), 0, sf>>>(pr.T, P, pr.leaf_of, PiR, MR, GS, GD,
+                                                                                pot, sH, sT);
+    }
   }
   prof_mark(pr, 6, true, st);
   if (overlap) {
@@ -1578,8 +1834,9 @@ static pie_status apply_near_t(Problem& pr, const void* xv, void* yv, cudaStream
   if constexpr (sizeof(Rm) == 8) {
     near_fixed(pr, coef, pot, 1, 0, st);
   } else if (pr.tune.near_kernel != 1) {  // the box-staged kernel, unless tuned off
-    k_near_box<Rio, H16, 1><<<unsigned(pr.nleaf), kNearBoxThreads, near_box_smem<1>(), st>>>(
-        pr.nleaf, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr,
+    const int nsplit = near_box_split(pr);
+    k_near_box<Rio, H16, 1><<<unsigned(pr.nleaf * nsplit), kNearBoxThreads, near_box_smem<1>(), st>>>(
+        pr.nleaf, nsplit, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr,
         static_cast<const cf*>(pr.mom), static_cast<const __half2*>(pr.mom), mom_scale(pr), ncoef, float(kMu0), pot);
   } else {
     k_near<Rm, Rio, 1, H16><<<nblk(pr.T * 32, 256), 256, 0, st>>>(
@@ -1625,11 +1882,6 @@ pie_status apply_batch(Problem& pr, const void* x, void* y, int nrhs, cudaStream
 }
 
 pie_status apply_one(Problem& pr, const void* x, void* y, cudaStream_t st) { return apply_batch(pr, x, y, 1, st); }
-
-pie_status prepare_apply(Problem& pr) {
-  if (pr.par.ntheta != 8) return PIE_OK;
-  return pr.far_f32() ? fft_prepare<8, float>() : fft_prepare<8, double>();
-}
 
 pie_status apply_cols(Problem& pr, const void* x, void* y, int nrhs, cudaStream_t st) {
   const size_t col = (pr.io_f32() ? sizeof(cf) : sizeof(cd)) * size_t(pr.N);

@@ -134,8 +134,6 @@ pie_status apply_one(Problem& pr, const void* x, void* y, cudaStream_t st);
 pie_status apply_batch(Problem& pr, const void* x, void* y, int nrhs, cudaStream_t st);
 // x, y: N x nrhs columns, passes of tune.rhs_chunk columns
 pie_status apply_cols(Problem& pr, const void* x, void* y, int nrhs, cudaStream_t st);
-// one-time kernel attributes of the product (not allowed inside a stream capture)
-pie_status prepare_apply(Problem& pr);
 // the shared-memory limit of the fixed-point near kernel on the current device (set-up of PIE_FP64 problems)
 pie_status near_fixed_prepare();
 // records the start (end = false) or end of stage `stage` of the current apply when profiling

@@ -278,7 +278,6 @@ pie_status pie_group_create(pie_problem* const* members, int n, pie_group** out)
     g->done.push_back(nullptr);
     s = cuda_check(cudaStreamCreateWithFlags(&g->branch.back(), cudaStreamNonBlocking), "group stream");
     if (s == PIE_OK) s = cuda_check(cudaEventCreateWithFlags(&g->done.back(), cudaEventDisableTiming), "event");
-    if (s == PIE_OK) s = prepare_apply(members[i]->p);
   }
   if (s == PIE_OK) s = cuda_check(cudaStreamCreateWithFlags(&g->cap, cudaStreamNonBlocking), "group stream");
   if (s == PIE_OK) s = cuda_check(cudaEventCreateWithFlags(&g->start, cudaEventDisableTiming), "event");
