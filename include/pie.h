@@ -418,14 +418,15 @@ pie_status pie_nearfield(pie_problem* pr, const void* x, const void* rho, const 
  *    threads per SM (each warp walks test triangles with a grid stride), so
  *    that it takes a bounded share of every SM beside the far kernels (a
  *    complex double near part: one block of 128 threads per SM for every two,
- *    as its integer multiply-adds leave the FP64 pipe to the far part);
- *    0 = one warp per test triangle.  0..32.
+ *    as its integer multiply-adds leave the FP64 pipe to the far part; a
+ *    box-staged float one with more than 16 blocks per SM: 32 times as many,
+ *    its blocks being short); 0 = one warp per test triangle.  0..32.
  *  rhs_chunk: right-hand sides per pass over the operator, 1..max_nrhs.
  *  near_rhs_block: right-hand sides that one pass of the near kernel
  *    carries (each pair's moments are read once for them): 1, 2, 4 or 8
  *    (8 only with the warp-per-triangle kernel), or 0 to pick by the pass
- *    width (1 for one column, 2 for two or a complex double near part, 4 up
- *    to four, else 8).
+ *    width (1 for one column, 2 for two, else 4; fewer where the box-staged
+ *    kernel's rows would not fit in shared memory).
  *  far_rows: tile shape of the per-box far kernels of angular grids other
  *    than N_theta = 8 (aggregation, dense interpolation and anterpolation,
  *    translation; one thread per sample): boxes per block, 1, 2, 4, 8, 16 or
@@ -435,9 +436,10 @@ pie_status pie_nearfield(pie_problem* pr, const void* x, const void* rho, const 
  *    test triangle reading the coefficients from global memory (1, 2, 4 or
  *    8 right-hand sides per thread), 2 = box-staged (one block per leaf box
  *    and group of up to 4 right-hand sides, the box's source coefficients
- *    in shared memory), 0 = automatic (box-staged for passes of one column,
- *    warp per triangle otherwise).  Both take the same operations in the
- *    same order.  near_rhs_block 8 always uses the warp-per-triangle kernel.
+ *    in shared memory), 0 = automatic (box-staged while the longest row's
+ *    coefficients fit in shared memory).  Both take the same operations in
+ *    the same order.  near_rhs_block 8 always uses the warp-per-triangle
+ *    kernel.
  *    A complex double near part runs in fixed point, one column per block,
  *    whatever near_rhs_block and near_kernel say.
  * Defaults at pie_problem_create: overlap 1, near_ctas_per_sm 2, rhs_chunk

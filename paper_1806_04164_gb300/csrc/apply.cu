@@ -172,45 +172,92 @@ __global__ void __launch_bounds__(256) k_near(int64_t T, int64_t nnz, const int3
   }
 }
 
+// The twelve components of six complex sums over a warp: each step of the
+// butterfly sum keeps half of the values on either side, so the adds of one
+// value are those of warp_sum (same bits) and a row takes 13 shuffles instead of
+// 60.  Component i ends on lane 16 (i / 6) + 8 (i % 6 / 3) + 4 (i % 3 / 2) + 2 (i % 3 % 2).
+__device__ __forceinline__ float warp_sum12(const cf* a, int lane, int* component) {
+  float v[12];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) v[2 * i] = a[i].x, v[2 * i + 1] = a[i].y;
+  const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4, h1 = lane & 2;
+  auto step = [](bool up, float lo, float hi, int o) {
+    const float keep = up ? hi : lo, send = up ? lo : hi;
+    return keep + __shfl_xor_sync(0xffffffffu, send, o);
+  };
+  float w[6], x[3], y[2];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) w[i] = step(h4, v[i], v[6 + i], 16);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) x[i] = step(h3, w[i], w[3 + i], 8);
+  y[0] = step(h2, x[0], x[2], 4);
+  y[1] = step(h2, x[1], 0.f, 4);
+  const float z = step(h1, y[0], y[1], 2);
+  // lanes 4 + 2 of each eight (and every odd lane) hold nothing of their own
+  *component = (lane & 1) || (h2 && h1) ? -1 : (h4 ? 6 : 0) + (h3 ? 3 : 0) + (h2 ? 2 : 0) + (h1 ? 1 : 0);
+  return z + __shfl_xor_sync(0xffffffffu, z, 1);
+}
+
 // a1, float near part: one block per leaf box (grid stride over boxes) and
 // per group of RB right-hand sides (blockIdx.y).  Every test triangle of a
 // box runs over the same source list (the concatenated source ranges of its
 // near boxes), so the block stages those sources' coefficients in shared
-// memory once per right-hand side, plane by plane ([RB][6][len], dynamic
-// shared memory), and its warps take the box's test triangles in turn,
-// lanes over the row as in k_near (lane j, j + 32, ...): each moment is read
-// once for the RB right-hand sides, and every right-hand side sees the same
-// operations in the same order as in k_near, so the same result to the last
-// bit.  nsplit shares a box's test triangles among several blocks when the
-// leaf boxes alone do not fill the SMs.  Rows longer than kNearStage read the coefficients from global
-// memory instead.
-constexpr int kNearStage = 512;
-constexpr int kNearBoxThreads = 128;  // threads per block (per leaf box); 256 measured 8 % slower (FP32H)
+// memory once per right-hand side, plane by plane ([RB][6][stage], dynamic
+// shared memory: stage is the problem's longest row), and its warps take the
+// box's test triangles in turn, lanes over the row as in k_near (lane j,
+// j + 32, ...): each moment is read once for the RB right-hand sides, and every
+// right-hand side sees the same operations in the same order as in k_near, so
+// the same result to the last bit.  nsplit shares a box's test triangles among
+// several blocks when the leaf boxes alone do not fill the SMs.  Rows longer
+// than stage (kNearSmemMax allows 1188 sources at RB = 4, 4752 at RB = 1) read the
+// coefficients from global memory instead.
+// Half-precision records of one right-hand side reach shared memory by cp.async
+// kNearAhead steps of 32 entries ahead, across rows: 327,680 triangles 607 -> 540 us
+// (loads of four records at a time left the memory idle at every row's end;
+// float moments read 94 % of the copy rate as they are).
+constexpr int kNearAhead = 3;
+constexpr size_t kNearSmemMax = 228096;  // a block's 227 KB less what the kernel declares itself
 template <int RB>
-constexpr size_t near_box_smem() {
-  return size_t(RB) * 6 * kNearStage * sizeof(cf);
+constexpr int near_box_threads() {
+  return 128 * RB;  // 256 threads per box measured 8 % slower than 128 (FP32H, RB = 1)
 }
+template <bool H16, int RB>
+constexpr size_t near_box_smem(int stage) {
+  return size_t(RB) * 6 * stage * sizeof(cf) + (H16 && RB == 1 ? size_t(4) * (kNearAhead + 1) * 64 * sizeof(uint4) : 0);
+}
+// Sources staged: the longest row, or as many as fit.
+template <bool H16, int RB>
+static int near_box_stage(const Problem& pr) {
+  const int row = int((pr.max_row + 31) / 32 * 32);
+  const int fit = int((kNearSmemMax - near_box_smem<H16, RB>(0)) / (size_t(RB) * 6 * sizeof(cf))) / 32 * 32;
+  return std::min(row, fit);
+}
+
 template <typename Rio, bool H16, int RB>
-__global__ void __launch_bounds__(kNearBoxThreads, RB == 1 ? 6 : (RB == 2 ? 4 : 2))
-    k_near_box(int64_t nleaf, int nsplit, int64_t nnz, const int32_t* __restrict__ leaf_start,
+__global__ void __launch_bounds__(near_box_threads<RB>(), RB == 1 ? 6 : (RB == 2 ? 2 : 1))
+    k_near_box(int64_t nleaf, int nsplit, int stage, int64_t nnz, const int32_t* __restrict__ leaf_start,
                const int32_t* __restrict__ near_ptr, const int32_t* __restrict__ near_idx,
                const int32_t* __restrict__ near_off, const int64_t* __restrict__ row_ptr,
                const cf* __restrict__ mom, const __half2* __restrict__ momh, MomScale msc,
                const cf* __restrict__ coef, float mu0, C2<Rio>* __restrict__ pot, int nrhs = 1, int64_t sc = 0,
                int64_t sp = 0) {
   extern __shared__ __align__(16) unsigned char near_smem[];
-  cf* cs = reinterpret_cast<cf*>(near_smem);  // [RB][6][kNearStage]
+  constexpr bool RING = H16 && RB == 1;
+  constexpr int NS = kNearAhead + 1;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  uint4* ring = reinterpret_cast<uint4*>(near_smem) + warp * NS * 64;  // [NS][2][32]
+  cf* cs = reinterpret_cast<cf*>(near_smem + (RING ? size_t(4) * NS * 64 * sizeof(uint4) : 0));  // [RB][6][stage]
   const int r0 = blockIdx.y * RB;             // right-hand sides r0 .. r0 + nr - 1
   const int nr = min(RB, nrhs - r0);
   coef += r0 * sc;
   pot += r0 * sp;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   for (int64_t bi = blockIdx.x; bi < nleaf * nsplit; bi += gridDim.x) {
     const int64_t b = bi / nsplit;
     const int q0 = near_ptr[b], q1 = near_ptr[b + 1];
     const int t0 = leaf_start[b], t1 = leaf_start[b + 1];
-    const int len = int(row_ptr[t0 + 1] - row_ptr[t0]);
-    const bool staged = len <= kNearStage;
+    const int64_t base = row_ptr[t0];
+    const int len = int(row_ptr[t0 + 1] - base);
+    const bool staged = len <= stage;
     __syncthreads();  // the previous box's readers are done with cs
     if (staged) {
       int qi = q0;  // j grows: the cursor only moves forward
@@ -219,13 +266,32 @@ __global__ void __launch_bounds__(kNearBoxThreads, RB == 1 ? 6 : (RB == 2 ? 4 : 
         const int64_t src = 6 * (int64_t(leaf_start[near_idx[qi]]) + (j - near_off[qi]));
         for (int r = 0; r < nr; ++r)
 #pragma unroll
-          for (int k = 0; k < 6; ++k) cp_async(&cs[(r * 6 + k) * kNearStage + j], coef + r * sc + src + k);
+          for (int k = 0; k < 6; ++k) cp_async(&cs[(r * 6 + k) * stage + j], coef + r * sc + src + k);
       }
     }
     cp_async_wait_all();
     __syncthreads();
-    for (int t = t0 + int(bi % nsplit) * nwarp + warp; t < t1; t += nwarp * nsplit) {
-      const int64_t e0 = row_ptr[t];
+    const int tfirst = t0 + int(bi % nsplit) * nwarp + warp, tstep = nwarp * nsplit;
+    // the (row, 32 entries) step after the last one sent on its way, and its slot
+    int ft = tfirst, fi = 0, fslot = 0;
+    const int per_row = (len + 31) / 32;
+    auto fetch = [&] {
+      // the step's records as 16-byte halves, 32 consecutive ones a copy (whole sectors)
+      const int n = ft < t1 ? 2 * min(32, len - 32 * fi) : 0;
+      const uint4* src = reinterpret_cast<const uint4*>(momh) + 2 * (base + int64_t(ft - t0) * len + 32 * fi);
+#pragma unroll
+      for (int c = lane; c < 64; c += 32)
+        if (c < n) cp_async(ring + fslot * 64 + c, src + c);
+      cp_async_commit();
+      fslot = (fslot + 1) % NS;
+      if (++fi == per_row) fi = 0, ft += tstep;
+    };
+    int slot = 0;
+    if constexpr (RING)
+#pragma unroll
+      for (int d = 0; d < kNearAhead; ++d) fetch();
+    for (int t = tfirst; t < t1; t += tstep) {
+      const int64_t e0 = base + int64_t(t - t0) * len;
       cf acc[RB][6];
 #pragma unroll
       for (int r = 0; r < RB; ++r)
@@ -238,7 +304,7 @@ __global__ void __launch_bounds__(kNearBoxThreads, RB == 1 ? 6 : (RB == 2 ? 4 : 
       auto coefs = [&](int r, int j, cf* c) {
         if (staged) {
 #pragma unroll
-          for (int k = 0; k < 6; ++k) c[k] = cs[(r * 6 + k) * kNearStage + j];
+          for (int k = 0; k < 6; ++k) c[k] = cs[(r * 6 + k) * stage + j];
         } else {
           while (qi + 1 < q1 && near_off[qi + 1] <= j) ++qi;
           const cf* src = coef + r * sc + 6 * (int64_t(leaf_start[near_idx[qi]]) + (j - near_off[qi]));
@@ -271,11 +337,25 @@ __global__ void __launch_bounds__(kNearBoxThreads, RB == 1 ? 6 : (RB == 2 ? 4 : 
             accumulate(acc[r], m, c);
           }
       };
-      if constexpr (H16) {
+      if constexpr (RING) {
+        for (int i = 0; i < per_row; ++i) {
+          cp_async_wait<kNearAhead - 1>();
+          __syncwarp();  // the step's records are here, and the slot before is read
+          fetch();
+          const int j = 32 * i + lane;
+          if (j < len) {
+            const uint4 lo = ring[slot * 64 + 2 * lane], hi = ring[slot * 64 + 2 * lane + 1];
+            cf m[kMom];
+            unpack_half<float>(lo, hi, msc, m);
+            entry(j, m);
+          }
+          slot = (slot + 1) % NS;
+        }
+      } else if constexpr (H16) {
         // entries j, j + 32, ... (U of them): their 32-byte records loaded
         // together, then accumulated in that order, the order of the
         // one-entry loop
-        constexpr int U = RB == 1 ? 4 : 2;
+        constexpr int U = 2;
         for (int j = lane; j < len; j += 32 * U) {
           uint4 lo[U], hi[U];
 #pragma unroll
@@ -307,26 +387,17 @@ __global__ void __launch_bounds__(kNearBoxThreads, RB == 1 ? 6 : (RB == 2 ? 4 : 
 #pragma unroll
       for (int r = 0; r < RB; ++r) {
         if (r >= nr) break;
-#pragma unroll
-        for (int i = 0; i < 6; ++i) {
-          acc[r][i].x = warp_sum(acc[r][i].x);
-          acc[r][i].y = warp_sum(acc[r][i].y);
-        }
-        if (lane == 0) {
-          C2<Rio>* o = pot + r * sp + 6 * int64_t(t);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) o[i] = mk<Rio>(Rio(mu0 * acc[r][i].x), Rio(mu0 * acc[r][i].y));
-          o[4] = cvt<Rio>(acc[r][4]);
-          o[5] = cvt<Rio>(acc[r][5]);
-        }
+        int i;
+        const float v = warp_sum12(acc[r], lane, &i);
+        if (i >= 0) reinterpret_cast<Rio*>(pot + r * sp + 6 * int64_t(t))[i] = Rio(i < 8 ? mu0 * v : v);
       }
     }
+    cp_async_wait_all();  // (steps past the last row: nothing in them)
   }
 }
 
-// The RB = 4 instance takes more than the 48 KB of shared memory a kernel
-// gets without asking: raise its limit once per instance and device (the
-// attribute belongs to the current device's copy of the kernel).
+// Raises the instance's shared-memory limit once per device (the attribute
+// belongs to the current device's copy of the kernel).
 static bool device_done(std::atomic<uint64_t>& mask, int* bit) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
@@ -342,10 +413,10 @@ template <typename Rio, bool H16, int RB>
 static pie_status near_box_prepare() {
   static std::atomic<uint64_t> done{0};
   int bit = -1;
-  if (near_box_smem<RB>() <= 49152 || device_done(done, &bit)) return PIE_OK;
-  pie_status s = cuda_check(cudaFuncSetAttribute(k_near_box<Rio, H16, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 int(near_box_smem<RB>())),
-                            "near smem attribute");
+  if (device_done(done, &bit)) return PIE_OK;
+  pie_status s = cuda_check(
+      cudaFuncSetAttribute(k_near_box<Rio, H16, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kNearSmemMax)),
+      "near smem attribute");
   if (s == PIE_OK && bit >= 0) done.fetch_or(uint64_t(1) << bit);
   return s;
 }
@@ -1616,27 +1687,33 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
           static_cast<const C2<Rm>*>(pr.mom), static_cast<const __half2*>(pr.mom), mom_scale(pr), ncoef, Rm(kMu0),
           pot2, nrhs, sT, sT);
   };
-  // float near part: the box-staged kernel (RB 1, 2 or 4) for one column,
-  // or for any pass when tune.near_kernel is 2; otherwise one warp per test
-  // triangle (RB 1, 2, 4 or 8).  The box kernel measured slower on passes of
-  // many columns of small meshes whose rows outgrow its staging buffer.
+  // float near part: the box-staged kernel (RB 1, 2 or 4), or one warp per
+  // test triangle (RB 1, 2, 4 or 8) when tuned so or when the rows outgrow the
+  // box kernel's shared memory
   int rb = pr.tune.near_rhs_block;
-  if (rb == 0) rb = nrhs == 1 ? 1 : nrhs == 2 ? 2 : nrhs <= 4 ? 4 : 8;
-  const bool boxed = sizeof(Rm) == 4 && (pr.tune.near_kernel == 2 || (pr.tune.near_kernel == 0 && rb == 1));
+  auto fits = [&](int n) { return size_t(n) * 6 * sizeof(cf) * size_t(pr.max_row + 31) < kNearSmemMax; };
+  bool boxed = sizeof(Rm) == 4 && pr.tune.near_kernel != 1;
+  if (rb == 0) {
+    rb = nrhs == 1 ? 1 : nrhs == 2 ? 2 : 4;
+    while (boxed && rb > 1 && !fits(rb)) rb /= 2;
+  }
+  if (pr.tune.near_kernel == 0) boxed = boxed && fits(rb);
   auto box_launch = [&](auto rbc) -> pie_status {
     if constexpr (sizeof(Rm) == 4) {
-      constexpr int RB = decltype(rbc)::value;
+      constexpr int RB = decltype(rbc)::value, TH = near_box_threads<RB>();
       pie_status s = near_box_prepare<Rio, H16, RB>();
       if (s != PIE_OK) return s;
-      const int nsplit = near_box_split(pr);
+      const int nsplit = near_box_split(pr), stage = near_box_stage<H16, RB>(pr);
       unsigned grid = unsigned(pr.nleaf * nsplit);
-      if (overlap && pr.tune.near_ctas_per_sm > 0)  // in CTAs of 256 threads per SM
-        grid = std::min<unsigned>(grid, unsigned(pr.nsm * pr.tune.near_ctas_per_sm * (256 / kNearBoxThreads)));
-      k_near_box<Rio, H16, RB><<<dim3(grid, unsigned((nrhs + RB - 1) / RB)), kNearBoxThreads, near_box_smem<RB>(),
-                                 sn>>>(pr.nleaf, nsplit, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off,
-                                       pr.row_ptr, static_cast<const cf*>(pr.mom),
-                                       static_cast<const __half2*>(pr.mom), mom_scale(pr),
-                                       reinterpret_cast<const cf*>(ncoef), float(kMu0), pot2, nrhs, sT, sT);
+      if (overlap && pr.tune.near_ctas_per_sm > 0)
+        // many short blocks make room for the far part's by themselves: a bound
+        // only where all of them would start at once
+        grid = std::min<unsigned>(grid, unsigned(pr.nsm * pr.tune.near_ctas_per_sm *
+                                                 (grid > unsigned(16 * pr.nsm) ? 8192 / TH : std::max(1, 256 / TH))));
+      k_near_box<Rio, H16, RB><<<dim3(grid, unsigned((nrhs + RB - 1) / RB)), TH, near_box_smem<H16, RB>(stage), sn>>>(
+          pr.nleaf, nsplit, stage, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr,
+          static_cast<const cf*>(pr.mom), static_cast<const __half2*>(pr.mom), mom_scale(pr),
+          reinterpret_cast<const cf*>(ncoef), float(kMu0), pot2, nrhs, sT, sT);
     }
     return PIE_OK;
   };
@@ -1834,9 +1911,11 @@ static pie_status apply_near_t(Problem& pr, const void* xv, void* yv, cudaStream
   if constexpr (sizeof(Rm) == 8) {
     near_fixed(pr, coef, pot, 1, 0, st);
   } else if (pr.tune.near_kernel != 1) {  // the box-staged kernel, unless tuned off
-    const int nsplit = near_box_split(pr);
-    k_near_box<Rio, H16, 1><<<unsigned(pr.nleaf * nsplit), kNearBoxThreads, near_box_smem<1>(), st>>>(
-        pr.nleaf, nsplit, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr,
+    pie_status s = near_box_prepare<Rio, H16, 1>();
+    if (s != PIE_OK) return s;
+    const int nsplit = near_box_split(pr), stage = near_box_stage<H16, 1>(pr);
+    k_near_box<Rio, H16, 1><<<unsigned(pr.nleaf * nsplit), near_box_threads<1>(), near_box_smem<H16, 1>(stage), st>>>(
+        pr.nleaf, nsplit, stage, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr,
         static_cast<const cf*>(pr.mom), static_cast<const __half2*>(pr.mom), mom_scale(pr), ncoef, float(kMu0), pot);
   } else {
     k_near<Rm, Rio, 1, H16><<<nblk(pr.T * 32, 256), 256, 0, st>>>(

@@ -46,6 +46,7 @@ struct Problem {
   int P = 0;
   int64_t T = 0, E = 0, N = 0;
   int64_t nnz = 0;      // near pair entries
+  int64_t max_row = 0;  // most near pair entries of a test triangle
   int64_t nleaf = 0;
   double h_max = 0;     // longest edge of the mesh
   double r_max = 0;     // largest distance of a centroid from the origin

@@ -853,6 +853,7 @@ static pie_status setup_t(Problem& pr, cudaStream_t st) {
       cnt += tr.leaf_start[nb + 1] - tr.leaf_start[nb];
     }
     row_ptr[i + 1] = row_ptr[i] + cnt;
+    pr.max_row = std::max(pr.max_row, cnt);
   }
   pr.nnz = row_ptr[T];
 
