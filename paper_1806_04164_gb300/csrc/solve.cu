@@ -6,9 +6,12 @@
 // Arnoldi runs on the device in complex double with classical Gram-Schmidt,
 // repeated when the first pass cancels most of the vector (DGKS criterion);
 // dot products use fixed-order two-pass reductions (results do not depend on
-// scheduling).  The small Hessenberg problem (Givens rotations)
-// is solved on the host.  Stopping test: ||b - Z x|| / ||b|| <= tol on the
+// scheduling).  The small Hessenberg problem (Givens rotations) is solved on
+// the host, which enqueues steps ahead of the ones it has read: the device
+// decides on the second Gram-Schmidt pass and normalises the new vector itself,
+// and publishes each step's coefficients in mapped host memory.  Stopping test: ||b - Z x|| / ||b|| <= tol on the
 // unscaled system, recomputed from the true residual at every restart.
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <complex>
@@ -130,19 +133,53 @@ __global__ void k_axs(int64_t N, double alpha, const C2<B>* __restrict__ x, C2<B
   if (i < N) y[i] = mk<B>(B(alpha * double(x[i].x)), B(alpha * double(x[i].y)));
 }
 
+// out = sum of the nblk partial sums, by one warp: lanes over the sums in a fixed
+// order, then a fixed shuffle tree.
+__device__ __forceinline__ void finish_sum(const cd* partial, int nblk, cd* out) {
+  const int lane = threadIdx.x & 31;
+  double r = 0, i = 0;
+  for (int b = lane; b < nblk; b += 32) {
+    const double2 p = __ldcg(reinterpret_cast<const double2*>(partial) + b);
+    r += p.x;
+    i += p.y;
+  }
+  r = warp_sum(r);
+  i = warp_sum(i);
+  if (lane == 0) *out = mk<double>(r, i);
+}
+
+// Whether this is the grid's last block to arrive here (the others' writes are
+// then visible); the ticket wraps back to zero.
+__device__ __forceinline__ bool last_block(unsigned* ticket) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const unsigned total = gridDim.x * gridDim.y;
+    last = atomicInc(ticket, total - 1) == total - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  return last;
+}
+
 // partial[v][tile] = sum over the tile's entries of conj(V[v][n]) w[n]
 // (accumulated in the basis type per lane, then in double).  Pass 1 of a
 // fixed-order reduction.  A block stages one tile of w in shared memory;
 // each warp runs it against its share of a chunk of kDotVecs vectors, every
 // lane streaming kDotTile / 32 entries of a vector before one warp
-// reduction; grid = (tiles, vector chunks).
+// reduction; grid = (tiles, vector chunks).  With out, the grid's last block
+// also does pass 2 (k_mdot_finish's sums in the same order: short vectors, where
+// another launch costs more); cond: do nothing unless *cond.
 constexpr int kTile = 2048;     // largest tile (entries of w per block)
 constexpr int kMinTile = 256;   // smallest, for short vectors
 constexpr int kDotVecs = 64;
 template <typename B>
 __global__ void __launch_bounds__(kRedThreads) k_mdot(int64_t N, int nv, const C2<B>* __restrict__ V, int64_t ldv,
                                                       const C2<B>* __restrict__ w, cd* __restrict__ partial,
-                                                      int tile) {
+                                                      int tile, cd* __restrict__ out, unsigned* ticket,
+                                                      const int* __restrict__ cond) {
+  if (cond && !*cond) return;
   __shared__ C2<B> ws[kTile];
   const int64_t n0 = int64_t(blockIdx.x) * tile;
   const int lim = int(min(int64_t(tile), N - n0));
@@ -163,31 +200,45 @@ __global__ void __launch_bounds__(kRedThreads) k_mdot(int64_t N, int nv, const C
     const double dr = warp_sum(double(ar)), di = warp_sum(double(ai));
     if (lane == 0) partial[int64_t(v) * gridDim.x + blockIdx.x] = mk<double>(dr, di);
   }
+  if (out && last_block(ticket))
+    for (int v = warp; v < nv; v += kRedThreads / 32) finish_sum(partial + int64_t(v) * gridDim.x, gridDim.x, out + v);
 }
 
 // Pass 2: out[v] = sum over tiles of partial[v][.], one warp per vector,
 // lanes over tiles in a fixed order, then a fixed shuffle tree.
-__global__ void k_mdot_finish(int nv, int nblk, const cd* __restrict__ partial, cd* __restrict__ out) {
-  const int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (v >= nv) return;
-  double r = 0, i = 0;
-  for (int b = lane; b < nblk; b += 32) {
-    r += partial[(int64_t)v * nblk + b].x;
-    i += partial[(int64_t)v * nblk + b].y;
-  }
-  r = warp_sum(r);
-  i = warp_sum(i);
-  if (lane == 0) out[v] = mk<double>(r, i);
+__global__ void k_mdot_finish(int nv, int nblk, const cd* __restrict__ partial, cd* __restrict__ out,
+                              const int* __restrict__ cond = nullptr) {
+  const int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (v >= nv || (cond && !*cond)) return;
+  finish_sum(partial + (int64_t)v * nblk, nblk, out + v);
 }
 
+// A step as the host reads it (mapped memory).
+struct StepRecord {
+  double hn;
+  int reorth;
+  unsigned seq;
+};
+
+// What the device knows of an Arnoldi step.
+struct StepScalars {
+  double hn;        // norm of the orthogonalised vector
+  int reorth;       // whether the second Gram-Schmidt pass runs
+  unsigned ticket;  // last_block
+};
+
 // w -= sum_v h[v] V[v] (in the basis type, h staged in shared memory),
-// followed by the squared norm of the updated w: per-block
-// partial sums (fixed order) in partial[blockIdx.x], finished by
-// k_mdot_finish.  Block size kRedThreads.
+// followed by the norm of the updated w: per-block partial sums (fixed order)
+// in partial[blockIdx.x], finished by the last block into sc->hn.  The first
+// pass (second = false) also decides on a second one, when it cancelled most of w:
+// hn below 0.7 of the norm before, h[nv] holding that norm's square; the second
+// pass does nothing unless so decided.  Block size kRedThreads.
 template <typename B>
 __global__ void __launch_bounds__(kRedThreads) k_mupdate_norm(int64_t N, int nv, const C2<B>* __restrict__ V,
                                                               int64_t ldv, const cd* __restrict__ h,
-                                                              C2<B>* __restrict__ w, cd* __restrict__ partial) {
+                                                              C2<B>* __restrict__ w, cd* __restrict__ partial,
+                                                              StepScalars* sc, bool second) {
+  if (second && !sc->reorth) return;
   extern __shared__ unsigned char hraw[];
   C2<B>* hs = reinterpret_cast<C2<B>*>(hraw);
   __shared__ double sn[kRedThreads / 32];
@@ -226,7 +277,40 @@ __global__ void __launch_bounds__(kRedThreads) k_mupdate_norm(int64_t N, int nv,
     for (int k = 0; k < kRedThreads / 32; ++k) t += sn[k];
     partial[blockIdx.x] = mk<double>(t, 0.0);
   }
+  if (!last_block(&sc->ticket) || threadIdx.x >= 32) return;
+  __shared__ cd n2;
+  finish_sum(partial, gridDim.x, &n2);
+  if (threadIdx.x == 0) {
+    const double hn = sqrt(n2.x);
+    sc->hn = hn;
+    if (!second) sc->reorth = hn < 0.7 * sqrt(h[nv].x);
+  }
 }
+
+// w /= hn, and the step's coefficients into mapped host memory, the sequence
+// number last: h [nh] of the first pass, h2 [nh - 1] of the second.
+template <typename B>
+__global__ void k_normalise(int64_t N, C2<B>* __restrict__ w, const StepScalars* __restrict__ sc, int nh,
+                            const cd* __restrict__ h, const cd* __restrict__ h2, StepRecord* rec, cd* out_h,
+                            cd* out_h2, unsigned seq) {
+  const double hn = sc->hn, alpha = 1.0 / hn;
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i < N) w[i] = mk<B>(B(alpha * double(w[i].x)), B(alpha * double(w[i].y)));
+  if (blockIdx.x != 0) return;
+  for (int k = threadIdx.x; k < nh; k += blockDim.x) {
+    out_h[k] = h[k];
+    if (sc->reorth && k + 1 < nh) out_h2[k] = h2[k];
+  }
+  __threadfence_system();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    rec->hn = hn;
+    rec->reorth = sc->reorth;
+    __threadfence_system();
+    *reinterpret_cast<volatile unsigned*>(&rec->seq) = seq;
+  }
+}
+
 
 // x += d (sum_v y[v] V[v]) in complex double (the solution stays FP64).
 template <typename B>
@@ -309,9 +393,26 @@ __global__ void k_cvt(int64_t N, const C2<A>* __restrict__ x, C2<B>* __restrict_
 // ---------------------------------------------------------------- host loop
 
 struct Work {
-  std::vector<void*> ptrs;
+  std::vector<void*> ptrs, pinned;
+  cudaStream_t st;
+  explicit Work(cudaStream_t st_) : st(st_) {}
   ~Work() {
+    if (!pinned.empty()) cudaStreamSynchronize(st);  // steps enqueued ahead may still write there
+    for (void* p : pinned) cudaFreeHost(p);
     for (void* p : ptrs) cudaFree(p);
+  }
+  template <typename T>
+  T* get_pinned(size_t n, pie_status& s) {
+    if (s != PIE_OK) return nullptr;
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, n * sizeof(T), cudaHostAllocMapped) != cudaSuccess) {
+      cudaGetLastError();
+      set_error("pie_solve: pinned host allocation failed");
+      s = PIE_ERR_OOM;
+      return nullptr;
+    }
+    pinned.push_back(p);
+    return static_cast<T*>(p);
   }
   template <typename T>
   T* get(size_t n, pie_status& s) {
@@ -328,6 +429,28 @@ struct Work {
   }
 };
 
+constexpr int kSlots = 4;  // steps, uploads and timed products that may be in flight
+
+// Events around the operator products (timing is left out if they cannot be made).
+struct ProductEvents {
+  cudaEvent_t e[kSlots][2] = {};
+  bool pending[kSlots] = {};
+  unsigned n = 0;
+  ProductEvents() {
+    for (auto& p : e)
+      for (auto& x : p)
+        if (cudaEventCreate(&x) != cudaSuccess) {
+          cudaGetLastError();
+          x = nullptr;
+        }
+  }
+  ~ProductEvents() {
+    for (auto& p : e)
+      for (auto& x : p)
+        if (x) cudaEventDestroy(x);
+  }
+};
+
 // Shared scratch of the Krylov loop.
 struct Ctx {
   Problem& pr;      // the problem whose operator the products apply
@@ -340,35 +463,84 @@ struct Ctx {
   cd* partial;      // reduction partials
   cd* hdev;         // small device vector
   int hcap = 0;     // its length (the last entry holds norms)
-  cudaEvent_t ev0 = nullptr, ev1 = nullptr;  // around the last operator product
-  bool pending = false;                      // ev0 / ev1 hold a product not yet counted
+  ProductEvents* ev = nullptr;
   double op_ms = 0;                          // time in operator products
   int reorth = 0;                            // second Gram-Schmidt passes
   cf* u32 = nullptr;                         // operator input / output of a problem with
   cf* w32 = nullptr;                         // complex-float vectors (PIE_FP32)
+  // Arnoldi steps: device scalars and projections, and the records the host reads
+  StepScalars* sc = nullptr;
+  cd *h1 = nullptr, *h2 = nullptr;
+  StepRecord* rec = nullptr;                 // mapped, [kSlots]
+  cd *p1 = nullptr, *p2 = nullptr;           // mapped, [kSlots][hcap]
+  unsigned* seq = nullptr;                   // steps enqueued so far (shared by the contexts of a solve)
+  cd* pin = nullptr;                         // pinned, [hcap]: results of dotc
+  cd* up = nullptr;                          // pinned, [kSlots][hcap]: vectors on their way to the device
+  cudaEvent_t* up_ev = nullptr;              // after each upload
+  unsigned* up_n = nullptr;
 };
 
-// Adds the last product's time (its events have completed: every product is
-// followed by a synchronising reduction before the next one).
-static void op_time_flush(Ctx& c) {
-  if (!c.pending || !c.ev0) return;
+// The parts of a context that the contexts of one solve share.
+struct StepBuffers {
+  unsigned seq = 0, up_n = 0;
+  cudaEvent_t up_ev[kSlots] = {};
+  ~StepBuffers() {
+    for (auto& e : up_ev)
+      if (e) cudaEventDestroy(e);
+  }
+  pie_status bind(Ctx& c, Work& wk, int hcap) {
+    pie_status s = PIE_OK;
+    c.hcap = hcap;
+    c.sc = wk.get<StepScalars>(1, s);
+    c.h1 = wk.get<cd>(hcap, s);
+    c.h2 = wk.get<cd>(hcap, s);
+    c.rec = wk.get_pinned<StepRecord>(kSlots, s);
+    c.p1 = wk.get_pinned<cd>(size_t(2 * kSlots + kSlots + 1) * hcap, s);
+    if (s != PIE_OK) return s;
+    c.p2 = c.p1 + size_t(kSlots) * hcap;
+    c.up = c.p2 + size_t(kSlots) * hcap;
+    c.pin = c.up + size_t(kSlots) * hcap;
+    c.seq = &seq;
+    c.up_ev = up_ev;
+    c.up_n = &up_n;
+    for (int i = 0; i < kSlots; ++i) c.rec[i].seq = 0;
+    for (auto& e : up_ev)
+      if ((s = cuda_check(cudaEventCreateWithFlags(&e, cudaEventDisableTiming), "event")) != PIE_OK) return s;
+    return cuda_check(cudaMemsetAsync(c.sc, 0, sizeof(StepScalars), c.st), "memset");
+  }
+};
+
+static void op_time_flush(Ctx& c, unsigned slot) {
+  ProductEvents* v = c.ev;
+  if (!v || !v->pending[slot]) return;
   float ms = 0;
-  if (cudaEventElapsedTime(&ms, c.ev0, c.ev1) == cudaSuccess)
+  if (cudaEventSynchronize(v->e[slot][1]) == cudaSuccess &&
+      cudaEventElapsedTime(&ms, v->e[slot][0], v->e[slot][1]) == cudaSuccess)
     c.op_ms += ms;
   else
     cudaGetLastError();
-  c.pending = false;
+  v->pending[slot] = false;
+}
+
+// Adds the times of the products still pending.
+static void op_time_flush(Ctx& c) {
+  for (unsigned i = 0; i < kSlots; ++i) op_time_flush(c, i);
 }
 
 // out = Z in, or out = S in for the single-layer operator of Eq. (3)
 // (vectors in the io precision of the context's problem).
 static pie_status op_apply(Ctx& c, const void* in, void* out) {
-  op_time_flush(c);
-  if (c.ev0) cudaEventRecord(c.ev0, c.st);
+  ProductEvents* v = c.ev;
+  const unsigned slot = v ? v->n++ % kSlots : 0;
+  const bool timed = v && v->e[slot][0] && v->e[slot][1];
+  if (timed) {
+    op_time_flush(c, slot);
+    cudaEventRecord(v->e[slot][0], c.st);
+  }
   pie_status s = c.op == 0 ? apply_one(c.pr, in, out, c.st) : single_layer_one(c.pr, in, out, c.st);
-  if (c.ev1) {
-    cudaEventRecord(c.ev1, c.st);
-    c.pending = true;
+  if (timed) {
+    cudaEventRecord(v->e[slot][1], c.st);
+    v->pending[slot] = true;
   }
   return s;
 }
@@ -391,64 +563,55 @@ static pie_status op_scaled(Ctx& c, const C2<B>* in, C2<B>* out) {
   return PIE_OK;
 }
 
-struct EventPair {
-  cudaEvent_t a = nullptr, b = nullptr;
-  EventPair() {
-    if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess) {
-      cudaGetLastError();
-      a = b = nullptr;  // timing of the products is then left out
-    }
-  }
-  ~EventPair() {
-    if (a) cudaEventDestroy(a);
-    if (b) cudaEventDestroy(b);
-  }
-};
-
-// conj(a) . b over N entries, deterministic; result on the host.
-template <typename B>
-static pie_status dotc(Ctx& c, int nv, const C2<B>* V, const C2<B>* w, zc* out_host) {
-  // tiles of kTile entries, smaller (down to kMinTile) when that leaves fewer
-  // than two blocks per SM
+// Tiles of the dot products over N entries: of kTile entries, smaller (down to
+// kMinTile) when that leaves fewer than two blocks per SM.
+static int dot_tile(const Ctx& c) {
   int tile = kTile;
   if ((c.N + kTile - 1) / kTile < 2 * int64_t(c.pr.nsm))
     tile = int(std::max<int64_t>(kMinTile, ((c.N / (2 * std::max(c.pr.nsm, 1)) + 31) / 32) * 32));
-  tile = std::min(tile, kTile);
-  const unsigned tiles = unsigned((c.N + tile - 1) / tile);
-  k_mdot<B><<<dim3(tiles, unsigned((nv + kDotVecs - 1) / kDotVecs)), kRedThreads, 0, c.st>>>(c.N, nv, V, c.N, w,
-                                                                                            c.partial, tile);
-  k_mdot_finish<<<nb_(int64_t(nv) * 32, 128), 128, 0, c.st>>>(nv, int(tiles), c.partial, c.hdev);
-  pie_status s = cuda_check(cudaMemcpyAsync(out_host, c.hdev, sizeof(cd) * nv, cudaMemcpyDeviceToHost, c.st), "dot");
-  if (s == PIE_OK) s = cuda_check(cudaStreamSynchronize(c.st), "dot sync");
-  return s;
+  return std::min(tile, kTile);
 }
 
-// w -= sum_{v<nv} hdev[v] V[v]; returns ||w|| (host) after the update.
+// out[v] = conj(V[v]) . w over N entries, deterministic.  The grid's last block
+// finishes the sums while they are few (8192 partial sums: about 3 us, less
+// than a launch); cond: nothing unless *cond.
 template <typename B>
-static pie_status update_norm(Ctx& c, int nv, const C2<B>* V, C2<B>* w, double* norm) {
-  const unsigned blocks = nb_(c.N, kRedThreads);
-  k_mupdate_norm<B><<<blocks, kRedThreads, sizeof(C2<B>) * nv, c.st>>>(c.N, nv, V, c.N, c.hdev, w, c.partial);
-  k_mdot_finish<<<1, 32, 0, c.st>>>(1, int(blocks), c.partial, c.hdev + c.hcap - 1);
-  cd out;
-  pie_status s = cuda_check(cudaMemcpyAsync(&out, c.hdev + c.hcap - 1, sizeof(cd), cudaMemcpyDeviceToHost, c.st),
-                            "norm");
-  if (s == PIE_OK) s = cuda_check(cudaStreamSynchronize(c.st), "norm sync");
-  *norm = std::sqrt(out.x);
+static void enqueue_dots(Ctx& c, int nv, const C2<B>* V, const C2<B>* w, cd* out, const int* cond) {
+  const int tile = dot_tile(c);
+  const unsigned tiles = unsigned((c.N + tile - 1) / tile);
+  const bool tail = int64_t(nv) * tiles <= 8192;
+  k_mdot<B><<<dim3(tiles, unsigned((nv + kDotVecs - 1) / kDotVecs)), kRedThreads, 0, c.st>>>(
+      c.N, nv, V, c.N, w, c.partial, tile, tail ? out : nullptr, &c.sc->ticket, cond);
+  if (!tail) k_mdot_finish<<<nb_(int64_t(nv) * 32, 128), 128, 0, c.st>>>(nv, int(tiles), c.partial, out, cond);
+}
+
+// conj(V[v]) . w over N entries; results on the host.
+template <typename B>
+static pie_status dotc(Ctx& c, int nv, const C2<B>* V, const C2<B>* w, zc* out_host) {
+  enqueue_dots<B>(c, nv, V, w, c.hdev, nullptr);
+  pie_status s = cuda_check(cudaMemcpyAsync(c.pin, c.hdev, sizeof(cd) * nv, cudaMemcpyDeviceToHost, c.st), "dot");
+  if (s == PIE_OK) s = cuda_check(cudaStreamSynchronize(c.st), "dot sync");
+  for (int i = 0; i < nv && s == PIE_OK; ++i) out_host[i] = zc(c.pin[i].x, c.pin[i].y);
   return s;
 }
 
+// n entries to c.hdev, through one of kSlots pinned buffers (waiting only for
+// the upload that last used it).
 static pie_status to_dev(Ctx& c, const std::vector<zc>& v, int n) {
-  std::vector<cd> h(n);
+  const unsigned slot = (*c.up_n)++ % kSlots;
+  pie_status s = cuda_check(cudaEventSynchronize(c.up_ev[slot]), "copy wait");
+  if (s != PIE_OK) return s;
+  cd* h = c.up + size_t(slot) * c.hcap;
   for (int i = 0; i < n; ++i) h[i] = cd{v[i].real(), v[i].imag()};
-  pie_status s = cuda_check(cudaMemcpyAsync(c.hdev, h.data(), sizeof(cd) * n, cudaMemcpyHostToDevice, c.st), "copy");
-  if (s == PIE_OK) s = cuda_check(cudaStreamSynchronize(c.st), "copy sync");  // h must outlive the copy
+  s = cuda_check(cudaMemcpyAsync(c.hdev, h, sizeof(cd) * n, cudaMemcpyHostToDevice, c.st), "copy");
+  if (s == PIE_OK) s = cuda_check(cudaEventRecord(c.up_ev[slot], c.st), "copy event");
   return s;
 }
 
 struct Cycle {
-  std::vector<zc> H, cs, sn, g, h, h2;
+  std::vector<zc> H, cs, sn, g, h;
   int m;
-  explicit Cycle(int m_) : H(size_t(m_ + 1) * m_), cs(m_), sn(m_), g(m_ + 1), h(m_ + 1), h2(m_ + 1), m(m_) {}
+  explicit Cycle(int m_) : H(size_t(m_ + 1) * m_), cs(m_), sn(m_), g(m_ + 1), h(m_ + 1), m(m_) {}
   void reset(double beta) {
     std::fill(H.begin(), H.end(), zc(0));
     std::fill(g.begin(), g.end(), zc(0));
@@ -458,20 +621,48 @@ struct Cycle {
 
 // Classical Gram-Schmidt of w (basis slot j + 1) against V[0..j]; a second
 // pass only when the first one cancelled most of w (Daniel-Gragg-Kaufman-
-// Stewart criterion).  One reduction gives (v_i, w) for i <= j and (w, w);
-// the update returns the new norm.  cy.h[0..j] gets the projections, *hn
-// the norm of the orthogonalised w.
+// Stewart criterion, decided on the device), then w is normalised.  One
+// reduction gives (v_i, w) for i <= j and (w, w); the update gives the new
+// norm.  Returns the step's sequence number, for wait_step.
 template <typename B>
-static pie_status orthogonalize(Ctx& c, const C2<B>* V, int j, C2<B>* w, Cycle& cy, double* hn) {
-  pie_status s;
-  if ((s = dotc<B>(c, j + 2, V, w, cy.h.data())) != PIE_OK) return s;
-  const double wn0 = std::sqrt(cy.h[j + 1].real());
-  if ((s = update_norm<B>(c, j + 1, V, w, hn)) != PIE_OK) return s;
-  if (*hn < 0.7 * wn0) {
+static unsigned enqueue_orthogonalize(Ctx& c, const C2<B>* V, int j, C2<B>* w) {
+  const unsigned blocks = nb_(c.N, kRedThreads);
+  enqueue_dots<B>(c, j + 2, V, w, c.h1, nullptr);
+  k_mupdate_norm<B><<<blocks, kRedThreads, sizeof(C2<B>) * (j + 1), c.st>>>(c.N, j + 1, V, c.N, c.h1, w, c.partial,
+                                                                           c.sc, false);
+  enqueue_dots<B>(c, j + 1, V, w, c.h2, &c.sc->reorth);
+  k_mupdate_norm<B><<<blocks, kRedThreads, sizeof(C2<B>) * (j + 1), c.st>>>(c.N, j + 1, V, c.N, c.h2, w, c.partial,
+                                                                           c.sc, true);
+  const unsigned seq = ++*c.seq, slot = seq % kSlots;
+  k_normalise<B><<<nb_(c.N, 256), 256, 0, c.st>>>(c.N, w, c.sc, j + 2, c.h1, c.h2, c.rec + slot,
+                                                  c.p1 + size_t(slot) * c.hcap, c.p2 + size_t(slot) * c.hcap, seq);
+  return seq;
+}
+
+// Waits for step seq (step j of its cycle): cy.h[0..j] gets the projections,
+// *hn the norm of the orthogonalised vector.
+static pie_status wait_step(Ctx& c, unsigned seq, int j, Cycle& cy, double* hn) {
+  const unsigned slot = seq % kSlots;
+  const StepRecord* r = c.rec + slot;
+  for (unsigned spins = 1;; ++spins) {
+    if (*reinterpret_cast<const volatile unsigned*>(&r->seq) == seq) break;
+    if (spins % 4096) continue;
+    const cudaError_t e = cudaStreamQuery(c.st);  // an error, or everything done
+    if (e == cudaErrorNotReady) continue;
+    pie_status s = cuda_check(e, "step wait");
+    if (s != PIE_OK) return s;
+    if (*reinterpret_cast<const volatile unsigned*>(&r->seq) == seq) break;
+    set_error("pie_solve: a step did not report");
+    return PIE_ERR_CUDA;
+  }
+  std::atomic_thread_fence(std::memory_order_acquire);
+  const cd* p1 = c.p1 + size_t(slot) * c.hcap;
+  const cd* p2 = c.p2 + size_t(slot) * c.hcap;
+  *hn = r->hn;
+  for (int i = 0; i <= j + 1; ++i) cy.h[i] = zc(p1[i].x, p1[i].y);
+  if (r->reorth) {
     ++c.reorth;
-    if ((s = dotc<B>(c, j + 1, V, w, cy.h2.data())) != PIE_OK) return s;
-    if ((s = update_norm<B>(c, j + 1, V, w, hn)) != PIE_OK) return s;
-    for (int i = 0; i <= j; ++i) cy.h[i] += cy.h2[i];
+    for (int i = 0; i <= j; ++i) cy.h[i] += zc(p2[i].x, p2[i].y);
   }
   for (int i = 0; i <= j; ++i)
     if (!std::isfinite(cy.h[i].real()) || !std::isfinite(cy.h[i].imag()) || !std::isfinite(*hn)) {
@@ -532,10 +723,9 @@ static pie_status unscaled_residual(Ctx& c, const C2<B>* V, const Cycle& cy, int
   const unsigned blocks = nb_(c.N, kRedThreads);
   k_resnorm<B><<<blocks, kRedThreads, sizeof(cd) * (j + 2), c.st>>>(c.N, j + 2, V, c.N, c.hdev, c.d, c.partial);
   k_mdot_finish<<<1, 32, 0, c.st>>>(1, int(blocks), c.partial, c.hdev + c.hcap - 1);
-  cd r;
-  s = cuda_check(cudaMemcpyAsync(&r, c.hdev + c.hcap - 1, sizeof(cd), cudaMemcpyDeviceToHost, c.st), "residual");
+  s = cuda_check(cudaMemcpyAsync(c.pin, c.hdev + c.hcap - 1, sizeof(cd), cudaMemcpyDeviceToHost, c.st), "residual");
   if (s == PIE_OK) s = cuda_check(cudaStreamSynchronize(c.st), "residual sync");
-  *out = std::sqrt(r.x);
+  *out = std::sqrt(c.pin[0].x);
   return s;
 }
 
@@ -559,12 +749,22 @@ static pie_status arnoldi_cycle(Ctx& c, C2<B>* V, Cycle& cy, double beta, double
   cy.reset(beta);
   int j = 0;
   breakdown = false;
+  // Steps are enqueued ahead of the one whose coefficients the host waits for
+  // (5120 triangles: 104 us of every inner step were round trips).  A step past
+  // the cycle's end is thrown away, so fewer run ahead where a product is long, and
+  // none where an estimate is likely to end the cycle between two products.
+  const int ahead = N < 200000 ? 2 : hint_every > 0 ? 0 : 1;
+  unsigned seq[kSlots];
+  int enqueued = 0;
   for (; j < m && j < max_steps; ++j) {
-    // the new vector is built in its own basis slot: w = D Op D v_j
-    C2<B>* w = V + size_t(j + 1) * N;
-    if ((s = op_scaled<B>(c, V + size_t(j) * N, w)) != PIE_OK) return s;
+    for (; enqueued <= j + ahead && enqueued < m && enqueued < max_steps; ++enqueued) {
+      // the new vector is built in its own basis slot: w = D Op D v_j
+      C2<B>* w = V + size_t(enqueued + 1) * N;
+      if ((s = op_scaled<B>(c, V + size_t(enqueued) * N, w)) != PIE_OK) return s;
+      seq[enqueued % kSlots] = enqueue_orthogonalize<B>(c, V, enqueued, w);
+    }
     double hn = 0;
-    if ((s = orthogonalize<B>(c, V, j, w, cy, &hn)) != PIE_OK) return s;
+    if ((s = wait_step(c, seq[j % kSlots], j, cy, &hn)) != PIE_OK) return s;
     const double den = hessenberg_column(cy, j, hn);
     ++steps_done;
     if (hn <= 1e-14 * den) {
@@ -572,7 +772,6 @@ static pie_status arnoldi_cycle(Ctx& c, C2<B>* V, Cycle& cy, double beta, double
       ++j;
       break;
     }
-    k_axs<B><<<nb_(N, 256), 256, 0, c.st>>>(N, 1.0 / hn, w, w);
     if (j + 1 < min_steps) continue;
     bool stop = std::abs(cy.g[j + 1]) <= stop_abs;
     if (!stop && hint_every > 0 && (j + 1) % hint_every == 0) {
@@ -622,7 +821,7 @@ static pie_status solve_t(Problem& pr, int op, const void* bv, void* xv, double 
   const int64_t N = op == 0 ? pr.N : pr.T;
   const int m = std::min(restart, maxit);
   pie_status s = PIE_OK;
-  Work wk;
+  Work wk(st);
   double* d = wk.get<double>(N, s);
   C2<B>* V = wk.get<C2<B>>(size_t(N) * (m + 1), s);
   cd* u = wk.get<cd>(N, s);
@@ -631,13 +830,11 @@ static pie_status solve_t(Problem& pr, int op, const void* bv, void* xv, double 
   cd* partial = wk.get<cd>(std::max(size_t((N + kMinTile - 1) / kMinTile) * (m + 2), size_t(nb_(N, kRedThreads))), s);
   cd* hdev = wk.get<cd>(m + 3, s);
   if (s != PIE_OK) return s;
-  EventPair evp;
+  ProductEvents events;
+  StepBuffers steps;
   Ctx c{pr, st, op, N, d, u, wd, partial, hdev};
-  c.hcap = m + 3;
-  if (evp.a && evp.b) {
-    c.ev0 = evp.a;
-    c.ev1 = evp.b;
-  }
+  c.ev = &events;
+  if ((s = steps.bind(c, wk, m + 3)) != PIE_OK) return s;
   const cd* b = static_cast<const cd*>(bv);
   cd* x = static_cast<cd*>(xv);
   diag_scaling(pr, op, N, d, st);
@@ -776,7 +973,7 @@ static pie_status nested_t(Problem& po, Problem& pi, const cd* b, cd* x, const p
   const bool ir = np.outer_restart == 0;
   const int mmax = std::max(mi, mo);
   pie_status s = PIE_OK;
-  Work wk;
+  Work wk(st);
   double* d = wk.get<double>(N, s);
   C2<Bi>* Vi = wk.get<C2<Bi>>(size_t(N) * (mi + 1), s);  // inner basis
   cd* Vo = wk.get<cd>(size_t(N) * (mo + 1), s);           // outer basis
@@ -790,14 +987,14 @@ static pie_status nested_t(Problem& po, Problem& pi, const cd* b, cd* x, const p
                            s);
   cd* hdev = wk.get<cd>(mmax + 3, s);
   if (s != PIE_OK) return s;
-  EventPair evo, evi;
+  ProductEvents evo, evi;
+  StepBuffers steps;
   Ctx co{po, st, 0, N, d, u, wd, partial, hdev};
-  Ctx ci{pi, st, 0, N, d, u, wd, partial, hdev};
-  co.hcap = ci.hcap = mmax + 3;
-  ci.u32 = u32;
-  ci.w32 = w32;
-  if (evo.a && evo.b) co.ev0 = evo.a, co.ev1 = evo.b;
-  if (evi.a && evi.b) ci.ev0 = evi.a, ci.ev1 = evi.b;
+  co.ev = &evo;
+  if ((s = steps.bind(co, wk, mmax + 3)) != PIE_OK) return s;
+  // the inner cycle's context: another operator, the same scratch
+  Ctx ci{pi, st, 0, N, d, u, wd, partial, hdev, co.hcap, &evi, 0.0, 0, u32, w32, co.sc, co.h1, co.h2, co.rec,
+         co.p1, co.p2, co.seq, co.pin, co.up, co.up_ev, co.up_n};
   diag_scaling(po, 0, N, d, st);
   cudaMemsetAsync(x, 0, sizeof(cd) * N, st);
   cudaMemcpyAsync(r, b, sizeof(cd) * N, cudaMemcpyDeviceToDevice, st);
@@ -866,7 +1063,7 @@ static pie_status nested_t(Problem& po, Problem& pi, const cd* b, cd* x, const p
         if ((s = op_scaled<double>(co, zj, w)) != PIE_OK) return s;
         ++outer_products;
         double hn = 0;
-        if ((s = orthogonalize<double>(co, Vo, j, w, cyo, &hn)) != PIE_OK) return s;
+        if ((s = wait_step(co, enqueue_orthogonalize<double>(co, Vo, j, w), j, cyo, &hn)) != PIE_OK) return s;
         const double den = hessenberg_column(cyo, j, hn);
         ++outer_steps;
         if (hn <= 1e-14 * den) {
@@ -874,7 +1071,6 @@ static pie_status nested_t(Problem& po, Problem& pi, const cd* b, cd* x, const p
           ++j;
           break;
         }
-        k_axs<double><<<nb_(N, 256), 256, 0, st>>>(N, 1.0 / hn, w, w);
         if (j + 1 < min_steps) continue;
         bool stop = std::abs(cyo.g[j + 1]) <= np.tol * dbn;
         if (!stop) {
