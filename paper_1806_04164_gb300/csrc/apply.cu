@@ -13,34 +13,43 @@ namespace pie {
 
 // a0: affine restriction of J to every triangle (tree order),
 // J|_t = a (r - c_t) + beta, and the pulse densities sigma, d = 2a + w^2 eps0 sigma.
+// tri_cdcp: tri_c times tri_dcp, multiplied once at set-up (the FP64 pipe bounds
+// the kernel).
 template <typename Rio>
 __global__ void k_coef(int64_t T, int64_t E, const C2<Rio>* __restrict__ x, const int64_t* __restrict__ perm,
                        const int32_t* __restrict__ tri_edge, const double* __restrict__ tri_c,
-                       const double* __restrict__ tri_dcp, double w2e, C2<Rio>* __restrict__ coef,
-                       cf* __restrict__ coef32, int64_t sx = 0, int64_t sc = 0) {
+                       const double* __restrict__ tri_cdcp, double w2e, C2<Rio>* __restrict__ coef,
+                       cf* __restrict__ coef32, int64_t sx = 0, int64_t sc = 0,
+                       const double* __restrict__ scale = nullptr) {
   int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= T) return;
   // right-hand side blockIdx.y (strides sx, sc between right-hand sides)
   x += blockIdx.y * sx;
   if (coef) coef += blockIdx.y * sc;
   if (coef32) coef32 += blockIdx.y * sc;
+  // scale (may be null): the input is scale x, rounded to the io precision
+  auto entry = [&](int64_t n) {
+    const C2<Rio> v = x[n];
+    return scale ? mk<Rio>(Rio(scale[n] * double(v.x)), Rio(scale[n] * double(v.y))) : v;
+  };
   double ar = 0, ai = 0, br[3] = {0, 0, 0}, bi[3] = {0, 0, 0};
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     int32_t n = tri_edge[3 * t + k];
     if (n < 0) continue;
     double c = tri_c[3 * t + k];
-    double xr = double(x[n].x), xi = double(x[n].y);
+    const C2<Rio> v = entry(n);
+    double xr = double(v.x), xi = double(v.y);
     ar += c * xr;
     ai += c * xi;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      double cd_ = c * tri_dcp[9 * t + 3 * k + d];
+      const double cd_ = tri_cdcp[9 * t + 3 * k + d];
       br[d] += cd_ * xr;
       bi[d] += cd_ * xi;
     }
   }
-  C2<Rio> s = x[E + perm[t]];
+  C2<Rio> s = entry(E + perm[t]);
   double sr = double(s.x), si = double(s.y);
   double v[12] = {ar, ai, br[0], bi[0], br[1], bi[1], br[2], bi[2], sr, si, 2.0 * ar + w2e * sr, 2.0 * ai + w2e * si};
   if (coef) {
@@ -826,8 +835,10 @@ __global__ void k_agg_split(int P, int ntheta, int64_t nb, const int32_t* __rest
 // per sample.  The children's patterns are staged in shared memory cg at a
 // time (all eight when they fit: one load latency per parent instead of one
 // per child), and with fs the filter F^T too (else it is read from global
-// memory); children are summed in order, whatever cg.
-template <typename Rf>
+// memory); children are summed in order, whatever cg.  A thread takes NC
+// components, the others threadIdx.z: five where the boxes fill the SMs, one on
+// small levels.
+template <typename Rf, int NC>
 __global__ void k_interp(int P, int64_t nb, const int32_t* __restrict__ child_start,
                          const int8_t* __restrict__ oct_child, const C2<Rf>* __restrict__ Sc,
                          const Rf* __restrict__ Ft, const C2<Rf>* __restrict__ phase, C2<Rf>* __restrict__ Sp,
@@ -840,47 +851,49 @@ __global__ void k_interp(int P, int64_t nb, const int32_t* __restrict__ child_st
   Rf* fsm = reinterpret_cast<Rf*>(smem_raw);
   const size_t fbytes = fs ? ((sizeof(Rf) * P * P + 15) / 16) * 16 : 0;
   C2<Rf>* sm = reinterpret_cast<C2<Rf>*>(smem_raw + fbytes) + threadIdx.y * cg * kComp * P;
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x, nth = blockDim.x * blockDim.y;
+  const int tid = (threadIdx.z * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x;
+  const int nth = blockDim.x * blockDim.y * blockDim.z;
+  const int row_tid = threadIdx.z * blockDim.x + threadIdx.x, row_nth = blockDim.x * blockDim.z, c0 = NC * threadIdx.z;
   if (fs)  // P x P reals as 8-byte words (P = 2 N_theta^2 is even)
     for (int i = tid; i < P * P * int(sizeof(Rf)) / 8; i += nth)
       cp_async(reinterpret_cast<uint2*>(fsm) + i, reinterpret_cast<const uint2*>(Ft) + i);
   const Rf* F = fs ? fsm : Ft;
   const int64_t b = int64_t(blockIdx.x) * blockDim.y + threadIdx.y;
   const bool live = b < nb;
-  const int c0 = live ? child_start[b] : 0, c1 = live ? child_start[b + 1] : 0;
+  const int b0 = live ? child_start[b] : 0, b1 = live ? child_start[b + 1] : 0;
   const int p = threadIdx.x;
-  C2<Rf> acc[kComp];
+  C2<Rf> acc[NC];
 #pragma unroll
-  for (int c = 0; c < kComp; ++c) acc[c] = mk<Rf>(0, 0);
-  for (int k0 = c0;; k0 += cg) {
-    const int nk = k0 < c1 ? min(cg, c1 - k0) : 0;
+  for (int c = 0; c < NC; ++c) acc[c] = mk<Rf>(0, 0);
+  for (int k0 = b0;; k0 += cg) {
+    const int nk = k0 < b1 ? min(cg, b1 - k0) : 0;
     if (!__syncthreads_or(nk > 0)) {  // every row of the block done
       cp_async_wait_all();            // (nothing may stay in flight at exit)
       break;
     }
     // the nk children are consecutive at level l+1: one contiguous copy
-    for (int i = threadIdx.x; i < nk * kComp * P; i += blockDim.x) cp_async(sm + i, Sc + (int64_t)k0 * kComp * P + i);
+    for (int i = row_tid; i < nk * kComp * P; i += row_nth) cp_async(sm + i, Sc + (int64_t)k0 * kComp * P + i);
     cp_async_wait_all();  // (also completes the filter's copy)
     __syncthreads();
     for (int k = 0; k < nk && p < P; ++k) {
-      const C2<Rf>* sk = sm + k * kComp * P;
-      C2<Rf> sum[kComp];
+      const C2<Rf>* sk = sm + (k * kComp + c0) * P;
+      C2<Rf> sum[NC];
 #pragma unroll
-      for (int c = 0; c < kComp; ++c) sum[c] = mk<Rf>(0, 0);
+      for (int c = 0; c < NC; ++c) sum[c] = mk<Rf>(0, 0);
 #pragma unroll 4
       for (int q = 0; q < P; ++q) {
         Rf f = F[(int64_t)q * P + p];
 #pragma unroll
-        for (int c = 0; c < kComp; ++c) rfma(sum[c], f, sk[c * P + q]);
+        for (int c = 0; c < NC; ++c) rfma(sum[c], f, sk[c * P + q]);
       }
       C2<Rf> ph = phase[oct_child[k0 + k] * P + p];
 #pragma unroll
-      for (int c = 0; c < kComp; ++c) cfma(acc[c], ph, sum[c]);
+      for (int c = 0; c < NC; ++c) cfma(acc[c], ph, sum[c]);
     }
   }
   if (live && p < P) {
 #pragma unroll
-    for (int c = 0; c < kComp; ++c) Sp[((int64_t)b * kComp + c) * P + p] = acc[c];
+    for (int c = 0; c < NC; ++c) Sp[((int64_t)b * kComp + c0 + c) * P + p] = acc[c];
   }
 }
 
@@ -1327,7 +1340,7 @@ __global__ void k_trans_split(int P, const TransArgs args) {
 // G_child += F^T (conj(phase_o) G_parent); one child box per threadIdx.y
 // row of a block (several rows for small angular grids).  With fs the
 // filter F is staged in shared memory first (else read from global memory).
-template <typename Rf>
+template <typename Rf, int NC>
 __global__ void k_anterp(int P, int64_t nc, const int32_t* __restrict__ parent, const int8_t* __restrict__ oct_child,
                          const C2<Rf>* __restrict__ Gp, const Rf* __restrict__ Fg, const C2<Rf>* __restrict__ phase,
                          C2<Rf>* __restrict__ Gc, int64_t sGp = 0, int64_t sGc = 0, bool fs = false) {
@@ -1337,7 +1350,9 @@ __global__ void k_anterp(int P, int64_t nc, const int32_t* __restrict__ parent, 
   Rf* fsm = reinterpret_cast<Rf*>(smem_raw);
   const size_t fbytes = fs ? ((sizeof(Rf) * P * P + 15) / 16) * 16 : 0;
   C2<Rf>* sm = reinterpret_cast<C2<Rf>*>(smem_raw + fbytes) + threadIdx.y * kComp * P;
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x, nth = blockDim.x * blockDim.y;
+  const int tid = (threadIdx.z * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x;
+  const int nth = blockDim.x * blockDim.y * blockDim.z;
+  const int row_tid = threadIdx.z * blockDim.x + threadIdx.x, row_nth = blockDim.x * blockDim.z, c0 = NC * threadIdx.z;
   if (fs)  // P x P reals as 8-byte words (P = 2 N_theta^2 is even)
     for (int i = tid; i < P * P * int(sizeof(Rf)) / 8; i += nth)
       cp_async(reinterpret_cast<uint2*>(fsm) + i, reinterpret_cast<const uint2*>(Fg) + i);
@@ -1348,9 +1363,9 @@ __global__ void k_anterp(int P, int64_t nc, const int32_t* __restrict__ parent, 
   const int o = live ? oct_child[ch] : 0;
   // the parent's pattern copied in, then turned in place by the thread
   // that copied each entry: conj(phase_o) G_parent
-  for (int i = threadIdx.x; live && i < kComp * P; i += blockDim.x) cp_async(sm + i, Gp + (int64_t)par * kComp * P + i);
+  for (int i = row_tid; live && i < kComp * P; i += row_nth) cp_async(sm + i, Gp + (int64_t)par * kComp * P + i);
   cp_async_wait_all();
-  for (int i = threadIdx.x; live && i < kComp * P; i += blockDim.x) {
+  for (int i = row_tid; live && i < kComp * P; i += row_nth) {
     const int q = i % P;
     const C2<Rf> g = sm[i], ph = phase[o * P + q];
     C2<Rf> h;
@@ -1361,18 +1376,18 @@ __global__ void k_anterp(int P, int64_t nc, const int32_t* __restrict__ parent, 
   __syncthreads();
   if (!live) return;
   for (int p = threadIdx.x; p < P; p += blockDim.x) {
-    C2<Rf> sum[kComp];
+    C2<Rf> sum[NC];
 #pragma unroll
-    for (int c = 0; c < kComp; ++c) sum[c] = mk<Rf>(0, 0);
+    for (int c = 0; c < NC; ++c) sum[c] = mk<Rf>(0, 0);
 #pragma unroll 4
     for (int q = 0; q < P; ++q) {
       Rf f = F[(int64_t)q * P + p];
 #pragma unroll
-      for (int c = 0; c < kComp; ++c) rfma(sum[c], f, sm[c * P + q]);
+      for (int c = 0; c < NC; ++c) rfma(sum[c], f, sm[(c0 + c) * P + q]);
     }
 #pragma unroll
-    for (int c = 0; c < kComp; ++c) {
-      C2<Rf>& g = Gc[((int64_t)ch * kComp + c) * P + p];
+    for (int c = 0; c < NC; ++c) {
+      C2<Rf>& g = Gc[((int64_t)ch * kComp + c0 + c) * P + p];
       g.x += sum[c].x;
       g.y += sum[c].y;
     }
@@ -1382,6 +1397,8 @@ __global__ void k_anterp(int P, int64_t nc, const int32_t* __restrict__ parent, 
 // Sum and difference of the incoming leaf patterns over antipodal sample
 // pairs, once per box: GS[b][c][q] = G(q) + G(-q), GD[b][c][q] = G(q) - G(-q)
 // (half grid q), shared by all triangles of the box in the disaggregation.
+// Double only: float adds are cheaper than the pass, so float disaggregation
+// forms them itself (the same sums).
 template <typename Rf>
 __global__ void k_gsgd(int P, int ntheta, const C2<Rf>* __restrict__ G, C2<Rf>* __restrict__ GS,
                        C2<Rf>* __restrict__ GD, int64_t sG = 0, int64_t sH = 0) {
@@ -1399,23 +1416,22 @@ __global__ void k_gsgd(int P, int ntheta, const C2<Rf>* __restrict__ G, C2<Rf>* 
   }
 }
 
-// a6: leaf disaggregation with the receiving (conjugate) patterns.  One
-// thread per triangle; the receiving tables are stored sample-major
+// a6: leaf disaggregation with the receiving (conjugate) patterns, float
+// patterns of many triangles (k_disagg_split otherwise).  One thread per
+// triangle; the receiving tables are stored sample-major
 // ([Ph][T], [3][Ph][T]) so that consecutive threads read consecutive
-// triangles, and the box's sum / difference patterns are shared through the
-// cache.  Over a sample pair (q, -q):
+// triangles, and the box's patterns are shared through the cache.  Over a sample pair (q, -q):
 // conj(X(q)) G(q) + X(q) G(-q) = Xr (G(q) + G(-q)) - i Xi (G(q) - G(-q)).
 // Adds to pot[t].
 template <typename Rf, typename Rio>
-__global__ void __launch_bounds__(256) k_disagg(int64_t T, int P, const int32_t* __restrict__ leaf_of,
+__global__ void __launch_bounds__(256) k_disagg(int64_t T, int P, int ntheta, const int32_t* __restrict__ leaf_of,
                                                 const C2<Rf>* __restrict__ PiR, const C2<Rf>* __restrict__ MR,
-                                                const C2<Rf>* __restrict__ GS, const C2<Rf>* __restrict__ GD,
-                                                C2<Rio>* __restrict__ pot, int64_t sH = 0, int64_t sp = 0) {
+                                                const C2<Rf>* __restrict__ G, C2<Rio>* __restrict__ pot,
+                                                int64_t sG = 0, int64_t sp = 0) {
   int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= T) return;
   const int Ph = P / 2;
-  GS += blockIdx.y * sH + (int64_t)leaf_of[t] * kComp * Ph;
-  GD += blockIdx.y * sH + (int64_t)leaf_of[t] * kComp * Ph;
+  G += blockIdx.y * sG + (int64_t)leaf_of[t] * kComp * P;
   pot += blockIdx.y * sp;
   C2<Rf> acc[6];
 #pragma unroll
@@ -1429,8 +1445,9 @@ __global__ void __launch_bounds__(256) k_disagg(int64_t T, int P, const int32_t*
   auto load = [&](int q, Sample& r) {
 #pragma unroll
     for (int c = 0; c < kComp; ++c) {
-      r.gs[c] = GS[c * Ph + q];
-      r.gd[c] = GD[c * Ph + q];
+      const C2<Rf> u = G[c * P + q], v = G[c * P + antipode(q, ntheta)];
+      r.gs[c] = mk<Rf>(u.x + v.x, u.y + v.y);
+      r.gd[c] = mk<Rf>(u.x - v.x, u.y - v.y);
     }
     r.pi = PiR[(int64_t)q * T + t];
 #pragma unroll
@@ -1477,15 +1494,17 @@ __global__ void __launch_bounds__(256) k_disagg(int64_t T, int P, const int32_t*
 // 1232 -> 1204 us).  Float patterns of many triangles keep k_disagg, which reads
 // each table entry once.
 template <typename Rf, typename Rio>
-__global__ void __launch_bounds__(160) k_disagg_split(int64_t T, int P, const int32_t* __restrict__ leaf_of,
+__global__ void __launch_bounds__(160) k_disagg_split(int64_t T, int P, int ntheta, const int32_t* __restrict__ leaf_of,
                                                       const C2<Rf>* __restrict__ PiR, const C2<Rf>* __restrict__ MR,
                                                       const C2<Rf>* __restrict__ GS, const C2<Rf>* __restrict__ GD,
                                                       C2<Rio>* __restrict__ pot, int64_t sH = 0, int64_t sp = 0) {
   const int64_t t = blockIdx.x * (int64_t)32 + threadIdx.x;
   if (t >= T) return;
   const int Ph = P / 2;
-  const Rf* gs = reinterpret_cast<const Rf*>(GS + blockIdx.y * sH + (int64_t)leaf_of[t] * kComp * Ph);
-  const Rf* gd = reinterpret_cast<const Rf*>(GD + blockIdx.y * sH + (int64_t)leaf_of[t] * kComp * Ph);
+  // double: the sum and difference patterns GS, GD; float: GS is the pattern G itself
+  constexpr bool WHOLE = sizeof(Rf) == 4;
+  const Rf* gs = reinterpret_cast<const Rf*>(GS + blockIdx.y * sH + (int64_t)leaf_of[t] * kComp * (WHOLE ? P : Ph));
+  const Rf* gd = WHOLE ? gs : reinterpret_cast<const Rf*>(GD + blockIdx.y * sH + (int64_t)leaf_of[t] * kComp * Ph);
   Rio* o = reinterpret_cast<Rio*>(pot + blockIdx.y * sp + 6 * t);
   // NS sums over the sample pairs: load(q, d) gives the operands of sum (or
   // step) d, step(d) its two multiply-adds; four sample pairs' loads are issued
@@ -1519,14 +1538,21 @@ __global__ void __launch_bounds__(160) k_disagg_split(int64_t T, int P, const in
       sum(q + U, b);
     }
   };
-  auto at = [&](const Rf* g, int c, int q, int im) { return g[2 * (c * Ph + q) + im]; };
+  auto at_s = [&](int c, int q, int im) {
+    if constexpr (WHOLE) return gs[2 * (c * P + q) + im] + gs[2 * (c * P + antipode(q, ntheta)) + im];
+    return gs[2 * (c * Ph + q) + im];
+  };
+  auto at_d = [&](int c, int q, int im) {
+    if constexpr (WHOLE) return gs[2 * (c * P + q) + im] - gs[2 * (c * P + antipode(q, ntheta)) + im];
+    return gd[2 * (c * Ph + q) + im];
+  };
   // im = 0: real part, += x.x s.x + x.y d.y; im = 1: imaginary part, += x.x s.y - x.y d.x
   auto U = [&](auto imc) {
     constexpr int im = decltype(imc)::value;
     Rf u = 0;
     run(
         std::integral_constant<int, 3>(),
-        [&](int q, int d) { return Op{MR[((int64_t)d * Ph + q) * T + t], at(gs, d, q, im), at(gd, d, q, 1 - im)}; },
+        [&](int q, int d) { return Op{MR[((int64_t)d * Ph + q) * T + t], at_s(d, q, im), at_d(d, q, 1 - im)}; },
         [&](int, const Op& v) {
           u = fma(v.x.x, v.s, u);
           u = fma(im ? -v.x.y : v.x.y, v.d, u);
@@ -1538,7 +1564,7 @@ __global__ void __launch_bounds__(160) k_disagg_split(int64_t T, int P, const in
     Rf v[3] = {0, 0, 0};
     run(
         std::integral_constant<int, 3>(),
-        [&](int q, int d) { return Op{PiR[(int64_t)q * T + t], at(gs, d, q, im), at(gd, d, q, 1 - im)}; },
+        [&](int q, int d) { return Op{PiR[(int64_t)q * T + t], at_s(d, q, im), at_d(d, q, 1 - im)}; },
         [&](int d, const Op& w) {
           v[d] = fma(w.x.x, w.s, v[d]);
           v[d] = fma(im ? -w.x.y : w.x.y, w.d, v[d]);
@@ -1555,7 +1581,7 @@ __global__ void __launch_bounds__(160) k_disagg_split(int64_t T, int P, const in
   Rf v[4] = {0, 0, 0, 0};  // T1 real, imaginary, T2 real, imaginary
   run(
       std::integral_constant<int, 4>(),
-      [&](int q, int d) { return Op{PiR[(int64_t)q * T + t], at(gs, 3 + d / 2, q, d % 2), at(gd, 3 + d / 2, q, 1 - d % 2)}; },
+      [&](int q, int d) { return Op{PiR[(int64_t)q * T + t], at_s(3 + d / 2, q, d % 2), at_d(3 + d / 2, q, 1 - d % 2)}; },
       [&](int d, const Op& w) {
         v[d] = fma(w.x.x, w.s, v[d]);
         v[d] = fma(d % 2 ? -w.x.y : w.x.y, w.d, v[d]);
@@ -1569,21 +1595,24 @@ __global__ void __launch_bounds__(160) k_disagg_split(int64_t T, int P, const in
 template <typename Rio>
 __device__ __forceinline__ C2<Rio> pot_sum(const C2<Rio>* pot, const C2<Rio>* pot2, int64_t j) {
   if (!pot2) return pot[j];
+  // (two floats summed in double and rounded again are the floats' rounded sum)
   const C2<Rio> a = pot2[j], b = pot[j];
-  return mk<Rio>(Rio(double(a.x) + double(b.x)), Rio(double(a.y) + double(b.y)));
+  return mk<Rio>(a.x + b.x, a.y + b.y);
 }
 
 // a7: Galerkin testing of the per-triangle potentials (Section 2):
 // RWG m: sum over its two triangles of c [U + (c_t - p).V] + 2c T1; pulse t: T2.
-// pot2 (may be null): near-part potentials, added to pot first.
+// pot2 (may be null): near-part potentials, added to pot first.  scale (may be
+// null): the result is scale y, y rounded to the io precision first.
 template <typename Rio>
 __global__ void k_assemble(int64_t N, int64_t E, const int32_t* __restrict__ edge_tt,
                            const int8_t* __restrict__ edge_k, const double* __restrict__ tri_c,
                            const double* __restrict__ tri_dcp, const int64_t* __restrict__ inv_perm,
                            const C2<Rio>* __restrict__ pot, C2<Rio>* __restrict__ y, int64_t sp = 0, int64_t sy = 0,
-                           const C2<Rio>* __restrict__ pot2 = nullptr) {
+                           const C2<Rio>* __restrict__ pot2 = nullptr, const double* __restrict__ scale = nullptr) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= N) return;
+  C2<Rio> out;
   pot += blockIdx.y * sp;
   if (pot2) pot2 += blockIdx.y * sp;
   y += blockIdx.y * sy;
@@ -1603,11 +1632,12 @@ __global__ void k_assemble(int64_t N, int64_t E, const int32_t* __restrict__ edg
       yr += c * (ur + 2.0 * double(p[4].x));
       yi += c * (ui + 2.0 * double(p[4].y));
     }
-    y[i] = mk<Rio>(Rio(yr), Rio(yi));
+    out = mk<Rio>(Rio(yr), Rio(yi));
   } else {
     int64_t t = inv_perm[i - E];
-    y[i] = pot_sum(pot, pot2, 6 * t + 5);
+    out = pot_sum(pot, pot2, 6 * t + 5);
   }
+  y[i] = scale ? mk<Rio>(Rio(scale[i] * double(out.x)), Rio(scale[i] * double(out.y))) : out;
 }
 
 // ---------------------------------------------------------------- orchestration
@@ -1633,7 +1663,7 @@ void prof_mark(Problem& pr, int stage, bool end, cudaStream_t st) {
 }
 
 template <typename Rm, typename Rf, typename Rio, bool H16 = false>
-static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaStream_t st) {
+static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaStream_t st, const double* scale) {
   const int P = pr.P;
   const int L = pr.tree.L;
   const C2<Rio>* x = static_cast<const C2<Rio>*>(xv);
@@ -1647,8 +1677,8 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
   cf* coef32 = split ? static_cast<cf*>(pr.coef32) : nullptr;
   const C2<Rm>* ncoef = split ? reinterpret_cast<const C2<Rm>*>(coef32) : reinterpret_cast<const C2<Rm>*>(coef);
   prof_mark(pr, 0, false, st);
-  k_coef<Rio><<<dim3(nblk(pr.T, 256), nr), 256, 0, st>>>(pr.T, pr.E, x, pr.perm, pr.tri_edge, pr.tri_c, pr.tri_dcp,
-                                                         w2e, coef, coef32, sN, sT);
+  k_coef<Rio><<<dim3(nblk(pr.T, 256), nr), 256, 0, st>>>(pr.T, pr.E, x, pr.perm, pr.tri_edge, pr.tri_c, pr.tri_cdcp,
+                                                         w2e, coef, coef32, sN, sT, scale);
   prof_mark(pr, 0, true, st);
   // near part into pot2, far part into pot.  With tune.overlap the near part
   // runs on the side stream (HBM-bound, a bounded grid) and the far part on
@@ -1805,12 +1835,22 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
     k_child_sum<Rf><<<dim3(unsigned(pr.lev[l].nb), nr, kComp), P, 0, sf>>>(
         P, pr.lev[l].child_start, U, static_cast<C2<Rf>*>(pr.lev[l].S), sl(l + 1), sl(l));
   }
-  for (int l = L - 1; l >= 3 && !fft8; --l) {
-    k_interp<Rf><<<dim3(nblk(pr.lev[l].nb, fbp), nr), dim3(tpb, fbp), fsm_bytes + sm * fbp * cg, sf>>>(
-        P, pr.lev[l].nb, pr.lev[l].child_start, pr.lev[l + 1].octant, static_cast<const C2<Rf>*>(pr.lev[l + 1].S),
-        static_cast<const Rf*>(pr.lev[l].Ft), static_cast<const C2<Rf>*>(pr.lev[l].phase),
-        static_cast<C2<Rf>*>(pr.lev[l].S), sl(l + 1), sl(l), cg, fsh);
-  }
+  // dense filter: (components a thread, boxes per block, children staged at a time)
+  auto dense = [&](int64_t nb, auto f) {
+    if (narrow(nb * (tpb / 32) * nr) && tpb * kComp <= 1024)
+      f(std::integral_constant<int, 1>(), 1, int(std::max<size_t>(1, std::min<size_t>(8, (49152 - fsm_bytes) / sm))));
+    else
+      f(std::integral_constant<int, kComp>(), fbp, cg);
+  };
+  for (int l = L - 1; l >= 3 && !fft8; --l)
+    dense(pr.lev[l].nb, [&](auto ncc, int rows, int kids) {
+      constexpr int NC = decltype(ncc)::value;
+      k_interp<Rf, NC><<<dim3(nblk(pr.lev[l].nb, rows), nr), dim3(tpb, rows, kComp / NC),
+                         fsm_bytes + sm * rows * kids, sf>>>(
+          P, pr.lev[l].nb, pr.lev[l].child_start, pr.lev[l + 1].octant, static_cast<const C2<Rf>*>(pr.lev[l + 1].S),
+          static_cast<const Rf*>(pr.lev[l].Ft), static_cast<const C2<Rf>*>(pr.lev[l].phase),
+          static_cast<C2<Rf>*>(pr.lev[l].S), sl(l + 1), sl(l), kids, fsh);
+    });
   prof_mark(pr, 3, true, st);
   prof_mark(pr, 4, false, st);
   TransArgs ta;
@@ -1853,30 +1893,35 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
         static_cast<const Rf*>(pr.lev[l].Kf), static_cast<const C2<Rf>*>(pr.lev[l].phase),
         static_cast<C2<Rf>*>(pr.lev[l + 1].G), sl(l), sl(l + 1));
   }
-  for (int l = 3; l < L && !fft8; ++l) {
-    k_anterp<Rf><<<dim3(nblk(pr.lev[l + 1].nb, fbp), nr), dim3(tpb, fbp), fsm_bytes + sm * fbp, sf>>>(
-        P, pr.lev[l + 1].nb, pr.lev[l + 1].parent, pr.lev[l + 1].octant, static_cast<const C2<Rf>*>(pr.lev[l].G),
-        static_cast<const Rf*>(pr.lev[l].F), static_cast<const C2<Rf>*>(pr.lev[l].phase),
-        static_cast<C2<Rf>*>(pr.lev[l + 1].G), sl(l), sl(l + 1), fsh);
-  }
+  for (int l = 3; l < L && !fft8; ++l)
+    dense(pr.lev[l + 1].nb, [&](auto ncc, int rows, int) {
+      constexpr int NC = decltype(ncc)::value;
+      k_anterp<Rf, NC><<<dim3(nblk(pr.lev[l + 1].nb, rows), nr), dim3(tpb, rows, kComp / NC), fsm_bytes + sm * rows,
+                         sf>>>(P, pr.lev[l + 1].nb, pr.lev[l + 1].parent, pr.lev[l + 1].octant,
+                               static_cast<const C2<Rf>*>(pr.lev[l].G), static_cast<const Rf*>(pr.lev[l].F),
+                               static_cast<const C2<Rf>*>(pr.lev[l].phase), static_cast<C2<Rf>*>(pr.lev[l + 1].G),
+                               sl(l), sl(l + 1), fsh);
+    });
   prof_mark(pr, 5, true, st);
   prof_mark(pr, 6, false, st);
   {
-    C2<Rf>* GS = static_cast<C2<Rf>*>(pr.gsgd);
-    C2<Rf>* GD = GS + int64_t(pr.par.max_nrhs) * pr.lev[L].nb * kComp * (P / 2);
-    const int64_t sH = int64_t(pr.lev[L].nb) * kComp * (P / 2);
-    k_gsgd<Rf><<<dim3(unsigned(pr.lev[L].nb), nr), 128, 0, sf>>>(P, pr.par.ntheta,
-                                                                 static_cast<const C2<Rf>*>(pr.lev[L].G), GS, GD,
-                                                                 sl(L), sH);
+    const C2<Rf>* G = static_cast<const C2<Rf>*>(pr.lev[L].G);
     const C2<Rf>* PiR = static_cast<const C2<Rf>*>(pr.PiR);
     const C2<Rf>* MR = static_cast<const C2<Rf>*>(pr.MR);
-    bool whole = false;  // a thread per triangle
-    if constexpr (sizeof(Rf) == 4) whole = !narrow((pr.T + 31) / 32 * nr);
-    if (whole) {
-      if constexpr (sizeof(Rf) == 4)
-        k_disagg<Rf, Rio><<<dim3(nblk(pr.T, 256), nr), 256, 0, sf>>>(pr.T, P, pr.leaf_of, PiR, MR, GS, GD, pot, sH, sT);
+    const int nt = pr.par.ntheta;
+    if constexpr (sizeof(Rf) == 4) {
+      if (narrow((pr.T + 31) / 32 * nr))
+        k_disagg_split<Rf, Rio><<<dim3(nblk(pr.T, 32), nr), dim3(32, 5), 0, sf>>>(pr.T, P, nt, pr.leaf_of, PiR, MR, G, G,
+                                                                                  pot, sl(L), sT);
+      else
+        k_disagg<Rf, Rio><<<dim3(nblk(pr.T, 256), nr), 256, 0, sf>>>(pr.T, P, nt, pr.leaf_of, PiR, MR, G, pot, sl(L),
+                                                                     sT);
     } else {
-      k_disagg_split<Rf, Rio><<<dim3(nblk(pr.T, 32), nr), dim3(32, 5), 0, sf>>>(pr.T, P, pr.leaf_of, PiR, MR, GS, GD,
+      C2<Rf>* GS = static_cast<C2<Rf>*>(pr.gsgd);
+      const int64_t sH = int64_t(pr.lev[L].nb) * kComp * (P / 2);
+      C2<Rf>* GD = GS + int64_t(pr.par.max_nrhs) * sH;
+      k_gsgd<Rf><<<dim3(unsigned(pr.lev[L].nb), nr), 128, 0, sf>>>(P, nt, G, GS, GD, sl(L), sH);
+      k_disagg_split<Rf, Rio><<<dim3(nblk(pr.T, 32), nr), dim3(32, 5), 0, sf>>>(pr.T, P, nt, pr.leaf_of, PiR, MR, GS, GD,
                                                                                 pot, sH, sT);
     }
   }
@@ -1892,7 +1937,7 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
   }
   prof_mark(pr, 7, false, st);
   k_assemble<Rio><<<dim3(nblk(pr.N, 256), nr), 256, 0, st>>>(pr.N, pr.E, pr.edge_tt, pr.edge_k, pr.tri_c,
-                                                             pr.tri_dcp, pr.inv_perm, pot, y, sT, sN, pot2);
+                                                             pr.tri_dcp, pr.inv_perm, pot, y, sT, sN, pot2, scale);
   prof_mark(pr, 7, true, st);
   if (pr.prof_n < pr.prof_cap) ++pr.prof_n;
   return cuda_check(cudaGetLastError(), "apply launch");
@@ -1907,7 +1952,7 @@ static pie_status apply_near_t(Problem& pr, const void* xv, void* yv, cudaStream
   cf* coef32 = split ? static_cast<cf*>(pr.coef32) : nullptr;
   const C2<Rm>* ncoef = split ? reinterpret_cast<const C2<Rm>*>(coef32) : reinterpret_cast<const C2<Rm>*>(coef);
   k_coef<Rio><<<nblk(pr.T, 256), 256, 0, st>>>(pr.T, pr.E, static_cast<const C2<Rio>*>(xv), pr.perm, pr.tri_edge,
-                                               pr.tri_c, pr.tri_dcp, pr.w * pr.w * eps0(), coef, coef32);
+                                               pr.tri_c, pr.tri_cdcp, pr.w * pr.w * eps0(), coef, coef32);
   if constexpr (sizeof(Rm) == 8) {
     near_fixed(pr, coef, pot, 1, 0, st);
   } else if (pr.tune.near_kernel != 1) {  // the box-staged kernel, unless tuned off
@@ -1941,26 +1986,28 @@ pie_status apply_near_one(Problem& pr, const void* x, void* y, cudaStream_t st) 
   }
 }
 
-pie_status apply_batch(Problem& pr, const void* x, void* y, int nrhs, cudaStream_t st) {
+pie_status apply_batch(Problem& pr, const void* x, void* y, int nrhs, cudaStream_t st, const double* scale) {
   if (nrhs < 1 || nrhs > pr.par.max_nrhs) {
     set_error("batch larger than max_nrhs");
     return PIE_ERR_PARAM;
   }
   switch (pr.par.precision) {
     case PIE_FP64:
-      return apply_t<double, double, double>(pr, x, y, nrhs, st);
+      return apply_t<double, double, double>(pr, x, y, nrhs, st, scale);
     case PIE_FP32:
-      return apply_t<float, float, float>(pr, x, y, nrhs, st);
+      return apply_t<float, float, float>(pr, x, y, nrhs, st, scale);
     case PIE_MIXED:
-      return apply_t<float, double, double>(pr, x, y, nrhs, st);
+      return apply_t<float, double, double>(pr, x, y, nrhs, st, scale);
     case PIE_FP32H:
-      return apply_t<float, float, float, true>(pr, x, y, nrhs, st);
+      return apply_t<float, float, float, true>(pr, x, y, nrhs, st, scale);
   }
   set_error("unknown precision");
   return PIE_ERR_PARAM;
 }
 
-pie_status apply_one(Problem& pr, const void* x, void* y, cudaStream_t st) { return apply_batch(pr, x, y, 1, st); }
+pie_status apply_one(Problem& pr, const void* x, void* y, cudaStream_t st, const double* scale) {
+  return apply_batch(pr, x, y, 1, st, scale);
+}
 
 pie_status apply_cols(Problem& pr, const void* x, void* y, int nrhs, cudaStream_t st) {
   const size_t col = (pr.io_f32() ? sizeof(cf) : sizeof(cd)) * size_t(pr.N);
@@ -2313,7 +2360,7 @@ template <typename Rio>
 static C2<Rio>* field_coef(Problem& pr, const void* x, cudaStream_t st) {
   C2<Rio>* coef = static_cast<C2<Rio>*>(pr.coef);
   k_coef<Rio><<<nblk(pr.T, 256), 256, 0, st>>>(pr.T, pr.E, static_cast<const C2<Rio>*>(x), pr.perm, pr.tri_edge,
-                                               pr.tri_c, pr.tri_dcp, pr.w * pr.w * eps0(), coef, nullptr);
+                                               pr.tri_c, pr.tri_cdcp, pr.w * pr.w * eps0(), coef, nullptr);
   if constexpr (sizeof(Rio) == 8) k_field_coef<<<nblk(pr.T, 256), 256, 0, st>>>(pr.T, pr.vert, pr.cent, coef);
   return coef;
 }
@@ -2371,7 +2418,7 @@ pie_status apply_near_scratch(Problem& pr, const void* x, void* y, void* coef, v
   const double w2e = pr.w * pr.w * eps0();
   if (pr.io_f32()) {
     k_coef<float><<<nblk(pr.T, 256), 256, 0, st>>>(pr.T, pr.E, static_cast<const cf*>(x), pr.perm, pr.tri_edge,
-                                                   pr.tri_c, pr.tri_dcp, w2e, static_cast<cf*>(coef), nullptr);
+                                                   pr.tri_c, pr.tri_cdcp, w2e, static_cast<cf*>(coef), nullptr);
     if (pr.near_h16())
       k_near<float, float, 1, true><<<nblk(pr.T * 32, 256), 256, 0, st>>>(
           pr.T, pr.nnz, pr.leaf_of, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr, nullptr,
@@ -2387,7 +2434,7 @@ pie_status apply_near_scratch(Problem& pr, const void* x, void* y, void* coef, v
   } else {
     const bool split = pr.near_f32();
     k_coef<double><<<nblk(pr.T, 256), 256, 0, st>>>(pr.T, pr.E, static_cast<const cd*>(x), pr.perm, pr.tri_edge,
-                                                    pr.tri_c, pr.tri_dcp, w2e, split ? nullptr : static_cast<cd*>(coef),
+                                                    pr.tri_c, pr.tri_cdcp, w2e, split ? nullptr : static_cast<cd*>(coef),
                                                     split ? static_cast<cf*>(coef) : nullptr);
     if (split)
       k_near<float, double><<<nblk(pr.T * 32, 256), 256, 0, st>>>(

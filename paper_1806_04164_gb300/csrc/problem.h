@@ -57,6 +57,7 @@ struct Problem {
   int32_t* tri_edge = nullptr;   // [T*3]
   double* tri_c = nullptr;       // [T*3]  s l / (2A)
   double* tri_dcp = nullptr;     // [T*9]  c_t - p
+  double* tri_cdcp = nullptr;    // [T*9]  tri_c (c_t - p)
   int64_t* perm = nullptr;       // [T] tree -> mesh
   int64_t* inv_perm = nullptr;   // [T] mesh -> tree
   int32_t* edge_tt = nullptr;    // [E*2] tree positions of T+, T-
@@ -131,8 +132,9 @@ struct Problem {
 // setup kernels (setup.cu)
 pie_status setup_device(Problem& pr, cudaStream_t st);
 // apply (apply.cu)
-pie_status apply_one(Problem& pr, const void* x, void* y, cudaStream_t st);
-pie_status apply_batch(Problem& pr, const void* x, void* y, int nrhs, cudaStream_t st);
+// scale (may be null, [N] double): y = scale Z (scale x), each vector rounded to the io precision
+pie_status apply_one(Problem& pr, const void* x, void* y, cudaStream_t st, const double* scale = nullptr);
+pie_status apply_batch(Problem& pr, const void* x, void* y, int nrhs, cudaStream_t st, const double* scale = nullptr);
 // x, y: N x nrhs columns, passes of tune.rhs_chunk columns
 pie_status apply_cols(Problem& pr, const void* x, void* y, int nrhs, cudaStream_t st);
 // the shared-memory limit of the fixed-point near kernel on the current device (set-up of PIE_FP64 problems)

@@ -782,7 +782,7 @@ static pie_status setup_t(Problem& pr, cudaStream_t st) {
 
   // tree-ordered triangle tables
   std::vector<int32_t> tri_edge(T * 3), leaf_of(T);
-  std::vector<double> tri_c(T * 3, 0.0), tri_dcp(T * 9, 0.0), vert(T * 9), cent(T * 3), h2(T), area(T);
+  std::vector<double> tri_c(T * 3, 0.0), tri_dcp(T * 9, 0.0), tri_cdcp(T * 9, 0.0), vert(T * 9), cent(T * 3), h2(T), area(T);
   for (int64_t i = 0; i < T; ++i) {
     int64_t tm = tr.perm[i];
     for (int k = 0; k < 3; ++k) {
@@ -805,7 +805,10 @@ static pie_status setup_t(Problem& pr, cudaStream_t st) {
       double len = std::sqrt((b[0] - a[0]) * (b[0] - a[0]) + (b[1] - a[1]) * (b[1] - a[1]) + (b[2] - a[2]) * (b[2] - a[2]));
       tri_c[3 * i + k] = sg * len / (2.0 * m.area[tm]);
       int32_t fv = m.edge_free[2 * n + (sg > 0 ? 0 : 1)];
-      for (int d = 0; d < 3; ++d) tri_dcp[9 * i + 3 * k + d] = m.centroid[3 * tm + d] - m.xyz[3 * fv + d];
+      for (int d = 0; d < 3; ++d) {
+        tri_dcp[9 * i + 3 * k + d] = m.centroid[3 * tm + d] - m.xyz[3 * fv + d];
+        tri_cdcp[9 * i + 3 * k + d] = tri_c[3 * i + k] * tri_dcp[9 * i + 3 * k + d];
+      }
     }
   }
   std::vector<int32_t> edge_tt(E * 2);
@@ -901,6 +904,7 @@ static pie_status setup_t(Problem& pr, cudaStream_t st) {
   pr.tri_edge = upload(pr, tri_edge, st, s);
   pr.tri_c = upload(pr, tri_c, st, s);
   pr.tri_dcp = upload(pr, tri_dcp, st, s);
+  pr.tri_cdcp = upload(pr, tri_cdcp, st, s);
   pr.perm = upload(pr, tr.perm, st, s);
   pr.inv_perm = upload(pr, tr.inv_perm, st, s);
   pr.edge_tt = upload(pr, edge_tt, st, s);

@@ -529,7 +529,7 @@ static void op_time_flush(Ctx& c) {
 
 // out = Z in, or out = S in for the single-layer operator of Eq. (3)
 // (vectors in the io precision of the context's problem).
-static pie_status op_apply(Ctx& c, const void* in, void* out) {
+static pie_status op_apply(Ctx& c, const void* in, void* out, const double* scale = nullptr) {
   ProductEvents* v = c.ev;
   const unsigned slot = v ? v->n++ % kSlots : 0;
   const bool timed = v && v->e[slot][0] && v->e[slot][1];
@@ -537,7 +537,7 @@ static pie_status op_apply(Ctx& c, const void* in, void* out) {
     op_time_flush(c, slot);
     cudaEventRecord(v->e[slot][0], c.st);
   }
-  pie_status s = c.op == 0 ? apply_one(c.pr, in, out, c.st) : single_layer_one(c.pr, in, out, c.st);
+  pie_status s = c.op == 0 ? apply_one(c.pr, in, out, c.st, scale) : single_layer_one(c.pr, in, out, c.st);
   if (timed) {
     cudaEventRecord(v->e[slot][1], c.st);
     v->pending[slot] = true;
@@ -546,11 +546,13 @@ static pie_status op_apply(Ctx& c, const void* in, void* out) {
 }
 
 // out = D Op D in for a Krylov vector in type B; the product runs on complex
-// double vectors, or on complex float ones for a PIE_FP32 problem.
+// double vectors, or on complex float ones for a PIE_FP32 problem.  Where that is
+// type B the product scales its own input and output.
 template <typename B>
 static pie_status op_scaled(Ctx& c, const C2<B>* in, C2<B>* out) {
   const int64_t N = c.N;
   pie_status s;
+  if (c.op == 0 && c.pr.io_f32() == (sizeof(B) == 4)) return op_apply(c, in, out, c.d);
   if (c.pr.io_f32()) {
     k_scale<B, float><<<nb_(N, 256), 256, 0, c.st>>>(N, c.d, in, c.u32);
     if ((s = op_apply(c, c.u32, c.w32)) != PIE_OK) return s;
