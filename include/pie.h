@@ -425,8 +425,7 @@ pie_status pie_nearfield(pie_problem* pr, const void* x, const void* rho, const 
  *  near_rhs_block: right-hand sides that one pass of the near kernel
  *    carries (each pair's moments are read once for them): 1, 2, 4 or 8
  *    (8 only with the warp-per-triangle kernel), or 0 to pick by the pass
- *    width (1 for one column, 2 for two, else 4; fewer where the box-staged
- *    kernel's rows would not fit in shared memory).
+ *    width (1 for one column, 2 for two, else 4).
  *  far_rows: tile shape of the per-box far kernels of angular grids other
  *    than N_theta = 8 (aggregation, dense interpolation and anterpolation,
  *    translation; one thread per sample): boxes per block, 1, 2, 4, 8, 16 or
@@ -436,9 +435,8 @@ pie_status pie_nearfield(pie_problem* pr, const void* x, const void* rho, const 
  *    test triangle reading the coefficients from global memory (1, 2, 4 or
  *    8 right-hand sides per thread), 2 = box-staged (one block per leaf box
  *    and group of up to 4 right-hand sides, the box's source coefficients
- *    in shared memory), 0 = automatic (box-staged while the longest row's
- *    coefficients fit in shared memory).  Both take the same operations in
- *    the same order.  near_rhs_block 8 always uses the warp-per-triangle
+ *    in shared memory), 0 = automatic (box-staged).  Both take the same
+ *    operations in the same order.  near_rhs_block 8 always uses the warp-per-triangle
  *    kernel.
  *    A complex double near part runs in fixed point, one column per block,
  *    whatever near_rhs_block and near_kernel say.

@@ -207,59 +207,66 @@ __device__ __forceinline__ float warp_sum12(const cf* a, int lane, int* componen
   return z + __shfl_xor_sync(0xffffffffu, z, 1);
 }
 
-// a1, float near part: one block per leaf box (grid stride over boxes) and
-// per group of RB right-hand sides (blockIdx.y).  Every test triangle of a
-// box runs over the same source list (the concatenated source ranges of its
-// near boxes), so the block stages those sources' coefficients in shared
-// memory once per right-hand side, plane by plane ([RB][6][stage], dynamic
-// shared memory: stage is the problem's longest row), and its warps take the
-// box's test triangles in turn, lanes over the row as in k_near (lane j,
-// j + 32, ...): each moment is read once for the RB right-hand sides, and every
-// right-hand side sees the same operations in the same order as in k_near, so
-// the same result to the last bit.  nsplit shares a box's test triangles among
-// several blocks when the leaf boxes alone do not fill the SMs.  Rows longer
-// than stage (kNearSmemMax allows 1188 sources at RB = 4, 4752 at RB = 1) read the
-// coefficients from global memory instead.
-// Half-precision records of one right-hand side reach shared memory by cp.async
-// kNearAhead steps of 32 entries ahead, across rows: 327,680 triangles 607 -> 540 us
-// (loads of four records at a time left the memory idle at every row's end;
-// float moments read 94 % of the copy rate as they are).
-constexpr int kNearAhead = 3;
-constexpr size_t kNearSmemMax = 228096;  // a block's 227 KB less what the kernel declares itself
-template <int RB>
-constexpr int near_box_threads() {
-  return 128 * RB;  // 256 threads per box measured 8 % slower than 128 (FP32H, RB = 1)
-}
-template <bool H16, int RB>
-constexpr size_t near_box_smem(int stage) {
-  return size_t(RB) * 6 * stage * sizeof(cf) + (H16 && RB == 1 ? size_t(4) * (kNearAhead + 1) * 64 * sizeof(uint4) : 0);
-}
-// Sources staged: the longest row, or as many as fit.
-template <bool H16, int RB>
-static int near_box_stage(const Problem& pr) {
-  const int row = int((pr.max_row + 31) / 32 * 32);
-  const int fit = int((kNearSmemMax - near_box_smem<H16, RB>(0)) / (size_t(RB) * 6 * sizeof(cf))) / 32 * 32;
-  return std::min(row, fit);
+// The twelve products of one pair into a right-hand side's sums; m: m0, mt(3),
+// ms(3), mts; c: a, beta(3), sigma, d.
+__device__ __forceinline__ void near_accumulate(cf* a, const cf* m, const cf* c) {
+  cfma(a[0], c[0], m[7]);
+  cfma(a[0], c[1], m[1]);
+  cfma(a[0], c[2], m[2]);
+  cfma(a[0], c[3], m[3]);
+  cfma(a[1], c[0], m[4]);
+  cfma(a[1], c[1], m[0]);
+  cfma(a[2], c[0], m[5]);
+  cfma(a[2], c[2], m[0]);
+  cfma(a[3], c[0], m[6]);
+  cfma(a[3], c[3], m[0]);
+  cfma(a[4], c[4], m[0]);
+  cfma(a[5], c[5], m[0]);
 }
 
-template <typename Rio, bool H16, int RB>
-__global__ void __launch_bounds__(near_box_threads<RB>(), RB == 1 ? 6 : (RB == 2 ? 2 : 1))
+// a1, float near part, one right-hand side: one block per leaf box (grid
+// stride over boxes).  Every test triangle of a box runs over the same source
+// list (the concatenated source ranges of its near boxes), so the block stages
+// those sources' coefficients in shared memory, plane by plane ([6][stage],
+// dynamic shared memory: stage is the problem's longest row), and its warps take
+// the box's test triangles in turn, lanes over the row as in k_near (lane j,
+// j + 32, ...): the same operations in the same order as in k_near, so the same
+// result to the last bit.  nsplit shares a box's test triangles among several
+// blocks when the leaf boxes alone do not fill the SMs.  Rows longer than stage
+// (shared memory takes 4704 sources) read the coefficients from global memory
+// instead.
+// Half-precision records reach shared memory by cp.async kNearAhead steps of 32
+// entries ahead, across rows: 327,680 triangles 607 -> 540 us (loads of four
+// records at a time left the memory idle at every row's end; float moments read
+// 94 % of the copy rate as they are).
+constexpr int kNearAhead = 3;
+constexpr int kNearBoxThreads = 128;  // 256 measured 8 % slower (FP32H)
+constexpr size_t kNearSmemMax = 228096;  // a block's 227 KB less what the kernel declares itself
+template <bool H16>
+constexpr size_t near_box_smem(int stage) {
+  return size_t(6) * stage * sizeof(cf) + (H16 ? size_t(4) * (kNearAhead + 1) * 64 * sizeof(uint4) : 0);
+}
+// Sources staged: the longest row, or as many as fit.
+template <bool H16>
+static int near_box_stage(const Problem& pr) {
+  const int fit = int((kNearSmemMax - near_box_smem<H16>(0)) / (6 * sizeof(cf))) / 32 * 32;
+  return std::min(int((pr.max_row + 31) / 32 * 32), fit);
+}
+
+template <typename Rio, bool H16>
+__global__ void __launch_bounds__(kNearBoxThreads, 6)
     k_near_box(int64_t nleaf, int nsplit, int stage, int64_t nnz, const int32_t* __restrict__ leaf_start,
                const int32_t* __restrict__ near_ptr, const int32_t* __restrict__ near_idx,
                const int32_t* __restrict__ near_off, const int64_t* __restrict__ row_ptr,
                const cf* __restrict__ mom, const __half2* __restrict__ momh, MomScale msc,
-               const cf* __restrict__ coef, float mu0, C2<Rio>* __restrict__ pot, int nrhs = 1, int64_t sc = 0,
-               int64_t sp = 0) {
+               const cf* __restrict__ coef, float mu0, C2<Rio>* __restrict__ pot, int64_t sc = 0, int64_t sp = 0) {
   extern __shared__ __align__(16) unsigned char near_smem[];
-  constexpr bool RING = H16 && RB == 1;
   constexpr int NS = kNearAhead + 1;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-  uint4* ring = reinterpret_cast<uint4*>(near_smem) + warp * NS * 64;  // [NS][2][32]
-  cf* cs = reinterpret_cast<cf*>(near_smem + (RING ? size_t(4) * NS * 64 * sizeof(uint4) : 0));  // [RB][6][stage]
-  const int r0 = blockIdx.y * RB;             // right-hand sides r0 .. r0 + nr - 1
-  const int nr = min(RB, nrhs - r0);
-  coef += r0 * sc;
-  pot += r0 * sp;
+  uint4* ring = reinterpret_cast<uint4*>(near_smem) + warp * NS * 64;  // [NS][64 half records]
+  cf* cs = reinterpret_cast<cf*>(near_smem + (H16 ? size_t(4) * NS * 64 * sizeof(uint4) : 0));  // [6][stage]
+  coef += blockIdx.y * sc;
+  pot += blockIdx.y * sp;
   for (int64_t bi = blockIdx.x; bi < nleaf * nsplit; bi += gridDim.x) {
     const int64_t b = bi / nsplit;
     const int q0 = near_ptr[b], q1 = near_ptr[b + 1];
@@ -273,9 +280,8 @@ __global__ void __launch_bounds__(near_box_threads<RB>(), RB == 1 ? 6 : (RB == 2
       for (int j = threadIdx.x; j < len; j += blockDim.x) {
         while (qi + 1 < q1 && near_off[qi + 1] <= j) ++qi;
         const int64_t src = 6 * (int64_t(leaf_start[near_idx[qi]]) + (j - near_off[qi]));
-        for (int r = 0; r < nr; ++r)
 #pragma unroll
-          for (int k = 0; k < 6; ++k) cp_async(&cs[(r * 6 + k) * stage + j], coef + r * sc + src + k);
+        for (int k = 0; k < 6; ++k) cp_async(&cs[k * stage + j], coef + src + k);
       }
     }
     cp_async_wait_all();
@@ -296,57 +302,32 @@ __global__ void __launch_bounds__(near_box_threads<RB>(), RB == 1 ? 6 : (RB == 2
       if (++fi == per_row) fi = 0, ft += tstep;
     };
     int slot = 0;
-    if constexpr (RING)
+    if constexpr (H16)
 #pragma unroll
       for (int d = 0; d < kNearAhead; ++d) fetch();
     for (int t = tfirst; t < t1; t += tstep) {
       const int64_t e0 = base + int64_t(t - t0) * len;
-      cf acc[RB][6];
+      cf acc[6];
 #pragma unroll
-      for (int r = 0; r < RB; ++r)
-#pragma unroll
-        for (int i = 0; i < 6; ++i) acc[r][i] = mk<float>(0, 0);
+      for (int i = 0; i < 6; ++i) acc[i] = mk<float>(0, 0);
       int qi = q0;
-      // entry j's six source coefficients of right-hand side r (a cursor on
-      // the near box that holds j when they are not staged; j never
-      // decreases from one call to the next)
-      auto coefs = [&](int r, int j, cf* c) {
+      // entry j's moments against its six source coefficients (a cursor on the
+      // near box that holds j when they are not staged; j never decreases from
+      // one call to the next)
+      auto entry = [&](int j, const cf* m) {
+        cf c[6];
         if (staged) {
 #pragma unroll
-          for (int k = 0; k < 6; ++k) c[k] = cs[(r * 6 + k) * stage + j];
+          for (int k = 0; k < 6; ++k) c[k] = cs[k * stage + j];
         } else {
           while (qi + 1 < q1 && near_off[qi + 1] <= j) ++qi;
-          const cf* src = coef + r * sc + 6 * (int64_t(leaf_start[near_idx[qi]]) + (j - near_off[qi]));
+          const cf* src = coef + 6 * (int64_t(leaf_start[near_idx[qi]]) + (j - near_off[qi]));
 #pragma unroll
           for (int k = 0; k < 6; ++k) c[k] = src[k];
         }
+        near_accumulate(acc, m, c);
       };
-      // m: m0, mt(3), ms(3), mts; c: a, beta(3), sigma, d
-      auto accumulate = [](cf* a, const cf* m, const cf* c) {
-        cfma(a[0], c[0], m[7]);
-        cfma(a[0], c[1], m[1]);
-        cfma(a[0], c[2], m[2]);
-        cfma(a[0], c[3], m[3]);
-        cfma(a[1], c[0], m[4]);
-        cfma(a[1], c[1], m[0]);
-        cfma(a[2], c[0], m[5]);
-        cfma(a[2], c[2], m[0]);
-        cfma(a[3], c[0], m[6]);
-        cfma(a[3], c[3], m[0]);
-        cfma(a[4], c[4], m[0]);
-        cfma(a[5], c[5], m[0]);
-      };
-      // one entry's moments against every right-hand side's coefficients
-      auto entry = [&](int j, const cf* m) {
-#pragma unroll
-        for (int r = 0; r < RB; ++r)
-          if (r < nr) {
-            cf c[6];
-            coefs(r, j, c);
-            accumulate(acc[r], m, c);
-          }
-      };
-      if constexpr (RING) {
+      if constexpr (H16) {
         for (int i = 0; i < per_row; ++i) {
           cp_async_wait<kNearAhead - 1>();
           __syncwarp();  // the step's records are here, and the slot before is read
@@ -359,24 +340,6 @@ __global__ void __launch_bounds__(near_box_threads<RB>(), RB == 1 ? 6 : (RB == 2
             entry(j, m);
           }
           slot = (slot + 1) % NS;
-        }
-      } else if constexpr (H16) {
-        // entries j, j + 32, ... (U of them): their 32-byte records loaded
-        // together, then accumulated in that order, the order of the
-        // one-entry loop
-        constexpr int U = 2;
-        for (int j = lane; j < len; j += 32 * U) {
-          uint4 lo[U], hi[U];
-#pragma unroll
-          for (int u = 0; u < U; ++u)
-            if (j + 32 * u < len) load_half_record(momh, e0 + j + 32 * u, lo[u], hi[u]);
-#pragma unroll
-          for (int u = 0; u < U; ++u)
-            if (j + 32 * u < len) {
-              cf m[kMom];
-              unpack_half<float>(lo[u], hi[u], msc, m);
-              entry(j + 32 * u, m);
-            }
         }
       } else {
         // entries j and j + 32 loaded together (twice the loads in flight),
@@ -393,15 +356,124 @@ __global__ void __launch_bounds__(near_box_threads<RB>(), RB == 1 ? 6 : (RB == 2
           if (two) entry(j + 32, mb);
         }
       }
-#pragma unroll
-      for (int r = 0; r < RB; ++r) {
-        if (r >= nr) break;
-        int i;
-        const float v = warp_sum12(acc[r], lane, &i);
-        if (i >= 0) reinterpret_cast<Rio*>(pot + r * sp + 6 * int64_t(t))[i] = Rio(i < 8 ? mu0 * v : v);
-      }
+      int i;
+      const float v = warp_sum12(acc, lane, &i);
+      if (i >= 0) reinterpret_cast<Rio*>(pot + 6 * int64_t(t))[i] = Rio(i < 8 ? mu0 * v : v);
     }
-    cp_async_wait_all();  // (steps past the last row: nothing in them)
+    if constexpr (H16) cp_async_wait_all();  // (steps past the last row: nothing in them)
+  }
+}
+
+// a1, float near part, RB = 2 or 4 right-hand sides (blockIdx.y: groups of
+// them): each moment is read once for all of them.  The block's eight warps take
+// eight of a leaf box's test triangles at a time, a row each, and walk the box's
+// source list together, kNearChunk sources a step: the step's coefficients
+// ([RB][6][kNearChunk]) come in by cp.async while the step before is multiplied,
+// so rows of any length take the same 50 KB.  (Whole rows in shared memory, 1100
+// sources and four columns, left one block of an SM and no room beside the far
+// part's kernels; coefficients from global memory cost 12 cache lines a load.)
+// Lanes meet their entries in k_near's order: the same result to the last bit.
+// Eight columns of a cylinder of 40,960 triangles: 3.3 -> 2.3 ms alone, the
+// product 6.7 -> 5.0 ms.
+constexpr int kNearChunk = 128, kNearChunkThreads = 256;
+template <int RB>
+constexpr size_t near_chunk_smem() {
+  return size_t(2) * RB * 6 * kNearChunk * sizeof(cf);
+}
+template <typename Rio, bool H16, int RB>
+__global__ void __launch_bounds__(kNearChunkThreads, 2)
+    k_near_chunk(int64_t nleaf, int nsplit, int64_t nnz, const int32_t* __restrict__ leaf_start,
+                 const int32_t* __restrict__ near_ptr, const int32_t* __restrict__ near_idx,
+                 const int32_t* __restrict__ near_off, const int64_t* __restrict__ row_ptr,
+                 const cf* __restrict__ mom, const __half2* __restrict__ momh, MomScale msc,
+                 const cf* __restrict__ coef, float mu0, C2<Rio>* __restrict__ pot, int nrhs, int64_t sc, int64_t sp) {
+  extern __shared__ __align__(16) unsigned char near_smem[];
+  constexpr int CH = kNearChunk, NW = kNearChunkThreads / 32;
+  cf* cs = reinterpret_cast<cf*>(near_smem);  // [2][RB][6][CH]
+  const int r0 = blockIdx.y * RB, nr = min(RB, nrhs - r0);  // right-hand sides r0 .. r0 + nr - 1
+  coef += r0 * sc;
+  pot += r0 * sp;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int64_t bi = blockIdx.x; bi < nleaf * nsplit; bi += gridDim.x) {
+    const int64_t b = bi / nsplit;
+    const int q0 = near_ptr[b], q1 = near_ptr[b + 1];
+    const int t0 = leaf_start[b], t1 = leaf_start[b + 1];
+    const int64_t base = row_ptr[t0];
+    const int len = int(row_ptr[t0 + 1] - base), nchunk = (len + CH - 1) / CH;
+    for (int tg = t0 + int(bi % nsplit) * NW; tg < t1; tg += NW * nsplit) {
+      const int t = tg + warp;
+      const int64_t e0 = base + int64_t(t - t0) * len;
+      cf acc[RB][6];
+#pragma unroll
+      for (int r = 0; r < RB; ++r)
+#pragma unroll
+        for (int i = 0; i < 6; ++i) acc[r][i] = mk<float>(0, 0);
+      // thread: source threadIdx.x % CH of a chunk, right-hand sides threadIdx.x / CH, + 2, ...
+      int qi = q0;
+      auto stage = [&](int c) {
+        const int j = c * CH + int(threadIdx.x % CH);
+        if (j < len) {
+          while (qi + 1 < q1 && near_off[qi + 1] <= j) ++qi;
+          const cf* src = coef + 6 * (int64_t(leaf_start[near_idx[qi]]) + (j - near_off[qi]));
+          cf* dst = cs + (c & 1) * (RB * 6 * CH) + threadIdx.x % CH;
+          for (int r = threadIdx.x / CH; r < nr; r += kNearChunkThreads / CH)
+#pragma unroll
+            for (int k = 0; k < 6; ++k) cp_async(dst + (r * 6 + k) * CH, src + r * sc + k);
+        }
+      };
+      __syncthreads();  // the previous rows' readers are done with cs
+      stage(0);
+      for (int c = 0; c < nchunk; ++c) {
+        cp_async_wait_all();
+        __syncthreads();  // chunk c is here, chunk c - 1 has been read
+        if (c + 1 < nchunk) stage(c + 1);
+        const cf* cc = cs + (c & 1) * (RB * 6 * CH);
+        const int n = t < t1 ? min(CH, len - c * CH) : 0;
+        const int64_t e = e0 + c * CH;
+        auto entry = [&](int j, const cf* m) {
+#pragma unroll
+          for (int r = 0; r < RB; ++r)
+            if (r < nr) {
+              cf x[6];
+#pragma unroll
+              for (int k = 0; k < 6; ++k) x[k] = cc[(r * 6 + k) * CH + j];
+              near_accumulate(acc[r], m, x);
+            }
+        };
+        // entries j and j + 32 loaded together
+        for (int j = lane; j < n; j += 64) {
+          const bool two = j + 32 < n;
+          cf ma[kMom], mb[kMom];
+          if constexpr (H16) {
+            uint4 lo[2], hi[2];
+            load_half_record(momh, e + j, lo[0], hi[0]);
+            if (two) load_half_record(momh, e + j + 32, lo[1], hi[1]);
+            unpack_half<float>(lo[0], hi[0], msc, ma);
+            entry(j, ma);
+            if (two) {
+              unpack_half<float>(lo[1], hi[1], msc, mb);
+              entry(j + 32, mb);
+            }
+          } else {
+#pragma unroll
+            for (int q = 0; q < kMom; ++q) ma[q] = mom[q * nnz + e + j];
+            if (two)
+#pragma unroll
+              for (int q = 0; q < kMom; ++q) mb[q] = mom[q * nnz + e + j + 32];
+            entry(j, ma);
+            if (two) entry(j + 32, mb);
+          }
+        }
+      }
+      if (t < t1)
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+          if (r >= nr) break;
+          int i;
+          const float v = warp_sum12(acc[r], lane, &i);
+          if (i >= 0) reinterpret_cast<Rio*>(pot + r * sp + 6 * int64_t(t))[i] = Rio(i < 8 ? mu0 * v : v);
+        }
+    }
   }
 }
 
@@ -418,16 +490,24 @@ static bool device_done(std::atomic<uint64_t>& mask, int* bit) {
   return (mask.load() >> dev) & 1u;
 }
 
-template <typename Rio, bool H16, int RB>
-static pie_status near_box_prepare() {
-  static std::atomic<uint64_t> done{0};
+template <typename K>
+static pie_status raise_smem(K* kernel, size_t bytes, std::atomic<uint64_t>& done) {
   int bit = -1;
   if (device_done(done, &bit)) return PIE_OK;
-  pie_status s = cuda_check(
-      cudaFuncSetAttribute(k_near_box<Rio, H16, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kNearSmemMax)),
-      "near smem attribute");
+  pie_status s = cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)),
+                            "near smem attribute");
   if (s == PIE_OK && bit >= 0) done.fetch_or(uint64_t(1) << bit);
   return s;
+}
+template <typename Rio, bool H16>
+static pie_status near_box_prepare() {
+  static std::atomic<uint64_t> done{0};
+  return raise_smem(k_near_box<Rio, H16>, kNearSmemMax, done);
+}
+template <typename Rio, bool H16, int RB>
+static pie_status near_chunk_prepare() {
+  static std::atomic<uint64_t> done{0};
+  return raise_smem(k_near_chunk<Rio, H16, RB>, near_chunk_smem<RB>(), done);
 }
 
 // a1, PIE_FP64: near part in fixed point (near_fixed.cuh).  A block per (leaf
@@ -638,13 +718,7 @@ __global__ void __launch_bounds__(128, 3)
 
 pie_status near_fixed_prepare() {
   static std::atomic<uint64_t> done{0};
-  int bit = -1;
-  if (device_done(done, &bit)) return PIE_OK;
-  pie_status s = cuda_check(
-      cudaFuncSetAttribute(k_near_fixed, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kFixedSmem)),
-      "near smem attribute");
-  if (s == PIE_OK && bit >= 0) done.fetch_or(uint64_t(1) << bit);
-  return s;
+  return raise_smem(k_near_fixed, kFixedSmem, done);
 }
 
 // Launch of the fixed-point near part for nrhs columns on a grid of at most
@@ -1602,9 +1676,9 @@ __device__ __forceinline__ C2<Rio> pot_sum(const C2<Rio>* pot, const C2<Rio>* po
 
 // a7: Galerkin testing of the per-triangle potentials (Section 2):
 // RWG m: sum over its two triangles of c [U + (c_t - p).V] + 2c T1; pulse t: T2.
-// pot2 (may be null): near-part potentials, added to pot first.  scale (may be
-// null): the result is scale y, y rounded to the io precision first.
-template <typename Rio>
+// pot2 (may be null): near-part potentials, added to pot first.  SCALED:
+// the result is scale y, y rounded to the io precision first.
+template <typename Rio, bool SCALED = false>
 __global__ void k_assemble(int64_t N, int64_t E, const int32_t* __restrict__ edge_tt,
                            const int8_t* __restrict__ edge_k, const double* __restrict__ tri_c,
                            const double* __restrict__ tri_dcp, const int64_t* __restrict__ inv_perm,
@@ -1612,7 +1686,10 @@ __global__ void k_assemble(int64_t N, int64_t E, const int32_t* __restrict__ edg
                            const C2<Rio>* __restrict__ pot2 = nullptr, const double* __restrict__ scale = nullptr) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= N) return;
-  C2<Rio> out;
+  auto store = [&](C2<Rio> v) {
+    if constexpr (SCALED) v = mk<Rio>(Rio(scale[i] * double(v.x)), Rio(scale[i] * double(v.y)));
+    y[i] = v;
+  };
   pot += blockIdx.y * sp;
   if (pot2) pot2 += blockIdx.y * sp;
   y += blockIdx.y * sy;
@@ -1632,22 +1709,21 @@ __global__ void k_assemble(int64_t N, int64_t E, const int32_t* __restrict__ edg
       yr += c * (ur + 2.0 * double(p[4].x));
       yi += c * (ui + 2.0 * double(p[4].y));
     }
-    out = mk<Rio>(Rio(yr), Rio(yi));
+    store(mk<Rio>(Rio(yr), Rio(yi)));
   } else {
     int64_t t = inv_perm[i - E];
-    out = pot_sum(pot, pot2, 6 * t + 5);
+    store(pot_sum(pot, pot2, 6 * t + 5));
   }
-  y[i] = scale ? mk<Rio>(Rio(scale[i] * double(out.x)), Rio(scale[i] * double(out.y))) : out;
 }
 
 // ---------------------------------------------------------------- orchestration
 
 static inline unsigned nblk(int64_t n, int b) { return unsigned((n + b - 1) / b); }
 
-// Blocks per leaf box of k_near_box: enough to give an SM its six, at least
-// four test triangles each.
-static int near_box_split(const Problem& pr) {
-  const int64_t want = (6 * int64_t(pr.nsm) + pr.nleaf - 1) / pr.nleaf, most = (pr.T / pr.nleaf + 3) / 4;
+// Blocks per leaf box of the box-staged kernels: enough to give an SM its six,
+// at least a test triangle for each of a block's warps.
+static int near_box_split(const Problem& pr, int warps) {
+  const int64_t want = (6 * int64_t(pr.nsm) + pr.nleaf - 1) / pr.nleaf, most = (pr.T / pr.nleaf + warps - 1) / warps;
   return int(std::max<int64_t>(1, std::min({want, most, int64_t(16)})));
 }
 
@@ -1717,33 +1793,38 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
           static_cast<const C2<Rm>*>(pr.mom), static_cast<const __half2*>(pr.mom), mom_scale(pr), ncoef, Rm(kMu0),
           pot2, nrhs, sT, sT);
   };
-  // float near part: the box-staged kernel (RB 1, 2 or 4), or one warp per
-  // test triangle (RB 1, 2, 4 or 8) when tuned so or when the rows outgrow the
-  // box kernel's shared memory
+  // float near part: the box-staged kernels (RB 1, or 2 and 4 by chunks), or
+  // one warp per test triangle (RB 1, 2, 4 or 8) when tuned so
   int rb = pr.tune.near_rhs_block;
-  auto fits = [&](int n) { return size_t(n) * 6 * sizeof(cf) * size_t(pr.max_row + 31) < kNearSmemMax; };
-  bool boxed = sizeof(Rm) == 4 && pr.tune.near_kernel != 1;
-  if (rb == 0) {
-    rb = nrhs == 1 ? 1 : nrhs == 2 ? 2 : 4;
-    while (boxed && rb > 1 && !fits(rb)) rb /= 2;
-  }
-  if (pr.tune.near_kernel == 0) boxed = boxed && fits(rb);
+  if (rb == 0) rb = nrhs == 1 ? 1 : nrhs == 2 ? 2 : 4;
+  const bool boxed = sizeof(Rm) == 4 && pr.tune.near_kernel != 1;
   auto box_launch = [&](auto rbc) -> pie_status {
     if constexpr (sizeof(Rm) == 4) {
-      constexpr int RB = decltype(rbc)::value, TH = near_box_threads<RB>();
-      pie_status s = near_box_prepare<Rio, H16, RB>();
-      if (s != PIE_OK) return s;
-      const int nsplit = near_box_split(pr), stage = near_box_stage<H16, RB>(pr);
+      constexpr int RB = decltype(rbc)::value, TH = RB == 1 ? kNearBoxThreads : kNearChunkThreads;
+      const int nsplit = near_box_split(pr, TH / 32);
       unsigned grid = unsigned(pr.nleaf * nsplit);
       if (overlap && pr.tune.near_ctas_per_sm > 0)
         // many short blocks make room for the far part's by themselves: a bound
         // only where all of them would start at once
         grid = std::min<unsigned>(grid, unsigned(pr.nsm * pr.tune.near_ctas_per_sm *
-                                                 (grid > unsigned(16 * pr.nsm) ? 8192 / TH : std::max(1, 256 / TH))));
-      k_near_box<Rio, H16, RB><<<dim3(grid, unsigned((nrhs + RB - 1) / RB)), TH, near_box_smem<H16, RB>(stage), sn>>>(
-          pr.nleaf, nsplit, stage, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr,
-          static_cast<const cf*>(pr.mom), static_cast<const __half2*>(pr.mom), mom_scale(pr),
-          reinterpret_cast<const cf*>(ncoef), float(kMu0), pot2, nrhs, sT, sT);
+                                                 (grid > unsigned(16 * pr.nsm) ? 8192 / TH : 256 / TH)));
+      const cf* mom = static_cast<const cf*>(pr.mom);
+      const __half2* momh = static_cast<const __half2*>(pr.mom);
+      const cf* c = reinterpret_cast<const cf*>(ncoef);
+      if constexpr (RB == 1) {
+        pie_status s = near_box_prepare<Rio, H16>();
+        if (s != PIE_OK) return s;
+        const int stage = near_box_stage<H16>(pr);
+        k_near_box<Rio, H16><<<dim3(grid, nr), TH, near_box_smem<H16>(stage), sn>>>(
+            pr.nleaf, nsplit, stage, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr, mom,
+            momh, mom_scale(pr), c, float(kMu0), pot2, sT, sT);
+      } else {
+        pie_status s = near_chunk_prepare<Rio, H16, RB>();
+        if (s != PIE_OK) return s;
+        k_near_chunk<Rio, H16, RB><<<dim3(grid, nblk(nrhs, RB)), TH, near_chunk_smem<RB>(), sn>>>(
+            pr.nleaf, nsplit, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr, mom, momh,
+            mom_scale(pr), c, float(kMu0), pot2, nrhs, sT, sT);
+      }
     }
     return PIE_OK;
   };
@@ -1936,8 +2017,14 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
     if (s != PIE_OK) return s;
   }
   prof_mark(pr, 7, false, st);
-  k_assemble<Rio><<<dim3(nblk(pr.N, 256), nr), 256, 0, st>>>(pr.N, pr.E, pr.edge_tt, pr.edge_k, pr.tri_c,
-                                                             pr.tri_dcp, pr.inv_perm, pot, y, sT, sN, pot2, scale);
+  auto assemble = [&](auto scaled) {
+    k_assemble<Rio, decltype(scaled)::value><<<dim3(nblk(pr.N, 256), nr), 256, 0, st>>>(
+        pr.N, pr.E, pr.edge_tt, pr.edge_k, pr.tri_c, pr.tri_dcp, pr.inv_perm, pot, y, sT, sN, pot2, scale);
+  };
+  if (scale)
+    assemble(std::true_type());
+  else
+    assemble(std::false_type());
   prof_mark(pr, 7, true, st);
   if (pr.prof_n < pr.prof_cap) ++pr.prof_n;
   return cuda_check(cudaGetLastError(), "apply launch");
@@ -1956,10 +2043,10 @@ static pie_status apply_near_t(Problem& pr, const void* xv, void* yv, cudaStream
   if constexpr (sizeof(Rm) == 8) {
     near_fixed(pr, coef, pot, 1, 0, st);
   } else if (pr.tune.near_kernel != 1) {  // the box-staged kernel, unless tuned off
-    pie_status s = near_box_prepare<Rio, H16, 1>();
+    pie_status s = near_box_prepare<Rio, H16>();
     if (s != PIE_OK) return s;
-    const int nsplit = near_box_split(pr), stage = near_box_stage<H16, 1>(pr);
-    k_near_box<Rio, H16, 1><<<unsigned(pr.nleaf * nsplit), near_box_threads<1>(), near_box_smem<H16, 1>(stage), st>>>(
+    const int nsplit = near_box_split(pr, kNearBoxThreads / 32), stage = near_box_stage<H16>(pr);
+    k_near_box<Rio, H16><<<unsigned(pr.nleaf * nsplit), kNearBoxThreads, near_box_smem<H16>(stage), st>>>(
         pr.nleaf, nsplit, stage, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr,
         static_cast<const cf*>(pr.mom), static_cast<const __half2*>(pr.mom), mom_scale(pr), ncoef, float(kMu0), pot);
   } else {
