@@ -4,6 +4,7 @@
 // Galerkin assembly (Section 2).
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdio>
 #include <type_traits>
 
@@ -224,11 +225,23 @@ __device__ __forceinline__ void near_accumulate(cf* a, const cf* m, const cf* c)
   cfma(a[5], c[5], m[0]);
 }
 
+// A source's six staged coefficients, source by source in shared memory: three
+// 16-byte loads, and eight lanes at 48 bytes apart meet every bank once.
+__device__ __forceinline__ void load_coefs(const cf* src, cf* c) {
+  const float4* p = reinterpret_cast<const float4*>(src);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const float4 v = p[k];
+    c[2 * k] = mk<float>(v.x, v.y);
+    c[2 * k + 1] = mk<float>(v.z, v.w);
+  }
+}
+
 // a1, float near part, one right-hand side: one block per leaf box (grid
 // stride over boxes).  Every test triangle of a box runs over the same source
 // list (the concatenated source ranges of its near boxes), so the block stages
-// those sources' coefficients in shared memory, plane by plane ([6][stage],
-// dynamic shared memory: stage is the problem's longest row), and its warps take
+// those sources' coefficients in shared memory ([stage][6], dynamic shared
+// memory: stage is the problem's longest row), and its warps take
 // the box's test triangles in turn, lanes over the row as in k_near (lane j,
 // j + 32, ...): the same operations in the same order as in k_near, so the same
 // result to the last bit.  nsplit shares a box's test triangles among several
@@ -264,7 +277,7 @@ __global__ void __launch_bounds__(kNearBoxThreads, 6)
   constexpr int NS = kNearAhead + 1;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   uint4* ring = reinterpret_cast<uint4*>(near_smem) + warp * NS * 64;  // [NS][64 half records]
-  cf* cs = reinterpret_cast<cf*>(near_smem + (H16 ? size_t(4) * NS * 64 * sizeof(uint4) : 0));  // [6][stage]
+  cf* cs = reinterpret_cast<cf*>(near_smem + (H16 ? size_t(4) * NS * 64 * sizeof(uint4) : 0));  // [stage][6]
   coef += blockIdx.y * sc;
   pot += blockIdx.y * sp;
   for (int64_t bi = blockIdx.x; bi < nleaf * nsplit; bi += gridDim.x) {
@@ -277,11 +290,11 @@ __global__ void __launch_bounds__(kNearBoxThreads, 6)
     __syncthreads();  // the previous box's readers are done with cs
     if (staged) {
       int qi = q0;  // j grows: the cursor only moves forward
-      for (int j = threadIdx.x; j < len; j += blockDim.x) {
+      for (int i = threadIdx.x; i < 3 * len; i += blockDim.x) {  // thirds of a source's 48 bytes
+        const int j = i / 3;
         while (qi + 1 < q1 && near_off[qi + 1] <= j) ++qi;
-        const int64_t src = 6 * (int64_t(leaf_start[near_idx[qi]]) + (j - near_off[qi]));
-#pragma unroll
-        for (int k = 0; k < 6; ++k) cp_async(&cs[k * stage + j], coef + src + k);
+        const cf* src = coef + 6 * (int64_t(leaf_start[near_idx[qi]]) + (j - near_off[qi])) + 2 * (i % 3);
+        cp_async(reinterpret_cast<float4*>(cs) + i, reinterpret_cast<const float4*>(src));
       }
     }
     cp_async_wait_all();
@@ -317,8 +330,7 @@ __global__ void __launch_bounds__(kNearBoxThreads, 6)
       auto entry = [&](int j, const cf* m) {
         cf c[6];
         if (staged) {
-#pragma unroll
-          for (int k = 0; k < 6; ++k) c[k] = cs[k * stage + j];
+          load_coefs(cs + 6 * j, c);
         } else {
           while (qi + 1 < q1 && near_off[qi + 1] <= j) ++qi;
           const cf* src = coef + 6 * (int64_t(leaf_start[near_idx[qi]]) + (j - near_off[qi]));
@@ -368,17 +380,19 @@ __global__ void __launch_bounds__(kNearBoxThreads, 6)
 // them): each moment is read once for all of them.  The block's eight warps take
 // eight of a leaf box's test triangles at a time, a row each, and walk the box's
 // source list together, kNearChunk sources a step: the step's coefficients
-// ([RB][6][kNearChunk]) come in by cp.async while the step before is multiplied,
+// ([RB][kNearChunk][6]) come in by cp.async while the step before is multiplied,
 // so rows of any length take the same 50 KB.  (Whole rows in shared memory, 1100
 // sources and four columns, left one block of an SM and no room beside the far
 // part's kernels; coefficients from global memory cost 12 cache lines a load.)
 // Lanes meet their entries in k_near's order: the same result to the last bit.
-// Eight columns of a cylinder of 40,960 triangles: 3.3 -> 2.3 ms alone, the
-// product 6.7 -> 5.0 ms.
-constexpr int kNearChunk = 128, kNearChunkThreads = 256;
-template <int RB>
+// Moments are kNearChunkSlots - 1 steps of 32 entries ahead, across rows.  Eight
+// columns of a cylinder of 40,960 triangles: 3.3 -> 2.1 ms alone, the product 6.7 ->
+// 4.84 ms.
+constexpr int kNearChunk = 128, kNearChunkThreads = 256, kNearChunkSlots = 3;
+template <bool H16, int RB>
 constexpr size_t near_chunk_smem() {
-  return size_t(2) * RB * 6 * kNearChunk * sizeof(cf);
+  return size_t(2) * RB * 6 * kNearChunk * sizeof(cf) +
+         size_t(kNearChunkThreads) * kNearChunkSlots * (H16 ? 2 * sizeof(uint4) : kMom * sizeof(cf));
 }
 template <typename Rio, bool H16, int RB>
 __global__ void __launch_bounds__(kNearChunkThreads, 2)
@@ -388,8 +402,12 @@ __global__ void __launch_bounds__(kNearChunkThreads, 2)
                  const cf* __restrict__ mom, const __half2* __restrict__ momh, MomScale msc,
                  const cf* __restrict__ coef, float mu0, C2<Rio>* __restrict__ pot, int nrhs, int64_t sc, int64_t sp) {
   extern __shared__ __align__(16) unsigned char near_smem[];
-  constexpr int CH = kNearChunk, NW = kNearChunkThreads / 32;
-  cf* cs = reinterpret_cast<cf*>(near_smem);  // [2][RB][6][CH]
+  constexpr int CH = kNearChunk, TH = kNearChunkThreads, NW = TH / 32, NS = kNearChunkSlots;
+  // moments on their way: half records [warp][NS][64 halves], or planes
+  // [NS][plane][thread] (each thread its own entries)
+  uint4* rh = reinterpret_cast<uint4*>(near_smem) + (threadIdx.x >> 5) * NS * 64;
+  cf* rf = reinterpret_cast<cf*>(near_smem) + threadIdx.x;
+  cf* cs = reinterpret_cast<cf*>(near_smem + near_chunk_smem<H16, RB>()) - 2 * RB * 6 * CH;  // [2][RB][CH][6]
   const int r0 = blockIdx.y * RB, nr = min(RB, nrhs - r0);  // right-hand sides r0 .. r0 + nr - 1
   coef += r0 * sc;
   pot += r0 * sp;
@@ -397,73 +415,92 @@ __global__ void __launch_bounds__(kNearChunkThreads, 2)
   for (int64_t bi = blockIdx.x; bi < nleaf * nsplit; bi += gridDim.x) {
     const int64_t b = bi / nsplit;
     const int q0 = near_ptr[b], q1 = near_ptr[b + 1];
-    const int t0 = leaf_start[b], t1 = leaf_start[b + 1];
+    const int t0 = leaf_start[b], t1 = leaf_start[b + 1], tstep = NW * nsplit;
     const int64_t base = row_ptr[t0];
-    const int len = int(row_ptr[t0 + 1] - base), nchunk = (len + CH - 1) / CH;
-    for (int tg = t0 + int(bi % nsplit) * NW; tg < t1; tg += NW * nsplit) {
+    const int len = int(row_ptr[t0 + 1] - base), nchunk = (len + CH - 1) / CH, per_row = (len + 31) / 32;
+    const int tg0 = t0 + int(bi % nsplit) * NW;
+    // the (row, 32 entries) step after the last one sent on its way, and its slot
+    int ft = tg0 + warp, fi = 0, fslot = 0;
+    auto fetch = [&] {
+      const int n = ft < t1 ? min(32, len - 32 * fi) : 0;
+      const int64_t e = base + int64_t(ft - t0) * len + 32 * fi;
+      if constexpr (H16) {
+        const uint4* src = reinterpret_cast<const uint4*>(momh) + 2 * e;
+#pragma unroll
+        for (int h = lane; h < 64; h += 32)
+          if (h < 2 * n) cp_async(rh + fslot * 64 + h, src + h);
+      } else if (lane < n) {
+#pragma unroll
+        for (int q = 0; q < kMom; ++q) cp_async(rf + (kMom * fslot + q) * TH, mom + q * nnz + e + lane);
+      }
+      cp_async_commit();
+      fslot = (fslot + 1) % NS;
+      if (++fi == per_row) fi = 0, ft += tstep;
+    };
+    int qi = q0, buf = 0;
+    auto stage = [&](int c, int to) {
+      if (c == 0) qi = q0;
+      float4* dst = reinterpret_cast<float4*>(cs + to * (RB * 6 * CH));
+      for (int i = threadIdx.x; i < 3 * CH; i += TH) {  // thirds of a source's 48 bytes
+        const int j = c * CH + i / 3;
+        if (j >= len) break;
+        while (qi + 1 < q1 && near_off[qi + 1] <= j) ++qi;
+        const cf* src = coef + 6 * (int64_t(leaf_start[near_idx[qi]]) + (j - near_off[qi])) + 2 * (i % 3);
+        for (int r = 0; r < nr; ++r) cp_async(dst + r * 3 * CH + i, reinterpret_cast<const float4*>(src + r * sc));
+      }
+    };
+    __syncthreads();  // the previous box's readers are done
+    int slot = 0;
+    if (tg0 < t1) {
+      stage(0, 0);  // (in the group of the first fetch)
+#pragma unroll
+      for (int d = 0; d < NS - 1; ++d) fetch();
+    }
+    for (int tg = tg0; tg < t1; tg += tstep) {
       const int t = tg + warp;
-      const int64_t e0 = base + int64_t(t - t0) * len;
       cf acc[RB][6];
 #pragma unroll
       for (int r = 0; r < RB; ++r)
 #pragma unroll
         for (int i = 0; i < 6; ++i) acc[r][i] = mk<float>(0, 0);
-      // thread: source threadIdx.x % CH of a chunk, right-hand sides threadIdx.x / CH, + 2, ...
-      int qi = q0;
-      auto stage = [&](int c) {
-        const int j = c * CH + int(threadIdx.x % CH);
-        if (j < len) {
-          while (qi + 1 < q1 && near_off[qi + 1] <= j) ++qi;
-          const cf* src = coef + 6 * (int64_t(leaf_start[near_idx[qi]]) + (j - near_off[qi]));
-          cf* dst = cs + (c & 1) * (RB * 6 * CH) + threadIdx.x % CH;
-          for (int r = threadIdx.x / CH; r < nr; r += kNearChunkThreads / CH)
-#pragma unroll
-            for (int k = 0; k < 6; ++k) cp_async(dst + (r * 6 + k) * CH, src + r * sc + k);
-        }
-      };
-      __syncthreads();  // the previous rows' readers are done with cs
-      stage(0);
       for (int c = 0; c < nchunk; ++c) {
-        cp_async_wait_all();
-        __syncthreads();  // chunk c is here, chunk c - 1 has been read
-        if (c + 1 < nchunk) stage(c + 1);
-        const cf* cc = cs + (c & 1) * (RB * 6 * CH);
-        const int n = t < t1 ? min(CH, len - c * CH) : 0;
-        const int64_t e = e0 + c * CH;
-        auto entry = [&](int j, const cf* m) {
+        const int n = min(CH, len - c * CH);
+        // the chunk's coefficients came with the first fetch of the chunk before,
+        // four fetches ago unless that was a row's short last chunk
+        if (c > 0)
+          cp_async_wait<NS - 1>();
+        else
+          cp_async_wait_all();
+        __syncthreads();  // every thread's part of them is here, the other buffer has been read
+        if (c + 1 < nchunk)
+          stage(c + 1, buf ^ 1);
+        else if (tg + tstep < t1)
+          stage(0, buf ^ 1);
+        const cf* cc = cs + buf * (RB * 6 * CH);
+        for (int i = 0; i < n; i += 32) {
+          cp_async_wait<NS - 2>();
+          __syncwarp();  // the step's moments are here, and the slot before is read
+          fetch();
+          const int j = i + lane;
+          if (t < t1 && j < n) {
+            cf m[kMom];
+            if constexpr (H16) {
+              unpack_half<float>(rh[slot * 64 + 2 * lane], rh[slot * 64 + 2 * lane + 1], msc, m);
+            } else {
 #pragma unroll
-          for (int r = 0; r < RB; ++r)
-            if (r < nr) {
-              cf x[6];
-#pragma unroll
-              for (int k = 0; k < 6; ++k) x[k] = cc[(r * 6 + k) * CH + j];
-              near_accumulate(acc[r], m, x);
+              for (int q = 0; q < kMom; ++q) m[q] = rf[(kMom * slot + q) * TH];
             }
-        };
-        // entries j and j + 32 loaded together
-        for (int j = lane; j < n; j += 64) {
-          const bool two = j + 32 < n;
-          cf ma[kMom], mb[kMom];
-          if constexpr (H16) {
-            uint4 lo[2], hi[2];
-            load_half_record(momh, e + j, lo[0], hi[0]);
-            if (two) load_half_record(momh, e + j + 32, lo[1], hi[1]);
-            unpack_half<float>(lo[0], hi[0], msc, ma);
-            entry(j, ma);
-            if (two) {
-              unpack_half<float>(lo[1], hi[1], msc, mb);
-              entry(j + 32, mb);
-            }
-          } else {
 #pragma unroll
-            for (int q = 0; q < kMom; ++q) ma[q] = mom[q * nnz + e + j];
-            if (two)
-#pragma unroll
-              for (int q = 0; q < kMom; ++q) mb[q] = mom[q * nnz + e + j + 32];
-            entry(j, ma);
-            if (two) entry(j + 32, mb);
+            for (int r = 0; r < RB; ++r)
+              if (r < nr) {
+                cf x[6];
+                load_coefs(cc + (r * CH + j) * 6, x);
+                near_accumulate(acc[r], m, x);
+              }
           }
+          slot = (slot + 1) % NS;
         }
+        buf ^= 1;
       }
       if (t < t1)
 #pragma unroll
@@ -474,6 +511,7 @@ __global__ void __launch_bounds__(kNearChunkThreads, 2)
           if (i >= 0) reinterpret_cast<Rio*>(pot + r * sp + 6 * int64_t(t))[i] = Rio(i < 8 ? mu0 * v : v);
         }
     }
+    cp_async_wait_all();  // (steps past the last row: nothing in them)
   }
 }
 
@@ -491,23 +529,20 @@ static bool device_done(std::atomic<uint64_t>& mask, int* bit) {
 }
 
 template <typename K>
-static pie_status raise_smem(K* kernel, size_t bytes, std::atomic<uint64_t>& done) {
-  int bit = -1;
-  if (device_done(done, &bit)) return PIE_OK;
-  pie_status s = cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)),
-                            "near smem attribute");
-  if (s == PIE_OK && bit >= 0) done.fetch_or(uint64_t(1) << bit);
-  return s;
+static pie_status raise_smem(K* kernel, size_t bytes) {
+  return cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)),
+                    "near smem attribute");
 }
 template <typename Rio, bool H16>
-static pie_status near_box_prepare() {
+static pie_status near_float_prepare() {
   static std::atomic<uint64_t> done{0};
-  return raise_smem(k_near_box<Rio, H16>, kNearSmemMax, done);
-}
-template <typename Rio, bool H16, int RB>
-static pie_status near_chunk_prepare() {
-  static std::atomic<uint64_t> done{0};
-  return raise_smem(k_near_chunk<Rio, H16, RB>, near_chunk_smem<RB>(), done);
+  int bit = -1;
+  if (device_done(done, &bit)) return PIE_OK;
+  pie_status s = raise_smem(k_near_box<Rio, H16>, kNearSmemMax);
+  if (s == PIE_OK) s = raise_smem(k_near_chunk<Rio, H16, 2>, near_chunk_smem<H16, 2>());
+  if (s == PIE_OK) s = raise_smem(k_near_chunk<Rio, H16, 4>, near_chunk_smem<H16, 4>());
+  if (s == PIE_OK && bit >= 0) done.fetch_or(uint64_t(1) << bit);
+  return s;
 }
 
 // a1, PIE_FP64: near part in fixed point (near_fixed.cuh).  A block per (leaf
@@ -579,16 +614,17 @@ __device__ __noinline__ double near_row_double(const FixedNear& nf, int64_t nnz,
 
 // Shared memory: the stage's coefficients [6][kFixedStage], then two buffers of
 // 32 entries' moments [2][8][32] per warp.
-constexpr size_t kFixedSmem = sizeof(int4) * (6 * kFixedStage + 4 * 2 * kMom * 32);
+constexpr int kFixedWarps = 4;  // (8 warps with 128 registers each: 15 % slower)
+constexpr size_t kFixedSmem = sizeof(int4) * (6 * kFixedStage + kFixedWarps * 2 * kMom * 32);
 
-__global__ void __launch_bounds__(128, 3)
+__global__ void __launch_bounds__(32 * kFixedWarps, 3)
     k_near_fixed(int64_t nleaf, int nsplit, int64_t nnz, const int32_t* __restrict__ leaf_start,
                  const int32_t* __restrict__ near_ptr, const int32_t* __restrict__ near_idx,
                  const int32_t* __restrict__ near_off, const int64_t* __restrict__ row_ptr, const FixedNear nf,
                  const cd* __restrict__ coef, double mu0, cd* __restrict__ pot, int64_t sc = 0, int64_t sp = 0) {
   extern __shared__ __align__(16) unsigned char fixed_smem[];
   int4(*cs)[kFixedStage] = reinterpret_cast<int4(*)[kFixedStage]>(fixed_smem);
-  __shared__ int fields[4][4];  // [warp][group]
+  __shared__ int fields[kFixedWarps][4];  // [warp][group]
   coef += blockIdx.y * sc;
   double* out = reinterpret_cast<double*>(pot + blockIdx.y * sp);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -596,7 +632,7 @@ __global__ void __launch_bounds__(128, 3)
   for (int64_t bi = blockIdx.x; bi < nleaf * nsplit; bi += gridDim.x) {
     const int64_t b = bi / nsplit;
     const int q0 = near_ptr[b], q1 = near_ptr[b + 1];
-    const int t0 = leaf_start[b] + int(bi % nsplit) * 4 + warp, t1 = leaf_start[b + 1];
+    const int t0 = leaf_start[b] + int(bi % nsplit) * kFixedWarps + warp, t1 = leaf_start[b + 1];
     const int len = int(row_ptr[leaf_start[b] + 1] - row_ptr[leaf_start[b]]);
     const int dl = nf.delta[b];
     for (int j0 = 0; j0 < len; j0 += kFixedStage) {
@@ -620,7 +656,9 @@ __global__ void __launch_bounds__(128, 3)
       if (lane < 4) fields[warp][lane] = lane == 0 ? x[0] : lane == 1 ? x[1] : lane == 2 ? x[2] : x[3];
       __syncthreads();
 #pragma unroll
-      for (int i = 0; i < 4; ++i) x[i] = max(max(fields[0][i], fields[1][i]), max(fields[2][i], fields[3][i]));
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int w = 0; w < kFixedWarps; ++w) x[i] = max(x[i], fields[w][i]);
       const bool finite = max(max(x[0], x[1]), max(x[2], x[3])) < 0x7ff;
       // beta's field covers a and delta; a takes beta's less delta
       x[1] = max(x[1], x[0] + dl);
@@ -656,7 +694,7 @@ __global__ void __launch_bounds__(128, 3)
       };
       int slot = 0;
       fetch(t0, 0, 0);
-      for (int t = t0; t < t1; t += 4 * nsplit) {
+      for (int t = t0; t < t1; t += kFixedWarps * nsplit) {
         const int64_t e0 = base + int64_t(t - leaf_start[b]) * len;
         double v;
         if (finite) {
@@ -665,7 +703,7 @@ __global__ void __launch_bounds__(128, 3)
           for (int i = 0; i < 12; ++i) sum[i] = FixedSum{0, 0};
           for (int i = 0; i < per_row; ++i) {
             const bool last = i + 1 == per_row;
-            fetch(last ? t + 4 * nsplit : t, last ? 0 : i + 1, slot ^ 1);
+            fetch(last ? t + kFixedWarps * nsplit : t, last ? 0 : i + 1, slot ^ 1);
             cp_async_wait<1>();
             const int j = 32 * i + lane;
             if (j0 + j < j1) {
@@ -716,18 +754,32 @@ __global__ void __launch_bounds__(128, 3)
   }
 }
 
-pie_status near_fixed_prepare() {
+static pie_status near_fixed_prepare() {
   static std::atomic<uint64_t> done{0};
-  return raise_smem(k_near_fixed, kFixedSmem, done);
+  int bit = -1;
+  if (device_done(done, &bit)) return PIE_OK;
+  pie_status s = raise_smem(k_near_fixed, kFixedSmem);
+  if (s == PIE_OK && bit >= 0) done.fetch_or(uint64_t(1) << bit);
+  return s;
+}
+
+pie_status near_prepare(const Problem& pr) {
+  switch (pr.par.precision) {
+    case PIE_FP64: return near_fixed_prepare();
+    case PIE_FP32: return near_float_prepare<float, false>();
+    case PIE_FP32H: return near_float_prepare<float, true>();
+    default: return near_float_prepare<double, false>();
+  }
 }
 
 // Launch of the fixed-point near part for nrhs columns on a grid of at most
 // max_blocks (0: no bound).
 static void near_fixed(const Problem& pr, const cd* coef, cd* pot, int nrhs, int64_t max_blocks, cudaStream_t st) {
   const FixedNear nf{static_cast<const int4*>(pr.mom), static_cast<const FixedRow*>(pr.fixed_row), pr.fixed_delta};
-  // shares per box: the least rounds of three blocks an SM, staging (about
-  // 1/50 of a box's rows) once a share; at least four test triangles each
-  const int64_t slots = 3 * int64_t(pr.nsm), most = std::min<int64_t>(16, (pr.T / pr.nleaf + 3) / 4);
+  // shares per box: the least rounds of three blocks an SM, staging (about 1/50
+  // of a box's rows) once a share; at least a test triangle for each warp
+  const int64_t slots = 3 * int64_t(pr.nsm),
+                most = std::min<int64_t>(16, (pr.T / pr.nleaf + kFixedWarps - 1) / kFixedWarps);
   int nsplit = 1;
   double best = 0;
   for (int64_t s = 1; s <= most; ++s) {
@@ -736,7 +788,7 @@ static void near_fixed(const Problem& pr, const cd* coef, cd* pot, int nrhs, int
   }
   int64_t grid = pr.nleaf * nsplit;
   if (max_blocks > 0) grid = std::min(grid, max_blocks);
-  k_near_fixed<<<dim3(unsigned(grid), unsigned(nrhs)), 128, kFixedSmem, st>>>(
+  k_near_fixed<<<dim3(unsigned(grid), unsigned(nrhs)), 32 * kFixedWarps, kFixedSmem, st>>>(
       pr.nleaf, nsplit, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr, nf, coef, kMu0, pot,
       6 * pr.T, 6 * pr.T);
 }
@@ -1798,7 +1850,7 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
   int rb = pr.tune.near_rhs_block;
   if (rb == 0) rb = nrhs == 1 ? 1 : nrhs == 2 ? 2 : 4;
   const bool boxed = sizeof(Rm) == 4 && pr.tune.near_kernel != 1;
-  auto box_launch = [&](auto rbc) -> pie_status {
+  auto box_launch = [&](auto rbc) {
     if constexpr (sizeof(Rm) == 4) {
       constexpr int RB = decltype(rbc)::value, TH = RB == 1 ? kNearBoxThreads : kNearChunkThreads;
       const int nsplit = near_box_split(pr, TH / 32);
@@ -1812,32 +1864,40 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
       const __half2* momh = static_cast<const __half2*>(pr.mom);
       const cf* c = reinterpret_cast<const cf*>(ncoef);
       if constexpr (RB == 1) {
-        pie_status s = near_box_prepare<Rio, H16>();
-        if (s != PIE_OK) return s;
         const int stage = near_box_stage<H16>(pr);
         k_near_box<Rio, H16><<<dim3(grid, nr), TH, near_box_smem<H16>(stage), sn>>>(
             pr.nleaf, nsplit, stage, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr, mom,
             momh, mom_scale(pr), c, float(kMu0), pot2, sT, sT);
       } else {
-        pie_status s = near_chunk_prepare<Rio, H16, RB>();
-        if (s != PIE_OK) return s;
-        k_near_chunk<Rio, H16, RB><<<dim3(grid, nblk(nrhs, RB)), TH, near_chunk_smem<RB>(), sn>>>(
+        k_near_chunk<Rio, H16, RB><<<dim3(grid, nblk(nrhs, RB)), TH, near_chunk_smem<H16, RB>(), sn>>>(
             pr.nleaf, nsplit, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr, mom, momh,
             mom_scale(pr), c, float(kMu0), pot2, nrhs, sT, sT);
       }
     }
-    return PIE_OK;
   };
   if (!with_near) {
     pot2 = nullptr;
   } else if constexpr (sizeof(Rm) == 8) {  // PIE_FP64: fixed point, each column by itself
+    // beside the far part: one block an SM where it ends with the far part, else
+    // two (three leave the filter kernels no shared memory until they are done:
+    // the 100 MHz plate 377 us beside 100 KB an SM, 440 beside 209).  One block takes
+    // 89 ps a pair (81,920 triangles: 1.95 ms), the far part 1.6 ps a double
+    // operation: 20 a list entry and sample, 32 a triangle and sample for
+    // aggregation and disaggregation, about 9000 a box and component for the filters
+    double far_ops = 32.0 * double(pr.T) * P;
+    for (int l = 3; l <= L; ++l)
+      far_ops += 20.0 * P * double(pr.lev[l].nlist) + (l > 3 ? 9000.0 * kComp * double(pr.lev[l].nb) : 0.0);
+    const int64_t per_sm = 89.0 * double(pr.nnz) > 1.6 * far_ops ? 2 : 1;
     near_fixed(pr, coef, pot2, nrhs,
-               overlap && pr.tune.near_ctas_per_sm > 0 ? int64_t(pr.nsm) * ((pr.tune.near_ctas_per_sm + 1) / 2) : 0, sn);
+               overlap && pr.tune.near_ctas_per_sm > 0
+                   ? int64_t(pr.nsm) * per_sm * ((pr.tune.near_ctas_per_sm + 1) / 2) : 0, sn);
   } else if (boxed && (rb == 1 || rb == 2 || rb == 4)) {
-    pie_status s = rb == 1   ? box_launch(std::integral_constant<int, 1>())
-                   : rb == 2 ? box_launch(std::integral_constant<int, 2>())
-                             : box_launch(std::integral_constant<int, 4>());
-    if (s != PIE_OK) return s;
+    if (rb == 1)
+      box_launch(std::integral_constant<int, 1>());
+    else if (rb == 2)
+      box_launch(std::integral_constant<int, 2>());
+    else
+      box_launch(std::integral_constant<int, 4>());
   } else if (rb == 1)
     near_launch(std::integral_constant<int, 1>());
   else if (rb == 2)
@@ -2043,8 +2103,6 @@ static pie_status apply_near_t(Problem& pr, const void* xv, void* yv, cudaStream
   if constexpr (sizeof(Rm) == 8) {
     near_fixed(pr, coef, pot, 1, 0, st);
   } else if (pr.tune.near_kernel != 1) {  // the box-staged kernel, unless tuned off
-    pie_status s = near_box_prepare<Rio, H16>();
-    if (s != PIE_OK) return s;
     const int nsplit = near_box_split(pr, kNearBoxThreads / 32), stage = near_box_stage<H16>(pr);
     k_near_box<Rio, H16><<<unsigned(pr.nleaf * nsplit), kNearBoxThreads, near_box_smem<H16>(stage), st>>>(
         pr.nleaf, nsplit, stage, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr,

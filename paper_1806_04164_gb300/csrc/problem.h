@@ -22,6 +22,7 @@ constexpr int kStages = 8;    // coef, near, aggregation, interpolation, transla
 
 struct LevelDev {
   int64_t nb = 0;
+  int64_t nlist = 0;           // interaction list entries
   int32_t* il_ptr = nullptr;   // [nb+1]
   int32_t* il_idx = nullptr;   // [nnz]
   int32_t* il_off = nullptr;   // [nnz]
@@ -137,8 +138,8 @@ pie_status apply_one(Problem& pr, const void* x, void* y, cudaStream_t st, const
 pie_status apply_batch(Problem& pr, const void* x, void* y, int nrhs, cudaStream_t st, const double* scale = nullptr);
 // x, y: N x nrhs columns, passes of tune.rhs_chunk columns
 pie_status apply_cols(Problem& pr, const void* x, void* y, int nrhs, cudaStream_t st);
-// the shared-memory limit of the fixed-point near kernel on the current device (set-up of PIE_FP64 problems)
-pie_status near_fixed_prepare();
+// shared-memory limits of the near kernels on the current device (set-up; not inside a stream capture)
+pie_status near_prepare(const Problem& pr);
 // records the start (end = false) or end of stage `stage` of the current apply when profiling
 void prof_mark(Problem& pr, int stage, bool end, cudaStream_t st);
 pie_status apply_near_one(Problem& pr, const void* x, void* y, cudaStream_t st);

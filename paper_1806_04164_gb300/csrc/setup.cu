@@ -978,7 +978,6 @@ static pie_status setup_t(Problem& pr, cudaStream_t st) {
   if constexpr (sizeof(Rm) == 8) {
     FixedRow* row = static_cast<FixedRow*>(pr.fixed_row = zalloc(pr, sizeof(FixedRow) * size_t(T), s));
     pr.fixed_delta = static_cast<int32_t*>(zalloc(pr, sizeof(int32_t) * size_t(nleaf), s));
-    if (s == PIE_OK) s = near_fixed_prepare();
     if (s != PIE_OK) return s;
     k_fixed_delta<<<unsigned((nleaf * 32 + 127) / 128), 128, 0, st>>>(nleaf, ng, pr.fixed_delta);
     k_moments_fixed<<<unsigned((T * 32 + 127) / 128), 128, 0, st>>>(T, pr.nnz, ng, pr.fixed_delta, row,
@@ -1027,6 +1026,7 @@ static pie_status setup_t(Problem& pr, cudaStream_t st) {
       std::vector<int32_t> idx(tr.il_idx[l].begin(), tr.il_idx[l].end());
       lv.il_ptr = upload(pr, ptr, st, s);
       lv.il_idx = upload(pr, idx, st, s);
+      lv.nlist = int64_t(idx.size());
       lv.il_off = upload(pr, tr.il_off[l], st, s);
       lv.S = zalloc(pr, sizeof(C2<Rf>) * size_t(pr.par.max_nrhs) * size_t(lv.nb) * kComp * P, s);
       lv.G = zalloc(pr, sizeof(C2<Rf>) * size_t(pr.par.max_nrhs) * size_t(lv.nb) * kComp * P, s);
@@ -1080,6 +1080,7 @@ static pie_status setup_t(Problem& pr, cudaStream_t st) {
   if ((s = cuda_check(cudaEventCreateWithFlags(&pr.ev_join, cudaEventDisableTiming), "event")) != PIE_OK) return s;
   if ((s = cuda_check(cudaEventCreateWithFlags(&pr.ev_far, cudaEventDisableTiming), "event")) != PIE_OK) return s;
   pr.tune = pie_tuning{1, 2, pr.par.max_nrhs, 0, 0, 0};
+  if ((s = near_prepare(pr)) != PIE_OK) return s;
   return cuda_check(cudaStreamSynchronize(st), "setup");
 }
 
