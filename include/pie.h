@@ -61,7 +61,10 @@ typedef enum {
 typedef enum { PIE_C128 = 0, PIE_C64 = 1 } pie_dtype;
 
 /* Arithmetic of the product:
- *  PIE_FP64  everything in complex double (inputs/outputs PIE_C128);
+ *  PIE_FP64  everything in complex double (inputs/outputs PIE_C128); the near
+ *            part multiplies 58-bit moments with 56-bit coefficients in fixed
+ *            point, scaled per test triangle and per leaf box, with exact
+ *            sums: an error no larger than that of FP64 multiply-adds;
  *  PIE_FP32  near and far parts in complex float (inputs/outputs PIE_C64);
  *  PIE_MIXED near part in complex float (pair moments stored as float),
  *            far part in complex double (inputs/outputs PIE_C128);

@@ -553,7 +553,7 @@ static pie_status near_float_prepare() {
 // leaf boxes alone do not fill the SMs.  81,920 triangles: 0.63 ms alone (2.2 ms
 // with FP64 multiply-adds), 24,576 of a cube: 0.66 ms (1.78); beside the far part
 // one block an SM does, since the two use different pipes: the product of 81,920
-// triangles 3.27 ms (5.11).
+// triangles 2.67 ms (3.27 when this came in, 5.11 before).
 
 // A warp-wide 64-bit multiply-add issues every two clocks and takes four, so the
 // limb products are taken kind by kind over all sums (KIND 0: h h', 1: h l',
@@ -2338,8 +2338,10 @@ static int field_terms(const Problem& pr) {
 
 // Phase of a centroid: 5 terms while k |c| stays below 0.2 (bodies well
 // below a wavelength, the method's range; a fifth of a pair's operations
-// less than sincos), else sincos (CT = 0).
-static bool field_small_phase(const Problem& pr) { return pr.k0 * pr.r_max < 0.2; }
+// less than sincos), else sincos (CT = 0).  reach: distance of the farthest
+// observation point from the origin, whose distances to the centroids are the
+// phases of the near-zone field.
+static bool field_small_phase(const Problem& pr, double reach = 0.0) { return pr.k0 * (pr.r_max + reach) < 0.2; }
 
 template <int NT>
 __device__ __forceinline__ double horner(const double* c, double z) {
@@ -2513,9 +2515,9 @@ static C2<Rio>* field_coef(Problem& pr, const void* x, cudaStream_t st) {
 // Runs f(integral_constant<NT>, integral_constant<CT>) for the problem's
 // numbers of series terms.
 template <typename F>
-static void with_field_terms(const Problem& pr, F f) {
+static void with_field_terms(const Problem& pr, F f, double reach = 0.0) {
   auto with_ct = [&](auto nt) {
-    if (field_small_phase(pr))
+    if (field_small_phase(pr, reach))
       f(nt, std::integral_constant<int, 5>());
     else
       f(nt, std::integral_constant<int, 0>());
@@ -2829,10 +2831,10 @@ pie_status rhs_potential(Problem& pr, const double* khat, const double* pol, dou
 // triangle, a short series per quadrature point, and 1/R from one rsqrt (no
 // division).  With g_q = w_q e^{ik(R_q - R_c)} / R_q and F_q = g_q (ik - 1/R_q)/R_q
 // the sums over an orbit need sum g, sum_o s_o g_ok, sum F, sum_o s_o F_ok only:
-// J and r - r' are affine in s_o v_k.  1024 points, 20,480 triangles: 14.6 ms;
+// J and r - r' are affine in s_o v_k.  1024 points, 20,480 triangles: 14.0 ms;
 // 42.0 ms with a block per point, a sincos and five divisions per quadrature
 // point.
-template <int NT>
+template <int NT, int CT>
 __global__ void __launch_bounds__(128) k_nearzone(int64_t T, int64_t npts, int64_t nchunk, int64_t len,
                                                   const double* __restrict__ vert, const double* __restrict__ cent,
                                                   const double* __restrict__ area, const int64_t* __restrict__ perm,
@@ -2853,7 +2855,7 @@ __global__ void __launch_bounds__(128) k_nearzone(int64_t T, int64_t npts, int64
     // common factor A e^{ik R_0} / (4 pi), times i w mu0 for J (ea: times a)
     // and -rho / eps0 for the gradient
     double sn, cs;
-    sincos(k0 * R0, &sn, &cs);
+    field_sincos<CT>(Q, k0 * R0, &sn, &cs);
     const double A = area[t] * (1.0 / (4.0 * kPi));
     const cd ej = mk<double>(-wmu * A * sn, wmu * A * cs), r = rho[perm[t]];
     const cd er = cmul(mk<double>(A * cs, A * sn), mk<double>(-inv_eps * r.x, -inv_eps * r.y));
@@ -2917,11 +2919,18 @@ pie_status nearzone(Problem& pr, const void* x, const void* rho, const double* p
   if (s != PIE_OK) return s;
   const cd* coef = field_coef<double>(pr, x, st);
   const FieldRule Q = field_rule(pr);
-  with_field_terms(pr, [&](auto nt, auto) {
-    k_nearzone<decltype(nt)::value><<<nblk(npts * nchunk * 32, 128), 128, 0, st>>>(
-        pr.T, npts, nchunk, len, pr.vert, pr.cent, pr.area, pr.perm, coef, static_cast<const cd*>(rho), d_pts, pr.k0,
-        pr.w * kMu0, 1.0 / eps0(), Q, partial);
-  });
+  double reach = 0;
+  for (int64_t i = 0; i < npts; ++i)
+    reach = std::max(reach, std::sqrt(pts[3 * i] * pts[3 * i] + pts[3 * i + 1] * pts[3 * i + 1] +
+                                      pts[3 * i + 2] * pts[3 * i + 2]));
+  with_field_terms(
+      pr,
+      [&](auto nt, auto ct) {
+        k_nearzone<decltype(nt)::value, decltype(ct)::value><<<nblk(npts * nchunk * 32, 128), 128, 0, st>>>(
+            pr.T, npts, nchunk, len, pr.vert, pr.cent, pr.area, pr.perm, coef, static_cast<const cd*>(rho), d_pts,
+            pr.k0, pr.w * kMu0, 1.0 / eps0(), Q, partial);
+      },
+      reach);
   k_field_finish<<<nblk(npts * 32, 128), 128, 0, st>>>(npts, nchunk, partial, nullptr, 0.0, static_cast<cd*>(E));
   return cuda_check(cudaGetLastError(), "nearfield launch");
 }

@@ -3,11 +3,11 @@
 // GB300 does two FP64 fused multiply-adds per clock and SM, and the near part
 // takes 48 per triangle pair: 24 clocks a pair on the pipe that also bounds the
 // far part, against 5.8 clocks of memory traffic (128 B a pair).  The integer
-// pipe multiplies 32 x 32 -> 64 bits and accumulates at 30 a clock and SM
+// pipe multiplies 32 x 32 -> 64 bits and accumulates at 54 a clock and SM
 // (measured).  With integers of two limbs, h 2^28 + l, a product takes three such
 // multiply-adds in two sums, h h' and h l' + l h' (l l' is below 2^-60 of the
-// largest product and left out), so a pair takes 4.8 clocks and leaves the FP64
-// pipe to the far part.
+// largest product and left out), so a pair takes 2.7 clocks of it and leaves the
+// FP64 pipe to the far part.
 //
 // A pair's moments are stored as integers of up to 58 bits times a power of two
 // that the test row shares (set-up), the sources' coefficients become 56-bit
