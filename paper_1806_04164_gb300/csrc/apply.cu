@@ -246,8 +246,8 @@ __device__ __forceinline__ void load_coefs(const cf* src, cf* c) {
 // j + 32, ...): the same operations in the same order as in k_near, so the same
 // result to the last bit.  nsplit shares a box's test triangles among several
 // blocks when the leaf boxes alone do not fill the SMs.  Rows longer than stage
-// (shared memory takes 4704 sources) read the coefficients from global memory
-// instead.
+// (shared memory takes 4736 sources, 4384 beside the half records) read the
+// coefficients from global memory instead.
 // Half-precision records reach shared memory by cp.async kNearAhead steps of 32
 // entries ahead, across rows: 327,680 triangles 607 -> 540 us (loads of four
 // records at a time left the memory idle at every row's end; float moments read
