@@ -433,8 +433,8 @@ pie_status pie_nearfield(pie_problem* pr, const void* x, const void* rho, const 
  *  far_rows: tile shape of the per-box far kernels of angular grids other
  *    than N_theta = 8 (aggregation, dense interpolation and anterpolation,
  *    translation; one thread per sample): boxes per block, 1, 2, 4, 8, 16 or
- *    32, reduced where a block would exceed 1024 threads or 48 KB of shared
- *    memory; 0 = automatic (enough boxes to fill 128 threads).
+ *    32, reduced where a block would exceed 1024 threads, an SM's registers or
+ *    48 KB of shared memory; 0 = automatic (enough boxes to fill 128 threads).
  *  near_kernel: near-part kernel for a float near part: 1 = one warp per
  *    test triangle reading the coefficients from global memory (1, 2, 4 or
  *    8 right-hand sides per thread), 2 = box-staged (one block per leaf box

@@ -801,6 +801,21 @@ __device__ __forceinline__ int antipode(int q, int ntheta) {
   return (ntheta - 1 - i) * nphi + (j + ntheta) % nphi;
 }
 
+// Largest blocks of the per-box far kernels, as their registers allow: a block
+// of n warps fits while each of the SM's four schedulers (16,384 registers) holds
+// its ceil(n / 4) of them, so 64 registers take 1024 threads, 80 take 768 and 88
+// to 96 take 640.  Kernels of up to 64 registers are bounded by 1024, the others
+// by what their main form takes, and the orchestration packs no more rows
+// into a block than fit; an angular grid whose one row is wider than that (20
+// and 22 theta rows) takes the WIDE form, held to 64 registers.
+constexpr int kFarThreads = 1024;
+template <typename Rf>
+constexpr int kAggThreads = sizeof(Rf) == 4 ? kFarThreads : 640;  // 59, 88 registers
+template <typename Rf, int NC, bool WIDE>
+constexpr int kInterpThreads = WIDE || NC == 1 ? kFarThreads : sizeof(Rf) == 4 ? 768 : 640;  // 80, 90 registers
+template <typename Rf, int NC, bool WIDE>
+constexpr int kTransThreads = WIDE || NC == 1 || sizeof(Rf) == 4 ? kFarThreads : 768;  // 77 registers in double
+
 // a2: leaf aggregation.  One block per leaf box, one thread per half-grid
 // sample q.  The radiation tables are stored for the half grid only, since
 // Pi(-khat) = conj(Pi(khat)) and M(-khat) = conj(M(khat)); with c X = c Xr +
@@ -808,7 +823,7 @@ __device__ __forceinline__ int antipode(int q, int ntheta) {
 // A = sum c Xr and B = sum c Xi.
 // Small angular grids pack several boxes into one block (threadIdx.y).
 template <typename Rf>
-__global__ void k_agg(int P, int ntheta, int64_t nb, const int32_t* __restrict__ leaf_start,
+__global__ void __launch_bounds__(kAggThreads<Rf>) k_agg(int P, int ntheta, int64_t nb, const int32_t* __restrict__ leaf_start,
                       const C2<Rf>* __restrict__ Pi, const C2<Rf>* __restrict__ M, const C2<Rf>* __restrict__ coef,
                       Rf mu0, C2<Rf>* __restrict__ S, int64_t sc = 0, int64_t sS = 0) {
   const int64_t b = int64_t(blockIdx.x) * blockDim.y + threadIdx.y;
@@ -884,9 +899,10 @@ __global__ void k_agg(int P, int ntheta, int64_t nb, const int32_t* __restrict__
 // 272 81 -> 35 us, 4400 (double) 358 -> 336 us; from about 10,000 boxes in double
 // and 9,000 in float k_agg is as fast or faster (its loads are wider).
 template <typename Rf, int NC>
-__global__ void k_agg_split(int P, int ntheta, int64_t nb, const int32_t* __restrict__ leaf_start,
-                      const C2<Rf>* __restrict__ Pi, const C2<Rf>* __restrict__ M, const C2<Rf>* __restrict__ coef,
-                      Rf mu0, C2<Rf>* __restrict__ S, int64_t sc = 0, int64_t sS = 0) {
+__global__ void __launch_bounds__(kFarThreads)
+    k_agg_split(int P, int ntheta, int64_t nb, const int32_t* __restrict__ leaf_start, const C2<Rf>* __restrict__ Pi,
+                const C2<Rf>* __restrict__ M, const C2<Rf>* __restrict__ coef, Rf mu0, C2<Rf>* __restrict__ S,
+                int64_t sc = 0, int64_t sS = 0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int X = threadIdx.z, part = blockIdx.z & 1, ri = X ? 1 - part : part, c0 = NC * int(blockIdx.z >> 1);
   const int nq = blockDim.x;
@@ -964,11 +980,11 @@ __global__ void k_agg_split(int P, int ntheta, int64_t nb, const int32_t* __rest
 // memory); children are summed in order, whatever cg.  A thread takes NC
 // components, the others threadIdx.z: five where the boxes fill the SMs, one on
 // small levels.
-template <typename Rf, int NC>
-__global__ void k_interp(int P, int64_t nb, const int32_t* __restrict__ child_start,
-                         const int8_t* __restrict__ oct_child, const C2<Rf>* __restrict__ Sc,
-                         const Rf* __restrict__ Ft, const C2<Rf>* __restrict__ phase, C2<Rf>* __restrict__ Sp,
-                         int64_t sSc = 0, int64_t sSp = 0, int cg = 1, bool fs = false) {
+template <typename Rf, int NC, bool WIDE = false>
+__global__ void __launch_bounds__(kInterpThreads<Rf, NC, WIDE>)
+    k_interp(int P, int64_t nb, const int32_t* __restrict__ child_start, const int8_t* __restrict__ oct_child,
+             const C2<Rf>* __restrict__ Sc, const Rf* __restrict__ Ft, const C2<Rf>* __restrict__ phase,
+             C2<Rf>* __restrict__ Sp, int64_t sSc = 0, int64_t sSp = 0, int cg = 1, bool fs = false) {
   Sc += blockIdx.y * sSc;
   Sp += blockIdx.y * sSp;
   extern __shared__ unsigned char smem_raw[];
@@ -1347,8 +1363,8 @@ __device__ __forceinline__ int trans_level(const TransArgs& a, int64_t box) {
 // left most SMs idle in turn: 327,680 triangles (double) 4.58 -> 4.40 ms, 81,920
 // 1.25 -> 1.12 ms, 56 boxes 46 -> 20 us, float patterns of 32 samples at 327,680
 // triangles 135 -> 97 us.
-template <typename Rf, int NC>
-__global__ void k_trans(int P, const TransArgs args) {
+template <typename Rf, int NC, bool WIDE = false>
+__global__ void __launch_bounds__(kTransThreads<Rf, NC, WIDE>) k_trans(int P, const TransArgs args) {
   constexpr int U = sizeof(Rf) == 4 ? 4 : 1;
   const int64_t box = int64_t(blockIdx.x) * blockDim.y + threadIdx.y;
   if (box >= args.total) return;
@@ -1400,7 +1416,7 @@ __global__ void k_trans(int P, const TransArgs args) {
 // order of operations depends on the list alone, never on the launch shape.
 constexpr int kTransSplit = 4;
 template <typename Rf, int NC>
-__global__ void k_trans_split(int P, const TransArgs args) {
+__global__ void __launch_bounds__(kFarThreads) k_trans_split(int P, const TransArgs args) {
   constexpr int U = 4;
   extern __shared__ unsigned char smem_raw[];
   C2<Rf>* part = reinterpret_cast<C2<Rf>*>(smem_raw);  // [row][chunk][component][P]
@@ -1467,9 +1483,10 @@ __global__ void k_trans_split(int P, const TransArgs args) {
 // row of a block (several rows for small angular grids).  With fs the
 // filter F is staged in shared memory first (else read from global memory).
 template <typename Rf, int NC>
-__global__ void k_anterp(int P, int64_t nc, const int32_t* __restrict__ parent, const int8_t* __restrict__ oct_child,
-                         const C2<Rf>* __restrict__ Gp, const Rf* __restrict__ Fg, const C2<Rf>* __restrict__ phase,
-                         C2<Rf>* __restrict__ Gc, int64_t sGp = 0, int64_t sGc = 0, bool fs = false) {
+__global__ void __launch_bounds__(kFarThreads)
+    k_anterp(int P, int64_t nc, const int32_t* __restrict__ parent, const int8_t* __restrict__ oct_child,
+             const C2<Rf>* __restrict__ Gp, const Rf* __restrict__ Fg, const C2<Rf>* __restrict__ phase,
+             C2<Rf>* __restrict__ Gc, int64_t sGp = 0, int64_t sGc = 0, bool fs = false) {
   Gp += blockIdx.y * sGp;
   Gc += blockIdx.y * sGc;
   extern __shared__ unsigned char smem_raw[];
@@ -1919,10 +1936,10 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
   // far coefficients in the far precision (MIXED and FP64: the io buffer)
   const C2<Rf>* fcoef = reinterpret_cast<const C2<Rf>*>(coef);
   // boxes per block of the per-box far kernels (threads: one per sample):
-  // tune.far_rows, or enough to fill 128 threads; at most 1024 threads
-  auto far_rows = [&](int threads) {
+  // tune.far_rows, or enough to fill 128 threads; at most the kernel's threads
+  auto far_rows = [&](int threads, int most = kFarThreads) {
     const int r = pr.tune.far_rows > 0 ? pr.tune.far_rows : (threads < 64 ? 128 / threads : 1);
-    return std::max(1, std::min(r, 1024 / threads));
+    return std::max(1, std::min(r, most / threads));
   };
   // grids of fewer warps than kWideWarps an SM (eight a scheduler) give each
   // warp less to do (components and sums over more threads); the arithmetic
@@ -1946,7 +1963,7 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
     } else if (narrow(sizeof(Rf) == 8 ? warps / 4 : warps)) {
       split(std::integral_constant<int, kComp>());
     } else {
-      const int abp = far_rows(ath);
+      const int abp = far_rows(ath, kAggThreads<Rf>);
       k_agg<Rf><<<dim3(nblk(pr.lev[L].nb, abp), nr), dim3(ath, abp), 0, sf>>>(
           P, pr.par.ntheta, pr.lev[L].nb, pr.leaf_start, Pi, M, fcoef, Rf(kMu0), SL, sT, sl(L));
     }
@@ -1986,11 +2003,18 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
   for (int l = L - 1; l >= 3 && !fft8; --l)
     dense(pr.lev[l].nb, [&](auto ncc, int rows, int kids) {
       constexpr int NC = decltype(ncc)::value;
-      k_interp<Rf, NC><<<dim3(nblk(pr.lev[l].nb, rows), nr), dim3(tpb, rows, kComp / NC),
-                         fsm_bytes + sm * rows * kids, sf>>>(
-          P, pr.lev[l].nb, pr.lev[l].child_start, pr.lev[l + 1].octant, static_cast<const C2<Rf>*>(pr.lev[l + 1].S),
-          static_cast<const Rf*>(pr.lev[l].Ft), static_cast<const C2<Rf>*>(pr.lev[l].phase),
-          static_cast<C2<Rf>*>(pr.lev[l].S), sl(l + 1), sl(l), kids, fsh);
+      auto launch = [&](auto wide, int n) {
+        k_interp<Rf, NC, decltype(wide)::value><<<dim3(nblk(pr.lev[l].nb, n), nr), dim3(tpb, n, kComp / NC),
+                                                  fsm_bytes + sm * n * kids, sf>>>(
+            P, pr.lev[l].nb, pr.lev[l].child_start, pr.lev[l + 1].octant, static_cast<const C2<Rf>*>(pr.lev[l + 1].S),
+            static_cast<const Rf*>(pr.lev[l].Ft), static_cast<const C2<Rf>*>(pr.lev[l].phase),
+            static_cast<C2<Rf>*>(pr.lev[l].S), sl(l + 1), sl(l), kids, fsh);
+      };
+      constexpr int most = kInterpThreads<Rf, NC, false> / (kComp / NC);
+      // (in double a grid that wide needs more than 48 KB a child: refused)
+      if constexpr (sizeof(Rf) == 4 && NC > 1)
+        if (tpb > most) return launch(std::true_type(), 1);
+      launch(std::false_type(), std::max(1, std::min(rows, most / tpb)));
     });
   prof_mark(pr, 3, true, st);
   prof_mark(pr, 4, false, st);
@@ -2017,7 +2041,13 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
                                   sizeof(C2<Rf>) * NC * P * kTransSplit * tbp, sf>>>(P, ta);
           return;
         }
-      const int tbp = far_rows(tpb);  // destination boxes per block
+      constexpr int most = kTransThreads<Rf, NC, false>;
+      if constexpr (most < kFarThreads)
+        if (tpb > most) {
+          k_trans<Rf, NC, true><<<dim3(unsigned(ta.total), nr, kComp / NC), tpb, 0, sf>>>(P, ta);
+          return;
+        }
+      const int tbp = far_rows(tpb, most);  // destination boxes per block
       k_trans<Rf, NC><<<dim3(nblk(ta.total, tbp), nr, kComp / NC), dim3(tpb, tbp), 0, sf>>>(P, ta);
     };
     if (one)
