@@ -2366,12 +2366,11 @@ static int field_terms(const Problem& pr) {
   return kh < 6e-3 ? 3 : kh < 0.13 ? 5 : 7;
 }
 
-// Phase of a centroid: 5 terms while k |c| stays below 0.2 (bodies well
-// below a wavelength, the method's range; a fifth of a pair's operations
-// less than sincos), else sincos (CT = 0).  reach: distance of the farthest
-// observation point from the origin, whose distances to the centroids are the
-// phases of the near-zone field.
-static bool field_small_phase(const Problem& pr, double reach = 0.0) { return pr.k0 * (pr.r_max + reach) < 0.2; }
+// Phase of a centroid: 6 terms while it stays below 0.2 (bodies well below a
+// wavelength, the method's range; a fifth of a pair's operations less than
+// sincos; first omitted term 0.2^12 / 12! = 9e-18), else sincos (CT = 0).
+constexpr double kSmallPhase = 0.2;
+constexpr int kSmallTerms = 6;
 
 template <int NT>
 __device__ __forceinline__ double horner(const double* c, double z) {
@@ -2543,12 +2542,12 @@ static C2<Rio>* field_coef(Problem& pr, const void* x, cudaStream_t st) {
 }
 
 // Runs f(integral_constant<NT>, integral_constant<CT>) for the problem's
-// numbers of series terms.
+// numbers of series terms; phase: largest phase of a centroid.
 template <typename F>
-static void with_field_terms(const Problem& pr, F f, double reach = 0.0) {
+static void with_field_terms(const Problem& pr, double phase, F f) {
   auto with_ct = [&](auto nt) {
-    if (field_small_phase(pr, reach))
-      f(nt, std::integral_constant<int, 5>());
+    if (phase < kSmallPhase)
+      f(nt, std::integral_constant<int, kSmallTerms>());
     else
       f(nt, std::integral_constant<int, 0>());
   };
@@ -2572,7 +2571,7 @@ static pie_status farfield_t(Problem& pr, const void* x, const double* rhat, int
   if (s != PIE_OK) return s;
   const C2<Rio>* coef = field_coef<Rio>(pr, x, st);
   const FieldRule R = field_rule(pr);
-  with_field_terms(pr, [&](auto nt, auto ct) {
+  with_field_terms(pr, pr.k0 * pr.r_max, [&](auto nt, auto ct) {
     k_farfield<Rio, decltype(nt)::value, decltype(ct)::value><<<nblk(ndir * nchunk * 32, 128), 128, 0, st>>>(
         pr.T, ndir, nchunk, len, pr.vert, pr.cent, pr.area, coef, d_rhat, pr.k0, R, partial);
   });
@@ -2778,7 +2777,7 @@ static pie_status farfield_adjoint_t(Problem& pr, const double* rhat, int64_t nd
   if (s != PIE_OK) return s;
   C2<Rio>* pot = static_cast<C2<Rio>*>(pr.pot);
   const FieldRule R = field_rule(pr);
-  with_field_terms(pr, [&](auto nt, auto ct) {
+  with_field_terms(pr, pr.k0 * pr.r_max, [&](auto nt, auto ct) {
     k_farfield_adj<Rio, decltype(nt)::value, decltype(ct)::value><<<dim3(nblk(pr.T, 128), unsigned(nchunk)), 128, 0, st>>>(
         pr.T, ndir, len, pr.vert, pr.cent, pr.area, d_rhat, static_cast<const cd*>(E), pr.k0,
         pr.w * kMu0 / (4.0 * kPi), R, pot, partial);
@@ -2953,14 +2952,12 @@ pie_status nearzone(Problem& pr, const void* x, const void* rho, const double* p
   for (int64_t i = 0; i < npts; ++i)
     reach = std::max(reach, std::sqrt(pts[3 * i] * pts[3 * i] + pts[3 * i + 1] * pts[3 * i + 1] +
                                       pts[3 * i + 2] * pts[3 * i + 2]));
-  with_field_terms(
-      pr,
-      [&](auto nt, auto ct) {
-        k_nearzone<decltype(nt)::value, decltype(ct)::value><<<nblk(npts * nchunk * 32, 128), 128, 0, st>>>(
-            pr.T, npts, nchunk, len, pr.vert, pr.cent, pr.area, pr.perm, coef, static_cast<const cd*>(rho), d_pts,
-            pr.k0, pr.w * kMu0, 1.0 / eps0(), Q, partial);
-      },
-      reach);
+  // the phases are k times the distances of the points from the centroids
+  with_field_terms(pr, pr.k0 * (pr.r_max + reach), [&](auto nt, auto ct) {
+    k_nearzone<decltype(nt)::value, decltype(ct)::value><<<nblk(npts * nchunk * 32, 128), 128, 0, st>>>(
+        pr.T, npts, nchunk, len, pr.vert, pr.cent, pr.area, pr.perm, coef, static_cast<const cd*>(rho), d_pts,
+        pr.k0, pr.w * kMu0, 1.0 / eps0(), Q, partial);
+  });
   k_field_finish<<<nblk(npts * 32, 128), 128, 0, st>>>(npts, nchunk, partial, nullptr, 0.0, static_cast<cd*>(E));
   return cuda_check(cudaGetLastError(), "nearfield launch");
 }

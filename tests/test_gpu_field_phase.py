@@ -1,0 +1,56 @@
+"""Phases of the field maps at the limits of their series: bodies whose
+farthest centroid (and point) lies just inside the range of the short series for
+the centroid's phase."""
+import numpy as np
+import pytest
+
+import pie_inputs as pi
+
+pytestmark = pytest.mark.gpu
+
+
+def _problem(k, offset=0.0, n=8, side=0.05, precision="PIE_MIXED"):
+    from oracle.mesh import build_topology
+    from tests._lib import ensure_built
+    ensure_built()
+    import paper_1806_04164_gb300 as pg
+    xyz, tri = pi.square_patch(n, side)
+    h = side / n * 2 ** 0.5
+    u = np.array([0.48, -0.6, 0.64])
+    xyz = xyz + offset * u
+    return build_topology(xyz, tri), pg.Problem(pg.Mesh(xyz, tri), k, 3, root_side=max(1.01 * side, 6.01 * h),
+                                                precision=getattr(pg, precision)), u
+
+
+@pytest.mark.parametrize("kr", [0.0899, 0.15, 0.1999, 0.21])
+def test_phase_series_at_its_limit(kr):
+    """Every triangle's phase is kr to a few per cent, the largest kr itself, so
+    that a series cut short shows in full.  Rounding: the phase to an ulp or two of
+    0.2, sine and cosine to an ulp each, a dozen multiply-adds a term: below 5e-15
+    of the norm."""
+    import torch
+    from oracle.farfield import far_field
+    from oracle.nearzone import scattered_field
+    top, _, u = _problem(0.1, offset=1.0)
+    far = np.linalg.norm(top.centroid, axis=1).max()
+    k = kr / far
+    top, pr, u = _problem(k, offset=1.0)
+    x = pi.complex_normal(pr.N, 3)
+    d = np.stack([u, -u])
+    xd = torch.from_numpy(x).cuda()
+    E, Eo = pr.farfield(xd, d).cpu().numpy(), far_field(top, k, x, d)
+    for i in range(2):
+        assert np.linalg.norm(E[i] - Eo[i]) <= 5e-15 * np.linalg.norm(Eo[i])
+    g = np.cross(u, pi.complex_normal(3, 4))[None]
+    v = pr.farfield_adjoint(torch.from_numpy(g).cuda(), d[:1]).cpu().numpy()
+    F = np.stack([far_field(top, k, e, d[:1])[0] for e in np.eye(pr.N)[:pr.E]])
+    vo = np.concatenate([F.conj() @ g[0], np.zeros(pr.T)])
+    assert np.linalg.norm(v - vo) <= 5e-15 * np.linalg.norm(vo)
+    # centroids 1 m to one side, a point 1 m to the other: the distance is the sum
+    k = kr / (far + 1.0)
+    top, pr, u = _problem(k, offset=1.0)
+    rho = pi.complex_normal(pr.T, 6) * 8.8e-12
+    p = -u[None]
+    E = pr.nearfield(xd, torch.from_numpy(rho).cuda(), p).cpu().numpy()
+    Eo = scattered_field(top, k, x, rho, p)
+    assert np.linalg.norm(E - Eo) <= 5e-15 * np.linalg.norm(Eo)
