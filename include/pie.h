@@ -272,7 +272,8 @@ pie_status pie_rhs_potentials(pie_problem* pr, const void* A_q, const void* Phi_
 
 /* Far-zone field from J (Section 2): E[d] = i w mu0/(4 pi) (I - rr) .
  * int J exp(-i k0 r.r') dr' (factor exp(i k0 r)/r removed).  rhat: host
- * ndir x 3; x: device solutions, N x nrhs (problem dtype, column j at
+ * ndir x 3 (unit vectors; for a vector r of another length the formula as it
+ * stands); x: device solutions, N x nrhs (problem dtype, column j at
  * offset j*N); E: device nrhs x ndir x 3 complex double. */
 pie_status pie_farfield(pie_problem* pr, const void* x, const double* rhat, int64_t ndir, void* E, int nrhs,
                         void* stream);

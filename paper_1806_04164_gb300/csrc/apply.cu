@@ -2359,11 +2359,19 @@ static FieldRule field_rule(const Problem& pr) {
   return r;
 }
 
-// Terms for phases up to 2/3 k h: 3 below k h = 6e-3, 5 below 0.13, else 7
-// (first omitted term (2/3 k h)^(2 NT) / (2 NT)! < 1e-17).
-static int field_terms(const Problem& pr) {
-  const double kh = pr.k0 * pr.h_max;
-  return kh < 6e-3 ? 3 : kh < 0.13 ? 5 : 7;
+// Terms for phases up to 2/3 k h: 3 below k h = 6e-3, 5 below 0.13, 7 up to
+// kMaxFieldKh (first omitted term (2/3 k h)^(2 NT) / (2 NT)! < 1e-17).  A longer
+// direction than a unit vector scales the phases and may leave that range: NT = 0,
+// sine and cosine of each orbit.
+constexpr double kMaxFieldKh = 0.52;
+static int field_terms(double kh) { return kh < 6e-3 ? 3 : kh < 0.13 ? 5 : kh <= kMaxFieldKh ? 7 : 0; }
+
+// Length of the longest of n vectors.
+static double longest(const double* v, int64_t n) {
+  double r2 = 0;
+  for (int64_t i = 0; i < n; ++i)
+    r2 = std::max(r2, v[3 * i] * v[3 * i] + v[3 * i + 1] * v[3 * i + 1] + v[3 * i + 2] * v[3 * i + 2]);
+  return std::sqrt(r2);
 }
 
 // Phase of a centroid: 6 terms while it stays below 0.2 (bodies well below a
@@ -2391,13 +2399,27 @@ __device__ __forceinline__ void field_sincos(const FieldRule& R, double p, doubl
   }
 }
 
-// f(p) added to C, D(p) returned.
+// f(p) added to C, D(p) returned (NT = 0: D but for a constant, which cancels in G_k).
 template <int NT>
 __device__ __forceinline__ cd field_phase(const FieldRule& R, double p, cd& C) {
-  const double z = p * p;
-  C.x += horner<NT>(R.fe, z);
-  C.y = fma(p, horner<NT>(R.fo, z), C.y);
-  return mk<double>(horner<NT>(R.de, z), p * horner<NT>(R.dO, z));
+  if constexpr (NT == 0) {
+    // (both orbits written out: as a loop, nvcc 13.0 left a term out of C)
+    cd D = mk<double>(0, 0);
+    double s0, c0, s1, c1;
+    sincos(R.s[0] * p, &s0, &c0);
+    sincos(R.s[1] * p, &s1, &c1);
+    const cd e0 = mk<double>(R.w[0] * c0, -R.w[0] * s0), e1 = mk<double>(R.w[1] * c1, -R.w[1] * s1);
+    C.x += e0.x + e1.x;
+    C.y += e0.y + e1.y;
+    rfma(D, R.s[0], e0);
+    rfma(D, R.s[1], e1);
+    return D;
+  } else {
+    const double z = p * p;
+    C.x += horner<NT>(R.fe, z);
+    C.y = fma(p, horner<NT>(R.fo, z), C.y);
+    return mk<double>(horner<NT>(R.de, z), p * horner<NT>(R.dO, z));
+  }
 }
 
 // C and G_k = D(p_k) - D(p_2), k = 0, 1 (sum_k v_k D_k = v_0 G_0 + v_1 G_1).
@@ -2541,17 +2563,20 @@ static C2<Rio>* field_coef(Problem& pr, const void* x, cudaStream_t st) {
   return coef;
 }
 
-// Runs f(integral_constant<NT>, integral_constant<CT>) for the problem's
-// numbers of series terms; phase: largest phase of a centroid.
-template <typename F>
-static void with_field_terms(const Problem& pr, double phase, F f) {
+// Runs f(integral_constant<NT>, integral_constant<CT>) for the numbers of
+// series terms at k h and at phase, the largest phase of a centroid.  ANY: k h
+// may exceed kMaxFieldKh.
+template <bool ANY, typename F>
+static void with_field_terms(double kh, double phase, F f) {
   auto with_ct = [&](auto nt) {
     if (phase < kSmallPhase)
       f(nt, std::integral_constant<int, kSmallTerms>());
     else
       f(nt, std::integral_constant<int, 0>());
   };
-  switch (field_terms(pr)) {
+  if constexpr (ANY)
+    if (field_terms(kh) == 0) return f(std::integral_constant<int, 0>(), std::integral_constant<int, 0>());
+  switch (field_terms(kh)) {
     case 3: return with_ct(std::integral_constant<int, 3>());
     case 5: return with_ct(std::integral_constant<int, 5>());
     default: return with_ct(std::integral_constant<int, 7>());
@@ -2571,7 +2596,8 @@ static pie_status farfield_t(Problem& pr, const void* x, const double* rhat, int
   if (s != PIE_OK) return s;
   const C2<Rio>* coef = field_coef<Rio>(pr, x, st);
   const FieldRule R = field_rule(pr);
-  with_field_terms(pr, pr.k0 * pr.r_max, [&](auto nt, auto ct) {
+  const double k = pr.k0 * longest(rhat, ndir);
+  with_field_terms<true>(k * pr.h_max, k * pr.r_max, [&](auto nt, auto ct) {
     k_farfield<Rio, decltype(nt)::value, decltype(ct)::value><<<nblk(ndir * nchunk * 32, 128), 128, 0, st>>>(
         pr.T, ndir, nchunk, len, pr.vert, pr.cent, pr.area, coef, d_rhat, pr.k0, R, partial);
   });
@@ -2777,7 +2803,8 @@ static pie_status farfield_adjoint_t(Problem& pr, const double* rhat, int64_t nd
   if (s != PIE_OK) return s;
   C2<Rio>* pot = static_cast<C2<Rio>*>(pr.pot);
   const FieldRule R = field_rule(pr);
-  with_field_terms(pr, pr.k0 * pr.r_max, [&](auto nt, auto ct) {
+  const double k = pr.k0 * longest(rhat, ndir);
+  with_field_terms<true>(k * pr.h_max, k * pr.r_max, [&](auto nt, auto ct) {
     k_farfield_adj<Rio, decltype(nt)::value, decltype(ct)::value><<<dim3(nblk(pr.T, 128), unsigned(nchunk)), 128, 0, st>>>(
         pr.T, ndir, len, pr.vert, pr.cent, pr.area, d_rhat, static_cast<const cd*>(E), pr.k0,
         pr.w * kMu0 / (4.0 * kPi), R, pot, partial);
@@ -2948,12 +2975,8 @@ pie_status nearzone(Problem& pr, const void* x, const void* rho, const double* p
   if (s != PIE_OK) return s;
   const cd* coef = field_coef<double>(pr, x, st);
   const FieldRule Q = field_rule(pr);
-  double reach = 0;
-  for (int64_t i = 0; i < npts; ++i)
-    reach = std::max(reach, std::sqrt(pts[3 * i] * pts[3 * i] + pts[3 * i + 1] * pts[3 * i + 1] +
-                                      pts[3 * i + 2] * pts[3 * i + 2]));
   // the phases are k times the distances of the points from the centroids
-  with_field_terms(pr, pr.k0 * (pr.r_max + reach), [&](auto nt, auto ct) {
+  with_field_terms<false>(pr.k0 * pr.h_max, pr.k0 * (pr.r_max + longest(pts, npts)), [&](auto nt, auto ct) {
     k_nearzone<decltype(nt)::value, decltype(ct)::value><<<nblk(npts * nchunk * 32, 128), 128, 0, st>>>(
         pr.T, npts, nchunk, len, pr.vert, pr.cent, pr.area, pr.perm, coef, static_cast<const cd*>(rho), d_pts,
         pr.k0, pr.w * kMu0, 1.0 / eps0(), Q, partial);

@@ -1,6 +1,7 @@
 """Phases of the field maps at the limits of their series: bodies whose
 farthest centroid (and point) lies just inside the range of the short series for
-the centroid's phase."""
+the centroid's phase, and directions that are not unit vectors (the maps are
+defined for any vector)."""
 import numpy as np
 import pytest
 
@@ -54,3 +55,28 @@ def test_phase_series_at_its_limit(kr):
     E = pr.nearfield(xd, torch.from_numpy(rho).cuda(), p).cpu().numpy()
     Eo = scattered_field(top, k, x, rho, p)
     assert np.linalg.norm(E - Eo) <= 5e-15 * np.linalg.norm(Eo)
+
+
+@pytest.mark.parametrize("length", [1e-3, 1.5, 4.0, 40.0, 1e4])
+@pytest.mark.parametrize("kh", [1e-3, 0.1, 0.5])
+def test_directions_of_any_length(length, kh):
+    """F(rhat) for |rhat| != 1: the phases are k rhat . r whatever its length
+    (rounding: 1e-16 of the largest phase, and 1e-12 as for unit vectors)."""
+    import torch
+    from oracle.farfield import far_field
+    h = 0.05 / 8 * 2 ** 0.5
+    k = kh / h
+    top, pr, _ = _problem(k, offset=0.02)
+    tol = 1e-12 + 4e-16 * k * length * 0.08
+    x = pi.complex_normal(pr.N, 3)
+    rng = np.random.default_rng(1)
+    d = rng.normal(size=(5, 3))
+    d *= length / np.linalg.norm(d, axis=1, keepdims=True)
+    d[3] /= 7
+    E, Eo = pr.farfield(torch.from_numpy(x).cuda(), d).cpu().numpy(), far_field(top, k, x, d)
+    assert np.linalg.norm(E - Eo) <= tol * np.linalg.norm(Eo)
+    g = pi.complex_normal(15, 4).reshape(5, 3)
+    v = pr.farfield_adjoint(torch.from_numpy(g).cuda(), d).cpu().numpy()
+    F = np.stack([far_field(top, k, e, d) for e in np.eye(pr.N)[:pr.E]])
+    vo = np.concatenate([np.einsum("end,nd->e", F.conj(), g), np.zeros(pr.T)])
+    assert np.linalg.norm(v - vo) <= tol * np.linalg.norm(vo)
