@@ -2436,26 +2436,29 @@ __device__ __forceinline__ void field_triangle(const FieldRule& R, double p0, do
 // A warp per (direction or point, chunk of triangles): lanes stride over the
 // chunk, the six sums are reduced once per warp and the chunks' partial sums
 // are added in order by k_field_finish, so the sum does not depend on
-// scheduling.  Chunks are cut so that there are about kFieldWarps warps per
-// SM: one block per direction left the pipe idle (181 directions on 152 SMs).
-constexpr int kFieldWarps = 32;
-static void field_chunks(const Problem& pr, int64_t rows, int64_t items, int64_t unit, int64_t* nchunk, int64_t* len) {
-  int64_t n = std::max<int64_t>(1, (int64_t(pr.nsm) * kFieldWarps + rows - 1) / rows);
-  n = std::min(n, std::max<int64_t>(1, (items + 2 * unit - 1) / (2 * unit)));
-  *len = ((items + n - 1) / n + unit - 1) / unit * unit;
-  *nchunk = (items + *len - 1) / *len;
+// scheduling.  Chunks are cut by the number of triangles alone, so that a field
+// does not depend on the directions or points beside it either: at least
+// kFieldChunk triangles (four a lane; the warp's reduction is eight adds) and at
+// most kFieldChunks chunks, which gives one direction a few hundred warps.
+// (One block per direction left the pipe idle: 181 directions on 152 SMs.)
+constexpr int64_t kFieldChunk = 128, kFieldChunks = 1024;
+static void field_chunks(const Problem& pr, int64_t* nchunk, int64_t* len) {
+  *len = std::max(kFieldChunk, ((pr.T + kFieldChunks - 1) / kFieldChunks + 31) / 32 * 32);
+  *nchunk = (pr.T + *len - 1) / *len;
 }
 
-// Scratch of one field call: the leaf sum / difference patterns, which only
-// live inside a product, or a stream-ordered allocation when they are too
-// small (many directions on a small problem).
+// Scratch of one field call: half of the leaf sum / difference patterns, which
+// only live inside a product (the adjoint map takes the upper half: it shares
+// no other buffer with the maps), or a stream-ordered allocation where that is
+// too small.
 struct FieldScratch {
   void* p = nullptr;
   cudaStream_t st;
   bool own = false;
-  FieldScratch(Problem& pr, size_t bytes, cudaStream_t s_, pie_status& s) : st(s_) {
-    if (bytes <= pr.gsgd_bytes) {
-      p = pr.gsgd;
+  FieldScratch(Problem& pr, size_t bytes, cudaStream_t s_, pie_status& s, bool adjoint = false) : st(s_) {
+    const size_t half = pr.gsgd_bytes / 512 * 256;
+    if (bytes <= half) {
+      p = static_cast<char*>(pr.gsgd) + (adjoint ? half : 0);
       return;
     }
     s = cuda_check(cudaMallocAsync(&p, bytes, st), "field scratch");
@@ -2466,12 +2469,30 @@ struct FieldScratch {
   }
 };
 
-__device__ __forceinline__ void field_partial(double (&S)[6], double* __restrict__ out) {
+// Directions or points of one launch: their partial sums take at most kFieldScratch bytes.
+constexpr size_t kFieldScratch = size_t(64) << 20;
+static int64_t field_batch(int64_t n, int64_t nchunk) {
+  return std::min<int64_t>(n, std::max<int64_t>(1, int64_t(kFieldScratch / (6 * sizeof(double) * size_t(nchunk)))));
+}
+
+// The warp's six sums into out[0..5], each step of the butterfly keeping half of
+// the values on either side (8 adds a lane instead of 30).
+__device__ __forceinline__ void field_partial(const double (&S)[6], double* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+  auto step = [](bool up, double lo, double hi, int o) {
+    const double keep = up ? hi : lo, send = up ? lo : hi;
+    return keep + __shfl_xor_sync(0xffffffffu, send, o);
+  };
+  double x[3], y[2];
 #pragma unroll
-  for (int i = 0; i < 6; ++i) S[i] = warp_sum(S[i]);
-  if ((threadIdx.x & 31) == 0)
-#pragma unroll
-    for (int i = 0; i < 6; ++i) out[i] = S[i];
+  for (int i = 0; i < 3; ++i) x[i] = step(h4, S[i], S[3 + i], 16);
+  y[0] = step(h3, x[0], x[2], 8);
+  y[1] = step(h3, x[1], 0.0, 8);
+  double z = step(h2, y[0], y[1], 4);
+  z += __shfl_xor_sync(0xffffffffu, z, 2);
+  z += __shfl_xor_sync(0xffffffffu, z, 1);
+  if ((lane & 3) == 0 && !(h3 && h2)) out[(h4 ? 3 : 0) + (h3 ? 2 : 0) + (h2 ? 1 : 0)] = z;
 }
 
 // Far field: partial sums of F = sum_t int J exp(-i k0 rhat.r).  181
@@ -2586,9 +2607,10 @@ static void with_field_terms(double kh, double phase, F f) {
 template <typename Rio>
 static pie_status farfield_t(Problem& pr, const void* x, const double* rhat, int64_t ndir, void* E, cudaStream_t st) {
   int64_t nchunk, len;
-  field_chunks(pr, ndir, pr.T, 32, &nchunk, &len);
+  field_chunks(pr, &nchunk, &len);
+  const int64_t batch = field_batch(ndir, nchunk);
   pie_status s = PIE_OK;
-  FieldScratch scratch(pr, sizeof(double) * size_t(ndir) * (3 + 6 * size_t(nchunk)), st, s);
+  FieldScratch scratch(pr, sizeof(double) * (3 * size_t(ndir) + 6 * size_t(nchunk * batch)), st, s);
   if (s != PIE_OK) return s;
   double* d_rhat = static_cast<double*>(scratch.p);
   double* partial = d_rhat + 3 * ndir;
@@ -2598,11 +2620,14 @@ static pie_status farfield_t(Problem& pr, const void* x, const double* rhat, int
   const FieldRule R = field_rule(pr);
   const double k = pr.k0 * longest(rhat, ndir);
   with_field_terms<true>(k * pr.h_max, k * pr.r_max, [&](auto nt, auto ct) {
-    k_farfield<Rio, decltype(nt)::value, decltype(ct)::value><<<nblk(ndir * nchunk * 32, 128), 128, 0, st>>>(
-        pr.T, ndir, nchunk, len, pr.vert, pr.cent, pr.area, coef, d_rhat, pr.k0, R, partial);
+    for (int64_t d = 0; d < ndir; d += batch) {
+      const int64_t n = std::min(batch, ndir - d);
+      k_farfield<Rio, decltype(nt)::value, decltype(ct)::value><<<nblk(n * nchunk * 32, 128), 128, 0, st>>>(
+          pr.T, n, nchunk, len, pr.vert, pr.cent, pr.area, coef, d_rhat + 3 * d, pr.k0, R, partial);
+      k_field_finish<<<nblk(n * 32, 128), 128, 0, st>>>(n, nchunk, partial, d_rhat + 3 * d, pr.w * kMu0 / (4.0 * kPi),
+                                                        static_cast<cd*>(E) + 3 * d);
+    }
   });
-  k_field_finish<<<nblk(ndir * 32, 128), 128, 0, st>>>(ndir, nchunk, partial, d_rhat, pr.w * kMu0 / (4.0 * kPi),
-                                                       static_cast<cd*>(E));
   return cuda_check(cudaGetLastError(), "farfield launch");
 }
 
@@ -2690,13 +2715,13 @@ pie_status apply_t_one(Problem& pr, const void* x, void* y, bool conj, cudaStrea
 // (F^H E)_m = sum_{t in m} c_t,m int_t (r - p_m) . h(r) dr, i.e. the Galerkin
 // testing of the potentials U = int (r - c_t).h, V = int h (T1 = T2 = 0).
 // One thread per triangle over a chunk of the directions (blockIdx.y; enough
-// chunks to give every SM warps), the conjugates of the far field's C and
+// chunks to give every SM kAdjWarps warps, of at least eight directions), the conjugates of the far field's C and
 // G_k per pair; kAdjTile directions at a time in shared memory, each as k rhat
 // and the vector -i pref (I - rr) E.  A launch of one chunk writes the
 // potentials, otherwise out holds the chunks' partial sums [chunk][8][T].
 // 181 directions on 32,768 triangles: 1.16 ms; 5.12 ms with a sincos per
 // quadrature point.
-constexpr int kAdjTile = 32;
+constexpr int kAdjTile = 32, kAdjWarps = 32;
 template <typename Rio, int NT, int CT>
 __global__ void __launch_bounds__(128) k_farfield_adj(int64_t T, int64_t ndir, int64_t len,
                                                       const double* __restrict__ vert,
@@ -2792,10 +2817,12 @@ __global__ void k_farfield_adj_finish(int64_t T, int64_t nchunk, const double* _
 template <typename Rio>
 static pie_status farfield_adjoint_t(Problem& pr, const double* rhat, int64_t ndir, const void* E, void* u,
                                      cudaStream_t st) {
-  int64_t nchunk, len;
-  field_chunks(pr, (pr.T + 31) / 32, ndir, 4, &nchunk, &len);
+  const int64_t warps = (pr.T + 31) / 32;
+  const int64_t most = std::min((int64_t(pr.nsm) * kAdjWarps + warps - 1) / warps, (ndir + 7) / 8);
+  const int64_t len = ((ndir + most - 1) / most + 3) / 4 * 4, nchunk = (ndir + len - 1) / len;
   pie_status s = PIE_OK;
-  FieldScratch scratch(pr, sizeof(double) * (3 * size_t(ndir) + (nchunk > 1 ? 8 * size_t(pr.T) * nchunk : 0)), st, s);
+  FieldScratch scratch(pr, sizeof(double) * (3 * size_t(ndir) + (nchunk > 1 ? 8 * size_t(pr.T) * nchunk : 0)), st, s,
+                       true);
   if (s != PIE_OK) return s;
   double* d_rhat = static_cast<double*>(scratch.p);
   double* partial = d_rhat + 3 * ndir;
@@ -2965,9 +2992,10 @@ __global__ void __launch_bounds__(128) k_nearzone(int64_t T, int64_t npts, int64
 pie_status nearzone(Problem& pr, const void* x, const void* rho, const double* pts, int64_t npts, void* E,
                     cudaStream_t st) {
   int64_t nchunk, len;
-  field_chunks(pr, npts, pr.T, 32, &nchunk, &len);
+  field_chunks(pr, &nchunk, &len);
+  const int64_t batch = field_batch(npts, nchunk);
   pie_status s = PIE_OK;
-  FieldScratch scratch(pr, sizeof(double) * size_t(npts) * (3 + 6 * size_t(nchunk)), st, s);
+  FieldScratch scratch(pr, sizeof(double) * (3 * size_t(npts) + 6 * size_t(nchunk * batch)), st, s);
   if (s != PIE_OK) return s;
   double* d_pts = static_cast<double*>(scratch.p);
   double* partial = d_pts + 3 * npts;
@@ -2977,11 +3005,14 @@ pie_status nearzone(Problem& pr, const void* x, const void* rho, const double* p
   const FieldRule Q = field_rule(pr);
   // the phases are k times the distances of the points from the centroids
   with_field_terms<false>(pr.k0 * pr.h_max, pr.k0 * (pr.r_max + longest(pts, npts)), [&](auto nt, auto ct) {
-    k_nearzone<decltype(nt)::value, decltype(ct)::value><<<nblk(npts * nchunk * 32, 128), 128, 0, st>>>(
-        pr.T, npts, nchunk, len, pr.vert, pr.cent, pr.area, pr.perm, coef, static_cast<const cd*>(rho), d_pts,
-        pr.k0, pr.w * kMu0, 1.0 / eps0(), Q, partial);
+    for (int64_t i = 0; i < npts; i += batch) {
+      const int64_t n = std::min(batch, npts - i);
+      k_nearzone<decltype(nt)::value, decltype(ct)::value><<<nblk(n * nchunk * 32, 128), 128, 0, st>>>(
+          pr.T, n, nchunk, len, pr.vert, pr.cent, pr.area, pr.perm, coef, static_cast<const cd*>(rho), d_pts + 3 * i,
+          pr.k0, pr.w * kMu0, 1.0 / eps0(), Q, partial);
+      k_field_finish<<<nblk(n * 32, 128), 128, 0, st>>>(n, nchunk, partial, nullptr, 0.0, static_cast<cd*>(E) + 3 * i);
+    }
   });
-  k_field_finish<<<nblk(npts * 32, 128), 128, 0, st>>>(npts, nchunk, partial, nullptr, 0.0, static_cast<cd*>(E));
   return cuda_check(cudaGetLastError(), "nearfield launch");
 }
 

@@ -1,7 +1,8 @@
 """Phases of the field maps at the limits of their series: bodies whose
 farthest centroid (and point) lies just inside the range of the short series for
-the centroid's phase, and directions that are not unit vectors (the maps are
-defined for any vector)."""
+the centroid's phase, directions that are not unit vectors (the maps are defined
+for any vector), and the order of the sums, which belongs to the body and not to
+the other directions or points of the call."""
 import numpy as np
 import pytest
 
@@ -80,3 +81,20 @@ def test_directions_of_any_length(length, kh):
     F = np.stack([far_field(top, k, e, d) for e in np.eye(pr.N)[:pr.E]])
     vo = np.concatenate([np.einsum("end,nd->e", F.conj(), g), np.zeros(pr.T)])
     assert np.linalg.norm(v - vo) <= tol * np.linalg.norm(vo)
+
+
+@pytest.mark.parametrize("n,most", [(4, 90001), (25, 3000), (60, 700)])
+def test_a_field_does_not_depend_on_its_neighbours(n, most):
+    """One direction or point gives the same bits alone and among many (more of
+    them than one launch's scratch holds in the first case)."""
+    import torch
+    _, pr, _ = _problem(0.3, offset=0.1, n=n)
+    rng = np.random.default_rng(2)
+    x = torch.from_numpy(pi.complex_normal(pr.N, 3)).cuda()
+    rho = torch.from_numpy(pi.complex_normal(pr.T, 6)).cuda()
+    d = rng.normal(size=(most, 3))
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    E, H = pr.farfield(x, d), pr.nearfield(x, rho, d)
+    for i, j in ((0, 1), (1, 182), (most - 1, most), (most // 2, most // 2 + 33)):
+        assert torch.equal(pr.farfield(x, d[i:j]), E[i:j]), (i, j)
+        assert torch.equal(pr.nearfield(x, rho, d[i:j]), H[i:j]), (i, j)
