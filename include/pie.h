@@ -63,8 +63,13 @@ typedef enum { PIE_C128 = 0, PIE_C64 = 1 } pie_dtype;
 /* Arithmetic of the product:
  *  PIE_FP64  everything in complex double (inputs/outputs PIE_C128); the near
  *            part multiplies 58-bit moments with 56-bit coefficients in fixed
- *            point, scaled per test triangle and per leaf box, with exact
- *            sums: an error no larger than that of FP64 multiply-adds;
+ *            point.  Real and imaginary parts are scaled apart, moments by the
+ *            largest of a test triangle's row and coefficients by the largest of
+ *            up to 384 sources near a leaf box; the rounding of a factor is
+ *            relative to those.  In the norm of either part of the result the error
+ *            is no larger than that of FP64 multiply-adds; a single entry far
+ *            below its neighbours has as many digits fewer of its own, and
+ *            pie_problem_stage returns the moments so rounded;
  *  PIE_FP32  near and far parts in complex float (inputs/outputs PIE_C64);
  *  PIE_MIXED near part in complex float (pair moments stored as float),
  *            far part in complex double (inputs/outputs PIE_C128);

@@ -387,7 +387,7 @@ pie_status pie_problem_stage(pie_problem* h, int which, int level, double* out, 
     f32 = pr.near_f32();
     if (!f32) {  // fixed point times the row's exponents (near_fixed.cuh)
       const size_t nnz = size_t(pr.nnz);
-      std::vector<int32_t> m(4 * n), row(2 * size_t(pr.T)), delta(size_t(pr.nleaf)), leaf(size_t(pr.T));
+      std::vector<int32_t> m(4 * n), row(4 * size_t(pr.T)), delta(size_t(pr.nleaf)), leaf(size_t(pr.T));
       std::vector<int64_t> ptr(size_t(pr.T) + 1);
       auto get = [&](auto& h, const void* d) {
         if (s == PIE_OK) s = cuda_check(cudaMemcpy(h.data(), d, h.size() * sizeof(h[0]), cudaMemcpyDeviceToHost), "stage copy");
@@ -401,12 +401,14 @@ pie_status pie_problem_stage(pie_problem* h, int which, int level, double* out, 
       for (size_t t = 0; t < size_t(pr.T); ++t)
         for (size_t q = 0; q < kMom; ++q) {
           const bool test = (q >= 1 && q <= 3) || q == 7;
-          const int x = row[2 * t + test] + (q >= 4 ? delta[leaf[t]] : 0);
-          for (size_t i = q * nnz + ptr[t]; i < q * nnz + ptr[t + 1]; ++i)
-            for (int c = 0; c < 2; ++c)
-              out[2 * i + c] = row[2 * t] == kFixedNan
-                                   ? std::nan("")
-                                   : std::ldexp(double(m[4 * i + 2 * c]) * (1 << kLimb) + m[4 * i + 2 * c + 1], x);
+          for (int c = 0; c < 2; ++c) {  // real, imaginary part
+            const int x = row[4 * t + 2 * test + c] + (q >= 4 ? delta[leaf[t]] : 0);
+            for (size_t e = ptr[t]; e < size_t(ptr[t + 1]); ++e) {
+              const int32_t* l = &m[4 * ((c * kFixedPlanes + q / 2) * nnz + e) + 2 * (q % 2)];
+              out[2 * (q * nnz + e) + c] =
+                  row[4 * t] == kFixedNan ? std::nan("") : std::ldexp(double(l[0]) * (1 << kLimb) + l[1], x);
+            }
+          }
         }
       return PIE_OK;
     }

@@ -550,25 +550,26 @@ static pie_status near_float_prepare() {
 // stride over the pairs: the box's source coefficients are staged as
 // integers kFixedStage at a time, then its warps take the test triangles in
 // turn, lanes over the row.  nsplit shares a box among several blocks when the
-// leaf boxes alone do not fill the SMs.  81,920 triangles: 0.63 ms alone (2.2 ms
-// with FP64 multiply-adds), 24,576 of a cube: 0.66 ms (1.78); beside the far part
+// leaf boxes alone do not fill the SMs.  81,920 triangles: 0.72 ms alone (2.2 ms
+// with FP64 multiply-adds; 0.65 with one exponent for both parts of a moment, in
+// one pass over the row), 24,576 of a cube: 0.69 ms (1.78); beside the far part
 // one block an SM does, since the two use different pipes: the product of 81,920
-// triangles 2.67 ms (3.27 when this came in, 5.11 before).
+// triangles 2.7 to 2.9 ms (5.1 with FP64 multiply-adds).
 
 // A warp-wide 64-bit multiply-add issues every two clocks and takes four, so the
 // limb products are taken kind by kind over all sums (KIND 0: h h', 1: h l',
-// 2: l h'; HALF 0: real, 1: imaginary part of c) and not sum by sum.
+// 2: l h') and not sum by sum.  s[2 i], s[2 i + 1]: real and imaginary part of c
+// times one part of the moment.
 struct FixedSum {
   int64_t hh, x;
 };
-template <int KIND, int HALF>
-__device__ __forceinline__ void fixed_cfma(FixedSum (&s)[12], int i, const int4& c, const int4& m) {
-  const int cc = HALF ? (KIND == 2 ? c.w : c.z) : (KIND == 2 ? c.y : c.x);
-  const int mx = KIND == 1 ? m.y : m.x, my = KIND == 1 ? m.w : m.z;
+template <int KIND>
+__device__ __forceinline__ void fixed_cfma(FixedSum (&s)[12], int i, const int4& c, const int2& m) {
+  const int mx = KIND == 1 ? m.y : m.x;
   int64_t& re = KIND == 0 ? s[2 * i].hh : s[2 * i].x;
   int64_t& im = KIND == 0 ? s[2 * i + 1].hh : s[2 * i + 1].x;
-  re += HALF ? int64_t(-cc) * my : int64_t(cc) * mx;
-  im += int64_t(cc) * (HALF ? mx : my);
+  re += int64_t(KIND == 2 ? c.y : c.x) * mx;
+  im += int64_t(KIND == 2 ? c.w : c.z) * mx;
 }
 
 // The twelve products of one pair; m: m0, mt(3), ms(3), mts; c: a, beta(3), sigma, d.
@@ -612,23 +613,28 @@ __device__ __noinline__ double near_row_double(const FixedNear& nf, int64_t nnz,
   return out;
 }
 
-// Shared memory: the stage's coefficients [6][kFixedStage], then two buffers of
-// 32 entries' moments [2][8][32] per warp.
-constexpr int kFixedWarps = 4;  // (8 warps with 128 registers each: 15 % slower)
-constexpr size_t kFixedSmem = sizeof(int4) * (6 * kFixedStage + kFixedWarps * 2 * kMom * 32);
+// Shared memory: the stage's coefficients [6][kFixedStage], then kFixedSlots
+// buffers of 32 entries' moments of one part [4][32] per warp.  (Three slots, 61 KB
+// a block, let blocks pile up on some SMs beside the far part: products of 81,920
+// triangles in a row 3.57 ms, 2.69 with four.)
+constexpr int kFixedWarps = 4, kFixedSlots = 4;
+constexpr size_t kFixedSmem = sizeof(int4) * (6 * kFixedStage + kFixedWarps * kFixedSlots * kFixedPlanes * 32);
 
-__global__ void __launch_bounds__(32 * kFixedWarps, 3)
+// BLOCKS: blocks of an SM that the registers allow (3: 158 registers, alone; 4: 128,
+// which leaves room for the far part's kernels beside it).
+template <int BLOCKS>
+__global__ void __launch_bounds__(32 * kFixedWarps, BLOCKS)
     k_near_fixed(int64_t nleaf, int nsplit, int64_t nnz, const int32_t* __restrict__ leaf_start,
                  const int32_t* __restrict__ near_ptr, const int32_t* __restrict__ near_idx,
                  const int32_t* __restrict__ near_off, const int64_t* __restrict__ row_ptr, const FixedNear nf,
                  const cd* __restrict__ coef, double mu0, cd* __restrict__ pot, int64_t sc = 0, int64_t sp = 0) {
   extern __shared__ __align__(16) unsigned char fixed_smem[];
   int4(*cs)[kFixedStage] = reinterpret_cast<int4(*)[kFixedStage]>(fixed_smem);
-  __shared__ int fields[kFixedWarps][4];  // [warp][group]
+  __shared__ int fields[kFixedWarps][8];  // [warp][part of a, beta, sigma, d]
   coef += blockIdx.y * sc;
   double* out = reinterpret_cast<double*>(pot + blockIdx.y * sp);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int4(*ms)[kMom][32] = reinterpret_cast<int4(*)[kMom][32]>(cs + 6) + 2 * warp;
+  int4(*ms)[kFixedPlanes][32] = reinterpret_cast<int4(*)[kFixedPlanes][32]>(cs + 6) + kFixedSlots * warp;
   for (int64_t bi = blockIdx.x; bi < nleaf * nsplit; bi += gridDim.x) {
     const int64_t b = bi / nsplit;
     const int q0 = near_ptr[b], q1 = near_ptr[b + 1];
@@ -637,8 +643,8 @@ __global__ void __launch_bounds__(32 * kFixedWarps, 3)
     const int dl = nf.delta[b];
     for (int j0 = 0; j0 < len; j0 += kFixedStage) {
       const int j1 = min(len, j0 + kFixedStage);
-      // largest exponent fields of the stage's a, beta, sigma, d
-      int x[4] = {1, 1, 1, 1};
+      // largest exponent fields of the stage's a, beta, sigma, d: real and imaginary parts
+      int x[8] = {1, 1, 1, 1, 1, 1, 1, 1};
       int qi = q0;
       for (int j = j0 + int(threadIdx.x); j < j1; j += blockDim.x) {
         while (qi + 1 < q1 && near_off[qi + 1] <= j) ++qi;
@@ -646,25 +652,34 @@ __global__ void __launch_bounds__(32 * kFixedWarps, 3)
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
           const cd v = c[k];
-          int& r = x[k == 0 ? 0 : k < 4 ? 1 : k - 2];
-          r = max(r, max(exponent_field(v.x), exponent_field(v.y)));
+          const int g = 2 * (k == 0 ? 0 : k < 4 ? 1 : k - 2);
+          x[g] = max(x[g], exponent_field(v.x));
+          x[g + 1] = max(x[g + 1], exponent_field(v.y));
         }
       }
 #pragma unroll
-      for (int i = 0; i < 4; ++i) x[i] = __reduce_max_sync(0xffffffffu, x[i]);
+      for (int i = 0; i < 8; ++i) x[i] = __reduce_max_sync(0xffffffffu, x[i]);
       __syncthreads();  // the previous stage's readers are done
-      if (lane < 4) fields[warp][lane] = lane == 0 ? x[0] : lane == 1 ? x[1] : lane == 2 ? x[2] : x[3];
-      __syncthreads();
+      if (lane == 0)
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 8; ++i) fields[warp][i] = x[i];
+      __syncthreads();
+      int top = 0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
 #pragma unroll
         for (int w = 0; w < kFixedWarps; ++w) x[i] = max(x[i], fields[w][i]);
-      const bool finite = max(max(x[0], x[1]), max(x[2], x[3])) < 0x7ff;
+        top = max(top, x[i]);
+      }
+      const bool finite = top < 0x7ff;
       // beta's field covers a and delta; a takes beta's less delta
-      x[1] = max(x[1], x[0] + dl);
-      x[0] = x[1] - dl;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) x[i] += 53 - kCoefBits;
+      for (int p = 0; p < 2; ++p) {
+        x[2 + p] = max(x[2 + p], x[p] + dl);
+        x[p] = x[2 + p] - dl;
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] += 53 - kCoefBits;
       qi = q0;
       for (int j = j0 + int(threadIdx.x); j < j1 && finite; j += blockDim.x) {
         while (qi + 1 < q1 && near_off[qi + 1] <= j) ++qi;
@@ -672,75 +687,103 @@ __global__ void __launch_bounds__(32 * kFixedWarps, 3)
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
           const cd v = c[k];
-          const int f = x[k == 0 ? 0 : k < 4 ? 1 : k - 2];
-          const int2 r = fixed_encode(v.x, f), i = fixed_encode(v.y, f);
+          const int g = 2 * (k == 0 ? 0 : k < 4 ? 1 : k - 2);
+          const int2 r = fixed_encode(v.x, x[g]), i = fixed_encode(v.y, x[g + 1]);
           cs[k][j - j0] = make_int4(r.x, r.y, i.x, i.y);
         }
       }
       __syncthreads();
-      // the warp's (test triangle, 32 entries) steps in one sequence: each step's
-      // moments are on their way while the step before is multiplied, across rows
-      // too (rows of a box have one length, one after the other)
+      // the warp's (test triangle, part, 32 entries) steps in one sequence: the next
+      // steps' moments are on their way while a step is multiplied, across rows
+      // too (rows of a box have one length, one after the other); a lane copies
+      // and reads its own entry
       const int64_t base = row_ptr[leaf_start[b]];
       const int per_row = (j1 - j0 + 31) / 32;
-      auto fetch = [&](int t, int i, int slot) {
-        const int j = j0 + 32 * i + lane;
-        if (t < t1 && j < j1 && finite) {
-          const int4* src = nf.mom + base + int64_t(t - leaf_start[b]) * len + j;
+      int ft = t0, fp = 0, fj = lane, fslot = 0;
+      const int count = j1 - j0;
+      // the part's first entry of the row, and how far the next row's lies from there
+      const int4* src = nf.mom + base + int64_t(t0 - leaf_start[b]) * len + j0;
+      const int64_t next_row = int64_t(kFixedWarps * nsplit) * len - kFixedPlanes * nnz;
+      auto fetch = [&] {
+        if (fj < count && ft < t1 && finite) {
+          const int4* from = src + fj;
 #pragma unroll
-          for (int q = 0; q < kMom; ++q) cp_async(&ms[slot][q][lane], src + q * nnz);
+          for (int g = 0; g < kFixedPlanes; ++g, from += nnz) cp_async(&ms[fslot][g][lane], from);
         }
         cp_async_commit();
+        fslot = fslot + 1 == kFixedSlots ? 0 : fslot + 1;
+        fj += 32;
+        if (fj - lane >= count) {
+          fj = lane;
+          src += fp ? next_row : kFixedPlanes * nnz;
+          ft += fp ? kFixedWarps * nsplit : 0;
+          fp ^= 1;
+        }
       };
+      // exponent of the coefficients in the lane's sum
+      const int ec = (lane & 1 ? (lane < 8 ? x[3] : lane < 10 ? x[5] : x[7])
+                               : (lane < 8 ? x[2] : lane < 10 ? x[4] : x[6])) - 1075;
+      // one part of row t: lane i < 12 gets the value of sum i
       int slot = 0;
-      fetch(t0, 0, 0);
+      auto part_sum = [&](int t, int part) {
+        FixedSum sum[12];
+#pragma unroll
+        for (int i = 0; i < 12; ++i) sum[i] = FixedSum{0, 0};
+        for (int i = 0; i < per_row; ++i) {
+          fetch();
+          cp_async_wait<kFixedSlots - 1>();
+          const int j = 32 * i + lane;
+          if (j0 + j < j1) {
+            int2 m[kMom];
+            int4 c[6];
+#pragma unroll
+            for (int g = 0; g < kFixedPlanes; ++g) {
+              const int4 v = ms[slot][g][lane];
+              m[2 * g] = make_int2(v.x, v.y);
+              m[2 * g + 1] = make_int2(v.z, v.w);
+            }
+#pragma unroll
+            for (int k = 0; k < 6; ++k) c[k] = cs[k][j];
+            near_products([&](int k, const int4& a, const int2& b) { fixed_cfma<0>(sum, k, a, b); }, c, m);
+            near_products([&](int k, const int4& a, const int2& b) { fixed_cfma<1>(sum, k, a, b); }, c, m);
+            near_products([&](int k, const int4& a, const int2& b) { fixed_cfma<2>(sum, k, a, b); }, c, m);
+          }
+          slot = slot + 1 == kFixedSlots ? 0 : slot + 1;
+        }
+        // value = hh 2^56 + x 2^28: x carried into hh but for 28 bits below it, and
+        // the warp's totals in pieces of 27 bits
+        int p0 = 0, p1 = 0, p2 = 0, p3 = 0;
+#pragma unroll
+        for (int i = 0; i < 12; ++i) {
+          const int64_t h = sum[i].hh + (sum[i].x >> kLimb);
+          const int r0 = int(__reduce_add_sync(0xffffffffu, (uint32_t(sum[i].x) & ((1u << kLimb) - 1)) >> 1));
+          const int r1 = int(__reduce_add_sync(0xffffffffu, uint32_t(h) & ((1u << 27) - 1)));
+          const int r2 = int(__reduce_add_sync(0xffffffffu, uint32_t(h >> 27) & ((1u << 27) - 1)));
+          const int r3 = __reduce_add_sync(0xffffffffu, int(h >> 54));
+          if (lane == i) p0 = r0, p1 = r1, p2 = r2, p3 = r3;
+        }
+        // 96 bits: the totals above the point less five bits, then 5 + 27 bits
+        const uint64_t mid = (uint64_t(uint32_t(p2)) << 27) + uint32_t(p1);
+        const uint64_t low = uint64_t(uint32_t(p0)) + ((mid & 31) << 27);
+        const int64_t hi = int64_t(p3) * (int64_t(1) << 49) + int64_t(mid >> 5) + int64_t(low >> 32);
+        const FixedRow row = nf.row[t];
+        if (row.m0[0] == kFixedNan) return nan("");
+        const int em = lane < 2 ? (part ? row.mt[1] : row.mt[0]) : part ? row.m0[1] : row.m0[0];
+        return fixed_scale(hi, uint32_t(low), em + ec + 2 * kLimb - 27);
+      };
+#pragma unroll
+      for (int d = 0; d < kFixedSlots - 1; ++d) fetch();
       for (int t = t0; t < t1; t += kFixedWarps * nsplit) {
         const int64_t e0 = base + int64_t(t - leaf_start[b]) * len;
         double v;
         if (finite) {
-          FixedSum sum[12];
-#pragma unroll
-          for (int i = 0; i < 12; ++i) sum[i] = FixedSum{0, 0};
-          for (int i = 0; i < per_row; ++i) {
-            const bool last = i + 1 == per_row;
-            fetch(last ? t + kFixedWarps * nsplit : t, last ? 0 : i + 1, slot ^ 1);
-            cp_async_wait<1>();
-            const int j = 32 * i + lane;
-            if (j0 + j < j1) {
-              int4 m[kMom], c[6];
-#pragma unroll
-              for (int q = 0; q < kMom; ++q) m[q] = ms[slot][q][lane];
-#pragma unroll
-              for (int k = 0; k < 6; ++k) c[k] = cs[k][j];
-              near_products([&](int k, const int4& a, const int4& b) { fixed_cfma<0, 0>(sum, k, a, b); }, c, m);
-              near_products([&](int k, const int4& a, const int4& b) { fixed_cfma<1, 0>(sum, k, a, b); }, c, m);
-              near_products([&](int k, const int4& a, const int4& b) { fixed_cfma<2, 0>(sum, k, a, b); }, c, m);
-              near_products([&](int k, const int4& a, const int4& b) { fixed_cfma<0, 1>(sum, k, a, b); }, c, m);
-              near_products([&](int k, const int4& a, const int4& b) { fixed_cfma<1, 1>(sum, k, a, b); }, c, m);
-              near_products([&](int k, const int4& a, const int4& b) { fixed_cfma<2, 1>(sum, k, a, b); }, c, m);
-            }
-            slot ^= 1;
+          // (re c + i im c) (re m + i im m): the imaginary moments' sums change places
+          v = 0;
+#pragma unroll 1
+          for (int part = 0; part < 2; ++part) {
+            const double w = part_sum(t, part), u = __shfl_xor_sync(0xffffffffu, w, 1);
+            v = part ? v + (lane & 1 ? u : -u) : w;
           }
-          // value = hh 2^56 + x 2^28: x carried into hh but for 28 bits below it, and
-          // the warp's totals in pieces of 27 bits
-          int p0 = 0, p1 = 0, p2 = 0, p3 = 0;
-#pragma unroll
-          for (int i = 0; i < 12; ++i) {
-            const int64_t h = sum[i].hh + (sum[i].x >> kLimb);
-            const int r0 = int(__reduce_add_sync(0xffffffffu, (uint32_t(sum[i].x) & ((1u << kLimb) - 1)) >> 1));
-            const int r1 = int(__reduce_add_sync(0xffffffffu, uint32_t(h) & ((1u << 27) - 1)));
-            const int r2 = int(__reduce_add_sync(0xffffffffu, uint32_t(h >> 27) & ((1u << 27) - 1)));
-            const int r3 = __reduce_add_sync(0xffffffffu, int(h >> 54));
-            if (lane == i) p0 = r0, p1 = r1, p2 = r2, p3 = r3;
-          }
-          // 96 bits: the totals above the point less five bits, then 5 + 27 bits
-          const uint64_t mid = (uint64_t(uint32_t(p2)) << 27) + uint32_t(p1);
-          const uint64_t low = uint64_t(uint32_t(p0)) + ((mid & 31) << 27);
-          const int64_t hi = int64_t(p3) * (int64_t(1) << 49) + int64_t(mid >> 5) + int64_t(low >> 32);
-          const FixedRow row = nf.row[t];
-          const int e = (lane < 2 ? row.mt : row.m0) + (lane < 8 ? x[1] : lane < 10 ? x[2] : x[3]) - 1075;
-          v = fixed_scale(hi, uint32_t(low), e + 2 * kLimb - 27);
-          if (row.m0 == kFixedNan) v = nan("");
         } else {
           v = near_row_double(nf, nnz, t, int(b), e0, j0, j1, q0, q1, leaf_start, near_idx, near_off, coef);
         }
@@ -758,7 +801,8 @@ static pie_status near_fixed_prepare() {
   static std::atomic<uint64_t> done{0};
   int bit = -1;
   if (device_done(done, &bit)) return PIE_OK;
-  pie_status s = raise_smem(k_near_fixed, kFixedSmem);
+  pie_status s = raise_smem(k_near_fixed<3>, kFixedSmem);
+  if (s == PIE_OK) s = raise_smem(k_near_fixed<4>, kFixedSmem);
   if (s == PIE_OK && bit >= 0) done.fetch_or(uint64_t(1) << bit);
   return s;
 }
@@ -777,18 +821,25 @@ pie_status near_prepare(const Problem& pr) {
 static void near_fixed(const Problem& pr, const cd* coef, cd* pot, int nrhs, int64_t max_blocks, cudaStream_t st) {
   const FixedNear nf{static_cast<const int4*>(pr.mom), static_cast<const FixedRow*>(pr.fixed_row), pr.fixed_delta};
   // shares per box: the least rounds of three blocks an SM, staging (about 1/50
-  // of a box's rows) once a share; at least a test triangle for each warp
+  // of a box's rows) once a share; at least a test triangle for each warp.  Boxes
+  // are uneven, so up to 8 % more by this count for finer shares, while a warp has
+  // three rows (alone: cube of 24,576 triangles 799 -> 695 us, ellipsoid of 32,768
+  // 2870 -> 1400; finer still: spheres lose 10 %)
   const int64_t slots = 3 * int64_t(pr.nsm),
                 most = std::min<int64_t>(16, (pr.T / pr.nleaf + kFixedWarps - 1) / kFixedWarps);
   int nsplit = 1;
-  double best = 0;
+  double best = 0, costs[17];
   for (int64_t s = 1; s <= most; ++s) {
     const double cost = double((pr.nleaf * s + slots - 1) / slots) * (1.0 / double(s) + 0.02);
     if (s == 1 || cost < best) best = cost, nsplit = int(s);
+    costs[s] = cost;
   }
+  for (int64_t s = nsplit + 1; s <= most && 3 * kFixedWarps * s <= pr.T / pr.nleaf; ++s)
+    if (costs[s] <= 1.08 * best) nsplit = int(s);
   int64_t grid = pr.nleaf * nsplit;
   if (max_blocks > 0) grid = std::min(grid, max_blocks);
-  k_near_fixed<<<dim3(unsigned(grid), unsigned(nrhs)), 32 * kFixedWarps, kFixedSmem, st>>>(
+  auto kernel = max_blocks > 0 ? k_near_fixed<4> : k_near_fixed<3>;
+  kernel<<<dim3(unsigned(grid), unsigned(nrhs)), 32 * kFixedWarps, kFixedSmem, st>>>(
       pr.nleaf, nsplit, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr, nf, coef, kMu0, pot,
       6 * pr.T, 6 * pr.T);
 }
@@ -1898,7 +1949,7 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
     // beside the far part: one block an SM where it ends with the far part, else
     // two (three leave the filter kernels no shared memory until they are done:
     // the 100 MHz plate 377 us beside 100 KB an SM, 440 beside 209).  One block takes
-    // 89 ps a pair (81,920 triangles: 1.95 ms), the far part 1.6 ps a double
+    // 89 ps a pair (81,920 triangles: 1.9 ms), the far part 1.6 ps a double
     // operation: 20 a list entry and sample, 32 a triangle and sample for
     // aggregation and disaggregation, about 9000 a box and component for the filters
     double far_ops = 32.0 * double(pr.T) * P;

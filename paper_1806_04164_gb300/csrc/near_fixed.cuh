@@ -12,10 +12,19 @@
 // A pair's moments are stored as integers of up to 58 bits times a power of two
 // that the test row shares (set-up), the sources' coefficients become 56-bit
 // integers times powers of two shared by a leaf box's sources when they are
-// staged.  Sums are exact: the error is that of the two roundings, 2^-59 and
-// 2^-57 of the largest factors, where FP64 rounds every product and partial sum
-// (24,576 triangles, against 64-bit sums: 1.4e-15 of the product, 1.6e-15 with
-// FP64 multiply-adds).
+// staged.  Real and imaginary parts have powers of their own, in moments and
+// coefficients alike: at low frequency the imaginary (radiated) part of a moment
+// is k h / 4 of the real one and less, and where the coefficients are real it
+// alone makes the imaginary part of the product.  So a row is summed twice, real
+// moments and then imaginary ones, and every sum takes products of one part with
+// one part.
+//
+// Error: the sums are exact but for l l' and the last bit of x, so what remains is the
+// rounding of the factors, to 2^-59 of the row's largest moment and 2^-57 of the
+// stage's largest coefficient of their part (FP64 rounds every product and partial
+// sum, to 2^-53 of itself).  In the norm of either part that is no more than
+// FP64's; an entry far below its neighbours in the row or stage
+// keeps as many digits fewer, as it adds as much less to their sum.
 #pragma once
 #include <cstdint>
 
@@ -24,26 +33,30 @@
 namespace pie {
 
 // Limbs: -2^27 <= l < 2^27, |h| <= 2^30 (moments) or 2^28 (coefficients).  A lane sums
-// at most kFixedStage / 32 = 12 entries, 8 real products each, before the sums
+// at most kFixedStage / 32 = 12 entries, 4 real products each, before the sums
 // are taken out.  The row's exponents keep the sum of the moments' integers over
 // those below 2^61 (2^33 in h), so |sum h h'| < 2^61 and |sum h l' + l h'| <
-// 2^28 96 2^27 + 2^27 2^33 < 2^62.
+// 2^28 48 2^27 + 2^27 2^33 < 2^62.
 constexpr int kLimb = 28;
 constexpr int kFixedStage = 384;
 constexpr int kMomentBits = 58, kCoefBits = 56, kLaneBits = 61;
 
-// Exponents of one test row: a moment is its integer times 2^e, with e = m0 for
-// m0, m0 + delta for ms, mt for mt and mt + delta for mts, delta the leaf box's
-// (about log2 of its edges, FixedNear::delta).  One delta for both pairs of groups lets
-// the products a mts and beta mt, a ms and beta m0 share a sum (a takes the
-// exponent of beta less delta).
-struct FixedRow {
-  int32_t m0, mt;
+// Exponents of one test row, [0] of the real and [1] of the imaginary parts: a
+// moment is its integer times 2^e, with e = m0 for m0, m0 + delta for ms, mt for mt
+// and mt + delta for mts, delta the leaf box's (about log2 of its edges,
+// FixedNear::delta).  One delta for both pairs of groups lets the products a mts and
+// beta mt, a ms and beta m0 share a sum (a takes the exponent of beta less delta).
+struct alignas(16) FixedRow {
+  int32_t m0[2], mt[2];
 };
 constexpr int32_t kFixedNan = 1 << 20;  // exponent of a row with a moment that is not finite
 
+// Moments: planes of int4, [part][4][nnz]: plane g holds moments 2 g and 2 g + 1 of
+// m0, mt(3), ms(3), mts as (h, l, h, l).
+constexpr int kFixedPlanes = 4;
+
 struct FixedNear {
-  const int4* mom;       // [8][nnz] (re h, re l, im h, im l)
+  const int4* mom;       // [2][kFixedPlanes][nnz]
   const FixedRow* row;   // [T]
   const int32_t* delta;  // [nleaf]
 };
@@ -63,9 +76,9 @@ __device__ __forceinline__ int2 fixed_encode(double v, int f) {
 
 __device__ __forceinline__ double fixed_value(int h, int l) { return fma(double(h), double(1 << kLimb), double(l)); }
 
-// (hi 2^32 + lo) 2^e, rounded once (the conversions are four operations on the FP64
-// pipe, which the far part needs; scalbn only where the result leaves the
-// normal range).
+// (hi 2^32 + lo) 2^e to about an ulp: hi is rounded where it has more than 53 bits,
+// then the sum (the conversions are four operations on the FP64 pipe, which the
+// far part needs; scalbn only where the result leaves the normal range).
 __device__ __forceinline__ double fixed_scale(int64_t hi, uint32_t lo, int e) {
   const double v = fma(double(hi), 4294967296.0, double(lo));
   const int f = exponent_field(v);
@@ -75,12 +88,17 @@ __device__ __forceinline__ double fixed_scale(int64_t hi, uint32_t lo, int e) {
 
 // Moment q of entry e in row t of leaf box b, as a double.
 __device__ __forceinline__ cd fixed_moment(const FixedNear& f, int64_t nnz, int q, int64_t e, int64_t t, int b) {
-  const int4 m = f.mom[q * nnz + e];
   const FixedRow r = f.row[t];
+  if (r.m0[0] == kFixedNan) return mk<double>(nan(""), nan(""));
   const bool test = (q >= 1 && q <= 3) || q == 7, source = q >= 4;
-  const int x = (test ? r.mt : r.m0) + (source ? f.delta[b] : 0);
-  if (r.m0 == kFixedNan) return mk<double>(nan(""), nan(""));
-  return mk<double>(scalbn(fixed_value(m.x, m.y), x), scalbn(fixed_value(m.z, m.w), x));
+  double v[2];
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    const int4 m = f.mom[(p * kFixedPlanes + q / 2) * nnz + e];
+    v[p] = scalbn(q % 2 ? fixed_value(m.z, m.w) : fixed_value(m.x, m.y),
+                  (test ? r.mt[p] : r.m0[p]) + (source ? f.delta[b] : 0));
+  }
+  return mk<double>(v[0], v[1]);
 }
 
 }  // namespace pie

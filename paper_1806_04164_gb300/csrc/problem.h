@@ -83,7 +83,7 @@ struct Problem {
   double* rule64 = nullptr;      // [64][4] collapsed Gauss 8 x 8
 
   // operator tables
-  void* mom = nullptr;           // [8][nnz] complex (near precision; PIE_FP64: fixed point, near_fixed.cuh)
+  void* mom = nullptr;           // [8][nnz] complex (near precision; PIE_FP64: fixed point, FixedNear::mom)
   void* fixed_row = nullptr;     // PIE_FP64: [T] FixedRow, exponents of the fixed-point moments
   int32_t* fixed_delta = nullptr;  // PIE_FP64: [nleaf]
   void* Pi = nullptr;            // [T][P/2]

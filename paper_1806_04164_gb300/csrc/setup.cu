@@ -511,7 +511,8 @@ __global__ void k_fixed_delta(int64_t nleaf, NearGeom g, int32_t* __restrict__ d
   if ((threadIdx.x & 31) == 0) delta[b] = (e >> 1) + 1;
 }
 
-// The FP64 pair moments into fixed point, in place (near_fixed.cuh): a warp per
+// The FP64 pair moments into fixed point, in place (near_fixed.cuh: the eight
+// 16-byte moments of an entry become its eight planes' entries): a warp per
 // row, one pass for the row's exponents and one to convert.
 __global__ void __launch_bounds__(128) k_moments_fixed(int64_t T, int64_t nnz, NearGeom g,
                                                        const int32_t* __restrict__ delta, FixedRow* __restrict__ row,
@@ -520,47 +521,71 @@ __global__ void __launch_bounds__(128) k_moments_fixed(int64_t T, int64_t nnz, N
   if (t >= T) return;
   const int lane = threadIdx.x & 31, dl = delta[g.leaf_of[t]];
   const int64_t e0 = g.row_ptr[t], e1 = g.row_ptr[t + 1];
-  int x[4] = {1, 1, 1, 1};  // largest exponent fields of m0, mt, ms, mts
-  // largest sums over one lane's entries of a product stage, as they meet in a
-  // sum of the product: m0 with one ms, mt's three with mts
-  double a0 = 0, at = 0, s0 = 0, st = 0;
+  // per part: largest exponent fields of m0, mt, ms, mts, and the largest sums
+  // over one lane's entries of a product stage, as they meet in a sum of the
+  // product: m0 with one ms, mt's three with mts
+  int x[2][4] = {{1, 1, 1, 1}, {1, 1, 1, 1}};
+  double a0[2] = {0, 0}, at[2] = {0, 0}, s0[2] = {0, 0}, st[2] = {0, 0};
   const double dw = scalbn(1.0, -dl);
   for (int64_t e = e0 + lane; e < e1; e += 32) {
-    if (((e - e0) % kFixedStage) < 32) s0 = st = 0;
-    double v[kMom];
+    cd m[kMom];
 #pragma unroll
-    for (int q = 0; q < kMom; ++q) {
-      const cd m = mom[q * nnz + e];
-      int& r = x[(q + 2) / 3];
-      r = max(r, max(exponent_field(m.x), exponent_field(m.y)));
-      v[q] = fabs(m.x) + fabs(m.y);
+    for (int q = 0; q < kMom; ++q) m[q] = mom[q * nnz + e];
+    const bool first = ((e - e0) % kFixedStage) < 32;
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      double v[kMom];
+#pragma unroll
+      for (int q = 0; q < kMom; ++q) {
+        v[q] = fabs(p ? m[q].y : m[q].x);
+        int& r = x[p][(q + 2) / 3];
+        r = max(r, exponent_field(v[q]));
+      }
+      s0[p] = (first ? 0.0 : s0[p]) + (v[0] + dw * fmax(v[4], fmax(v[5], v[6])));
+      st[p] = (first ? 0.0 : st[p]) + (v[1] + v[2] + v[3] + dw * v[7]);
+      a0[p] = fmax(a0[p], s0[p]);
+      at[p] = fmax(at[p], st[p]);
     }
-    s0 += v[0] + dw * fmax(v[4], fmax(v[5], v[6]));
-    st += v[1] + v[2] + v[3] + dw * v[7];
-    a0 = fmax(a0, s0);
-    at = fmax(at, st);
   }
   int top = 0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    x[i] = __reduce_max_sync(0xffffffffu, x[i]);
-    top = max(top, x[i]);
-  }
+  for (int p = 0; p < 2; ++p)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      x[p][i] = __reduce_max_sync(0xffffffffu, x[p][i]);
+      top = max(top, x[p][i]);
+    }
   // exponent fields: the largest integer below 2^kMomentBits, the sums below 2^kLaneBits
   auto field = [&](int xa, int xb, double sum) {
     const int lane_e = __reduce_max_sync(0xffffffffu, sum > 0 ? exponent_field(sum) + 53 - kLaneBits : -100000);
     return max(max(xa, xb - dl) + 53 - kMomentBits, lane_e);
   };
-  const int f0 = field(x[0], x[2], a0), ft = field(x[1], x[3], at);
-  if (lane == 0) row[t] = top == 0x7ff ? FixedRow{kFixedNan, kFixedNan} : FixedRow{f0 - 1075, ft - 1075};
-  for (int64_t e = e0 + lane; e < e1; e += 32)
+  int f0[2], ft[2];
 #pragma unroll
-    for (int q = 0; q < kMom; ++q) {
-      const cd m = mom[q * nnz + e];
-      const int f = ((q >= 1 && q <= 3) || q == 7 ? ft : f0) + (q >= 4 ? dl : 0);
-      const int2 r = fixed_encode(m.x, f), i = fixed_encode(m.y, f);
-      reinterpret_cast<int4*>(mom)[q * nnz + e] = make_int4(r.x, r.y, i.x, i.y);
-    }
+  for (int p = 0; p < 2; ++p) {
+    f0[p] = field(x[p][0], x[p][2], a0[p]);
+    ft[p] = field(x[p][1], x[p][3], at[p]);
+  }
+  if (lane == 0)
+    row[t] = top == 0x7ff ? FixedRow{{kFixedNan, kFixedNan}, {kFixedNan, kFixedNan}}
+                          : FixedRow{{f0[0] - 1075, f0[1] - 1075}, {ft[0] - 1075, ft[1] - 1075}};
+  for (int64_t e = e0 + lane; e < e1; e += 32) {
+    cd m[kMom];
+#pragma unroll
+    for (int q = 0; q < kMom; ++q) m[q] = mom[q * nnz + e];
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+      for (int g = 0; g < kFixedPlanes; ++g) {
+        int2 r[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int q = 2 * g + u;
+          r[u] = fixed_encode(p ? m[q].y : m[q].x, ((q >= 1 && q <= 3) || q == 7 ? ft[p] : f0[p]) + (q >= 4 ? dl : 0));
+        }
+        reinterpret_cast<int4*>(mom)[(p * kFixedPlanes + g) * nnz + e] = make_int4(r[0].x, r[0].y, r[1].x, r[1].y);
+      }
+  }
 }
 
 // Leaf radiation tables at kappa_L: Pi_t(p) = int_t exp(-i kappa khat_p.(r - C_b)),
