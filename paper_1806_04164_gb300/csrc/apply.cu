@@ -241,29 +241,44 @@ __device__ __forceinline__ void load_coefs(const cf* src, cf* c) {
 // stride over boxes).  Every test triangle of a box runs over the same source
 // list (the concatenated source ranges of its near boxes), so the block stages
 // those sources' coefficients in shared memory ([stage][6], dynamic shared
-// memory: stage is the problem's longest row), and its warps take
+// memory), and its warps take
 // the box's test triangles in turn, lanes over the row as in k_near (lane j,
 // j + 32, ...): the same operations in the same order as in k_near, so the same
 // result to the last bit.  nsplit shares a box's test triangles among several
-// blocks when the leaf boxes alone do not fill the SMs.  Rows longer than stage
-// (shared memory takes 4736 sources, 4384 beside the half records) read the
-// coefficients from global memory instead.
+// blocks when the leaf boxes alone do not fill the SMs.  Rows longer than stage read
+// the coefficients from global memory instead (near_box_stage).
 // Half-precision records reach shared memory by cp.async kNearAhead steps of 32
 // entries ahead, across rows: 327,680 triangles 607 -> 540 us (loads of four
 // records at a time left the memory idle at every row's end; float moments read
 // 94 % of the copy rate as they are).
 constexpr int kNearAhead = 3;
 constexpr int kNearBoxThreads = 128;  // 256 measured 8 % slower (FP32H)
-constexpr size_t kNearSmemMax = 228096;  // a block's 227 KB less what the kernel declares itself
+constexpr size_t kNearSmemMax = 232448;  // what a block may have: 227 KB
 template <bool H16>
 constexpr size_t near_box_smem(int stage) {
   return size_t(6) * stage * sizeof(cf) + (H16 ? size_t(4) * (kNearAhead + 1) * 64 * sizeof(uint4) : 0);
 }
-// Sources staged: the longest row, or as many as fit.
+// Sources staged, one size for all boxes: the longest row while that pays, for long
+// rows take blocks off every SM, short ones' too, and room from the far part.  Float
+// moments: up to 1344 sources, three blocks an SM and 60 KB of first-level cache
+// (81,920 triangles, rows of 838 to 1311: 1.28 ms, 1.33 from global memory; up to
+// 1541: 2.17, 1.71; 2947: 4.90, 2.74); up to 2400, two blocks, where one box is the
+// critical path (cylinder of 40,960 triangles, rows to 2030 and one box with 2.7
+// times an SM's share of the pairs: 1.48, 1.88).  Half records, whose loads hide less: as
+// many as fit (up to 1541: 1.03, 1.64; 2947: 2.48, 2.50, the product 2.72, 4.30).
+// Beyond, the short rows only, at six blocks an SM, where they hold half of the
+// pairs (327,680 triangles of rows near 270 and 5120 of rows to 2377: the product
+// 11.4 ms with the longest row staged, 10.0 with short rows, 10.1 with none), else
+// none: the first-level cache then has the memory (rows of 3244 to 5170: near part
+// 12.5 ms with those staged that fit, 5.0 with room for 512 sources, 4.6 with none).
+constexpr int kNearFloatRow = 1344, kNearPathRow = 2400;
 template <bool H16>
 static int near_box_stage(const Problem& pr) {
   const int fit = int((kNearSmemMax - near_box_smem<H16>(0)) / (6 * sizeof(cf))) / 32 * 32;
-  return std::min(int((pr.max_row + 31) / 32 * 32), fit);
+  const bool path = 2 * pr.box_pairs * pr.nsm > 3 * pr.nnz;  // 1.5 times an SM's share
+  const int64_t most = H16 ? fit : path ? kNearPathRow : kNearFloatRow;
+  const int64_t row = pr.max_row <= most ? pr.max_row : 2 * pr.short_pairs >= pr.nnz ? pr.short_row : 0;
+  return int((row + 31) / 32 * 32);
 }
 
 template <typename Rio, bool H16>

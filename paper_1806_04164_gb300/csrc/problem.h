@@ -18,6 +18,7 @@ typedef C2<float> cf;
 constexpr int kComp = 5;      // radiated densities per box: mu0 J (3), sigma, d
 constexpr int kNoffs = 316;   // one-box-buffer translation offsets
 constexpr int kMom = 8;       // moments per triangle pair: m0, mt(3), ms(3), mts
+constexpr int kNearShortRow = 448;  // rows that the near kernel stages at six blocks an SM in every precision
 constexpr int kStages = 8;    // coef, near, aggregation, interpolation, translation, anterpolation, disaggregation, assembly
 
 struct LevelDev {
@@ -48,6 +49,9 @@ struct Problem {
   int64_t T = 0, E = 0, N = 0;
   int64_t nnz = 0;      // near pair entries
   int64_t max_row = 0;  // most near pair entries of a test triangle
+  int64_t short_row = 0;    // the same among rows of at most kNearShortRow entries
+  int64_t short_pairs = 0;  // entries in those rows
+  int64_t box_pairs = 0;    // most entries in one leaf box's rows
   int64_t nleaf = 0;
   double h_max = 0;     // longest edge of the mesh
   double r_max = 0;     // largest distance of a centroid from the origin

@@ -882,6 +882,11 @@ static pie_status setup_t(Problem& pr, cudaStream_t st) {
     }
     row_ptr[i + 1] = row_ptr[i] + cnt;
     pr.max_row = std::max(pr.max_row, cnt);
+    if (cnt <= kNearShortRow) {
+      pr.short_row = std::max(pr.short_row, cnt);
+      pr.short_pairs += cnt;
+    }
+    pr.box_pairs = std::max(pr.box_pairs, cnt * (tr.leaf_start[b + 1] - tr.leaf_start[b]));
   }
   pr.nnz = row_ptr[T];
 
