@@ -427,9 +427,9 @@ pie_status pie_nearfield(pie_problem* pr, const void* x, const void* rho, const 
  *    threads per SM (each warp walks test triangles with a grid stride), so
  *    that it takes a bounded share of every SM beside the far kernels;
  *    0 = one warp per test triangle.  0..32.  A complex double near part
- *    takes, for every two, one or two blocks of 128 threads per SM, whichever
- *    ends with the far part (its integer multiply-adds leave the FP64 pipe to
- *    it); a box-staged float one with more than 16 blocks per SM takes 32
+ *    takes, for every two, one to three blocks of 128 threads per SM, by how
+ *    its work compares with the far part's (its integer multiply-adds leave the
+ *    FP64 pipe to it); a box-staged float one with more than 16 blocks per SM takes 32
  *    times the bound, its blocks being short.
  *  rhs_chunk: right-hand sides per pass over the operator, 1..max_nrhs.
  *  near_rhs_block: right-hand sides that one pass of the near kernel

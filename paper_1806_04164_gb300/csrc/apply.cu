@@ -565,43 +565,23 @@ static pie_status near_float_prepare() {
 // stride over the pairs: the box's source coefficients are staged as
 // integers kFixedStage at a time, then its warps take the test triangles in
 // turn, lanes over the row.  nsplit shares a box among several blocks when the
-// leaf boxes alone do not fill the SMs.  81,920 triangles: 0.72 ms alone (2.2 ms
-// with FP64 multiply-adds; 0.65 with one exponent for both parts of a moment, in
-// one pass over the row), 24,576 of a cube: 0.69 ms (1.78); beside the far part
+// leaf boxes alone do not fill the SMs.  81,920 triangles: 0.68 ms alone (2.2 ms
+// with FP64 multiply-adds), 24,576 of a cube: 0.65 ms (1.78); beside the far part
 // one block an SM does, since the two use different pipes: the product of 81,920
 // triangles 2.7 to 2.9 ms (5.1 with FP64 multiply-adds).
 
-// A warp-wide 64-bit multiply-add issues every two clocks and takes four, so the
-// limb products are taken kind by kind over all sums (KIND 0: h h', 1: h l',
-// 2: l h') and not sum by sum.  s[2 i], s[2 i + 1]: real and imaginary part of c
-// times one part of the moment.
+// A product's limbs: hh += h h', x += h l' + l h'; s[0], s[1]: real and imaginary
+// part of c times one part of the moment, m = (h, l).
 struct FixedSum {
   int64_t hh, x;
 };
-template <int KIND>
-__device__ __forceinline__ void fixed_cfma(FixedSum (&s)[12], int i, const int4& c, const int2& m) {
-  const int mx = KIND == 1 ? m.y : m.x;
-  int64_t& re = KIND == 0 ? s[2 * i].hh : s[2 * i].x;
-  int64_t& im = KIND == 0 ? s[2 * i + 1].hh : s[2 * i + 1].x;
-  re += int64_t(KIND == 2 ? c.y : c.x) * mx;
-  im += int64_t(KIND == 2 ? c.w : c.z) * mx;
-}
-
-// The twelve products of one pair; m: m0, mt(3), ms(3), mts; c: a, beta(3), sigma, d.
-template <typename F, typename C, typename M>
-__device__ __forceinline__ void near_products(F f, const C& c, const M& m) {
-  f(1, c[0], m[4]);
-  f(2, c[0], m[5]);
-  f(3, c[0], m[6]);
-  f(0, c[0], m[7]);
-  f(4, c[4], m[0]);
-  f(1, c[1], m[0]);
-  f(0, c[1], m[1]);
-  f(2, c[2], m[0]);
-  f(5, c[5], m[0]);
-  f(0, c[2], m[2]);
-  f(3, c[3], m[0]);
-  f(0, c[3], m[3]);
+__device__ __forceinline__ void fixed_cfma(FixedSum* s, const int4& c, const int2& m) {
+  s[0].hh += int64_t(c.x) * m.x;
+  s[1].hh += int64_t(c.z) * m.x;
+  s[0].x += int64_t(c.x) * m.y;
+  s[1].x += int64_t(c.z) * m.y;
+  s[0].x += int64_t(c.y) * m.x;
+  s[1].x += int64_t(c.w) * m.x;
 }
 
 // Entries j0 .. j1 of row t in double, for a stage with a coefficient that is
@@ -618,7 +598,14 @@ __device__ __noinline__ double near_row_double(const FixedNear& nf, int64_t nnz,
     const cd* c = coef + 6 * (int64_t(leaf_start[near_idx[qi]]) + (j - near_off[qi]));
     cd m[kMom];
     for (int q = 0; q < kMom; ++q) m[q] = fixed_moment(nf, nnz, q, e0 + j, t, b);
-    near_products([&](int i, cd x, cd y) { cfma(acc[i], x, y); }, c, m);
+    cfma(acc[0], c[0], m[7]);
+    for (int d = 0; d < 3; ++d) {
+      cfma(acc[0], c[1 + d], m[1 + d]);
+      cfma(acc[1 + d], c[0], m[4 + d]);
+      cfma(acc[1 + d], c[1 + d], m[0]);
+    }
+    cfma(acc[4], c[4], m[0]);
+    cfma(acc[5], c[5], m[0]);
   }
   double out = 0;
   for (int i = 0; i < 12; ++i) {
@@ -628,28 +615,31 @@ __device__ __noinline__ double near_row_double(const FixedNear& nf, int64_t nnz,
   return out;
 }
 
-// Shared memory: the stage's coefficients [6][kFixedStage], then kFixedSlots
-// buffers of 32 entries' moments of one part [4][32] per warp.  (Three slots, 61 KB
-// a block, let blocks pile up on some SMs beside the far part: products of 81,920
-// triangles in a row 3.57 ms, 2.69 with four.)
-constexpr int kFixedWarps = 4, kFixedSlots = 4;
-constexpr size_t kFixedSmem = sizeof(int4) * (6 * kFixedStage + kFixedWarps * kFixedSlots * kFixedPlanes * 32);
+// PARTS: moments' parts of a pass over the row.  Both at once take 48 sums and 164
+// registers, one after the other 24 and 128 and the coefficients from shared memory
+// twice: 81,920 triangles alone 0.68 ms, 0.72, but beside the far part, whose
+// kernels the registers hold up, the product 2.97 ms, 2.88.  BLOCKS: blocks of an SM that
+// the registers allow.  Shared memory: the stage's coefficients [6][kFixedStage], then
+// per warp SLOTS buffers of 32 entries' moments [PARTS][4][32], as much for either
+// number (with 61 KB a block three fit, and blocks pile up on some SMs beside the far
+// part: products of 81,920 triangles in a row 3.57 ms, 2.69).
+constexpr int kFixedWarps = 4;
+constexpr size_t kFixedSmem = sizeof(int4) * (6 * kFixedStage + kFixedWarps * 4 * kFixedPlanes * 32);
 
-// BLOCKS: blocks of an SM that the registers allow (3: 158 registers, alone; 4: 128,
-// which leaves room for the far part's kernels beside it).
-template <int BLOCKS>
+template <int PARTS, int BLOCKS>
 __global__ void __launch_bounds__(32 * kFixedWarps, BLOCKS)
     k_near_fixed(int64_t nleaf, int nsplit, int64_t nnz, const int32_t* __restrict__ leaf_start,
                  const int32_t* __restrict__ near_ptr, const int32_t* __restrict__ near_idx,
                  const int32_t* __restrict__ near_off, const int64_t* __restrict__ row_ptr, const FixedNear nf,
                  const cd* __restrict__ coef, double mu0, cd* __restrict__ pot, int64_t sc = 0, int64_t sp = 0) {
+  constexpr int PASSES = 2 / PARTS, PLANES = kFixedPlanes * PARTS, SLOTS = 4 / PARTS;
   extern __shared__ __align__(16) unsigned char fixed_smem[];
   int4(*cs)[kFixedStage] = reinterpret_cast<int4(*)[kFixedStage]>(fixed_smem);
   __shared__ int fields[kFixedWarps][8];  // [warp][part of a, beta, sigma, d]
   coef += blockIdx.y * sc;
   double* out = reinterpret_cast<double*>(pot + blockIdx.y * sp);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int4(*ms)[kFixedPlanes][32] = reinterpret_cast<int4(*)[kFixedPlanes][32]>(cs + 6) + kFixedSlots * warp;
+  int4(*ms)[PLANES][32] = reinterpret_cast<int4(*)[PLANES][32]>(cs + 6) + SLOTS * warp;
   for (int64_t bi = blockIdx.x; bi < nleaf * nsplit; bi += gridDim.x) {
     const int64_t b = bi / nsplit;
     const int q0 = near_ptr[b], q1 = near_ptr[b + 1];
@@ -708,97 +698,111 @@ __global__ void __launch_bounds__(32 * kFixedWarps, BLOCKS)
         }
       }
       __syncthreads();
-      // the warp's (test triangle, part, 32 entries) steps in one sequence: the next
+      // the warp's (test triangle, pass, 32 entries) steps in one sequence: the next
       // steps' moments are on their way while a step is multiplied, across rows
       // too (rows of a box have one length, one after the other); a lane copies
       // and reads its own entry
       const int64_t base = row_ptr[leaf_start[b]];
-      const int per_row = (j1 - j0 + 31) / 32;
+      const int count = j1 - j0, tstep = kFixedWarps * nsplit;
       int ft = t0, fp = 0, fj = lane, fslot = 0;
-      const int count = j1 - j0;
-      // the part's first entry of the row, and how far the next row's lies from there
+      // the pass's first entry of the row, and how far the next row's lies from there
       const int4* src = nf.mom + base + int64_t(t0 - leaf_start[b]) * len + j0;
-      const int64_t next_row = int64_t(kFixedWarps * nsplit) * len - kFixedPlanes * nnz;
+      const int64_t next_row = int64_t(tstep) * len - (PASSES - 1) * PLANES * nnz;
       auto fetch = [&] {
         if (fj < count && ft < t1 && finite) {
           const int4* from = src + fj;
 #pragma unroll
-          for (int g = 0; g < kFixedPlanes; ++g, from += nnz) cp_async(&ms[fslot][g][lane], from);
+          for (int g = 0; g < PLANES; ++g, from += nnz) cp_async(&ms[fslot][g][lane], from);
         }
         cp_async_commit();
-        fslot = fslot + 1 == kFixedSlots ? 0 : fslot + 1;
+        fslot = fslot + 1 == SLOTS ? 0 : fslot + 1;
         fj += 32;
         if (fj - lane >= count) {
           fj = lane;
-          src += fp ? next_row : kFixedPlanes * nnz;
-          ft += fp ? kFixedWarps * nsplit : 0;
-          fp ^= 1;
+          const bool next = fp + 1 == PASSES;
+          src += next ? next_row : PLANES * nnz;
+          ft += next ? tstep : 0;
+          fp = next ? 0 : fp + 1;
         }
       };
       // exponent of the coefficients in the lane's sum
       const int ec = (lane & 1 ? (lane < 8 ? x[3] : lane < 10 ? x[5] : x[7])
                                : (lane < 8 ? x[2] : lane < 10 ? x[4] : x[6])) - 1075;
-      // one part of row t: lane i < 12 gets the value of sum i
       int slot = 0;
-      auto part_sum = [&](int t, int part) {
-        FixedSum sum[12];
+      // a pass over row t, part and (PARTS = 2) the next: lane i < 12 gets the value of
+      // sum i of the (re c + i im c) (re m + i im m) so far, v of the passes before
+      auto pass = [&](int t, int part, double v) {
+        FixedSum sum[PARTS][12];
 #pragma unroll
-        for (int i = 0; i < 12; ++i) sum[i] = FixedSum{0, 0};
-        for (int i = 0; i < per_row; ++i) {
+        for (int i = 0; i < 12 * PARTS; ++i) sum[i / 12][i % 12] = FixedSum{0, 0};
+        for (int j = lane; j - lane < count; j += 32) {
           fetch();
-          cp_async_wait<kFixedSlots - 1>();
-          const int j = 32 * i + lane;
-          if (j0 + j < j1) {
-            int2 m[kMom];
-            int4 c[6];
+          cp_async_wait<SLOTS - 1>();
+          if (j < count) {
+            int2 m[PARTS][kMom];
 #pragma unroll
-            for (int g = 0; g < kFixedPlanes; ++g) {
-              const int4 v = ms[slot][g][lane];
-              m[2 * g] = make_int2(v.x, v.y);
-              m[2 * g + 1] = make_int2(v.z, v.w);
+            for (int g = 0; g < PLANES; ++g) {
+              const int4 w = ms[slot][g][lane];
+              m[g / kFixedPlanes][2 * (g % kFixedPlanes)] = make_int2(w.x, w.y);
+              m[g / kFixedPlanes][2 * (g % kFixedPlanes) + 1] = make_int2(w.z, w.w);
             }
+            // (one coefficient after the other: the sums fill the registers)
+            auto product = [&](int i, const int4& c, int q) {
 #pragma unroll
-            for (int k = 0; k < 6; ++k) c[k] = cs[k][j];
-            near_products([&](int k, const int4& a, const int2& b) { fixed_cfma<0>(sum, k, a, b); }, c, m);
-            near_products([&](int k, const int4& a, const int2& b) { fixed_cfma<1>(sum, k, a, b); }, c, m);
-            near_products([&](int k, const int4& a, const int2& b) { fixed_cfma<2>(sum, k, a, b); }, c, m);
+              for (int u = 0; u < PARTS; ++u) fixed_cfma(&sum[u][2 * i], c, m[u][q]);
+            };
+            const int4 a = cs[0][j];
+            product(0, a, 7);
+            product(1, a, 4);
+            product(2, a, 5);
+            product(3, a, 6);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+              const int4 c = cs[1 + d][j];
+              product(0, c, 1 + d);
+              product(1 + d, c, 0);
+            }
+            product(4, cs[4][j], 0);
+            product(5, cs[5][j], 0);
           }
-          slot = slot + 1 == kFixedSlots ? 0 : slot + 1;
+          slot = slot + 1 == SLOTS ? 0 : slot + 1;
         }
-        // value = hh 2^56 + x 2^28: x carried into hh but for 28 bits below it, and
-        // the warp's totals in pieces of 27 bits
-        int p0 = 0, p1 = 0, p2 = 0, p3 = 0;
-#pragma unroll
-        for (int i = 0; i < 12; ++i) {
-          const int64_t h = sum[i].hh + (sum[i].x >> kLimb);
-          const int r0 = int(__reduce_add_sync(0xffffffffu, (uint32_t(sum[i].x) & ((1u << kLimb) - 1)) >> 1));
-          const int r1 = int(__reduce_add_sync(0xffffffffu, uint32_t(h) & ((1u << 27) - 1)));
-          const int r2 = int(__reduce_add_sync(0xffffffffu, uint32_t(h >> 27) & ((1u << 27) - 1)));
-          const int r3 = __reduce_add_sync(0xffffffffu, int(h >> 54));
-          if (lane == i) p0 = r0, p1 = r1, p2 = r2, p3 = r3;
-        }
-        // 96 bits: the totals above the point less five bits, then 5 + 27 bits
-        const uint64_t mid = (uint64_t(uint32_t(p2)) << 27) + uint32_t(p1);
-        const uint64_t low = uint64_t(uint32_t(p0)) + ((mid & 31) << 27);
-        const int64_t hi = int64_t(p3) * (int64_t(1) << 49) + int64_t(mid >> 5) + int64_t(low >> 32);
         const FixedRow row = nf.row[t];
-        if (row.m0[0] == kFixedNan) return nan("");
-        const int em = lane < 2 ? (part ? row.mt[1] : row.mt[0]) : part ? row.m0[1] : row.m0[0];
-        return fixed_scale(hi, uint32_t(low), em + ec + 2 * kLimb - 27);
+#pragma unroll
+        for (int u = 0; u < PARTS; ++u) {
+          // value = hh 2^56 + x 2^28: x carried into hh but for 28 bits below it, and
+          // the warp's totals in pieces of 27 bits
+          int p0 = 0, p1 = 0, p2 = 0, p3 = 0;
+#pragma unroll
+          for (int i = 0; i < 12; ++i) {
+            const FixedSum& s = sum[u][i];
+            const int64_t h = s.hh + (s.x >> kLimb);
+            const int r0 = int(__reduce_add_sync(0xffffffffu, (uint32_t(s.x) & ((1u << kLimb) - 1)) >> 1));
+            const int r1 = int(__reduce_add_sync(0xffffffffu, uint32_t(h) & ((1u << 27) - 1)));
+            const int r2 = int(__reduce_add_sync(0xffffffffu, uint32_t(h >> 27) & ((1u << 27) - 1)));
+            const int r3 = __reduce_add_sync(0xffffffffu, int(h >> 54));
+            if (lane == i) p0 = r0, p1 = r1, p2 = r2, p3 = r3;
+          }
+          // 96 bits: the totals above the point less five bits, then 5 + 27 bits
+          const uint64_t mid = (uint64_t(uint32_t(p2)) << 27) + uint32_t(p1);
+          const uint64_t low = uint64_t(uint32_t(p0)) + ((mid & 31) << 27);
+          const int64_t hi = int64_t(p3) * (int64_t(1) << 49) + int64_t(mid >> 5) + int64_t(low >> 32);
+          const bool im = part + u;
+          const int em = lane < 2 ? (im ? row.mt[1] : row.mt[0]) : im ? row.m0[1] : row.m0[0];
+          const double w = fixed_scale(hi, uint32_t(low), em + ec + 2 * kLimb - 27);
+          const double other = __shfl_xor_sync(0xffffffffu, w, 1);
+          v = im ? v + (lane & 1 ? other : -other) : w;  // i im m: the parts change places
+        }
+        return row.m0[0] == kFixedNan ? nan("") : v;
       };
 #pragma unroll
-      for (int d = 0; d < kFixedSlots - 1; ++d) fetch();
-      for (int t = t0; t < t1; t += kFixedWarps * nsplit) {
+      for (int d = 0; d < SLOTS - 1; ++d) fetch();
+      for (int t = t0; t < t1; t += tstep) {
         const int64_t e0 = base + int64_t(t - leaf_start[b]) * len;
-        double v;
+        double v = 0;
         if (finite) {
-          // (re c + i im c) (re m + i im m): the imaginary moments' sums change places
-          v = 0;
 #pragma unroll 1
-          for (int part = 0; part < 2; ++part) {
-            const double w = part_sum(t, part), u = __shfl_xor_sync(0xffffffffu, w, 1);
-            v = part ? v + (lane & 1 ? u : -u) : w;
-          }
+          for (int part = 0; part < 2; part += PARTS) v = pass(t, part, v);
         } else {
           v = near_row_double(nf, nnz, t, int(b), e0, j0, j1, q0, q1, leaf_start, near_idx, near_off, coef);
         }
@@ -816,8 +820,8 @@ static pie_status near_fixed_prepare() {
   static std::atomic<uint64_t> done{0};
   int bit = -1;
   if (device_done(done, &bit)) return PIE_OK;
-  pie_status s = raise_smem(k_near_fixed<3>, kFixedSmem);
-  if (s == PIE_OK) s = raise_smem(k_near_fixed<4>, kFixedSmem);
+  pie_status s = raise_smem(k_near_fixed<2, 3>, kFixedSmem);
+  if (s == PIE_OK) s = raise_smem(k_near_fixed<1, 4>, kFixedSmem);
   if (s == PIE_OK && bit >= 0) done.fetch_or(uint64_t(1) << bit);
   return s;
 }
@@ -832,14 +836,15 @@ pie_status near_prepare(const Problem& pr) {
 }
 
 // Launch of the fixed-point near part for nrhs columns on a grid of at most
-// max_blocks (0: no bound).
-static void near_fixed(const Problem& pr, const cd* coef, cd* pot, int nrhs, int64_t max_blocks, cudaStream_t st) {
+// max_blocks (0: no bound).  lean: the kernel of fewer registers.
+static void near_fixed(const Problem& pr, const cd* coef, cd* pot, int nrhs, int64_t max_blocks, bool lean,
+                       cudaStream_t st) {
   const FixedNear nf{static_cast<const int4*>(pr.mom), static_cast<const FixedRow*>(pr.fixed_row), pr.fixed_delta};
   // shares per box: the least rounds of three blocks an SM, staging (about 1/50
   // of a box's rows) once a share; at least a test triangle for each warp.  Boxes
   // are uneven, so up to 8 % more by this count for finer shares, while a warp has
   // three rows (alone: cube of 24,576 triangles 799 -> 695 us, ellipsoid of 32,768
-  // 2870 -> 1400; finer still: spheres lose 10 %)
+  // 2870 -> 1400; finer still, spheres lose 10 %)
   const int64_t slots = 3 * int64_t(pr.nsm),
                 most = std::min<int64_t>(16, (pr.T / pr.nleaf + kFixedWarps - 1) / kFixedWarps);
   int nsplit = 1;
@@ -853,7 +858,7 @@ static void near_fixed(const Problem& pr, const cd* coef, cd* pot, int nrhs, int
     if (costs[s] <= 1.08 * best) nsplit = int(s);
   int64_t grid = pr.nleaf * nsplit;
   if (max_blocks > 0) grid = std::min(grid, max_blocks);
-  auto kernel = max_blocks > 0 ? k_near_fixed<4> : k_near_fixed<3>;
+  auto kernel = lean ? k_near_fixed<1, 4> : k_near_fixed<2, 3>;
   kernel<<<dim3(unsigned(grid), unsigned(nrhs)), 32 * kFixedWarps, kFixedSmem, st>>>(
       pr.nleaf, nsplit, pr.nnz, pr.leaf_start, pr.near_ptr, pr.near_idx, pr.near_off, pr.row_ptr, nf, coef, kMu0, pot,
       6 * pr.T, 6 * pr.T);
@@ -1961,19 +1966,25 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
   if (!with_near) {
     pot2 = nullptr;
   } else if constexpr (sizeof(Rm) == 8) {  // PIE_FP64: fixed point, each column by itself
-    // beside the far part: one block an SM where it ends with the far part, else
-    // two (three leave the filter kernels no shared memory until they are done:
-    // the 100 MHz plate 377 us beside 100 KB an SM, 440 beside 209).  One block takes
-    // 89 ps a pair (81,920 triangles: 1.9 ms), the far part 1.6 ps a double
-    // operation: 20 a list entry and sample, 32 a triangle and sample for
-    // aggregation and disaggregation, about 9000 a box and component for the filters
+    // beside the far part: one block an SM where it ends with the far part, else two
+    // (three leave the filter kernels no shared memory until they are done: the 100 MHz
+    // plate 377 us beside 100 KB an SM, 440 beside 209), and three where the near part
+    // takes four times as long (cylinder of 9472 triangles 834 us with two, 625;
+    // ellipsoid of 8192 750, 575).  One block takes 89 ps a pair (81,920 triangles: 1.9
+    // ms), the far part 1.6 ps a double operation: 20 a list entry and sample, 32 a
+    // triangle and sample for aggregation and disaggregation, about 9000 a box and
+    // component for the filters
     double far_ops = 32.0 * double(pr.T) * P;
     for (int l = 3; l <= L; ++l)
       far_ops += 20.0 * P * double(pr.lev[l].nlist) + (l > 3 ? 9000.0 * kComp * double(pr.lev[l].nb) : 0.0);
-    const int64_t per_sm = 89.0 * double(pr.nnz) > 1.6 * far_ops ? 2 : 1;
+    const double near_part = 89.0 * double(pr.nnz) / (1.6 * far_ops);  // over the far part
+    const int64_t per_sm = near_part > 4.0 ? 3 : near_part > 1.0 ? 2 : 1;
+    // (the kernel of fewer registers up to there: plates, at 2.9, 356 us, 381 with the
+    // other; 1120, 1314)
     near_fixed(pr, coef, pot2, nrhs,
                overlap && pr.tune.near_ctas_per_sm > 0
-                   ? int64_t(pr.nsm) * per_sm * ((pr.tune.near_ctas_per_sm + 1) / 2) : 0, sn);
+                   ? int64_t(pr.nsm) * per_sm * ((pr.tune.near_ctas_per_sm + 1) / 2) : 0,
+               overlap && near_part <= 4.0, sn);
   } else if (boxed && (rb == 1 || rb == 2 || rb == 4)) {
     if (rb == 1)
       box_launch(std::integral_constant<int, 1>());
@@ -2197,7 +2208,7 @@ static pie_status apply_near_t(Problem& pr, const void* xv, void* yv, cudaStream
   k_coef<Rio><<<nblk(pr.T, 256), 256, 0, st>>>(pr.T, pr.E, static_cast<const C2<Rio>*>(xv), pr.perm, pr.tri_edge,
                                                pr.tri_c, pr.tri_cdcp, pr.w * pr.w * eps0(), coef, coef32);
   if constexpr (sizeof(Rm) == 8) {
-    near_fixed(pr, coef, pot, 1, 0, st);
+    near_fixed(pr, coef, pot, 1, 0, false, st);
   } else if (pr.tune.near_kernel != 1) {  // the box-staged kernel, unless tuned off
     const int nsplit = near_box_split(pr, kNearBoxThreads / 32), stage = near_box_stage<H16>(pr);
     k_near_box<Rio, H16><<<unsigned(pr.nleaf * nsplit), kNearBoxThreads, near_box_smem<H16>(stage), st>>>(
@@ -2735,7 +2746,7 @@ pie_status apply_near_scratch(Problem& pr, const void* x, void* y, void* coef, v
           static_cast<const cf*>(pr.mom), nullptr, mom_scale(pr), static_cast<const cf*>(coef), float(kMu0),
           static_cast<cd*>(pot));
     else
-      near_fixed(pr, static_cast<const cd*>(coef), static_cast<cd*>(pot), 1, 0, st);
+      near_fixed(pr, static_cast<const cd*>(coef), static_cast<cd*>(pot), 1, 0, false, st);
     k_assemble<double><<<nblk(pr.N, 256), 256, 0, st>>>(pr.N, pr.E, pr.edge_tt, pr.edge_k, pr.tri_c, pr.tri_dcp,
                                                         pr.inv_perm, static_cast<const cd*>(pot), static_cast<cd*>(y));
   }

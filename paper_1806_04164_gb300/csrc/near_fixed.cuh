@@ -15,9 +15,8 @@
 // staged.  Real and imaginary parts have powers of their own, in moments and
 // coefficients alike: at low frequency the imaginary (radiated) part of a moment
 // is k h / 4 of the real one and less, and where the coefficients are real it
-// alone makes the imaginary part of the product.  So a row is summed twice, real
-// moments and then imaginary ones, and every sum takes products of one part with
-// one part.
+// alone makes the imaginary part of the product.  So every sum takes products of one
+// part with one part: four where a complex product has two.
 //
 // Error: the sums are exact but for l l' and the last bit of x, so what remains is the
 // rounding of the factors, to 2^-59 of the row's largest moment and 2^-57 of the
