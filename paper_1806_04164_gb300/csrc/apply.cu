@@ -872,20 +872,25 @@ __device__ __forceinline__ int antipode(int q, int ntheta) {
   return (ntheta - 1 - i) * nphi + (j + ntheta) % nphi;
 }
 
-// Largest blocks of the per-box far kernels, as their registers allow: a block
-// of n warps fits while each of the SM's four schedulers (16,384 registers) holds
-// its ceil(n / 4) of them, so 64 registers take 1024 threads, 80 take 768 and 88
-// to 96 take 640.  Kernels of up to 64 registers are bounded by 1024, the others
-// by what their main form takes, and the orchestration packs no more rows
-// into a block than fit; an angular grid whose one row is wider than that (20
-// and 22 theta rows) takes the WIDE form, held to 64 registers.
-constexpr int kFarThreads = 1024;
-template <typename Rf>
-constexpr int kAggThreads = sizeof(Rf) == 4 ? kFarThreads : 640;  // 59, 88 registers
-template <typename Rf, int NC, bool WIDE>
-constexpr int kInterpThreads = WIDE || NC == 1 ? kFarThreads : sizeof(Rf) == 4 ? 768 : 640;  // 80, 90 registers
-template <typename Rf, int NC, bool WIDE>
-constexpr int kTransThreads = WIDE || NC == 1 || sizeof(Rf) == 4 ? kFarThreads : 768;  // 77 registers in double
+// Largest block of a per-box far kernel, as its registers allow (up to 64 a
+// thread: 1024 threads, up to 80: 768).  The orchestration packs no more rows into
+// a block; an angular grid whose one row is wider (20 and 22 theta rows) takes the
+// kernel's WIDE form, held to 64 registers.  Asked of the kernel and not set by launch
+// bounds: bounds of 1024 cost the float aggregation 61 -> 94 us at 327,680
+// triangles, although its 62 registers meet them.
+template <auto Kernel>
+static int max_threads() {
+  static std::atomic<int> most{0};
+  if (const int n = most.load()) return n;
+  cudaFuncAttributes a;
+  if (cudaFuncGetAttributes(&a, Kernel) != cudaSuccess) {
+    cudaGetLastError();
+    return 512;  // the widest row of any of them but WIDE ones
+  }
+  most.store(a.maxThreadsPerBlock);
+  return a.maxThreadsPerBlock;
+}
+constexpr int kWideThreads = 1024;
 
 // a2: leaf aggregation.  One block per leaf box, one thread per half-grid
 // sample q.  The radiation tables are stored for the half grid only, since
@@ -894,7 +899,7 @@ constexpr int kTransThreads = WIDE || NC == 1 || sizeof(Rf) == 4 ? kFarThreads :
 // A = sum c Xr and B = sum c Xi.
 // Small angular grids pack several boxes into one block (threadIdx.y).
 template <typename Rf>
-__global__ void __launch_bounds__(kAggThreads<Rf>) k_agg(int P, int ntheta, int64_t nb, const int32_t* __restrict__ leaf_start,
+__global__ void k_agg(int P, int ntheta, int64_t nb, const int32_t* __restrict__ leaf_start,
                       const C2<Rf>* __restrict__ Pi, const C2<Rf>* __restrict__ M, const C2<Rf>* __restrict__ coef,
                       Rf mu0, C2<Rf>* __restrict__ S, int64_t sc = 0, int64_t sS = 0) {
   const int64_t b = int64_t(blockIdx.x) * blockDim.y + threadIdx.y;
@@ -970,10 +975,10 @@ __global__ void __launch_bounds__(kAggThreads<Rf>) k_agg(int P, int ntheta, int6
 // 272 81 -> 35 us, 4400 (double) 358 -> 336 us; from about 10,000 boxes in double
 // and 9,000 in float k_agg is as fast or faster (its loads are wider).
 template <typename Rf, int NC>
-__global__ void __launch_bounds__(kFarThreads)
-    k_agg_split(int P, int ntheta, int64_t nb, const int32_t* __restrict__ leaf_start, const C2<Rf>* __restrict__ Pi,
-                const C2<Rf>* __restrict__ M, const C2<Rf>* __restrict__ coef, Rf mu0, C2<Rf>* __restrict__ S,
-                int64_t sc = 0, int64_t sS = 0) {
+__global__ void k_agg_split(int P, int ntheta, int64_t nb, const int32_t* __restrict__ leaf_start,
+                            const C2<Rf>* __restrict__ Pi, const C2<Rf>* __restrict__ M,
+                            const C2<Rf>* __restrict__ coef, Rf mu0, C2<Rf>* __restrict__ S, int64_t sc = 0,
+                            int64_t sS = 0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int X = threadIdx.z, part = blockIdx.z & 1, ri = X ? 1 - part : part, c0 = NC * int(blockIdx.z >> 1);
   const int nq = blockDim.x;
@@ -1051,11 +1056,11 @@ __global__ void __launch_bounds__(kFarThreads)
 // memory); children are summed in order, whatever cg.  A thread takes NC
 // components, the others threadIdx.z: five where the boxes fill the SMs, one on
 // small levels.
-template <typename Rf, int NC, bool WIDE = false>
-__global__ void __launch_bounds__(kInterpThreads<Rf, NC, WIDE>)
-    k_interp(int P, int64_t nb, const int32_t* __restrict__ child_start, const int8_t* __restrict__ oct_child,
-             const C2<Rf>* __restrict__ Sc, const Rf* __restrict__ Ft, const C2<Rf>* __restrict__ phase,
-             C2<Rf>* __restrict__ Sp, int64_t sSc = 0, int64_t sSp = 0, int cg = 1, bool fs = false) {
+template <typename Rf, int NC>
+__device__ __forceinline__ void interp_boxes(int P, int64_t nb, const int32_t* __restrict__ child_start,
+                                             const int8_t* __restrict__ oct_child, const C2<Rf>* __restrict__ Sc,
+                                             const Rf* __restrict__ Ft, const C2<Rf>* __restrict__ phase,
+                                             C2<Rf>* __restrict__ Sp, int64_t sSc, int64_t sSp, int cg, bool fs) {
   Sc += blockIdx.y * sSc;
   Sp += blockIdx.y * sSp;
   extern __shared__ unsigned char smem_raw[];
@@ -1108,6 +1113,21 @@ __global__ void __launch_bounds__(kInterpThreads<Rf, NC, WIDE>)
 #pragma unroll
     for (int c = 0; c < NC; ++c) Sp[((int64_t)b * kComp + c0 + c) * P + p] = acc[c];
   }
+}
+
+template <typename Rf, int NC>
+__global__ void k_interp(int P, int64_t nb, const int32_t* __restrict__ child_start,
+                         const int8_t* __restrict__ oct_child, const C2<Rf>* __restrict__ Sc,
+                         const Rf* __restrict__ Ft, const C2<Rf>* __restrict__ phase, C2<Rf>* __restrict__ Sp,
+                         int64_t sSc, int64_t sSp, int cg, bool fs) {
+  interp_boxes<Rf, NC>(P, nb, child_start, oct_child, Sc, Ft, phase, Sp, sSc, sSp, cg, fs);
+}
+template <typename Rf, int NC>
+__global__ void __launch_bounds__(kWideThreads)
+    k_interp_wide(int P, int64_t nb, const int32_t* __restrict__ child_start, const int8_t* __restrict__ oct_child,
+                  const C2<Rf>* __restrict__ Sc, const Rf* __restrict__ Ft, const C2<Rf>* __restrict__ phase,
+                  C2<Rf>* __restrict__ Sp, int64_t sSc, int64_t sSp, int cg, bool fs) {
+  interp_boxes<Rf, NC>(P, nb, child_start, oct_child, Sc, Ft, phase, Sp, sSc, sSp, cg, fs);
 }
 
 // ---- factorised filter: F is block-circulant in azimuth (its entries depend
@@ -1434,8 +1454,8 @@ __device__ __forceinline__ int trans_level(const TransArgs& a, int64_t box) {
 // left most SMs idle in turn: 327,680 triangles (double) 4.58 -> 4.40 ms, 81,920
 // 1.25 -> 1.12 ms, 56 boxes 46 -> 20 us, float patterns of 32 samples at 327,680
 // triangles 135 -> 97 us.
-template <typename Rf, int NC, bool WIDE = false>
-__global__ void __launch_bounds__(kTransThreads<Rf, NC, WIDE>) k_trans(int P, const TransArgs args) {
+template <typename Rf, int NC>
+__device__ __forceinline__ void trans_boxes(int P, const TransArgs& args) {
   constexpr int U = sizeof(Rf) == 4 ? 4 : 1;
   const int64_t box = int64_t(blockIdx.x) * blockDim.y + threadIdx.y;
   if (box >= args.total) return;
@@ -1478,6 +1498,15 @@ __global__ void __launch_bounds__(kTransThreads<Rf, NC, WIDE>) k_trans(int P, co
   }
 }
 
+template <typename Rf, int NC>
+__global__ void k_trans(int P, const TransArgs args) {
+  trans_boxes<Rf, NC>(P, args);
+}
+template <typename Rf, int NC>
+__global__ void __launch_bounds__(kWideThreads) k_trans_wide(int P, const TransArgs args) {
+  trans_boxes<Rf, NC>(P, args);
+}
+
 // a4 for float patterns of at most 128 samples (the inner operator of the
 // nested solve): the interaction list of a box is cut into kTransSplit
 // contiguous chunks, one per threadIdx.y sub-row, walked as in k_trans (four
@@ -1487,7 +1516,7 @@ __global__ void __launch_bounds__(kTransThreads<Rf, NC, WIDE>) k_trans(int P, co
 // order of operations depends on the list alone, never on the launch shape.
 constexpr int kTransSplit = 4;
 template <typename Rf, int NC>
-__global__ void __launch_bounds__(kFarThreads) k_trans_split(int P, const TransArgs args) {
+__global__ void k_trans_split(int P, const TransArgs args) {
   constexpr int U = 4;
   extern __shared__ unsigned char smem_raw[];
   C2<Rf>* part = reinterpret_cast<C2<Rf>*>(smem_raw);  // [row][chunk][component][P]
@@ -1554,10 +1583,9 @@ __global__ void __launch_bounds__(kFarThreads) k_trans_split(int P, const TransA
 // row of a block (several rows for small angular grids).  With fs the
 // filter F is staged in shared memory first (else read from global memory).
 template <typename Rf, int NC>
-__global__ void __launch_bounds__(kFarThreads)
-    k_anterp(int P, int64_t nc, const int32_t* __restrict__ parent, const int8_t* __restrict__ oct_child,
-             const C2<Rf>* __restrict__ Gp, const Rf* __restrict__ Fg, const C2<Rf>* __restrict__ phase,
-             C2<Rf>* __restrict__ Gc, int64_t sGp = 0, int64_t sGc = 0, bool fs = false) {
+__global__ void k_anterp(int P, int64_t nc, const int32_t* __restrict__ parent, const int8_t* __restrict__ oct_child,
+                         const C2<Rf>* __restrict__ Gp, const Rf* __restrict__ Fg, const C2<Rf>* __restrict__ phase,
+                         C2<Rf>* __restrict__ Gc, int64_t sGp = 0, int64_t sGc = 0, bool fs = false) {
   Gp += blockIdx.y * sGp;
   Gc += blockIdx.y * sGc;
   extern __shared__ unsigned char smem_raw[];
@@ -2014,7 +2042,7 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
   const C2<Rf>* fcoef = reinterpret_cast<const C2<Rf>*>(coef);
   // boxes per block of the per-box far kernels (threads: one per sample):
   // tune.far_rows, or enough to fill 128 threads; at most the kernel's threads
-  auto far_rows = [&](int threads, int most = kFarThreads) {
+  auto far_rows = [&](int threads, int most) {
     const int r = pr.tune.far_rows > 0 ? pr.tune.far_rows : (threads < 64 ? 128 / threads : 1);
     return std::max(1, std::min(r, most / threads));
   };
@@ -2030,7 +2058,8 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
     C2<Rf>* SL = static_cast<C2<Rf>*>(pr.lev[L].S);
     auto split = [&](auto ncc) {
       constexpr int NC = decltype(ncc)::value;
-      const int sth = std::min(512, ath), abp = std::max(1, std::min(far_rows(2 * sth), 512 / sth));
+      const int most = max_threads<k_agg_split<Rf, NC>>(), sth = std::min(most / 64 * 32, ath);
+      const int abp = far_rows(2 * sth, most);
       k_agg_split<Rf, NC><<<dim3(nblk(pr.lev[L].nb, abp), nr, 2 * kComp / NC), dim3(sth, abp, 2),
                             sizeof(Rf) * 2 * NC * sth * abp, sf>>>(P, pr.par.ntheta, pr.lev[L].nb, pr.leaf_start, Pi,
                                                                    M, fcoef, Rf(kMu0), SL, sT, sl(L));
@@ -2040,7 +2069,7 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
     } else if (narrow(sizeof(Rf) == 8 ? warps / 4 : warps)) {
       split(std::integral_constant<int, kComp>());
     } else {
-      const int abp = far_rows(ath, kAggThreads<Rf>);
+      const int abp = far_rows(ath, max_threads<k_agg<Rf>>());
       k_agg<Rf><<<dim3(nblk(pr.lev[L].nb, abp), nr), dim3(ath, abp), 0, sf>>>(
           P, pr.par.ntheta, pr.lev[L].nb, pr.leaf_start, Pi, M, fcoef, Rf(kMu0), SL, sT, sl(L));
     }
@@ -2053,7 +2082,7 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
   const size_t fsb = ((sizeof(Rf) * size_t(P) * P + 15) / 16) * 16;
   const bool fsh = fsb <= 16384;
   const size_t fsm_bytes = fsh ? fsb : 0;
-  const int fbp = std::max(1, std::min(far_rows(tpb), int((49152 - fsm_bytes) / sm)));
+  const int fbp = std::max(1, std::min(far_rows(tpb, kWideThreads), int((49152 - fsm_bytes) / sm)));
   const int cg = int(std::max<size_t>(1, std::min<size_t>(8, (49152 - fsm_bytes) / (sm * fbp))));
   const bool fft8 = pr.par.ntheta == 8;
   prof_mark(pr, 3, false, st);
@@ -2072,7 +2101,8 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
   }
   // dense filter: (components a thread, boxes per block, children staged at a time)
   auto dense = [&](int64_t nb, auto f) {
-    if (narrow(nb * (tpb / 32) * nr) && tpb * kComp <= 1024)
+    if (narrow(nb * (tpb / 32) * nr) &&
+        tpb * kComp <= std::min(max_threads<k_interp<Rf, 1>>(), max_threads<k_anterp<Rf, 1>>()))
       f(std::integral_constant<int, 1>(), 1, int(std::max<size_t>(1, std::min<size_t>(8, (49152 - fsm_bytes) / sm))));
     else
       f(std::integral_constant<int, kComp>(), fbp, cg);
@@ -2080,18 +2110,16 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
   for (int l = L - 1; l >= 3 && !fft8; --l)
     dense(pr.lev[l].nb, [&](auto ncc, int rows, int kids) {
       constexpr int NC = decltype(ncc)::value;
-      auto launch = [&](auto wide, int n) {
-        k_interp<Rf, NC, decltype(wide)::value><<<dim3(nblk(pr.lev[l].nb, n), nr), dim3(tpb, n, kComp / NC),
-                                                  fsm_bytes + sm * n * kids, sf>>>(
-            P, pr.lev[l].nb, pr.lev[l].child_start, pr.lev[l + 1].octant, static_cast<const C2<Rf>*>(pr.lev[l + 1].S),
-            static_cast<const Rf*>(pr.lev[l].Ft), static_cast<const C2<Rf>*>(pr.lev[l].phase),
-            static_cast<C2<Rf>*>(pr.lev[l].S), sl(l + 1), sl(l), kids, fsh);
-      };
-      constexpr int most = kInterpThreads<Rf, NC, false> / (kComp / NC);
+      const int most = max_threads<k_interp<Rf, NC>>() / (kComp / NC);
+      auto kernel = k_interp<Rf, NC>;
       // (in double a grid that wide needs more than 48 KB a child: refused)
       if constexpr (sizeof(Rf) == 4 && NC > 1)
-        if (tpb > most) return launch(std::true_type(), 1);
-      launch(std::false_type(), std::max(1, std::min(rows, most / tpb)));
+        if (tpb > most) kernel = k_interp_wide<Rf, NC>;
+      const int n = std::max(1, std::min(rows, most / tpb));
+      kernel<<<dim3(nblk(pr.lev[l].nb, n), nr), dim3(tpb, n, kComp / NC), fsm_bytes + sm * n * kids, sf>>>(
+          P, pr.lev[l].nb, pr.lev[l].child_start, pr.lev[l + 1].octant, static_cast<const C2<Rf>*>(pr.lev[l + 1].S),
+          static_cast<const Rf*>(pr.lev[l].Ft), static_cast<const C2<Rf>*>(pr.lev[l].phase),
+          static_cast<C2<Rf>*>(pr.lev[l].S), sl(l + 1), sl(l), kids, fsh);
     });
   prof_mark(pr, 3, true, st);
   prof_mark(pr, 4, false, st);
@@ -2113,19 +2141,17 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
       constexpr int NC = decltype(ncc)::value;
       if constexpr (sizeof(Rf) == 4)
         if (tpb <= 128) {  // float, small grid: each list cut into kTransSplit chunks
-          const int tbp = far_rows(tpb * kTransSplit);
+          const int tbp = far_rows(tpb * kTransSplit, max_threads<k_trans_split<Rf, NC>>());
           k_trans_split<Rf, NC><<<dim3(nblk(ta.total, tbp), nr, kComp / NC), dim3(tpb, tbp * kTransSplit),
                                   sizeof(C2<Rf>) * NC * P * kTransSplit * tbp, sf>>>(P, ta);
           return;
         }
-      constexpr int most = kTransThreads<Rf, NC, false>;
-      if constexpr (most < kFarThreads)
-        if (tpb > most) {
-          k_trans<Rf, NC, true><<<dim3(unsigned(ta.total), nr, kComp / NC), tpb, 0, sf>>>(P, ta);
-          return;
-        }
+      const int most = max_threads<k_trans<Rf, NC>>();
+      auto kernel = k_trans<Rf, NC>;
+      if constexpr (sizeof(Rf) == 8 && NC > 1)
+        if (tpb > most) kernel = k_trans_wide<Rf, NC>;
       const int tbp = far_rows(tpb, most);  // destination boxes per block
-      k_trans<Rf, NC><<<dim3(nblk(ta.total, tbp), nr, kComp / NC), dim3(tpb, tbp), 0, sf>>>(P, ta);
+      kernel<<<dim3(nblk(ta.total, tbp), nr, kComp / NC), dim3(tpb, tbp), 0, sf>>>(P, ta);
     };
     if (one)
       launch(std::integral_constant<int, 1>());
@@ -2144,11 +2170,11 @@ static pie_status apply_t(Problem& pr, const void* xv, void* yv, int nrhs, cudaS
   for (int l = 3; l < L && !fft8; ++l)
     dense(pr.lev[l + 1].nb, [&](auto ncc, int rows, int) {
       constexpr int NC = decltype(ncc)::value;
-      k_anterp<Rf, NC><<<dim3(nblk(pr.lev[l + 1].nb, rows), nr), dim3(tpb, rows, kComp / NC), fsm_bytes + sm * rows,
-                         sf>>>(P, pr.lev[l + 1].nb, pr.lev[l + 1].parent, pr.lev[l + 1].octant,
-                               static_cast<const C2<Rf>*>(pr.lev[l].G), static_cast<const Rf*>(pr.lev[l].F),
-                               static_cast<const C2<Rf>*>(pr.lev[l].phase), static_cast<C2<Rf>*>(pr.lev[l + 1].G),
-                               sl(l), sl(l + 1), fsh);
+      const int n = std::max(1, std::min(rows, max_threads<k_anterp<Rf, NC>>() / (kComp / NC) / tpb));
+      k_anterp<Rf, NC><<<dim3(nblk(pr.lev[l + 1].nb, n), nr), dim3(tpb, n, kComp / NC), fsm_bytes + sm * n, sf>>>(
+          P, pr.lev[l + 1].nb, pr.lev[l + 1].parent, pr.lev[l + 1].octant, static_cast<const C2<Rf>*>(pr.lev[l].G),
+          static_cast<const Rf*>(pr.lev[l].F), static_cast<const C2<Rf>*>(pr.lev[l].phase),
+          static_cast<C2<Rf>*>(pr.lev[l + 1].G), sl(l), sl(l + 1), fsh);
     });
   prof_mark(pr, 5, true, st);
   prof_mark(pr, 6, false, st);
