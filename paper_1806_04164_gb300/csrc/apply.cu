@@ -1664,7 +1664,7 @@ __global__ void k_gsgd(int P, int ntheta, const C2<Rf>* __restrict__ G, C2<Rf>* 
 // ([Ph][T], [3][Ph][T]) so that consecutive threads read consecutive
 // triangles, and the box's patterns are shared through the cache.  Over a sample pair (q, -q):
 // conj(X(q)) G(q) + X(q) G(-q) = Xr (G(q) + G(-q)) - i Xi (G(q) - G(-q)).
-// Adds to pot[t].
+// Writes pot[t].
 template <typename Rf, typename Rio>
 __global__ void __launch_bounds__(256) k_disagg(int64_t T, int P, int ntheta, const int32_t* __restrict__ leaf_of,
                                                 const C2<Rf>* __restrict__ PiR, const C2<Rf>* __restrict__ MR,
@@ -2477,11 +2477,11 @@ static double longest(const double* v, int64_t n) {
   return std::sqrt(r2);
 }
 
-// Phase of a centroid: 6 terms while it stays below 0.2 (bodies well below a
+// Phase of a centroid: 5 terms below 0.09 and 6 below 0.2 (bodies well below a
 // wavelength, the method's range; a fifth of a pair's operations less than
-// sincos; first omitted term 0.2^12 / 12! = 9e-18), else sincos (CT = 0).
-constexpr double kSmallPhase = 0.2;
-constexpr int kSmallTerms = 6;
+// sincos, a term 2 % of the adjoint map; first omitted terms 0.09^10 / 10! = 1e-17 and
+// 0.2^12 / 12! = 9e-18), else sincos (CT = 0).
+static int centroid_terms(double phase) { return phase < 0.09 ? 5 : phase < 0.2 ? 6 : 0; }
 
 template <int NT>
 __device__ __forceinline__ double horner(const double* c, double z) {
@@ -2599,7 +2599,7 @@ __device__ __forceinline__ void field_partial(const double (&S)[6], double* __re
 }
 
 // Far field: partial sums of F = sum_t int J exp(-i k0 rhat.r).  181
-// directions on 81,920 triangles: 3.32 ms; a block per direction with a sincos
+// directions on 81,920 triangles: 3.12 ms; a block per direction with a sincos
 // per quadrature point took 20.4 ms.
 template <typename Rio, int NT, int CT>
 __global__ void __launch_bounds__(128) k_farfield(int64_t T, int64_t ndir, int64_t nchunk, int64_t len,
@@ -2693,10 +2693,11 @@ static C2<Rio>* field_coef(Problem& pr, const void* x, cudaStream_t st) {
 template <bool ANY, typename F>
 static void with_field_terms(double kh, double phase, F f) {
   auto with_ct = [&](auto nt) {
-    if (phase < kSmallPhase)
-      f(nt, std::integral_constant<int, kSmallTerms>());
-    else
-      f(nt, std::integral_constant<int, 0>());
+    switch (centroid_terms(phase)) {
+      case 5: return f(nt, std::integral_constant<int, 5>());
+      case 6: return f(nt, std::integral_constant<int, 6>());
+      default: return f(nt, std::integral_constant<int, 0>());
+    }
   };
   if constexpr (ANY)
     if (field_terms(kh) == 0) return f(std::integral_constant<int, 0>(), std::integral_constant<int, 0>());
@@ -3017,7 +3018,7 @@ pie_status rhs_potential(Problem& pr, const double* khat, const double* pol, dou
 // triangle, a short series per quadrature point, and 1/R from one rsqrt (no
 // division).  With g_q = w_q e^{ik(R_q - R_c)} / R_q and F_q = g_q (ik - 1/R_q)/R_q
 // the sums over an orbit need sum g, sum_o s_o g_ok, sum F, sum_o s_o F_ok only:
-// J and r - r' are affine in s_o v_k.  1024 points, 20,480 triangles: 14.0 ms;
+// J and r - r' are affine in s_o v_k.  1024 points, 20,480 triangles: 13.3 ms;
 // 42.0 ms with a block per point, a sincos and five divisions per quadrature
 // point.
 template <int NT, int CT>
