@@ -116,7 +116,8 @@ typedef struct {
   double rel_residual;        /* ||b - Z x|| / ||b||, recomputed in FP64 */
   double seconds;             /* wall time of the solve */
   int32_t reorthogonalizations; /* Arnoldi steps that took a second Gram-Schmidt pass */
-  double product_seconds;     /* part of `seconds` in operator products (CUDA events) */
+  double product_seconds;     /* part of `seconds` in operator products (CUDA events), those of the
+                               * one or two steps enqueued past a cycle's end included */
 } pie_solve_stats;
 
 /* Message of the last failed call on this thread ("" if none). */
@@ -228,7 +229,8 @@ pie_status pie_apply_near_noalloc(pie_problem* pr, const void* x, void* y, int d
 
 /* Per-stage timing of products (CUDA events recorded on the apply stream
  * around each stage).  pie_profile_begin arms recording for the next
- * max_applies single-column products; pie_profile_end waits for them and
+ * max_applies single-column products (a solve's include the one or two it
+ * enqueues past a cycle's end); pie_profile_end waits for them and
  * writes the summed milliseconds of the PIE_NSTAGES stages to stage_ms
  * (host, may be NULL) and the number of recorded products to applies.
  * Stages, in order: 0 local coefficients, 1 near part, 2 leaf aggregation,
@@ -378,7 +380,8 @@ typedef struct {
   int32_t outer_products;       /* products with the outer operator, true residuals included */
   double rel_residual;          /* ||b - Z x|| / ||b|| with the outer operator, FP64 */
   double seconds;               /* wall time of the solve */
-  double inner_product_seconds; /* part of `seconds` in inner products (CUDA events) */
+  double inner_product_seconds; /* part of `seconds` in inner products (CUDA events), steps past a
+                                 * cycle's end included */
   double outer_product_seconds; /* part of `seconds` in outer products (CUDA events) */
 } pie_nested_stats;
 

@@ -826,15 +826,6 @@ static pie_status near_fixed_prepare() {
   return s;
 }
 
-pie_status near_prepare(const Problem& pr) {
-  switch (pr.par.precision) {
-    case PIE_FP64: return near_fixed_prepare();
-    case PIE_FP32: return near_float_prepare<float, false>();
-    case PIE_FP32H: return near_float_prepare<float, true>();
-    default: return near_float_prepare<double, false>();
-  }
-}
-
 // Launch of the fixed-point near part for nrhs columns on a grid of at most
 // max_blocks (0: no bound).  lean: the kernel of fewer registers.
 static void near_fixed(const Problem& pr, const cd* coef, cd* pot, int nrhs, int64_t max_blocks, bool lean,
@@ -1904,6 +1895,37 @@ static inline MomScale mom_scale(const Problem& pr) {
 void prof_mark(Problem& pr, int stage, bool end, cudaStream_t st) {
   if (pr.prof_n >= pr.prof_cap) return;
   cudaEventRecord(pr.prof_ev[(size_t(pr.prof_n) * kStages + stage) * 2 + (end ? 1 : 0)], st);
+}
+
+// Asks the far kernels for their limits, once per process (set-up).
+template <typename Rf>
+static void far_prepare() {
+  max_threads<k_agg<Rf>>();
+  max_threads<k_agg_split<Rf, 1>>();
+  max_threads<k_agg_split<Rf, kComp>>();
+  max_threads<k_interp<Rf, 1>>();
+  max_threads<k_interp<Rf, kComp>>();
+  max_threads<k_anterp<Rf, 1>>();
+  max_threads<k_anterp<Rf, kComp>>();
+  max_threads<k_trans<Rf, 1>>();
+  max_threads<k_trans<Rf, kComp>>();
+  if constexpr (sizeof(Rf) == 4) {
+    max_threads<k_trans_split<Rf, 1>>();
+    max_threads<k_trans_split<Rf, kComp>>();
+  }
+}
+
+pie_status product_prepare(const Problem& pr) {
+  if (pr.far_f32())
+    far_prepare<float>();
+  else
+    far_prepare<double>();
+  switch (pr.par.precision) {
+    case PIE_FP64: return near_fixed_prepare();
+    case PIE_FP32: return near_float_prepare<float, false>();
+    case PIE_FP32H: return near_float_prepare<float, true>();
+    default: return near_float_prepare<double, false>();
+  }
 }
 
 template <typename Rm, typename Rf, typename Rio, bool H16 = false>

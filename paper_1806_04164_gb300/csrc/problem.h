@@ -104,7 +104,7 @@ struct Problem {
   void* coef = nullptr;          // [max_nrhs][T][6] complex (io precision)
   void* coef32 = nullptr;        // [T][6] complex float copy for the MIXED near part
   void* gsgd = nullptr;          // 2 x [max_nrhs][nleaf][5][P/2] antipodal sum / difference leaf patterns
-  size_t gsgd_bytes = 0;         // (the field maps use the same buffer as scratch)
+  size_t gsgd_bytes = 0;         // (double far part; scratch of the field maps in every precision)
   void* vec = nullptr;           // [N] complex (io precision), adjoint scratch
   void* vec2 = nullptr;          // [N] complex (io precision), single-layer scratch
   void* pot = nullptr;           // [max_nrhs][T][6] far-part potentials (near part too when pot2 is unused)
@@ -142,8 +142,9 @@ pie_status apply_one(Problem& pr, const void* x, void* y, cudaStream_t st, const
 pie_status apply_batch(Problem& pr, const void* x, void* y, int nrhs, cudaStream_t st, const double* scale = nullptr);
 // x, y: N x nrhs columns, passes of tune.rhs_chunk columns
 pie_status apply_cols(Problem& pr, const void* x, void* y, int nrhs, cudaStream_t st);
-// shared-memory limits of the near kernels on the current device (set-up; not inside a stream capture)
-pie_status near_prepare(const Problem& pr);
+// shared-memory limits of the near kernels on the current device and block sizes of the far
+// kernels (set-up; not inside a stream capture)
+pie_status product_prepare(const Problem& pr);
 // records the start (end = false) or end of stage `stage` of the current apply when profiling
 void prof_mark(Problem& pr, int stage, bool end, cudaStream_t st);
 pie_status apply_near_one(Problem& pr, const void* x, void* y, cudaStream_t st);

@@ -753,7 +753,8 @@ static pie_status arnoldi_cycle(Ctx& c, C2<B>* V, Cycle& cy, double beta, double
   breakdown = false;
   // Steps are enqueued ahead of the one whose coefficients the host waits for
   // (5120 triangles: 104 us of every inner step were round trips).  A step past
-  // the cycle's end is thrown away, so fewer run ahead where a product is long, and
+  // the cycle's end is thrown away (after a breakdown it runs on vectors that are not
+  // finite, which nothing reads), so fewer run ahead where a product is long, and
   // none where an estimate is likely to end the cycle between two products.
   const int ahead = N < 200000 ? 2 : hint_every > 0 ? 0 : 1;
   unsigned seq[kSlots];

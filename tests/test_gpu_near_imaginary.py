@@ -35,3 +35,22 @@ def test_parts_of_the_near_product_keep_their_own_accuracy(shape, k):
             for f in (np.real, np.imag):
                 a, b = f(y[part]), f(yo[part])
                 assert np.linalg.norm(a - b) <= 1e-13 * np.linalg.norm(b), (part, f)
+
+
+@pytest.mark.parametrize("mesh,levels,side", [("sphere", 4, 2.0), ("cube", 3, 1.2)])
+def test_both_kernels_give_the_same_bits(mesh, levels, side):
+    """Beside a far part of its own length the near part runs in two passes over a
+    row, alone (overlap off) and beside a short far part in one: exact sums, so the
+    order and the pass make no difference."""
+    import torch
+    from tests._lib import ensure_built
+    ensure_built()
+    import paper_1806_04164_gb300 as pg
+    pr = pg.Problem(pg.Mesh(*(pi.icosphere(3) if mesh == "sphere" else pi.cube(6))), 1e-3, levels, root_side=side,
+                    max_nrhs=3)
+    x = torch.from_numpy(np.stack([pi.complex_normal(pr.N, s) for s in (1, 2, 3)])).cuda()
+    y = pr.apply(x)
+    pr.tuning = dict(overlap=0)
+    assert torch.equal(pr.apply(x), y)
+    pr.tuning = dict(overlap=1, near_ctas_per_sm=0)
+    assert torch.equal(pr.apply(x), y)
