@@ -98,8 +98,9 @@ static void free_problem(Problem& pr) {
   if (pr.ev_fork) cudaEventDestroy(pr.ev_fork);
   if (pr.ev_join) cudaEventDestroy(pr.ev_join);
   if (pr.ev_far) cudaEventDestroy(pr.ev_far);
+  if (pr.ev_field) cudaEventDestroy(pr.ev_field);
   pr.side = pr.far = nullptr;
-  pr.ev_fork = pr.ev_join = pr.ev_far = nullptr;
+  pr.ev_fork = pr.ev_join = pr.ev_far = pr.ev_field = nullptr;
   for (void* p : pr.allocs) cudaFree(p);
   pr.allocs.clear();
 }

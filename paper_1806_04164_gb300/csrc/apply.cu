@@ -2572,18 +2572,24 @@ static void field_chunks(const Problem& pr, int64_t* nchunk, int64_t* len) {
   *nchunk = (pr.T + *len - 1) / *len;
 }
 
-// Scratch of one field call: half of the leaf sum / difference patterns, which
-// only live inside a product (the adjoint map takes the upper half: it shares
-// no other buffer with the maps), or a stream-ordered allocation where that is
-// too small.
+// Scratch of one field call: the leaf sum / difference patterns, which only
+// live inside a product, or a stream-ordered allocation where they are too
+// small.  The maps and the adjoint map share no other buffer, so a call waits on
+// the device for the last one that used the patterns, whatever its stream (not
+// inside a stream capture, whose launches are the caller's to order).
 struct FieldScratch {
   void* p = nullptr;
   cudaStream_t st;
+  cudaEvent_t done = nullptr;
   bool own = false;
-  FieldScratch(Problem& pr, size_t bytes, cudaStream_t s_, pie_status& s, bool adjoint = false) : st(s_) {
-    const size_t half = pr.gsgd_bytes / 512 * 256;
-    if (bytes <= half) {
-      p = static_cast<char*>(pr.gsgd) + (adjoint ? half : 0);
+  FieldScratch(Problem& pr, size_t bytes, cudaStream_t s_, pie_status& s) : st(s_) {
+    if (bytes <= pr.gsgd_bytes) {
+      p = pr.gsgd;
+      cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+      s = cuda_check(cudaStreamIsCapturing(st, &cap), "capture status");
+      if (s != PIE_OK || cap != cudaStreamCaptureStatusNone) return;
+      done = pr.ev_field;
+      s = cuda_check(cudaStreamWaitEvent(st, done, 0), "field scratch");
       return;
     }
     s = cuda_check(cudaMallocAsync(&p, bytes, st), "field scratch");
@@ -2591,6 +2597,7 @@ struct FieldScratch {
   }
   ~FieldScratch() {
     if (own) cudaFreeAsync(p, st);
+    if (done) cudaEventRecord(done, st);
   }
 };
 
@@ -2947,8 +2954,7 @@ static pie_status farfield_adjoint_t(Problem& pr, const double* rhat, int64_t nd
   const int64_t most = std::min((int64_t(pr.nsm) * kAdjWarps + warps - 1) / warps, (ndir + 7) / 8);
   const int64_t len = ((ndir + most - 1) / most + 3) / 4 * 4, nchunk = (ndir + len - 1) / len;
   pie_status s = PIE_OK;
-  FieldScratch scratch(pr, sizeof(double) * (3 * size_t(ndir) + (nchunk > 1 ? 8 * size_t(pr.T) * nchunk : 0)), st, s,
-                       true);
+  FieldScratch scratch(pr, sizeof(double) * (3 * size_t(ndir) + (nchunk > 1 ? 8 * size_t(pr.T) * nchunk : 0)), st, s);
   if (s != PIE_OK) return s;
   double* d_rhat = static_cast<double*>(scratch.p);
   double* partial = d_rhat + 3 * ndir;

@@ -116,6 +116,7 @@ struct Problem {
   // near part's many blocks instead of queueing behind them
   cudaStream_t side = nullptr, far = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_far = nullptr;
+  cudaEvent_t ev_field = nullptr;  // last use of gsgd by a field map
   int nsm = 0;                   // SMs of the device
   int device = 0;                // the device the problem was built on (current at pie_problem_create)
   void* noalloc_scratch = nullptr;  // device address of the fixed scratch of pie_apply_near_noalloc

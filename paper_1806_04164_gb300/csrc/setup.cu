@@ -1109,6 +1109,7 @@ static pie_status setup_t(Problem& pr, cudaStream_t st) {
   if ((s = cuda_check(cudaEventCreateWithFlags(&pr.ev_fork, cudaEventDisableTiming), "event")) != PIE_OK) return s;
   if ((s = cuda_check(cudaEventCreateWithFlags(&pr.ev_join, cudaEventDisableTiming), "event")) != PIE_OK) return s;
   if ((s = cuda_check(cudaEventCreateWithFlags(&pr.ev_far, cudaEventDisableTiming), "event")) != PIE_OK) return s;
+  if ((s = cuda_check(cudaEventCreateWithFlags(&pr.ev_field, cudaEventDisableTiming), "event")) != PIE_OK) return s;
   pr.tune = pie_tuning{1, 2, pr.par.max_nrhs, 0, 0, 0};
   if ((s = product_prepare(pr)) != PIE_OK) return s;
   return cuda_check(cudaStreamSynchronize(st), "setup");
