@@ -615,7 +615,7 @@ __device__ __noinline__ double near_row_double(const FixedNear& nf, int64_t nnz,
   return out;
 }
 
-// PARTS: moments' parts of a pass over the row.  Both at once take 48 sums and 164
+// PARTS: moments' parts of a pass over the row.  Both at once take 48 sums and 166
 // registers, one after the other 24 and 128 and the coefficients from shared memory
 // twice: 81,920 triangles alone 0.68 ms, 0.72, but beside the far part, whose
 // kernels the registers hold up, the product 2.97 ms, 2.88.  BLOCKS: blocks of an SM that
@@ -831,8 +831,8 @@ static pie_status near_fixed_prepare() {
 static void near_fixed(const Problem& pr, const cd* coef, cd* pot, int nrhs, int64_t max_blocks, bool lean,
                        cudaStream_t st) {
   const FixedNear nf{static_cast<const int4*>(pr.mom), static_cast<const FixedRow*>(pr.fixed_row), pr.fixed_delta};
-  // shares per box: the least rounds of three blocks an SM, staging (about 1/50
-  // of a box's rows) once a share; at least a test triangle for each warp.  Boxes
+  // shares per box: the least rounds of three blocks an SM over all columns, staging
+  // (about 1/50 of a box's rows) once a share; at least a test triangle for each warp.  Boxes
   // are uneven, so up to 8 % more by this count for finer shares, while a warp has
   // three rows (alone: cube of 24,576 triangles 799 -> 695 us, ellipsoid of 32,768
   // 2870 -> 1400; finer still, spheres lose 10 %)
@@ -841,7 +841,7 @@ static void near_fixed(const Problem& pr, const cd* coef, cd* pot, int nrhs, int
   int nsplit = 1;
   double best = 0, costs[17];
   for (int64_t s = 1; s <= most; ++s) {
-    const double cost = double((pr.nleaf * s + slots - 1) / slots) * (1.0 / double(s) + 0.02);
+    const double cost = double((pr.nleaf * nrhs * s + slots - 1) / slots) * (1.0 / double(s) + 0.02);
     if (s == 1 || cost < best) best = cost, nsplit = int(s);
     costs[s] = cost;
   }
