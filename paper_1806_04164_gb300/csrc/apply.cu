@@ -2628,7 +2628,7 @@ __device__ __forceinline__ void field_partial(const double (&S)[6], double* __re
 }
 
 // Far field: partial sums of F = sum_t int J exp(-i k0 rhat.r).  181
-// directions on 81,920 triangles: 3.12 ms; a block per direction with a sincos
+// directions on 81,920 triangles: 3.06 ms; a block per direction with a sincos
 // per quadrature point took 20.4 ms.
 template <typename Rio, int NT, int CT>
 __global__ void __launch_bounds__(128) k_farfield(int64_t T, int64_t ndir, int64_t nchunk, int64_t len,
@@ -3046,7 +3046,7 @@ pie_status rhs_potential(Problem& pr, const double* khat, const double* pol, dou
 // triangle, a short series per quadrature point, and 1/R from one rsqrt (no
 // division).  With g_q = w_q e^{ik(R_q - R_c)} / R_q and F_q = g_q (ik - 1/R_q)/R_q
 // the sums over an orbit need sum g, sum_o s_o g_ok, sum F, sum_o s_o F_ok only:
-// J and r - r' are affine in s_o v_k.  1024 points, 20,480 triangles: 13.3 ms;
+// J and r - r' are affine in s_o v_k.  1024 points, 20,480 triangles: 13.2 ms;
 // 42.0 ms with a block per point, a sincos and five divisions per quadrature
 // point.
 template <int NT, int CT>
